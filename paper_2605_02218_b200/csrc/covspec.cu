@@ -68,7 +68,8 @@ struct Plan {
   int tile_rows = 128;                        // rows of a subspace-block tile: 64 when that still gives every tile a CTA
   int tile_ctas = 0, servers = 0;             // CTAs of the subspace kernel that carry tiles / that only factor
   int pow_grid = 0;                           // CTAs of the power step
-  std::vector<int> sched;                     // [pow_grid + 1] offsets + item lists (longest first)
+  std::vector<int> sched;                     // [pow_grid + 1] offsets + item lists (longest first) + places (see FusedParams)
+  bool one_request_ctas = false;              // no CTA of the subspace kernel carries tiles of two requests
   long long total_vis = 0, total_txt = 0, total_keep = 0, total_presel = 0;
   bool valid = false;
 };
@@ -290,7 +291,7 @@ int get_plan(covspec_ctx* ctx, const covspec_problem* p, cudaStream_t stream) {
   pl.tile_ctas = std::min(pl.n_ptiles, ctx->num_sms);
   pl.servers = (pl.n_ptiles > 0 && pl.n_ptiles + pl.n_stage2 <= ctx->num_sms) ? pl.n_stage2 : 0;
   pl.pow_grid = pl.tile_ctas + pl.servers;
-  pl.sched.assign((size_t)pl.pow_grid + 1 + pl.n_ptiles, 0);
+  pl.sched.assign((size_t)2 * pl.pow_grid + 1 + pl.n_ptiles, 0);
   if (pl.n_ptiles > 0) {
     auto tile_cost = [&](const ReqPlan& r, int t) {
       int rows = std::min(pl.tile_rows, r.m - t * pl.tile_rows);
@@ -304,7 +305,7 @@ int get_plan(covspec_ctx* ctx, const covspec_problem* p, cudaStream_t stream) {
     // groups per request (sum = CTAs) minimises the largest step time: the smallest feasible bound
     // is found among the step times every request can have; CTAs that are left then go, one at a
     // time, to the request that is slowest at that moment.  Requests are never mixed inside a group.
-    struct Group { double cost; int first, count, req; };
+    struct Group { double cost; int first, count, req, index, of; };
     struct Share { int req, nt, g; };
     std::vector<Group> groups;
     std::vector<Share> shares;
@@ -364,10 +365,13 @@ int get_plan(covspec_ctx* ctx, const covspec_problem* p, cudaStream_t stream) {
         ++shares[worst].g;
       }
     }
-    for (const Share& sh : shares)
+    for (const Share& sh : shares) {
+      int index = 0;
       split(sh, sh.g, [&](int t, int count, double cost) {
-        groups.push_back(Group{cost, pl.req[sh.req].ptile_off + t, count, sh.req});
+        groups.push_back(Group{cost, pl.req[sh.req].ptile_off + t, count, sh.req, index++, sh.g});
       });
+    }
+    pl.one_request_ctas = (int)groups.size() <= pl.tile_ctas;
     std::stable_sort(groups.begin(), groups.end(), [](const Group& a, const Group& b2) { return a.cost > b2.cost; });
     std::vector<double> load(pl.tile_ctas, 0.0);
     std::vector<std::vector<int>> lists(pl.tile_ctas);
@@ -375,6 +379,7 @@ int get_plan(covspec_ctx* ctx, const covspec_problem* p, cudaStream_t stream) {
       int best = 0;
       for (int c = 1; c < pl.tile_ctas; ++c) if (load[c] < load[best]) best = c;
       load[best] += g.cost;
+      pl.sched[(size_t)pl.pow_grid + 1 + pl.n_ptiles + best] = g.index | g.of << 16;
       for (int t = 0; t < g.count; ++t) lists[best].push_back(g.first + t);
     }
     // more groups than CTAs is guaranteed to leave no CTA empty only if groups >= CTAs
@@ -798,7 +803,7 @@ int select_impl(covspec_ctx* ctx, const covspec_problem* p, const float* s_fused
     sub::FusedParams fp{};
     fp.plan = ctx->d_plan; fp.batch = B; fp.n_items = pl.n_ptiles; fp.sched = ctx->d_sched;
     fp.tile_rows = pl.tile_rows;
-    fp.spread_sum = pl.n_ptiles <= pl.tile_ctas ? 1 : 0;     // one tile per CTA (see the schedule above)
+    fp.spread_sum = pl.one_request_ctas ? 1 : 0;
     fp.n_tile_ctas = pl.tile_ctas; fp.n_servers = pl.servers;
     fp.steps = cfg.eig_iters + 1;
     fp.lbuf = ctx->Lbuf;
@@ -935,7 +940,7 @@ int covspec_prune_init(const covspec_config* cfg, covspec_ctx** out) {
   long long o_status = carve(256);
   long long o_plan = carve(sizeof(ReqPlan) * c.max_batch);
   long long o_tab = carve(sizeof(GemmProb) * (long long)T_COUNT * c.max_batch);
-  long long sched_ints = 1024 + ctx->cap_ptiles;   // offsets of up to 1023 CTAs + one entry per tile
+  long long sched_ints = 1024 + ctx->cap_ptiles;   // offsets and places of up to 511 CTAs + one entry per tile
   long long o_sched = carve(4 * sched_ints);
   long long o_qn = carve(4ll * c.max_total_txt * ctx->P);
   long long o_kp = carve(4ll * ctx->kp_rows * ctx->P);

@@ -113,6 +113,90 @@ __device__ __forceinline__ bool jacobi_sweeps(float* C, int ldc, int w, float s1
   return converged;
 }
 
+// The same rotations for w <= 32 (the usual window), same pairs in the same order and the same sums in
+// the same order, by one warp: two lanes per pair, the rows of a column dealt over them as the four
+// partial sums above want it (lane h adds up the rows 4 q + h, then the rows 4 q + h + 2), so that one
+// shuffle joins the sums and no barrier separates the rounds.  The search ends as soon as np - 1
+// consecutive rounds (every pair once) have passed without a rotation, wherever in a sweep that
+// happens.  A round is a chain of shared load, eight-term sums, shuffle, threshold and, where a pair
+// rotates, root, quotient, reciprocal root and store: w = 32 took 640 cycles a round on two warps with a
+// barrier per round.
+__host__ __device__ __forceinline__ int ritz_row(int row) {      // place of a row inside its column
+  return (row & 1) * 16 + (row & 2) * 4 + (row >> 2);
+}
+constexpr int kRitzLd32 = 36;            // column stride: the columns of neighbouring pairs hit distinct banks
+// c_off: place of C in the kernel's shared memory (floats from the base).  Out of line: see the rehearsal in
+// subspace_kernel.
+__device__ __noinline__ bool jacobi_warp32(int c_off, int w, float s1, int max_sweeps) {
+  float* C = reinterpret_cast<float*>(sub::pow_smem()) + c_off;
+  const int lane = threadIdx.x & 31, g = lane >> 1, h = lane & 1;
+  const int np = (w + 1) & ~1, half = np >> 1;
+  const float abs2 = (2e-5f * s1) * (2e-5f * s1);
+  if (w < 2) return true;
+  const int limit = max_sweeps * (np - 1);
+  int quiet = 0;                         // rounds since the last rotation
+  // columns of this group's pair, one step of the round-robin further each round: ra runs upwards and rb
+  // with it through 0 .. np - 2 (their sum is 2 round modulo np - 1), column np - 1 stays with group 0
+  int ra = g, rb = g == 0 ? np - 1 : np - 1 - g;
+  for (int it = 0; it < limit; ++it) {
+    const int a = min(ra, rb), b = max(ra, rb);
+    const bool active = g < half && b < w;
+    float4* ca = reinterpret_cast<float4*>(C + (active ? a : 0) * kRitzLd32 + h * 16);
+    float4* cb = reinterpret_cast<float4*>(C + (active ? b : 0) * kRitzLd32 + h * 16);
+    float xa[16], xb[16];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float4 u = ca[q], v = cb[q];
+      xa[4 * q] = u.x; xa[4 * q + 1] = u.y; xa[4 * q + 2] = u.z; xa[4 * q + 3] = u.w;
+      xb[4 * q] = v.x; xb[4 * q + 1] = v.y; xb[4 * q + 2] = v.z; xb[4 * q + 3] = v.w;
+    }
+    float al = 0.f, be = 0.f, ga = 0.f, al2 = 0.f, be2 = 0.f, ga2 = 0.f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      al += xa[q] * xa[q]; be += xb[q] * xb[q]; ga += xa[q] * xb[q];
+      al2 += xa[q + 8] * xa[q + 8]; be2 += xb[q + 8] * xb[q + 8]; ga2 += xa[q + 8] * xb[q + 8];
+    }
+    al += al2; be += be2; ga += ga2;
+    al += __shfl_xor_sync(0xffffffffu, al, 1);
+    be += __shfl_xor_sync(0xffffffffu, be, 1);
+    ga += __shfl_xor_sync(0xffffffffu, ga, 1);
+    if (++ra == np - 1) ra = 0;
+    if (g != 0 && ++rb == np - 1) rb = 0;
+    const float g2 = ga * ga;
+    const float thr2 = fmaxf(1e-12f * al * be, abs2 * fminf(al, be));
+    const bool rotate = active && g2 > thr2 && g2 > 1e-37f;
+    if (__any_sync(0xffffffffu, rotate)) {
+      // tan of the rotation angle: t = sign(d g) 2|g| / (|d| + sqrt(d^2 + 4 g^2)), d = |b|^2 - |a|^2
+      // (hardware root, quotient and reciprocal root, a few units in the last place each: the
+      // rotation is orthogonal to float32 accuracy for whatever t comes out)
+      float d = be - al, r, t, c;
+      asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d * d + 4.f * g2));
+      asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(t) : "f"(2.f * ga), "f"(fabsf(d) + r));
+      if (d < 0.f) t = -t;
+      asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(c) : "f"(t * t + 1.f));
+      const float sn = t * c;
+      if (rotate) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          float ya[4], yb[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            ya[e] = c * xa[4 * q + e] - sn * xb[4 * q + e];
+            yb[e] = sn * xa[4 * q + e] + c * xb[4 * q + e];
+          }
+          ca[q] = make_float4(ya[0], ya[1], ya[2], ya[3]);
+          cb[q] = make_float4(yb[0], yb[1], yb[2], yb[3]);
+        }
+      }
+      __syncwarp();
+      quiet = 0;
+    } else if (++quiet >= np - 1) {
+      return true;
+    }
+  }
+  return false;
+}
+
 // Column stride of the window factor in shared memory: >= w and congruent to 4 modulo 32, so that
 // the eight 4-lane groups of a warp, which hold consecutive columns, hit distinct banks.
 __host__ __device__ inline int ritz_ldc(int w) { return (w + 27) / 32 * 32 + 4; }

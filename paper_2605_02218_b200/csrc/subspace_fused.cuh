@@ -16,8 +16,8 @@
 //               factor, reads "is this the last step?" with it, and the producer and MMA roles, which
 //               only ask "is step s skipped?", can first be affected at step k + 2, whose start
 //               every tile's arrival of step k + 1 precedes
-//   summed[b]   tiles of request b that have added up their slice of the partial Gram matrices of a
-//               step (only when every CTA holds exactly one tile, see spread_sum)
+//   summed[b]   CTAs of request b that have added up their slice of the partial Gram matrices of a
+//               step (CTAs of request b, only when every CTA holds tiles of one request, see spread_sum)
 // With SMs to spare the grid carries one more CTA per request that holds no tile and only factors for
 // that request (n_servers); otherwise
 // the tile that makes arrive[b] reach tiles(b) * (k + 1) (an atomic ticket; nobody waits for it to be
@@ -43,19 +43,22 @@ struct FusedParams {
   int batch;
   int n_items;              // row tiles over all stage-2 requests
   int tile_rows;            // rows of a tile: 128, or 64 (the MMA still computes 128 rows; the upper half is dropped)
-  const int* sched;         // [gridDim.x + 1] offsets, then the item lists of every CTA
+  const int* sched;         // [gridDim.x + 1] offsets, the item lists of every CTA, [gridDim.x] place among the CTAs of the
+                            // request: index | count << 16
   int steps;                // multiplications by G (eig_iters + 1, >= 2)
   float* lbuf;              // [batch][kLbufStride] triangular factor + reciprocal diagonal
   __nv_bfloat16* y_hi[2];   // plane buffers: step k reads [k & 1], writes [(k & 1) ^ 1]
   __nv_bfloat16* y_lo[2];
   int ld;
-  float* yf[2];             // [sum M_b, kPMax], window columns only: the orthonormal basis Q of the block
-                            // before the last multiplication, and the block after it (Eq. 15)
+  float* yf[2];             // [sum M_b * kPMax], window columns only: the orthonormal basis Q of the block
+                            // before the last multiplication, and the block after it (Eq. 15); the tile that
+                            // starts at row i owns the floats from i * kPMax on, as [window column][row of the tile]
   double* partial;          // [tiles][kTileDoubles], see tile_offset
   float* ub;                // [batch][kPMax * kPMax] Ritz vectors of the discarded pairs
   float* energy;            // [sum M_b] (out)
   unsigned* sync;           // [batch][kSyncStride] counters (zero on entry), then the abort word
-  int spread_sum;           // every CTA holds exactly one tile: the tiles of a request sum the partial matrices together
+  int spread_sum;           // every CTA holds tiles of one request only: the CTAs of a request can add up the partial
+                            // matrices together (the schedule then carries every CTA's place among them)
   int n_tile_ctas;          // CTAs that carry tiles: blockIdx.x < n_tile_ctas
   int n_servers;            // CTAs after those, one per stage-2 request, that only factor (0: the last tile to
                             // finish a step factors)
@@ -181,21 +184,24 @@ __device__ __forceinline__ void team_sum_partials(double* T, const double* pbase
   }
 }
 
-// 1 / sqrt(x) for x > 0 without a range test on the pivot chain: x = m 4^k with m in [1, 4) (integer
-// operations on the exponent field), float32 estimate of 1 / sqrt(m) refined in float32 and by one
-// Newton step in float64, then scaled by 2^-k.  Subnormal or non-finite x give a meaningless value;
-// the caller clamps pivots to a positive floor first.
-__device__ __forceinline__ double rsqrt_f64_scaled(double x) {
+// 1 / sqrt(x) for x > 0: float32 estimate of 1 / sqrt(x) refined in float32 and by one Newton step in
+// float64.  kScale: x = m 4^k with m in [1, 4) first (integer operations on the exponent field) and the
+// result scaled by 2^-k, for pivots beyond the float32 range; the result is the same, bit for bit, where
+// both forms apply (every operation scales by a power of two).  Subnormal or non-finite x give a
+// meaningless value; the caller clamps pivots to a positive floor.
+template <bool kScale>
+__device__ __forceinline__ double rsqrt_f64(double x) {
   const int hi = __double2hiint(x), lo = __double2loint(x);
-  const int k = ((((hi >> 20) & 0x7ff) - 1023)) >> 1;
-  const double m = __hiloint2double(hi - (k << 21), lo);
+  const int k = kScale ? ((((hi >> 20) & 0x7ff) - 1023)) >> 1 : 0;
+  const double m = kScale ? __hiloint2double(hi - (k << 21), lo) : x;
   const float xf = (float)m;
-  float yf = rsqrtf(xf);
+  float yf;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(xf));
   yf = yf * (1.5f - 0.5f * xf * yf * yf);
   double y = (double)yf;
   const double e = fma(-0.5 * m * y, y, 0.5);
   y = fma(y, e, y);
-  return __hiloint2double(__double2hiint(y) - (k << 20), __double2loint(y));
+  return kScale ? __hiloint2double(__double2hiint(y) - (k << 20), __double2loint(y)) : y;
 }
 
 // Diagonal 8 x 8 tile, factored by one thread in registers: measured faster than a lane-per-row
@@ -204,23 +210,37 @@ __device__ __forceinline__ double rsqrt_f64_scaled(double x) {
 // l22 = sqrt(de / al) with de = al ga - be^2, so the two reciprocal square roots (of al and de) run
 // side by side instead of one after the other.  The chain of dependent pivots is the critical path
 // of the whole factorisation.  A pivot below 1e-12 of its original diagonal entry (a numerically
-// dependent direction) is clamped there; the next multiplication by G restores the direction.
+// dependent direction) is clamped there; the next multiplication by G restores the direction.  The
+// tests for that, and for pivots whose reciprocal root needs the scaled form, stay off the chain:
+// the roots are taken first and taken again where a test fails.
 __device__ __forceinline__ void factor_diag_thread(double* D, const double* d0, double* rd) {
-  double a[8][8];
+  double a[8][8], fl[8];
 #pragma unroll
-  for (int l = 0; l < 8; ++l)
+  for (int l = 0; l < 8; ++l) {
 #pragma unroll
-    for (int m = 0; m <= l; ++m) a[l][m] = D[l * 8 + m];
+    for (int m = 0; m <= l; m += 2) {
+      const double2 v = *reinterpret_cast<const double2*>(D + l * 8 + m);
+      a[l][m] = v.x;
+      if (m < l) a[l][m + 1] = v.y;
+    }
+    fl[l] = 1e-12 * d0[l];
+  }
 #pragma unroll
   for (int c = 0; c < 8; c += 2) {
-    const double f0 = 1e-12 * d0[c], f1 = 1e-12 * d0[c + 1];
     double al = a[c][c];
-    if (!(al > f0)) al = f0 > 0.0 ? f0 : 1.0;
     const double be = a[c + 1][c], ga = a[c + 1][c + 1];
     double de = fma(al, ga, -be * be);                  // al * (second pivot)
-    const double fd = f1 * al;
-    if (!(de > fd)) de = fd > 0.0 ? fd : al;
-    const double ra = rsqrt_f64_scaled(al), rq = rsqrt_f64_scaled(de);
+    double ra = rsqrt_f64<false>(al), rq = rsqrt_f64<false>(de);
+    // 2^-100 < al, de < 2^100 by the exponent fields (a negative value's field is out of range too)
+    const unsigned ea = (unsigned)__double2hiint(al) - (923u << 20), ed = (unsigned)__double2hiint(de) - (923u << 20);
+    if (!(al > fl[c]) || !(de > fl[c + 1] * al) || ea >= (200u << 20) || ed >= (200u << 20)) {
+      if (!(al > fl[c])) al = fl[c] > 0.0 ? fl[c] : 1.0;
+      de = fma(al, ga, -be * be);
+      const double fd = fl[c + 1] * al;
+      if (!(de > fd)) de = fd > 0.0 ? fd : al;
+      ra = rsqrt_f64<true>(al);
+      rq = rsqrt_f64<true>(de);
+    }
     const double l11 = al * ra, l21 = be * ra, inv22 = rq * l11, l22 = de * rq * ra;
     a[c][c] = l11; a[c + 1][c] = l21; a[c + 1][c + 1] = l22;
     rd[c] = ra; rd[c + 1] = inv22;
@@ -238,30 +258,106 @@ __device__ __forceinline__ void factor_diag_thread(double* D, const double* d0, 
 #pragma unroll
   for (int l = 0; l < 8; ++l)
 #pragma unroll
-    for (int m = 0; m <= l; ++m) D[l * 8 + m] = a[l][m];
+    for (int m = 0; m <= l; m += 2)
+      if (m < l) *reinterpret_cast<double2*>(D + l * 8 + m) = make_double2(a[l][m], a[l][m + 1]);
+      else D[l * 8 + m] = a[l][m];
 }
 
-// The matrix is already in T (tile layout, see tile_offset); entries beyond n inside the last row of
-// tiles are replaced by the identity here.
-//   store(I, J, tile, rd)   receives the factor tile (I, J) (64 doubles, row-major) and the array of
-//                           reciprocal diagonal entries; called by a whole warp
-// kEarlyStore: warp 4 (idle in the panel loop) hands panel J - 1 to store() during iteration J (the
-// panel is final since the last barrier) instead of leaving all tiles to the end; the team then has
-// at least five warps.
-template <bool kEarlyStore = false, typename Store, typename Sync>
-__device__ __forceinline__ void cholesky_blocked_team(int n, double* T, double* aux, int tid, int nthreads,
-                                                      Store store, Sync sync) {
-  const int lane = tid & 31, warp = tid >> 5, nw = nthreads >> 5;
-  const int nb = (n + 7) >> 3, ntile = nb * (nb + 1) / 2;
+constexpr int kEpiThreads = 256;         // warps 0-7
+
+// The part behind the ring: the triangular factor, its reciprocal diagonal (a scratch array of p floats
+// while a factor is being made), barriers, then single words.
+struct PowTail {
+  float *lt, *dinv;
+  uint64_t* bars;
+  uint32_t* tmem_slot;
+  volatile int *abort_flag, *s_word;     // s_word: [2] broadcast slots of the epilogue
+  int* s_flag;                           // Jacobi rotation flag
+  float* s_scale;
+};
+__device__ __forceinline__ PowTail pow_tail() {
+  PowTail t;
+  t.lt = reinterpret_cast<float*>(pow_smem() + kPowRegion);
+  t.dinv = t.lt + kLtFloats;
+  t.bars = reinterpret_cast<uint64_t*>(t.lt + kLbufStride);
+  t.tmem_slot = reinterpret_cast<uint32_t*>(t.bars + 8);
+  t.abort_flag = reinterpret_cast<volatile int*>(t.tmem_slot + 1);
+  t.s_word = reinterpret_cast<volatile int*>(t.tmem_slot + 2);
+  t.s_flag = reinterpret_cast<int*>(t.tmem_slot + 4);
+  t.s_scale = reinterpret_cast<float*>(t.tmem_slot + 6);
+  return t;
+}
+
+// float64 Gram matrix of the staged block (columns coff .. coff + 8 nb8 - 1, 16 nslab rows) on the FP64
+// tensor cores, by the eight epilogue warps.  A warp takes 16 x 16 blocks of the lower triangle (dealt
+// round-robin, `first` = the warp's place in the deal) and runs through all rows of a block before it
+// starts the next: the four fragments of four rows (two per block row / column, one shared-memory word
+// and one conversion per lane each) feed four instructions, so that nothing is staged and the warps
+// never wait for one another.  Rows enter in ascending groups of four, whatever the split.  Bound by the
+// FP64 pipe (16 cycles an instruction and scheduler): p = 144, 128 rows 68 -> 29 k cycles against
+// float64 slabs in shared memory with a barrier every 16 rows; p = 48, 64 rows 12.5 -> 3 k.
+constexpr int kEpiWarps = kEpiThreads / 32;
+__device__ __forceinline__ void gram_tile_f64(const float* xs, int coff, int nb8, int nslab, int first, int lane,
+                                              double* __restrict__ out) {
+  const int fr = lane >> 2, fk = lane & 3;
+  const int nb = (nb8 + 1) >> 1, nblk = nb * (nb + 1) / 2, t0 = coff >> 3;
+  for (int q = first; q < nblk; q += kEpiWarps) {
+    int bi, bj;
+    tri_decode(q, bi, bj);
+    // an odd number of tiles leaves half of the last block row unused: its reads are turned to the first half
+    const bool hi_i = 2 * bi + 1 < nb8, hi_j = 2 * bj + 1 < nb8, off_diag = bi != bj;
+    const float* a0 = xs + (size_t)(coff + bi * 16 + fr) * kXsLd + fk;
+    const float* b0 = xs + (size_t)(coff + bj * 16 + fr) * kXsLd + fk;
+    const float* a1 = a0 + (hi_i ? 8 * kXsLd : 0);
+    const float* b1 = b0 + (hi_j ? 8 * kXsLd : 0);
+    double c00[2] = {0.0, 0.0}, c10[2] = {0.0, 0.0}, c11[2] = {0.0, 0.0}, c01[2] = {0.0, 0.0};
+    for (int sl = 0; sl < nslab; ++sl) {
+#pragma unroll
+      for (int ks = 0; ks < kSlabRows / 4; ++ks) {
+        const int o = sl * kSlabRows + 4 * ks;
+        const double x0 = (double)a0[o], x1 = (double)a1[o], y0 = (double)b0[o], y1 = (double)b1[o];
+        dmma_8x8x4(c00[0], c00[1], x0, y0);
+        if (hi_i) {
+          dmma_8x8x4(c10[0], c10[1], x1, y0);
+          dmma_8x8x4(c11[0], c11[1], x1, y1);
+        }
+        if (off_diag) dmma_8x8x4(c01[0], c01[1], x0, y1);
+      }
+    }
+    auto put = [&](int I, int J, const double (&c)[2]) {
+      *reinterpret_cast<double2*>(out + tri_index(t0 + I, t0 + J) * 64 + fr * 8 + 2 * fk) = make_double2(c[0], c[1]);
+    };
+    put(2 * bi, 2 * bj, c00);
+    if (hi_i) { put(2 * bi + 1, 2 * bj, c10); put(2 * bi + 1, 2 * bj + 1, c11); }
+    if (off_diag) put(2 * bi, 2 * bj + 1, c01);
+  }
+}
+
+template <int N> struct IntTag { static constexpr int value = N; };
+
+// Blocked right-looking Cholesky factorisation in float64 by the eight epilogue warps.  The matrix is
+// already in shared memory, t_off doubles behind the base (tile layout, see tile_offset; 16-byte
+// aligned), followed by room for 16 nb doubles (original diagonal, reciprocal pivots); entries beyond n
+// inside the last row of tiles are replaced by the identity here.  out != nullptr: the factor goes to
+// global memory in the layout the triangular solve reads (see lt_row_offset) with the reciprocal
+// diagonal behind it, panel by panel while the later ones are factored.  One function for the
+// factor and for the Rayleigh-Ritz window, kept out of line: code that runs once per launch is fetched
+// from L2, and the window's factorisation finds this code where the steps before it left it.
+__device__ __noinline__ void cholesky_team(int n, int t_off, float* out) {
+  double* T = reinterpret_cast<double*>(pow_smem()) + t_off;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  auto sync = [&]() { named_barrier(1, kEpiThreads); };
+  const int nb = (n + 7) >> 3;
+  double* aux = T + nb * (nb + 1) / 2 * 64;
   double* d0 = aux;                 // original diagonal
   double* rd = aux + 8 * nb;        // 1 / L[j][j]
   // identity padding of rows / columns n .. 8 nb - 1 (last row of tiles), then the diagonal
-  for (int e = tid; e < nb * 64; e += nthreads) {
+  for (int e = tid; e < nb * 64; e += kEpiThreads) {
     const int J = e >> 6, i = 8 * (nb - 1) + ((e >> 3) & 7), j = 8 * J + (e & 7);
     if (i >= n || j >= n) T[tri_index(nb - 1, J) * 64 + (e & 63)] = (i == j) ? 1.0 : 0.0;
   }
   sync();
-  for (int i = tid; i < 8 * nb; i += nthreads) d0[i] = T[tile_offset(i, i)];
+  for (int i = tid; i < 8 * nb; i += kEpiThreads) d0[i] = T[tile_offset(i, i)];
   sync();
   const int fr = lane >> 2, fk = lane & 3;
   auto update_tile = [&](int J, int I, int K) {
@@ -274,52 +370,112 @@ __device__ __forceinline__ void cholesky_blocked_team(int n, double* T, double* 
     C[0] = c0; C[1] = c1;
   };
   // row `i` of the tile (I, J) <- row * L_JJ^-T (forward substitution over the 8 columns)
-  auto solve_row = [&](int J, int i) {
-    const double* D = T + tri_index(J, J) * 64;
-    double* row = T + tri_index(i >> 3, J) * 64 + (i & 7) * 8;
-    double x[8];
+  auto solve_row = [&](int J, int i, double (&x)[8]) {
+    const double2* D = reinterpret_cast<const double2*>(T + tri_index(J, J) * 64);
+    double2* row = reinterpret_cast<double2*>(T + tri_index(i >> 3, J) * 64 + (i & 7) * 8);
+    double r[8];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) x[c] = row[c];
+    for (int c = 0; c < 4; ++c) {
+      const double2 v = row[c], q = reinterpret_cast<const double2*>(rd + 8 * J)[c];
+      x[2 * c] = v.x; x[2 * c + 1] = v.y;
+      r[2 * c] = q.x; r[2 * c + 1] = q.y;
+    }
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
       double v = x[c];
 #pragma unroll
-      for (int k = 0; k < c; ++k) v -= x[k] * D[c * 8 + k];
-      x[c] = v * rd[8 * J + c];
+      for (int k = 0; k < c; k += 2) {
+        const double2 l = D[c * 4 + (k >> 1)];
+        v -= x[k] * l.x;
+        if (k + 1 < c) v -= x[k + 1] * l.y;
+      }
+      x[c] = v * r[c];
     }
 #pragma unroll
-    for (int c = 0; c < 8; ++c) row[c] = x[c];
+    for (int c = 0; c < 4; ++c) row[c] = make_double2(x[2 * c], x[2 * c + 1]);
   };
-  auto update_tile2 = [&](int J, int Ia, int Ka, int Ib, int Kb) {
-    const double* XIa = T + tri_index(Ia, J) * 64 + fr * 8 + fk;
-    const double* XKa = T + tri_index(Ka, J) * 64 + fr * 8 + fk;
-    const double* XIb = T + tri_index(Ib, J) * 64 + fr * 8 + fk;
-    const double* XKb = T + tri_index(Kb, J) * 64 + fr * 8 + fk;
-    double* Ca = T + tri_index(Ia, Ka) * 64 + fr * 8 + 2 * fk;
-    double* Cb = T + tri_index(Ib, Kb) * 64 + fr * 8 + 2 * fk;
-    double a0 = Ca[0], a1 = Ca[1], b0 = Cb[0], b1 = Cb[1];
-    const double xa0 = -XIa[0], xa4 = -XIa[4], xb0 = -XIb[0], xb4 = -XIb[4];
-    const double ka0 = XKa[0], ka4 = XKa[4], kb0 = XKb[0], kb4 = XKb[4];
-    dmma_8x8x4(a0, a1, xa0, ka0);
-    dmma_8x8x4(b0, b1, xb0, kb0);
-    dmma_8x8x4(a0, a1, xa4, ka4);
-    dmma_8x8x4(b0, b1, xb4, kb4);
-    Ca[0] = a0; Ca[1] = a1; Cb[0] = b0; Cb[1] = b1;
+  // NT tiles (I, K), (I + step, K), ... -= sum over the panels 0 .. J of X_I X_K^T, accumulators in registers
+  auto accumulate = [&](auto nt_tag, int J, int I, int step, int K) {
+    constexpr int NT = decltype(nt_tag)::value;
+    double c[NT][2];
+#pragma unroll
+    for (int u = 0; u < NT; ++u) {
+      const double2 v = *reinterpret_cast<const double2*>(T + tri_index(I + u * step, K) * 64 + fr * 8 + 2 * fk);
+      c[u][0] = v.x; c[u][1] = v.y;
+    }
+    const double* XK = T + tri_index(K, 0) * 64 + fr * 8 + fk;
+    const double* XI = T + tri_index(I, 0) * 64 + fr * 8 + fk;
+    int skip[NT];                                        // from tile (I, .) to tile (I + u step, .)
+#pragma unroll
+    for (int u = 0; u < NT; ++u) skip[u] = (tri_index(I + u * step, 0) - tri_index(I, 0)) * 64;
+    double k0[2], k4[2], x0[2][NT], x4[2][NT];           // fragments of two panels: one in flight, one in use
+    auto load = [&](int buf) {
+      k0[buf] = XK[0]; k4[buf] = XK[4];
+#pragma unroll
+      for (int u = 0; u < NT; ++u) { x0[buf][u] = XI[skip[u]]; x4[buf][u] = XI[skip[u] + 4]; }
+      XK += 64; XI += 64;
+    };
+    auto apply = [&](int buf) {
+#pragma unroll
+      for (int u = 0; u < NT; ++u) dmma_8x8x4(c[u][0], c[u][1], -x0[buf][u], k0[buf]);
+#pragma unroll
+      for (int u = 0; u < NT; ++u) dmma_8x8x4(c[u][0], c[u][1], -x4[buf][u], k4[buf]);
+    };
+    load(0);
+#pragma unroll 1
+    for (int q = 0; q <= J; q += 2) {                    // (the loads beyond panel J stay inside the matrix)
+      load(1);
+      apply(0);
+      if (q + 1 > J) break;
+      load(0);
+      apply(1);
+    }
+#pragma unroll
+    for (int u = 0; u < NT; ++u)
+      *reinterpret_cast<double2*>(T + tri_index(I + u * step, K) * 64 + fr * 8 + 2 * fk) = make_double2(c[u][0], c[u][1]);
+  };
+  // Factor entries in the layout of the triangular solve (row j holds L[i][j] for i >= (j & ~3)): the
+  // tiles (J, J) and (J + 1, J) with the reciprocal diagonal by one warp, the rows below by the threads
+  // that solved them (consecutive rows, so a column is one coalesced store).
+  const int P8 = nb * 8;
+  auto column = [&](int j) { return out + lt_row_offset(j, P8) - (j & ~3); };
+  auto store_tiles = [&](int J) {
+    const int jl = lane >> 2, j = 8 * J + jl;
+    if (j >= n) return;
+    float* dst = column(j);
+    for (int I = J; I < min(J + 2, nb); ++I)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int i0 = (lane & 3) * 2 + q, i = 8 * I + i0;
+        if (i >= j && i < n) dst[i] = (float)T[tri_index(I, J) * 64 + i0 * 8 + jl];
+      }
+    if ((lane & 3) == 0) out[kLtFloats + j] = (float)rd[j];
+  };
+  auto store_row = [&](int J, int i, const double (&x)[8]) {
+    if (i >= n) return;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) column(8 * J + c)[i] = (float)x[c];
   };
   if (tid == 0) factor_diag_thread(T, d0, rd);
   sync();
   // One barrier of the whole team per 8-column panel.  The chain that bounds the factorisation -
   // panel J's diagonal tile -> tile (J+1, J) -> its update of tile (J+1, J+1) -> that tile's eight
   // dependent pivots - runs on warp 0 alone; the warps of the other three schedulers (the FP64 pipe
-  // is per scheduler: warp w issues on scheduler w & 3, so warp 4 stays idle) solve the rest of the
-  // panel and update the rest of the trailing matrix meanwhile.  They need tile (J+1, J) for the
-  // tiles of column J+1: warp 0 arrives on barrier 4 once it is solved.
+  // is per scheduler: warp w issues on scheduler w & 3, so warp 4 stays idle) meanwhile solve the rest of
+  // panel J and bring the columns J+1 and J+2 up to date.  They look two columns ahead: column J+2 takes
+  // its contributions of all panels up to J in one go, with the tile in registers, and column J+1 only
+  // that of panel J (it had the others an iteration before).  Updating the whole trailing matrix after
+  // every panel, every tile through shared memory, made the first half of the panels wait for it
+  // (n = 144: 80-100 k cycles); now every panel takes what its pivot chain takes.  The bulk warps need
+  // tile (J+1, J) for column J+1: warp 0 arrives on barrier 4 once it is solved.
   const bool bulk = (warp & 3) != 0;
-  const int nbulk = nw - (nw + 3) / 4, me = warp - (warp >> 2) - 1;          // bulk warps, in order
-  const int bulk_threads = nbulk * 32, btid = me * 32 + lane;
+  const int me = warp - (warp >> 2) - 1;                                     // bulk warps, in order
+  constexpr int nbulk = kEpiWarps - (kEpiWarps + 3) / 4, bulk_threads = nbulk * 32;
+  const int btid = me * 32 + lane;
   for (int J = 0; J + 1 < nb; ++J) {
     if (warp == 0) {
-      if (lane < 8) solve_row(J, 8 * (J + 1) + lane);
+      double x[8];
+      if (lane < 8) solve_row(J, 8 * (J + 1) + lane, x);
       __syncwarp();
       asm volatile("bar.arrive 4, %0;" ::"r"(bulk_threads + 32) : "memory");
       update_tile(J, J + 1, J + 1);
@@ -327,84 +483,35 @@ __device__ __forceinline__ void cholesky_blocked_team(int n, double* T, double* 
       if (lane == 0) factor_diag_thread(T + tri_index(J + 1, J + 1) * 64, d0 + 8 * (J + 1), rd + 8 * (J + 1));
       __syncwarp();
     } else if (bulk) {
-      for (int i = 8 * (J + 2) + btid; i < 8 * nb; i += bulk_threads) solve_row(J, i);
+      const int i = 8 * (J + 2) + btid;              // at most 18 tiles below: fewer rows than bulk threads
+      double x[8];
+      if (i < 8 * nb) solve_row(J, i, x);
       asm volatile("bar.sync 4, %0;" ::"r"(bulk_threads + 32) : "memory");
-      // tiles (I, K), J+1 <= K <= I, I >= J+2, dealt one by one to the bulk warps (row-major
-      // order); two tiles at a time so that their tensor-core instructions overlap
-      int I = J + 2, K = J + 1 + me;
-      auto settle = [&]() { while (I < nb && K > I) { K -= I - J; ++I; } };
-      settle();
-      while (I < nb) {
-        const int I1 = I, K1 = K;
-        K += nbulk; settle();
-        if (I < nb) {
-          update_tile2(J, I1, K1, I, K);
-          K += nbulk; settle();
-        } else {
-          update_tile(J, I1, K1);
-        }
+      if (out != nullptr && i < 8 * nb) store_row(J, i, x);
+      for (int I = J + 2 + me; I < nb; I += nbulk) update_tile(J, I, J + 1);
+      // column J + 2: the tiles are dealt from the other end, so that the warps with one tile less
+      // above come first here
+      for (int I = J + 2 + (nbulk - 1 - me); I < nb; I += 3 * nbulk) {
+        if (I + 2 * nbulk < nb) accumulate(IntTag<3>{}, J, I, nbulk, J + 2);
+        else if (I + nbulk < nb) accumulate(IntTag<2>{}, J, I, nbulk, J + 2);
+        else accumulate(IntTag<1>{}, J, I, nbulk, J + 2);
       }
-    } else if (kEarlyStore && warp == 4 && J >= 1) {
-      for (int I = J - 1; I < nb; ++I) store(I, J - 1, T + tri_index(I, J - 1) * 64, rd);
+    } else if (out != nullptr && warp == 4 && J >= 1) {
+      store_tiles(J - 1);                        // final since the last barrier
     }
     sync();
   }
-  if constexpr (kEarlyStore) {
-    // the last two panels (or the only one)
-    int t = 0;
-    for (int J = nb >= 2 ? nb - 2 : 0; J < nb; ++J)
-      for (int I = J; I < nb; ++I, ++t)
-        if (t % nw == warp) store(I, J, T + tri_index(I, J) * 64, rd);
-  } else {
-    for (int t = warp; t < ntile; t += nw) {
-      int I, J;
-      tri_decode(t, I, J);
-      store(I, J, T + t * 64, rd);
-    }
+  if (out != nullptr) {
+    if (nb >= 2 && warp == 1) store_tiles(nb - 2);
+    if (warp == 2) store_tiles(nb - 1);
   }
 }
-
-constexpr int kEpiThreads = 256;         // warps 0-7
-
-// Writes the accumulated 8 x 8 tiles of one warp unit (see gram_unit_accumulate) to the tile layout;
-// t0 = index of the first tile row / column the unit's coordinates are relative to.
-__device__ __forceinline__ void gram_unit_store_tiles(const GramAcc& acc, int ta, int tz, int t0, int lane,
-                                                      double* __restrict__ out) {
-  const int fr = lane >> 2, fk = lane & 3;
-#pragma unroll
-  for (int u = 0; u <= kMaxTiles8; ++u) {
-    int strip = -1, tb = 0;
-    if (u < kMaxTiles8 && u <= ta) { strip = ta; tb = u; }
-    else if (u >= 1 && kMaxTiles8 - u <= tz && tz != ta) { strip = tz; tb = kMaxTiles8 - u; }
-    if (strip < 0) continue;
-    *reinterpret_cast<double2*>(out + tri_index(t0 + strip, t0 + tb) * 64 + fr * 8 + 2 * fk) =
-        make_double2(acc.a[u][0], acc.a[u][1]);
-  }
-}
-
-// 8 x 8 tiles of the partial Gram matrix that do not fit the eight warp units (see the kernel): the
-// strips ta = u and tz = nb8 - 1 - u of the units u = 8 .. units - 1, listed strip by strip.
-// nb8 <= 20 leaves at most 2 units = 42 tiles, six per warp.
-constexpr int kExtraTiles = 6;
-__device__ __forceinline__ bool extra_tile(int e, int nb8, int units, int& ta, int& tb) {
-  for (int u = 8; u < units; ++u) {
-    const int a = u, z = nb8 - 1 - u;
-    if (e <= a) { ta = a; tb = e; return true; }
-    e -= a + 1;
-    if (z != a) {
-      if (e <= z) { ta = z; tb = e; return true; }
-      e -= z + 1;
-    }
-  }
-  return false;
-}
-
 
 // ---- work of the tile that finishes a step last (all 256 epilogue threads) ----------------------
 // Kept out of line: the tile epilogue is register-bound, and these run once per request and step.
 
 // Cholesky factor of the summed Gram matrix, written in the layout the triangular solve reads
-// (see lt_row_offset) followed by the reciprocal diagonal.  Tm: cholesky_smem_bytes(p) of scratch.
+// (see lt_row_offset) followed by the reciprocal diagonal.  Uses the operand ring as scratch.
 // Returns (to every thread) whether the next step may be the last one: from the diagonal of
 // the summed Gram matrix B = Y'^T Y' (theta_i = sqrt(B_ii) estimates the i-th eigenvalue of G once the
 // basis has started to order itself) the energy error after q_final multiplications is predicted as
@@ -413,9 +520,11 @@ __device__ __forceinline__ bool extra_tile(int e, int nb8, int units, int& ta, i
 // team_ritz reports at the end; stop_below is the bound it has to stay under (0: never stop early).
 // pad: also write the entries of the layout that no factor touches (the first factorisation of a
 // launch does; they stay as they are for the later ones).
-__device__ __noinline__ bool team_cholesky(const double* pbase, int nt, int p, int r, float* out, double* Tm,
-                                           float* dg, volatile int* s_word, int q_final, float stop_below,
-                                           bool pad) {
+__device__ __noinline__ bool team_cholesky(const double* pbase, int nt, int p, int r, float* out, int q_final,
+                                           float stop_below, bool pad) {
+  double* Tm = reinterpret_cast<double*>(pow_smem());
+  float* dg = pow_tail().dinv;
+  volatile int* s_word = pow_tail().s_word;
   const int et = threadIdx.x, warp = et >> 5, lane = et & 31;
   const int P = (p + 7) & ~7, nb = (p + 7) >> 3;
   auto epi_sync = [&]() { named_barrier(1, kEpiThreads); };
@@ -448,34 +557,24 @@ __device__ __noinline__ bool team_cholesky(const double* pbase, int nt, int p, i
     epi_sync();
   }
   const bool stop = stop_below > 0.f && *s_word != 0;
-  // row j of the layout holds L[i][j] for i >= (j & ~3): lane -> (j, half of the tile's rows), so that
-  // a lane's four entries are consecutive floats
-  auto store = [&](int I, int J, const double* tile, const double* rd) {
-    const int jl = lane >> 2, i0 = (lane & 3) * 2;
-    const int j = 8 * J + jl;
-    if (j < p) {
-      float* dst = out + lt_row_offset(j, P) - (j & ~3);
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int i = 8 * I + i0 + q;
-        if (i < p && i >= j) dst[i] = (float)tile[(i0 + q) * 8 + jl];
-      }
-      if (I == J && (lane & 3) == 0) out[kLtFloats + j] = (float)rd[j];
-    }
-  };
-  cholesky_blocked_team<true>(p, Tm, Tm + (size_t)nb * (nb + 1) / 2 * 64, et, kEpiThreads, store, epi_sync);
+  cholesky_team(p, 0, out);
   return stop;
 }
 
 // Rayleigh-Ritz on the window next to the cut (see eig_kernels.cuh) and the convergence estimate.
-// C: ritz_smem_bytes(w) of scratch; dg: p floats of scratch.
+// Uses the operand ring and the factor's place behind it as scratch.
 __device__ __noinline__ void team_ritz(const double* pbase, int nt, int p, int w, int r, int m, float* out_u,
-                                       float* C, float* dg, float* s_scale, int* s_flag, int max_sweeps,
-                                       float conv_tol, int steps, int* status) {
+                                       int max_sweeps, float conv_tol, int steps, int* status) {
+  float* C = reinterpret_cast<float*>(pow_smem());
+  float* dg = pow_tail().lt;
+  float* s_scale = pow_tail().s_scale;
+  int* s_flag = pow_tail().s_flag;
   const int et = threadIdx.x, warp = et >> 5, lane = et & 31;
   auto epi_sync = [&]() { named_barrier(1, kEpiThreads); };
   const int w0 = p - w, nbot = p - r;
-  const int ldc = ritz_ldc(w);
+  const bool small = w <= 32;            // the usual window: see jacobi_warp32 for the row order of a column
+  const int ldc = small ? kRitzLd32 : ritz_ldc(w);
+  auto at = [&](int col, int row) { return col * ldc + (small ? ritz_row(row) : row); };
   float* sig = C + (size_t)w * ldc;
   for (int e = et; e < w * ldc; e += kEpiThreads) C[e] = 0.f;
   if (et == 0) *s_scale = 0.f;
@@ -493,7 +592,8 @@ __device__ __noinline__ void team_ritz(const double* pbase, int nt, int p, int w
   {
     // the window block of B' (rows / columns w0 .. p-1), gathered into a tile layout of its own
     const int nbw = (w + 7) >> 3, cnt = nbw * (nbw + 1) / 2 * 64;
-    double* Tw = reinterpret_cast<double*>(C + (((size_t)w * ldc + w + 1) & ~(size_t)1));
+    const int tw_off = (w * ldc + w + 3) / 4 * 2;          // doubles from the base, a multiple of two
+    double* Tw = reinterpret_cast<double*>(C) + tw_off;
     for (int e = et; e < cnt; e += kEpiThreads) {
       int I, J;
       tri_decode(e >> 6, I, J);
@@ -503,13 +603,14 @@ __device__ __noinline__ void team_ritz(const double* pbase, int nt, int p, int w
       Tw[e] = v;
     }
     epi_sync();
-    auto store = [&](int I, int J, const double* tile, const double*) {
-      for (int q = lane; q < 64; q += 32) {
-        const int i = 8 * I + (q >> 3), j = 8 * J + (q & 7);
-        if (i < w && j <= i) C[j * ldc + i] = (float)tile[q];
-      }
-    };
-    cholesky_blocked_team(w, Tw, Tw + (size_t)cnt, et, kEpiThreads, store, epi_sync);
+    cholesky_team(w, tw_off, nullptr);
+    epi_sync();
+    for (int e = et; e < cnt; e += kEpiThreads) {
+      int I, J;
+      tri_decode(e >> 6, I, J);
+      const int i = 8 * I + ((e >> 3) & 7), j = 8 * J + (e & 7);
+      if (i < w && j <= i) C[at(j, i)] = (float)Tw[e];
+    }
   }
   epi_sync();
   const float s1 = sqrtf(*s_scale);
@@ -533,12 +634,12 @@ __device__ __noinline__ void team_ritz(const double* pbase, int nt, int p, int w
     worst = warp_max(worst);
     if (lane == 0 && worst > conv_tol) atomicOr(status, kStatusNoConverge);
   }
-  const int nact = min(kEpiThreads, ((((w + 1) >> 1) * 4) + 31) & ~31);
+  const int nact = small ? 32 : min(kEpiThreads, ((((w + 1) >> 1) * 4) + 31) & ~31);
   if (et == 0) *s_flag = 0;
   epi_sync();
   if (et < nact) {
     bool converged;
-    if (w <= 32) converged = jacobi_sweeps<8>(C, ldc, w, s1, max_sweeps, nact, s_flag);
+    if (small) converged = jacobi_warp32(0, w, s1, max_sweeps);
     else if (w <= 64) converged = jacobi_sweeps<16>(C, ldc, w, s1, max_sweeps, nact, s_flag);
     else if (w <= 96) converged = jacobi_sweeps<24>(C, ldc, w, s1, max_sweeps, nact, s_flag);
     else converged = jacobi_sweeps<(kPMax + 3) / 4>(C, ldc, w, s1, max_sweeps, nact, s_flag);
@@ -547,7 +648,7 @@ __device__ __noinline__ void team_ritz(const double* pbase, int nt, int p, int w
   named_barrier(3, kEpiThreads);
   for (int k = warp; k < w; k += 8) {
     float sm = 0.f;
-    for (int row = lane; row < w; row += 32) { float x = C[k * ldc + row]; sm += x * x; }
+    for (int row = lane; row < w; row += 32) { float x = C[at(k, row)]; sm += x * x; }
     sm = warp_sum(sm);
     if (lane == 0) sig[k] = sqrtf(sm);
   }
@@ -565,7 +666,7 @@ __device__ __noinline__ void team_ritz(const double* pbase, int nt, int p, int w
     for (int o = 16; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
     if (rank < nbot) {
       float scale = sk > 0.f ? 1.f / sk : 0.f;
-      for (int j = lane; j < w; j += 32) out_u[j * nbot + rank] = C[k * ldc + j] * scale;
+      for (int j = lane; j < w; j += 32) out_u[j * nbot + rank] = C[at(k, j)] * scale;
     }
   }
 }
@@ -575,23 +676,19 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
                 const __grid_constant__ CUtensorMap map_y0h, const __grid_constant__ CUtensorMap map_y0l,
                 const __grid_constant__ CUtensorMap map_y1h, const __grid_constant__ CUtensorMap map_y1l,
                 const FusedParams prm) {
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = pow_smem();
   float* xs = reinterpret_cast<float*>(smem);                       // aliases the ring after the MMAs
   float* xq = reinterpret_cast<float*>(smem + kXsBytes);            // previous block (last step)
-  float* lt = reinterpret_cast<float*>(smem + kPowRegion);
-  float* dinv = lt + kLtFloats;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(lt + kLbufStride);
-  uint64_t* full = bars;                 // [2]
-  uint64_t* empty = bars + 2;            // [2]
-  uint64_t* acc_full = bars + 4;
-  uint64_t* acc_empty = bars + 5;
-  uint64_t* epi_done = bars + 6;         // the region no longer belongs to the epilogue
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 8);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  volatile int* s_word = reinterpret_cast<volatile int*>(tmem_slot + 2);      // [2] broadcast slots of the epilogue
-  int* s_flag = reinterpret_cast<int*>(tmem_slot + 4);                        // Jacobi rotation flag
-  float* s_scale = reinterpret_cast<float*>(tmem_slot + 5);
+  const PowTail tail = pow_tail();
+  float *lt = tail.lt, *dinv = tail.dinv;
+  uint64_t* full = tail.bars;            // [2]
+  uint64_t* empty = tail.bars + 2;       // [2]
+  uint64_t* acc_full = tail.bars + 4;
+  uint64_t* acc_empty = tail.bars + 5;
+  uint64_t* epi_done = tail.bars + 6;    // the region no longer belongs to the epilogue
+  uint32_t* tmem_slot = tail.tmem_slot;
+  volatile int* abort_flag = tail.abort_flag;
+  volatile int* s_word = tail.s_word;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned* gabort = prm.sync + (size_t)prm.batch * kSyncStride;
 
@@ -611,6 +708,8 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
 
   const int s_begin = prm.sched[blockIdx.x], s_end = prm.sched[blockIdx.x + 1];
   const int* s_items = prm.sched + gridDim.x + 1;
+  const int my_group = prm.sched[gridDim.x + 1 + prm.n_items + blockIdx.x] & 0xffff;
+  const int n_groups = prm.sched[gridDim.x + 1 + prm.n_items + blockIdx.x] >> 16;
   const int last_step = prm.steps - 1;
   const int R = prm.tile_rows;
   auto decode = [&](int item, int& b, ReqPlan& rp, int& tile) {
@@ -660,6 +759,20 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
       }
     }
     __syncwarp();
+  } else if (warp == 9 && prm.n_servers > 0 && (int)blockIdx.x >= prm.n_tile_ctas) {
+    // ------------------------------------------------------------ rehearsal (factor servers)
+    // A server has nothing to multiply.  While it waits for the tiles this warp runs the eigenvalue
+    // rotations of the Ritz window once on a made-up matrix, in the part of the ring that the team
+    // does not use: the code is then in the SM's instruction cache when the last step needs it, instead of
+    // being fetched line by line from L2 in the middle of the request's critical path.
+    constexpr int kOff = (kPowRegion - 32 * kRitzLd32 * 4) / 4;
+    float* C = reinterpret_cast<float*>(smem) + kOff;
+    for (int e = lane; e < 32 * kRitzLd32; e += 32) C[e] = 0.f;
+    __syncwarp();
+    C[lane * kRitzLd32 + ritz_row(lane)] = 1.f;
+    if (lane == 0) C[ritz_row(1)] = 0.5f;
+    __syncwarp();
+    jacobi_warp32(kOff, 32, 1.f, 1);
   } else if (warp == 9) {
     // ------------------------------------------------------------ MMA issuer
     if (lane == 0) {
@@ -716,6 +829,13 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
       epi_sync();
       return *s_word != 0;
     };
+    // Do the CTAs of a request with nt tiles add up its partial matrices slice by slice?  One CTA reads
+    // about 64 bytes a cycle, the two more rounds through L2 that sharing takes cost 5-6 k cycles: worth it
+    // from 48 k entries over all tiles on (11 tiles at p = 88, 4 at p = 144), and only if there is somebody
+    // to share with (a server's request has one CTA per tile).
+    auto spread_of = [&](int nt, int P) {
+      return prm.spread_sum && nt * ((P >> 3) * ((P >> 3) + 1) / 2 * 64) > 48000 && (prm.n_servers > 0 || n_groups > 1);
+    };
     uint32_t n = 0;
     int cached_b = -1, cached_step = -1;
     bool ok = true;
@@ -724,10 +844,8 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
     // declared the last one.  Uses the operand ring as scratch.
     auto factor_request = [&](int b, const ReqPlan& rp, unsigned* sync_b, int step, bool is_last, int last_b,
                               int nt_sum) -> bool {
-      __threadfence();
       const int p = rp.p;
       const double* pbase = prm.partial + (size_t)rp.ptile_off * kTileDoubles;
-      double* Tm = reinterpret_cast<double*>(smem);        // the region is free: every thread passed the barrier
       bool stop = false;
       if (!is_last) {
         // after the second multiplication and later: may the next step be the last one?  (asked with a
@@ -735,20 +853,19 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
         // the basis is still mixing)
         const bool may_stop = prm.early_stop && step >= 1 && step + 1 < last_b && p < rp.m;
         const float margin = step == 1 ? 0.015625f : 0.125f;
-        stop = team_cholesky(pbase, nt_sum, p, rp.r, prm.lbuf + (size_t)b * kLbufStride, Tm, dinv,
-                             s_word, step + 2, may_stop ? margin * prm.conv_tol : 0.f, step == 0);
-        __threadfence();
-        epi_sync();
+        stop = team_cholesky(pbase, nt_sum, p, rp.r, prm.lbuf + (size_t)b * kLbufStride, step + 2,
+                             may_stop ? margin * prm.conv_tol : 0.f, step == 0);
+        epi_sync();                                // then one fence for the team's stores (it is cumulative)
         if (et == 0) {
+          __threadfence();
           if (stop) st_release_u32(sync_b + 3, (unsigned)(step + 1));
           st_release_u32(sync_b + 1, (unsigned)(step + 1));
         }
       } else {
-        team_ritz(pbase, nt_sum, p, rp.win, rp.r, rp.m, prm.ub + (size_t)b * kPMax * kPMax, reinterpret_cast<float*>(smem), lt,
-                  s_scale, s_flag, prm.max_sweeps, prm.conv_tol, step + 1, prm.status);
-        __threadfence();
+        team_ritz(pbase, nt_sum, p, rp.win, rp.r, rp.m, prm.ub + (size_t)b * kPMax * kPMax,
+                  prm.max_sweeps, prm.conv_tol, step + 1, prm.status);
         epi_sync();
-        if (et == 0) st_release_u32(sync_b + 2, 1u);
+        if (et == 0) { __threadfence(); st_release_u32(sync_b + 2, 1u); }
       }
       return stop;
     };
@@ -765,7 +882,7 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
         const ReqPlan rp = prm.plan[b];
         unsigned* sync_b = prm.sync + (size_t)b * kSyncStride;
         const unsigned nt = (unsigned)((rp.m + R - 1) / R);
-        const bool summed = prm.spread_sum && nt >= 4;      // the tiles have added up the partial matrices
+        const bool summed = spread_of((int)nt, (rp.p + 7) & ~7);   // the tiles have added up the partial matrices
         int last_b = last_step;
         for (int step = 0; step <= last_b; ++step) {
           if (!team_wait(summed ? sync_b + 4 : sync_b, nt * (unsigned)(step + 1))) break;
@@ -805,8 +922,15 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
           if (ok) {
             const float4* src = reinterpret_cast<const float4*>(prm.lbuf + (size_t)b * kLbufStride);
             float4* dst = reinterpret_cast<float4*>(lt);
-            int n4 = (lt_row_offset(P, P) + 3) / 4;    // floats used by the P-wide layout
-            for (int e = et; e < n4; e += kEpiThreads) dst[e] = __ldcg(src + e);
+            const int n4 = (lt_row_offset(P, P) + 3) / 4;    // 16-byte vectors the P-wide layout takes, eight in flight
+            for (int e0 = et; e0 < n4; e0 += 8 * kEpiThreads) {
+              float4 v[8];
+#pragma unroll
+              for (int u = 0; u < 8; ++u) v[u] = __ldcg(src + min(e0 + u * kEpiThreads, n4 - 1));
+#pragma unroll
+              for (int u = 0; u < 8; ++u)
+                if (e0 + u * kEpiThreads < n4) dst[e0 + u * kEpiThreads] = v[u];
+            }
             const float* dsrc = prm.lbuf + (size_t)b * kLbufStride + kLtFloats;
             for (int e = et; e < P; e += kEpiThreads) dinv[e] = __ldcg(dsrc + e);
           }
@@ -825,113 +949,72 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
         float* yf = is_last ? prm.yf[1] : nullptr;
         float* qprev = is_last ? prm.yf[0] : nullptr;
         const int nrows = min(R, rp.m - tile * R);
-        // ---- Y_next row = T row * L^-T (forward substitution per row), staged as xs[c][r] ----
-        // Between the first and the last step two threads share a row: warps 0-3 own the 32-column
-        // super-block S being solved (contributions of the previous super-block and of its own
-        // columns), warps 4-7 run one super-block ahead and sum what the columns before that
-        // contribute to super-block S + 1 (hs, double-buffered behind the staged block).
-        const bool split = !identity && !is_last;
+        // ---- Y_next = T L^-T (forward substitution), staged as xs[c][r]; see solve_gemm / solve_diag ----
         const int nS = (P + 31) >> 5;
-        float* hs = reinterpret_cast<float*>(smem + kXsBytes);          // [2][32][kXsLd]
+        const bool row_ok = r < nrows;
+        // 32-row groups that lie wholly beyond the tile's rows (64-row tiles, ragged last tiles) are left
+        // out; their rows of the staged block stay unwritten and are not read below
+        const bool active = (warp & 3) * 32 < nrows;
         if (warp < 4) {
           ok = ok && mbar_wait(acc_full, n & 1u, abort_flag);
           tc_fence_after();
-        }
-        const bool row_ok = r < nrows;
-        // warps whose 32 rows all lie beyond the tile's rows (64-row tiles, ragged last tiles), and
-        // their helpers, have nothing to solve; they keep taking part in the barriers.  Their rows
-        // of the staged block stay unwritten and are not read below.
-        const bool active = (warp & 3) * 32 < nrows;
+          if (active) {
 #pragma unroll 1
-        for (int S = 0; S < nS; ++S) {
-          if (warp < 4) {
-            if (active) {
-            float v[32];
-            tmem_ld32(t_lane + S * 32, v);
-            const float* hcur = hs + (S & 1) * 32 * kXsLd;
+            for (int S = 0; S < nS; ++S) {
+              float v[32];
+              tmem_ld32(t_lane + S * 32, v);
 #pragma unroll
-            for (int sb = 0; sb < 4; ++sb) {
-              const int jb = S * 32 + sb * 8;
-              if (jb < P) {
-                float acc[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) acc[e] = v[sb * 8 + e];
-                if (!identity) {
-                  int g0 = 0;
-                  if (split && S >= 2) {
-                    g0 = 8 * (S - 1);
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) acc[e] += hcur[(sb * 8 + e) * kXsLd + r];
-                  }
-                  solve_apply_groups(acc, jb, g0, jb >> 2, smem_u32(lt), smem_u32(xs), r, P);
-                  solve_inblock8(acc, jb, smem_u32(lt), smem_u32(dinv), P);
-                }
-#pragma unroll
-                for (int e = 0; e < 8; ++e) xs[(jb + e) * kXsLd + r] = (row_ok && ok) ? acc[e] : 0.f;
-              }
-            }
-            }
-          } else if (active && split && S >= 1 && S + 1 < nS) {
-            // minus the contributions of the columns before 32 S to super-block S + 1
-            float* hnext = hs + ((S + 1) & 1) * 32 * kXsLd;
-#pragma unroll 1
-            for (int sb = 0; sb < 4; ++sb) {
-              const int jb = (S + 1) * 32 + sb * 8;
-              if (jb < P) {
-                float acc[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-                solve_apply_groups(acc, jb, 0, 8 * S, smem_u32(lt), smem_u32(xs), r, P);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) hnext[(sb * 8 + e) * kXsLd + r] = acc[e];
-              }
+              for (int e = 0; e < 32; ++e)
+                if (S * 32 + (e & ~7) < P) xs[(S * 32 + e) * kXsLd + r] = (row_ok && ok) ? v[e] : 0.f;
             }
           }
-          if (split) epi_sync();
-        }
-        if (warp < 4) {
           tc_fence_before();
           mbar_arrive(acc_empty);
         } else if (is_last) {
-          // ---- last step, warps 4-7: rows of Q = Y L^-T for the previous block Y, in place ----
+          // last step, warps 4-7: the block this step multiplied, from its two bf16 planes (eight rows of a
+          // column per vector), becomes Q = Y L^-T
           ok = ok && mbar_wait(acc_full, n & 1u, abort_flag);      // the ring is no longer read
-          const int t4 = et - 128;
-          float* qrows = qprev + ((size_t)rp.presel_off + tile * R) * kPMax;
-          {
-            // the block this step multiplied, row t4 of the tile, from its two bf16 planes
-            const __nv_bfloat16* ph = prm.y_hi[step & 1] + (size_t)b * kPMax * prm.ld + tile * R + t4;
-            const __nv_bfloat16* pl = prm.y_lo[step & 1] + (size_t)b * kPMax * prm.ld + tile * R + t4;
-            const unsigned short* uh = reinterpret_cast<const unsigned short*>(ph);
-            const unsigned short* ul = reinterpret_cast<const unsigned short*>(pl);
-            const bool have_row = t4 < nrows;
-#pragma unroll 1
-            for (int c0 = 0; c0 < P; c0 += 8) {
-              unsigned short vh[8], vl[8];
+          const int t4 = et - 128, chunks = (nrows + 7) >> 3;
+          const size_t base = (size_t)b * kPMax * prm.ld + tile * R;
+          const int ch = t4 & 15;
+          if (ch < chunks) {
+#pragma unroll 4
+            for (int c = t4 >> 4; c < P; c += 8) {
+              uint4 h = make_uint4(0u, 0u, 0u, 0u), l = h;
+              if (c < p) {
+                h = __ldcg(reinterpret_cast<const uint4*>(prm.y_hi[step & 1] + base + (size_t)c * prm.ld) + ch);
+                l = __ldcg(reinterpret_cast<const uint4*>(prm.y_lo[step & 1] + base + (size_t)c * prm.ld) + ch);
+              }
+              const uint32_t uh[4] = {h.x, h.y, h.z, h.w}, ul[4] = {l.x, l.y, l.z, l.w};
+              float f[8];
 #pragma unroll
-              for (int u = 0; u < 8; ++u) {
-                const bool in = have_row && c0 + u < p;
-                vh[u] = in ? __ldcg(uh + (size_t)(c0 + u) * prm.ld) : (unsigned short)0;
-                vl[u] = in ? __ldcg(ul + (size_t)(c0 + u) * prm.ld) : (unsigned short)0;
+              for (int e = 0; e < 4; ++e) {
+                f[2 * e] = __uint_as_float(uh[e] << 16) + __uint_as_float(ul[e] << 16);
+                f[2 * e + 1] = __uint_as_float(uh[e] & 0xffff0000u) + __uint_as_float(ul[e] & 0xffff0000u);
               }
 #pragma unroll
-              for (int u = 0; u < 8; ++u)
-                xq[(c0 + u) * kXsLd + t4] = __uint_as_float((uint32_t)vh[u] << 16) + __uint_as_float((uint32_t)vl[u] << 16);
+              for (int e = 0; e < 8; ++e)
+                if (ch * 8 + e >= nrows) f[e] = 0.f;
+              float4* dst = reinterpret_cast<float4*>(xq + c * kXsLd + ch * 8);
+              dst[0] = make_float4(f[0], f[1], f[2], f[3]);
+              dst[1] = make_float4(f[4], f[5], f[6], f[7]);
             }
           }
-          named_barrier(2, 128);
-          for (int jb = 0; jb < P && active; jb += 8) {
-            float acc[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) acc[e] = xq[(jb + e) * kXsLd + t4];
-            solve_apply_groups(acc, jb, 0, jb >> 2, smem_u32(lt), smem_u32(xq), t4, P);
-            solve_inblock8(acc, jb, smem_u32(lt), smem_u32(dinv), P);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) xq[(jb + e) * kXsLd + t4] = acc[e];
+          // 32-row groups that the diagonal solves touch are complete
+          if (active && chunks * 8 + (t4 & 31) < ((nrows + 31) & ~31) && t4 < 32)
+            for (int c = 0; c < P; ++c) xq[c * kXsLd + chunks * 8 + t4] = 0.f;
+        }
+        if (!identity) {
+          for (int q = 0; q < (is_last ? 2 : 1); ++q) {     // the block, then (last step) Q
+            if (is_last) epi_sync();
+            solve_team(q * (kXsBytes / 4), P, R, !is_last, nrows, ok);
           }
-          named_barrier(2, 128);
-          // only the window columns are read again (second half of Eq. 15)
-          for (int c = (p - rp.win) + (t4 & 31); c < p; c += 32)
-            for (int rr = t4 >> 5; rr < nrows; rr += 4) qrows[(size_t)rr * kPMax + c] = xq[c * kXsLd + rr];
+        }
+        if (is_last) {
+          // only the window columns of Q are read again (second half of Eq. 15)
+          float* qrows = qprev + ((size_t)rp.presel_off + tile * R) * kPMax;      // [win][nrows]
+          for (int c = warp; c < rp.win; c += 8)
+            for (int rr = lane; rr < nrows; rr += 32) qrows[c * nrows + rr] = xq[(p - rp.win + c) * kXsLd + rr];
         }
         epi_sync();                                  // the staged block is complete
         if (is_last && et < nrows) {
@@ -941,9 +1024,6 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
           for (int c = 0; c < p; ++c) total += xs[c * kXsLd + et] * xq[c * kXsLd + et];
           prm.energy[(size_t)rp.presel_off + tile * R + et] = total;
         }
-        // the partial Gram below stages its slabs where the previous block (xq) lives: nobody may
-        // start on them while a row still reads xq
-        if (is_last) epi_sync();
         // ---- bf16 planes of the new block (K-major operand of the next step): 8 positions per thread
         if (!is_last) {
           const int cols = (rp.m + kBK - 1) / kBK * kBK;
@@ -973,102 +1053,44 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
           }
         }
         if (yf != nullptr) {
-          // float32 window columns of the final block, one token per row (second half of Eq. 15)
-          float* yrows = yf + ((size_t)rp.presel_off + tile * R) * kPMax;
-          for (int c = (p - rp.win) + (et & 31); c < p; c += 32)
-            for (int rr = et >> 5; rr < nrows; rr += 8) yrows[(size_t)rr * kPMax + c] = xs[c * kXsLd + rr];
+          // float32 window columns of the final block (second half of Eq. 15)
+          float* yrows = yf + ((size_t)rp.presel_off + tile * R) * kPMax;          // [win][nrows]
+          for (int c = warp; c < rp.win; c += 8)
+            for (int rr = lane; rr < nrows; rr += 32) yrows[c * nrows + rr] = xs[(p - rp.win + c) * kXsLd + rr];
         }
         // ---- float64 partial Gram of the tile on the FP64 tensor cores ----
         const int coff = is_last ? ((p - rp.win) & ~7) : 0;
         {
           // The last step only feeds the Rayleigh-Ritz window: the trailing block of columns from
           // coff on, plus the diagonal of the leading columns (the scale of the problem).
-          const int pw = p - coff;
-          const int nb8 = (pw + 7) >> 3, units = (nb8 + 1) / 2, nslab = (nrows + kSlabRows - 1) / kSlabRows;
-          double* slabs = reinterpret_cast<double*>(smem + kXsBytes);
           double* out = prm.partial + (size_t)item * kTileDoubles;
           for (int c = et; c < coff; c += kEpiThreads) {
             double sq = 0.0;
             for (int rr = 0; rr < nrows; ++rr) { double x = (double)xs[c * kXsLd + rr]; sq += x * x; }
             out[tile_offset(c, c)] = sq;
           }
-          // Units 0-7 go to the eight warps.  With more than 128 columns one or two units are left
-          // over: a second, short pass over the slabs deals their 8 x 8 tiles round-robin to the
-          // warps (at most kExtraTiles each) instead of leaving them to one or two warps.
-          const int fr = lane >> 2, fk = lane & 3;
-          auto fill_slab = [&](double* slab, int sl) {
-            for (int e = et; e < nb8 * 8 * kSlabRows; e += kEpiThreads) {
-              int c = e >> 4, rr = e & 15;
-              slab[c * kSlabLd + rr] = (double)xs[(coff + c) * kXsLd + sl * kSlabRows + rr];
-            }
-          };
-          {
-            const bool have = warp < units;
-            const int ta = have ? warp : 0, tz = have ? nb8 - 1 - warp : 0;
-            GramAcc acc;
-#pragma unroll
-            for (int u = 0; u <= kMaxTiles8; ++u) { acc.a[u][0] = 0.0; acc.a[u][1] = 0.0; }
-            for (int sl = 0; sl < nslab; ++sl) {
-              double* slab = slabs + (sl & 1) * (kPMax * kSlabLd);
-              fill_slab(slab, sl);
-              epi_sync();
-              if (have) gram_unit_accumulate(acc, slab, ta, tz, lane);
-              // the other buffer is refilled next; this one is reused two slabs later, after the
-              // barrier of the next slab
-            }
-            if (have) gram_unit_store_tiles(acc, ta, tz, coff >> 3, lane, out);
-            epi_sync();
-          }
-          if (units > 8) {
-            int xa_t[kExtraTiles], xb_t[kExtraTiles];
-            double xacc[kExtraTiles][2];
-            int n_extra = 0;
-#pragma unroll
-            for (int q = 0; q < kExtraTiles; ++q) {
-              xacc[q][0] = 0.0; xacc[q][1] = 0.0; xa_t[q] = 0; xb_t[q] = 0;
-              if (extra_tile(warp + 8 * q, nb8, units, xa_t[q], xb_t[q])) n_extra = q + 1;
-            }
-            for (int sl = 0; sl < nslab; ++sl) {
-              double* slab = slabs + (sl & 1) * (kPMax * kSlabLd);
-              fill_slab(slab, sl);
-              epi_sync();
-              const double* base = slab + fr * kSlabLd + fk;
-#pragma unroll 1
-              for (int ks = 0; ks < kSlabRows / 4; ++ks) {
-#pragma unroll
-                for (int q = 0; q < kExtraTiles; ++q)
-                  if (q < n_extra)
-                    dmma_8x8x4(xacc[q][0], xacc[q][1], base[xa_t[q] * 8 * kSlabLd + 4 * ks],
-                               base[xb_t[q] * 8 * kSlabLd + 4 * ks]);
-              }
-            }
-#pragma unroll
-            for (int q = 0; q < kExtraTiles; ++q) {
-              if (q < n_extra)
-                *reinterpret_cast<double2*>(out + tri_index((coff >> 3) + xa_t[q], (coff >> 3) + xb_t[q]) * 64 +
-                                            fr * 8 + 2 * fk) = make_double2(xacc[q][0], xacc[q][1]);
-            }
-            epi_sync();
-          }
+          gram_tile_f64(xs, coff, (p - coff + 7) >> 3, (nrows + kSlabRows - 1) / kSlabRows, kEpiWarps - 1 - warp, lane, out);
         }
         // ---- arrival: this tile's slab and partial sums are published -------------------------
-        __threadfence();
+        // (one thread's fence covers what the others wrote before the barrier; a fence of every thread
+        // cost 2-3 k cycles more)
         fence_proxy_async_all();
         epi_sync();
         int nt_sum = (int)nt;                        // partial matrices the factoring tile has to add up
-        if (prm.spread_sum && nt >= 4) {             // with fewer tiles the extra round trip costs more than it saves
-          // Every CTA holds one tile, so all tiles of the request are being worked on at the same
-          // time: instead of leaving the sum of the partial matrices to the last tile alone, every
-          // tile waits for the others and adds up its own slice of the matrix (in tile order, into
-          // the slot of tile 0); the last one to finish its slice factors the summed matrix.
-          if (et == 0) atomicAdd(sync_b, 1u);
+        const bool spread = spread_of((int)nt, P);
+        if (spread && si + 1 == s_end) {
+          // All tiles of the request are being worked on at the same time, one group of them per CTA:
+          // instead of leaving the sum of the partial matrices to one CTA, every CTA waits for the last
+          // of the tiles and adds up its own slice of the matrix (in tile order, into the slot of
+          // tile 0); the last one to finish its slice factors the summed matrix.
+          if (et == 0) { __threadfence(); atomicAdd(sync_b, 1u); }
           ok = team_wait(sync_b, nt * (unsigned)(step + 1)) && ok;
           double* sum0 = prm.partial + (size_t)rp.ptile_off * kTileDoubles;
           const int used = (P >> 3) * ((P >> 3) + 1) / 2 * 64;
-          const int chunk = ((used + (int)nt - 1) / (int)nt + 1) & ~1;
-          const int e1 = min(used, (tile + 1) * chunk);
+          const int chunk = ((used + n_groups - 1) / n_groups + 1) & ~1;
+          const int e1 = min(used, (my_group + 1) * chunk);
           if (ok) {
-            for (int e = tile * chunk + 2 * et; e < e1; e += 2 * kEpiThreads) {
+            for (int e = my_group * chunk + 2 * et; e < e1; e += 2 * kEpiThreads) {
               double2 acc = make_double2(0.0, 0.0);
               for (int t0 = 0; t0 < (int)nt; t0 += 8) {
                 double2 v[8];
@@ -1082,17 +1104,20 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
               *reinterpret_cast<double2*>(sum0 + e) = acc;
             }
           }
-          __threadfence();
           epi_sync();
           if (et == 0) {
+            __threadfence();
             unsigned old = atomicAdd(sync_b + 4, 1u);
-            *s_word = (old + 1u == nt * (unsigned)(step + 1) && !*abort_flag) ? 1 : 0;
+            __threadfence();
+            *s_word = (old + 1u == (unsigned)n_groups * (unsigned)(step + 1) && !*abort_flag) ? 1 : 0;
           }
           nt_sum = 1;
         } else if (et == 0) {
+          __threadfence();
           unsigned old = atomicAdd(sync_b, 1u);
+          __threadfence();
           // one decision for the whole team (a CTA that has given up factors nothing)
-          *s_word = (old + 1u == nt * (unsigned)(step + 1) && !*abort_flag) ? 1 : 0;
+          *s_word = (!spread && old + 1u == nt * (unsigned)(step + 1) && !*abort_flag) ? 1 : 0;
         }
         epi_sync();
         if (*s_word && prm.n_servers == 0) {
@@ -1101,65 +1126,97 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_arrive(epi_done);
+        if (identity && prm.n_servers > 0) {
+          // Rehearsal: this CTA's only tile now waits for the first factor.  The solve runs once on whatever
+          // the factor's place holds (a narrow block with the same remainder of columns, so that the same
+          // code runs): it is in the instruction cache when the factor arrives, instead of being fetched line
+          // by line from L2 on the critical path (batch of 16 requests: 27 -> 11 k cycles).
+          const int dry = P <= 95 ? P : 64 + (P & 31);
+          solve_team(kPowRegion / 4, dry, R, true, nrows, true);
+        }
       }
     }
     // ------------------------------------------------------------ Eq. 15 for this CTA's tiles
     // c_i = sum_j Y'_ij Q_ij - sum_k (Y'_{i,win} u_k)(Q_{i,win} u_k)  (see eig_kernels.cuh)
+    // The discarded Ritz pairs take only the window columns of the two blocks, which lie column by
+    // column in global memory (coalesced over the rows; one token per row of 640 bytes took a sector
+    // for every value: 28-40 k cycles a tile, now about 4 k).  Two threads share a row: of every
+    // sixteen Ritz vectors the first projects the row on eight and the second on the next eight; the
+    // products are added up in the order of the vectors, the second thread going on from the
+    // first's sum.
     {
-      float* us = reinterpret_cast<float*>(smem);                      // [w][nbot]
+      float* us = reinterpret_cast<float*>(smem);                      // [w][nb8], zero-padded columns
+      float* part = us + kPMax * kPMax;                                // [128] running sums
       int cached_u = -1;
       for (int si = s_begin; si < s_end; ++si) {
         const int item = s_items[si];
         int b, tile; ReqPlan rp;
         decode(item, b, rp, tile);
-        const int p = rp.p, w = rp.win, w0 = p - w, nbot = p - rp.r;
+        const int p = rp.p, w = rp.win, nbot = p - rp.r, nb8 = (nbot + 7) & ~7;
+        const int nrows = min(R, rp.m - tile * R);
+        const int rr = et & 127, second = et >> 7;
+        const size_t grow = (size_t)rp.presel_off + tile * R;
+        const float* yw = prm.yf[1] + grow * kPMax + rr;
+        const float* qw = prm.yf[0] + grow * kPMax + rr;
+        const bool have = rr < nrows;
+        float yv[32], qv[32];
+        auto load_chunk = [&](int j0) {
+#pragma unroll
+          for (int jj = 0; jj < 32; ++jj) {
+            const bool in = have && j0 + jj < w;
+            yv[jj] = in ? __ldcg(yw + (j0 + jj) * nrows) : 0.f;
+            qv[jj] = in ? __ldcg(qw + (j0 + jj) * nrows) : 0.f;
+          }
+        };
+        load_chunk(0);                                 // this CTA's own rows: before the wait for the Ritz vectors
+        float total = have && !second ? __ldcg(prm.energy + grow + rr) : 0.f;
         if (b != cached_u) {
           ok = team_wait(prm.sync + (size_t)b * kSyncStride + 2, 1u) && ok;
           const float* usrc = prm.ub + (size_t)b * kPMax * kPMax;
-          if (ok) for (int e = et; e < w * nbot; e += kEpiThreads) us[e] = __ldcg(usrc + e);
+          for (int e = et; e < w * nb8; e += kEpiThreads) {
+            const int j = e / nb8, k = e - j * nb8;
+            us[e] = ok && k < nbot ? __ldcg(usrc + j * nbot + k) : 0.f;
+          }
           epi_sync();
           cached_u = b;
         }
-        const int nrows = min(R, rp.m - tile * R);
-        // the discarded Ritz pairs take only the window columns of the two blocks: one thread per
-        // row, window slices read straight from the float32 blocks
-        for (int rr = et; rr < nrows; rr += kEpiThreads) {
-          const size_t grow = (size_t)rp.presel_off + tile * R + rr;
-          const float* yrow = prm.yf[1] + grow * kPMax + w0;
-          const float* qrow = prm.yf[0] + grow * kPMax + w0;
-          // projections of the two window slices on every discarded Ritz vector, accumulated over
-          // chunks of 32 window columns (all loads of a chunk in flight together)
-          float sub_ = 0.f;
-          for (int k0 = 0; k0 < nbot; k0 += 8) {
-            float ya[8], qa[8];
+        float sub_ = 0.f;
+        for (int k0 = 0; k0 < nbot; k0 += 16) {
+          const int kk = k0 + 8 * second;
+          float ya[8], qa[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) { ya[u] = 0.f; qa[u] = 0.f; }
+          for (int u = 0; u < 8; ++u) { ya[u] = 0.f; qa[u] = 0.f; }
+          if (have && kk < nbot) {
             for (int j0 = 0; j0 < w; j0 += 32) {
-              float yv[32], qv[32];
-#pragma unroll
-              for (int jj = 0; jj < 32; ++jj) {
-                const bool in = ok && j0 + jj < w;
-                yv[jj] = in ? __ldcg(yrow + j0 + jj) : 0.f;
-                qv[jj] = in ? __ldcg(qrow + j0 + jj) : 0.f;
-              }
+              if (w > 32) load_chunk(j0);
 #pragma unroll
               for (int jj = 0; jj < 32; ++jj) {
                 if (j0 + jj < w) {
-                  const float* ur = us + (j0 + jj) * nbot + k0;
+                  const float4* ur = reinterpret_cast<const float4*>(us + (j0 + jj) * nb8 + kk);
+                  const float4 u0 = ur[0], u1 = ur[1];
+                  const float uu[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
 #pragma unroll
-                  for (int u = 0; u < 8; ++u) {
-                    const float uu = k0 + u < nbot ? ur[u] : 0.f;
-                    ya[u] += yv[jj] * uu; qa[u] += qv[jj] * uu;
-                  }
+                  for (int u = 0; u < 8; ++u) { ya[u] += yv[jj] * uu[u]; qa[u] += qv[jj] * uu[u]; }
                 }
               }
             }
+          }
+          if (!second) {
 #pragma unroll
             for (int u = 0; u < 8; ++u) sub_ += ya[u] * qa[u];
+            part[rr] = sub_;
           }
-          const float total = ok ? __ldcg(prm.energy + grow) : 0.f;
-          prm.energy[grow] = fmaxf(total - sub_, 0.f);
+          epi_sync();
+          if (second) {
+            sub_ = part[rr];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) sub_ += ya[u] * qa[u];
+            part[rr] = sub_;
+          }
+          epi_sync();
+          if (!second) sub_ = part[rr];
         }
+        if (have && !second) prm.energy[grow + rr] = fmaxf((ok ? total : 0.f) - sub_, 0.f);
       }
     }
   }

@@ -311,72 +311,177 @@ constexpr int kPowTmemCols = 256;
 constexpr int kPowThreads = 320;                         // 8 epilogue warps, TMA producer, MMA issuer
 static_assert(kPMax * kXsLd * 4 <= kPowStages * kPowStageBytes, "staged block must fit in the ring");
 
-__device__ __forceinline__ float lds_f32(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
-  return v;
+// Base of the kernel's dynamic shared memory, rounded up to 1024 bytes by an offset (not by integer
+// arithmetic on the address), and taken from the array itself in every function that is not inlined: so
+// the compiler knows that what it reaches through the result is shared memory.
+__device__ __forceinline__ uint8_t* pow_smem() {
+  extern __shared__ uint8_t smem_raw[];
+  return smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);
 }
-__device__ __forceinline__ float4 lds_v4(uint32_t addr) {
-  float4 v;
-  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
-  return v;
+// ---- T L^-T by super-blocks of 32 columns (x[c * kXsLd + row] holds T and becomes the result) ------
+// solve_gemm takes the contributions of the columns before super-block S off its 32 columns: a product
+// of (rows) x (32 S) with (32 S) x 32, by the eight warps, RT rows x 4 columns per thread.  A warp
+// covers 16 RT rows x 8 columns, so that a column step reads 16 RT + 8 words of shared memory for
+// 128 RT products (three wavefronts for sixteen multiply-adds per thread when RT = 4): bound by the FP32
+// pipe, where one thread per row needed a word for every product and was bound by shared memory.
+// solve_diag then solves inside the super-block, one thread per row, the row's 32 values in
+// registers.  p = 144, 128 rows: 40 -> 14 k cycles.
+// The products enter every sum in ascending column order; `split` (steps before the last one): the
+// columns before 32 (S - 1) are summed from zero and T is added to that sum.
+template <int RT, int RG>
+__device__ __forceinline__ void solve_gemm(float* x, const float* lt, int P, int S, bool split, int nrows, int warp,
+                                           int lane) {
+  const int rg = warp % RG, row0 = 16 * RT * rg + RT * (lane & 15);
+  const int j0 = 32 * S + 8 * (warp / RG);
+  if (16 * RT * rg >= ((nrows + 31) & ~31) || j0 >= P) return;       // whole warp
+  const int j = j0 + 4 * (lane >> 4);
+  float acc[4][RT];
+  auto t_at = [&](int c) { return x + (j + c) * kXsLd + row0; };
+  auto rows_load = [&](const float* src, float (&v)[RT]) {
+    if constexpr (RT == 4) {
+      float4 t = *reinterpret_cast<const float4*>(src);
+      v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+    } else if constexpr (RT == 2) {
+      float2 t = *reinterpret_cast<const float2*>(src);
+      v[0] = t.x; v[1] = t.y;
+    } else {
+      v[0] = *src;
+    }
+  };
+  const float* xp = x + row0;
+  const float* lp = lt + j;                // row i of the layout starts at column i & ~3
+  int stride = P;                          // rows 4a .. 4a+3 have P - 4a entries
+  float xv[2][4][RT];
+  float4 lv[2][4];
+  auto load = [&](int buf) {               // one group of four columns, then step to the next
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      rows_load(xp + q * kXsLd, xv[buf][q]);
+      lv[buf][q] = *reinterpret_cast<const float4*>(lp + q * stride);
+    }
+    xp += 4 * kXsLd;
+    lp += 4 * stride - 4;
+    stride -= 4;
+  };
+  auto apply = [&](int buf) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int e = 0; e < RT; ++e) {
+        acc[0][e] -= xv[buf][q][e] * lv[buf][q].x; acc[1][e] -= xv[buf][q][e] * lv[buf][q].y;
+        acc[2][e] -= xv[buf][q][e] * lv[buf][q].z; acc[3][e] -= xv[buf][q][e] * lv[buf][q].w;
+      }
+  };
+  // `count` (even) groups; the loads of a group are in flight while the one before is applied.  The
+  // group loaded beyond the last one is dropped (its addresses lie inside the staged block and the factor).
+  auto groups = [&](int count) {
+#pragma unroll 1
+    for (int g = 0; g < count; g += 2) {
+      load(1);
+      apply(0);
+      load(0);
+      apply(1);
+    }
+  };
+  load(0);
+  if (split && S >= 2) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int e = 0; e < RT; ++e) acc[c][e] = 0.f;
+    groups(8 * (S - 1));
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      float t[RT];
+      rows_load(t_at(c), t);
+#pragma unroll
+      for (int e = 0; e < RT; ++e) acc[c][e] = t[e] + acc[c][e];
+    }
+    groups(8);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) rows_load(t_at(c), acc[c]);
+    groups(8 * S);
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    if constexpr (RT == 4) *reinterpret_cast<float4*>(t_at(c)) = make_float4(acc[c][0], acc[c][1], acc[c][2], acc[c][3]);
+    else if constexpr (RT == 2) *reinterpret_cast<float2*>(t_at(c)) = make_float2(acc[c][0], acc[c][1]);
+    else *t_at(c) = acc[c][0];
+  }
+}
+// RT and the split of the eight warps over row groups (RG) and columns: all 32 columns, or at most 16 of them in the
+// last super-block (the column groups would otherwise leave half the warps without work).
+__device__ __forceinline__ void solve_gemm_any(int tile_rows, float* x, const float* lt, int P, int S, bool split,
+                                               int nrows, int warp, int lane) {
+  const bool narrow = P - 32 * S <= 16;
+  if (tile_rows == kTile) {
+    if (narrow) solve_gemm<2, 4>(x, lt, P, S, split, nrows, warp, lane);
+    else solve_gemm<4, 2>(x, lt, P, S, split, nrows, warp, lane);
+  } else {
+    if (narrow) solve_gemm<1, 4>(x, lt, P, S, split, nrows, warp, lane);
+    else solve_gemm<2, 2>(x, lt, P, S, split, nrows, warp, lane);
+  }
+}
+// NG: groups of eight columns in the super-block (four but for the last one of a width that is not a multiple of 32)
+template <int NG>
+__device__ __forceinline__ void solve_diag_n(float* xr, const float* lt, const float* dinv, int P, int S, bool keep) {
+  float acc[8 * NG];
+  float* xb = xr + 32 * S * kXsLd;
+#pragma unroll
+  for (int e = 0; e < 8 * NG; ++e) acc[e] = xb[e * kXsLd];
+  const int a0 = 8 * S;
+  const float* lp = lt + 4 * a0 * P - 8 * a0 * (a0 - 1);      // row 32 S of the layout, at its first column 32 S
+  int stride = P - 32 * S;
+#pragma unroll
+  for (int a = 0; a < 2 * NG; ++a) {
+    const float4 d4 = *reinterpret_cast<const float4*>(dinv + 32 * S + 4 * a);
+    const float dv[4] = {d4.x, d4.y, d4.z, d4.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = 4 * a + q;
+      const float xi = acc[i] * dv[q];
+      acc[i] = xi;
+#pragma unroll
+      for (int v = a; v < 2 * NG; ++v) {
+        if (v == a && q == 3) continue;
+        const float4 l = *reinterpret_cast<const float4*>(lp + q * stride + 4 * (v - a));
+        const float lv[4] = {l.x, l.y, l.z, l.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (4 * v + e > i) acc[4 * v + e] -= xi * lv[e];
+      }
+    }
+    lp += 4 * stride;
+    stride -= 4;
+  }
+#pragma unroll
+  for (int e = 0; e < 8 * NG; ++e) xb[e * kXsLd] = keep ? acc[e] : 0.f;
+}
+__device__ __forceinline__ void solve_diag(float* xr, const float* lt, const float* dinv, int P, int S, bool keep) {
+  const int ng = (P - 32 * S) >> 3;
+  if (ng >= 4) solve_diag_n<4>(xr, lt, dinv, P, S, keep);
+  else if (ng == 3) solve_diag_n<3>(xr, lt, dinv, P, S, keep);
+  else if (ng == 2) solve_diag_n<2>(xr, lt, dinv, P, S, keep);
+  else solve_diag_n<1>(xr, lt, dinv, P, S, keep);
 }
 
-// Four rows i .. i+3 of the triangular layout (two float4 each) and the matching four x_i.
-struct SolveGroup {
-  float x[4];
-  float4 l[4][2];
-};
-__device__ __forceinline__ void solve_group_load(SolveGroup& g, uint32_t xs_row, uint32_t lt_at, int stride) {
-#pragma unroll
-  for (int q = 0; q < 4; ++q) g.x[q] = lds_f32(xs_row + q * kXsLd * 4);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    g.l[q][0] = lds_v4(lt_at + q * stride * 4);
-    g.l[q][1] = lds_v4(lt_at + q * stride * 4 + 16);
-  }
-}
-__device__ __forceinline__ void solve_group_apply(const SolveGroup& g, float (&acc)[8]) {
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    acc[0] -= g.x[q] * g.l[q][0].x; acc[1] -= g.x[q] * g.l[q][0].y;
-    acc[2] -= g.x[q] * g.l[q][0].z; acc[3] -= g.x[q] * g.l[q][0].w;
-    acc[4] -= g.x[q] * g.l[q][1].x; acc[5] -= g.x[q] * g.l[q][1].y;
-    acc[6] -= g.x[q] * g.l[q][1].z; acc[7] -= g.x[q] * g.l[q][1].w;
-  }
-}
-
-// acc[0..7] -= sum over the groups g0 .. g1-1 (four solved columns i each; g1 - g0 even) of
-// x_i * L[jb + e][i]: the part of the forward substitution for columns jb .. jb+7 that only needs
-// x_i already staged in xs[i * kXsLd + r].  The loads of one group are in flight while the previous
-// group is applied.
-__device__ __forceinline__ void solve_apply_groups(float (&acc)[8], int jb, int g0, int g1, uint32_t lt,
-                                                   uint32_t xs, int r, int P) {
-  if (g1 <= g0) return;
-  uint32_t xr = xs + (r + 4 * g0 * kXsLd) * 4;
-  uint32_t at = lt + (4 * g0 * P - 8 * g0 * (g0 - 1) + jb - 4 * g0) * 4;   // row 4 g0 of the layout, column jb
-  int stride = P - 4 * g0;                         // rows 4a .. 4a+3 have P - 4a entries
-  SolveGroup ga, gb;
-  solve_group_load(ga, xr, at, stride);
-  for (int g = g0; g < g1; g += 2) {
-    xr += 4 * kXsLd * 4; at += (4 * stride - 4) * 4; stride -= 4;
-    solve_group_load(gb, xr, at, stride);
-    solve_group_apply(ga, acc);
-    xr += 4 * kXsLd * 4; at += (4 * stride - 4) * 4; stride -= 4;
-    if (g + 2 < g1) solve_group_load(ga, xr, at, stride);
-    solve_group_apply(gb, acc);
-  }
-}
-// Triangular solve inside the block of columns jb .. jb+7: acc holds t - (contributions of the
-// columns before jb) on entry and x[jb..jb+7] on return.
-__device__ __forceinline__ void solve_inblock8(float (&acc)[8], int jb, uint32_t lt, uint32_t dinv, int P) {
-#pragma unroll
-  for (int jj = 0; jj < 8; ++jj) {
-    float x = acc[jj] * lds_f32(dinv + (jb + jj) * 4);
-    acc[jj] = x;
-    uint32_t lr = lt + (lt_row_offset(jb + jj, P) - (jj & ~3)) * 4;
-#pragma unroll
-    for (int j2 = jj + 1; j2 < 8; ++j2) acc[j2] -= x * lds_f32(lr + j2 * 4);
+// The whole solve of a staged block that starts x_off floats behind the base of shared memory, by the eight
+// epilogue warps; rows nrows and beyond (and all rows when keep_rows is false) come out as zeros.  Out of
+// line: see the rehearsal in subspace_kernel.
+__device__ __noinline__ void solve_team(int x_off, int P, int tile_rows, bool split, int nrows, bool keep_rows) {
+  float* x = reinterpret_cast<float*>(pow_smem()) + x_off;
+  const float* lt = reinterpret_cast<float*>(pow_smem() + kPowRegion);
+  const float* dinv = lt + kLtFloats;
+  const int et = threadIdx.x, warp = et >> 5, lane = et & 31, nS = (P + 31) >> 5;
+#pragma unroll 1
+  for (int S = 0; S < nS; ++S) {
+    if (S > 0) {
+      solve_gemm_any(tile_rows, x, lt, P, S, split, nrows, warp, lane);
+      named_barrier(1, 256);
+    }
+    if (warp < 4 && warp * 32 < nrows) solve_diag(x + et, lt, dinv, P, S, keep_rows && et < nrows);
+    named_barrier(1, 256);
   }
 }
 
@@ -387,55 +492,7 @@ __device__ __forceinline__ void dmma_8x8x4(double& c0, double& c1, double a, dou
                : "d"(a), "d"(b));
 }
 
-// The float64 Gram of the staged block is accumulated from 16-row slabs converted to float64 in
-// shared memory (slab[c * kSlabLd + row]); a warp owns two strips of 8x8 tiles, (ta, tb <= ta) and
-// (tz = nb8-1-ta, tb <= tz), so that every warp carries nb8 + 1 tiles.
-constexpr int kSlabRows = 16;
-constexpr int kSlabLd = 20;                      // doubles; conflict-free fragment loads
-constexpr int kMaxTiles8 = kPMax / 8;            // 20
-static_assert(kXsBytes + 2 * kPMax * kSlabLd * 8 <= kPowRegion, "slabs must fit behind the staged block");
-
-// Accumulator slots of one warp: strip ta (the shorter one) uses slots 0 .. ta for tb = slot,
-// strip tz uses slots kMaxTiles8 - tb for tb = 0 .. tz; ta + tz = nb8 - 1 <= 19, so they never meet.
-struct GramAcc {
-  double a[kMaxTiles8 + 1][2];
-};
-
-// The tensor-core instructions sit behind warp-uniform jump tables (switch fall-through), not
-// predicates: a predicated-off mma still occupies the FP64 pipe.
-#define COVSPEC_GRAM_A(u) case u: dmma_8x8x4(acc.a[u][0], acc.a[u][1], xa, b[u]);
-#define COVSPEC_GRAM_Z(t) case t: dmma_8x8x4(acc.a[kMaxTiles8 - t][0], acc.a[kMaxTiles8 - t][1], xz, b[t]);
-__device__ __forceinline__ void gram_unit_accumulate(GramAcc& acc, const double* slab, int ta, int tz,
-                                                     int lane) {
-  const int fr = lane >> 2, fk = lane & 3;
-  const double* base = slab + fr * kSlabLd + fk;
-#pragma unroll 1
-  for (int ks = 0; ks < kSlabRows / 4; ++ks) {
-    double b[kMaxTiles8];
-#pragma unroll
-    for (int t = 0; t < kMaxTiles8; ++t)
-      if (t <= tz) b[t] = base[t * 8 * kSlabLd + 4 * ks];
-    const double xa = base[ta * 8 * kSlabLd + 4 * ks], xz = base[tz * 8 * kSlabLd + 4 * ks];
-    switch (ta) {
-      COVSPEC_GRAM_A(19) COVSPEC_GRAM_A(18) COVSPEC_GRAM_A(17) COVSPEC_GRAM_A(16) COVSPEC_GRAM_A(15)
-      COVSPEC_GRAM_A(14) COVSPEC_GRAM_A(13) COVSPEC_GRAM_A(12) COVSPEC_GRAM_A(11) COVSPEC_GRAM_A(10)
-      COVSPEC_GRAM_A(9) COVSPEC_GRAM_A(8) COVSPEC_GRAM_A(7) COVSPEC_GRAM_A(6) COVSPEC_GRAM_A(5)
-      COVSPEC_GRAM_A(4) COVSPEC_GRAM_A(3) COVSPEC_GRAM_A(2) COVSPEC_GRAM_A(1) COVSPEC_GRAM_A(0)
-      default: break;
-    }
-    if (tz != ta) {
-      switch (tz) {
-        COVSPEC_GRAM_Z(19) COVSPEC_GRAM_Z(18) COVSPEC_GRAM_Z(17) COVSPEC_GRAM_Z(16) COVSPEC_GRAM_Z(15)
-        COVSPEC_GRAM_Z(14) COVSPEC_GRAM_Z(13) COVSPEC_GRAM_Z(12) COVSPEC_GRAM_Z(11) COVSPEC_GRAM_Z(10)
-        COVSPEC_GRAM_Z(9) COVSPEC_GRAM_Z(8) COVSPEC_GRAM_Z(7) COVSPEC_GRAM_Z(6) COVSPEC_GRAM_Z(5)
-        COVSPEC_GRAM_Z(4) COVSPEC_GRAM_Z(3) COVSPEC_GRAM_Z(2) COVSPEC_GRAM_Z(1) COVSPEC_GRAM_Z(0)
-        default: break;
-      }
-    }
-  }
-}
-#undef COVSPEC_GRAM_A
-#undef COVSPEC_GRAM_Z
+constexpr int kSlabRows = 16;            // the float64 Gram of a block takes its rows in groups of this many
 
 }  // namespace sub
 }  // namespace covspec
