@@ -231,6 +231,13 @@ int covspec_branch_candidates(int logit_dtype, int rows, int vocab, long long ld
                               const int* drafted, const int* cand_offsets, int max_fanout, int* cand,
                               void* stream);
 
+/* The same with cand_offsets on the host (read before the call returns; no copy to the device is made).
+ * Fan-outs up to 64, rows of at least 32 KB and a 16-byte aligned z_draft; else COVSPEC_ERR_UNSUPPORTED and
+ * nothing is launched. */
+int covspec_branch_candidates_host(int logit_dtype, int rows, int vocab, long long ld, const void* z_draft,
+                                   const int* drafted, const int* cand_offsets, int max_fanout, int* cand,
+                                   void* stream);
+
 /* Scalar host-side formulas of the link model and the draft-length controller.  No device work.
  *  covspec_uplink_bits       Eq. 7: N_draft * b_id + N_logit_draft * b_logit
  *  covspec_downlink_bits     Eq. 8: b_acc + b_bonus if all drafted tokens were accepted, else

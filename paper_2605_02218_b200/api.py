@@ -28,7 +28,7 @@ EXPORTS = [
     "covspec_last_launch_count", "covspec_strerror", "covspec_last_cuda_error",
     "covspec_profile_begin", "covspec_profile_end", "covspec_profile_stage_count",
     "covspec_profile_stage_name", "covspec_query_score_static", "covspec_selftest_wait_timeout",
-    "covspec_correct", "covspec_fanout", "covspec_branch_candidates",
+    "covspec_correct", "covspec_fanout", "covspec_branch_candidates", "covspec_branch_candidates_host",
     "covspec_uplink_bits", "covspec_downlink_bits", "covspec_comm_latency", "covspec_ema_update",
     "covspec_draft_length", "covspec_get_iteration_counts", "covspec_build_has_bounds_checks",
     "covspec_selftest_fill_workspace",
@@ -112,6 +112,7 @@ def load_library():
     lib.covspec_ema_update.restype = C.c_double
     lib.covspec_draft_length.argtypes = [C.c_int] + [C.c_double] * 6 + [C.c_int, C.c_int]
     lib.covspec_branch_candidates.argtypes = [C.c_int, C.c_int, C.c_int, C.c_longlong, vp, vp, vp, C.c_int, vp, vp]
+    lib.covspec_branch_candidates_host.argtypes = lib.covspec_branch_candidates.argtypes
     lib.covspec_correct.argtypes = [C.c_int, C.c_int, C.c_int, C.c_longlong, vp, vp, vp, vp, C.c_float,
                                     vp, vp, vp, vp, vp, vp]
     lib.covspec_last_launch_count.argtypes = [vp]
@@ -185,8 +186,13 @@ class _Marshalled:
                                keep_p, float(keep_ratio))
 
 
+def _raw_stream() -> int:
+    """The address torch.cuda.current_stream().cuda_stream gives, without making the Stream object (2-3 us)."""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return C.c_void_p(_raw_stream())
 
 
 class Pruner:
@@ -407,20 +413,19 @@ def correct(z_draft: torch.Tensor, z_target: torch.Tensor, uniforms: torch.Tenso
     """covspec_correct: gating (Eq. 16-17), acceptance probability (Eq. 5) and the residual
     correction draw (Eq. 6) for every row of two logit matrices [rows, ld] (ld >= vocab).
     Returns (margin, gate, accept, resid_mass, token) device tensors."""
-    lib = load_library()
+    lib = _lib or load_library()
     assert z_draft.is_cuda and z_draft.is_contiguous() and z_target.is_contiguous()
     assert z_draft.shape == z_target.shape and z_draft.dtype == z_target.dtype
     rows, ld = z_draft.shape
-    vocab = ld if vocab is None else vocab
     dev = z_draft.device
-    margin = torch.empty(rows, dtype=torch.float32, device=dev)
-    gate = torch.empty(rows, dtype=torch.int32, device=dev)
-    accept = torch.empty(rows, dtype=torch.float32, device=dev)
-    mass = torch.empty(rows, dtype=torch.float32, device=dev)
-    token = torch.empty(rows, dtype=torch.int32, device=dev)
-    st = lib.covspec_correct(_LOGIT_DTYPES[z_draft.dtype], rows, vocab, ld, _ptr(z_draft), _ptr(z_target),
-                             _ptr(drafted), _ptr(uniforms), float(gamma), _ptr(margin), _ptr(gate),
-                             _ptr(accept), _ptr(mass), _ptr(token), _stream())
+    # two allocations for the five results; plain integers for the addresses: on a drafted block of a few
+    # positions the call takes longer here than on the device
+    margin, accept, mass = torch.empty((3, rows), dtype=torch.float32, device=dev).unbind(0)
+    gate, token = torch.empty((2, rows), dtype=torch.int32, device=dev).unbind(0)
+    st = lib.covspec_correct(_LOGIT_DTYPES[z_draft.dtype], rows, ld if vocab is None else vocab, ld, z_draft.data_ptr(),
+                             z_target.data_ptr(), None if drafted is None else drafted.data_ptr(), uniforms.data_ptr(), gamma,
+                             margin.data_ptr(), gate.data_ptr(), accept.data_ptr(), mass.data_ptr(), token.data_ptr(),
+                             _raw_stream())
     if st:
         raise CovspecError(st, "covspec_correct")
     return margin, gate, accept, mass, token
@@ -438,17 +443,21 @@ def branch_candidates(z_draft: torch.Tensor, fanouts, drafted: Optional[torch.Te
                       vocab: Optional[int] = None):
     """covspec_branch_candidates: the F_j largest draft logits of every row, the drafted token
     excluded.  `fanouts`: one int per row.  Returns (cand int32 device tensor, offsets numpy)."""
-    lib = load_library()
+    lib = _lib or load_library()
     rows, ld = z_draft.shape
     vocab = ld if vocab is None else vocab
     f = np.asarray(fanouts, dtype=np.int64)
     assert len(f) == rows
-    off = np.concatenate([[0], np.cumsum(f)]).astype(np.int32)
-    d_off = torch.from_numpy(off).to(z_draft.device)
-    cand = torch.empty(max(int(off[-1]), 1), dtype=torch.int32, device=z_draft.device)
-    st = lib.covspec_branch_candidates(_LOGIT_DTYPES[z_draft.dtype], rows, vocab, ld, _ptr(z_draft),
-                                       _ptr(drafted), _ptr(d_off), int(f.max()) if rows else 0,
-                                       _ptr(cand), _stream())
+    off = np.zeros(rows + 1, dtype=np.int32)
+    np.cumsum(f, out=off[1:])
+    total, most = int(off[-1]), int(f.max()) if rows else 0
+    cand = torch.empty(max(total, 1), dtype=torch.int32, device=z_draft.device)
+    dtype, z, out = _LOGIT_DTYPES[z_draft.dtype], z_draft.data_ptr(), cand.data_ptr()
+    y, stream = None if drafted is None else drafted.data_ptr(), _raw_stream()
+    st = lib.covspec_branch_candidates_host(dtype, rows, vocab, ld, z, y, off.ctypes.data, most, out, stream)
+    if st == -3:                         # a fan-out or a row length that the host-offset form does not take
+        d_off = torch.from_numpy(off).to(z_draft.device)
+        st = lib.covspec_branch_candidates(dtype, rows, vocab, ld, z, y, d_off.data_ptr(), most, out, stream)
     if st:
         raise CovspecError(st, "covspec_branch_candidates")
-    return cand[:int(off[-1])], off
+    return (cand if total else cand[:0]), off

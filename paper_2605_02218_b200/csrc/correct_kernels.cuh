@@ -488,5 +488,134 @@ branch_candidates_kernel(const T* __restrict__ zd, long long ldz, int w, const i
                 cand + off, nullptr);
 }
 
+// The same for small fan-outs (the usual case: F_j = ceil(F_0 rho^j) of a handful): one cluster of eight
+// CTAs per position streams the row once.  The F_j-th largest of the 128 warps' maxima bounds the F_j-th
+// largest key of the row from below, so only the few threads that saw a key that large look at
+// their vectors again, and what they find (F_j entries and a few more) is ranked by one CTA.  One block
+// per position with five passes over the row read it at one SM's rate: 32 positions x 151,674 float16
+// logits 290 us.
+constexpr int kFastFanout = 64;                      // largest fan-out of this kernel
+constexpr int kFastCtas = 8, kFastThreads = 512;
+constexpr int kFastWarps = kFastCtas * kFastThreads / 32;
+constexpr int kFastMinVec = 32 * kFastFanout;        // shorter rows give fewer warps with a vector than F_j may ask for
+constexpr int kFastList = 1024;                      // entries that are ranked directly; more (mass ties): block_topk_by
+constexpr int kFastRows = 512;                       // positions per launch: their offsets travel as kernel arguments
+struct FanOffsets { int v[kFastRows + 1]; };
+
+__device__ __forceinline__ unsigned peer_addr(const void* p, unsigned cta) {
+  unsigned local = (unsigned)__cvta_generic_to_shared(p), remote;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(cta));
+  return remote;
+}
+
+template <typename T>
+__global__ void __cluster_dims__(kFastCtas, 1, 1) __launch_bounds__(kFastThreads)
+branch_fast_kernel(const T* __restrict__ zd, long long ldz, int w, const int* __restrict__ drafted,
+                   const int* __restrict__ dev_offsets, const __grid_constant__ FanOffsets host_offsets,
+                   int* __restrict__ cand) {
+  constexpr int N = Vec<T>::N;
+  __shared__ __align__(16) unsigned keys[kFastWarps];
+  __shared__ unsigned warp_best[kFastThreads / 32];
+  __shared__ unsigned s_threshold, s_count;
+  __shared__ unsigned list_key[kFastList];
+  __shared__ int list_id[kFastList];
+  __shared__ unsigned chosen[kFastList / 32];
+  const unsigned crank = cluster_rank();
+  const int row = blockIdx.x / kFastCtas, tid = threadIdx.x;
+  const int off = dev_offsets != nullptr ? dev_offsets[row] : host_offsets.v[row];
+  const int f = min((dev_offsets != nullptr ? dev_offsets[row + 1] : host_offsets.v[row + 1]) - off, w);
+  if (f <= 0) return;                                // the whole cluster
+  const T* r = zd + (size_t)row * ldz;
+  const int y = drafted != nullptr ? __ldg(drafted + row) : -1;
+  const int nvec = (w + N - 1) / N, first = (int)crank * kFastThreads + tid;
+  constexpr int kStep = kFastCtas * kFastThreads;
+  if (tid == 0) s_count = 0u;
+  auto key_at = [&](int i) { return order_key(i == y ? -INFINITY : cvt(r[i])); };
+  auto special = [&](int v) { return (v + 1) * N > w || (y >= v * N && y < (v + 1) * N); };   // row end, drafted token
+  unsigned mine = 0u;
+#pragma unroll 4
+  for (int v = first; v < nvec; v += kStep) {
+    if (special(v)) {
+      for (int i = v * N; i < min(w, (v + 1) * N); ++i) mine = max(mine, key_at(i));
+    } else {
+      mine = max(mine, order_key(vec_max(__ldg(reinterpret_cast<const uint4*>(r) + v), (const T*)nullptr)));
+    }
+  }
+  {
+    const unsigned m = __reduce_max_sync(0xffffffffu, mine);
+    if ((tid & 31) == 0) warp_best[tid >> 5] = m;
+  }
+  cluster_sync();                                    // every CTA's maxima are in its shared memory
+  if (tid < kFastWarps) {
+    unsigned k;
+    const unsigned a = peer_addr(&warp_best[tid & (kFastThreads / 32 - 1)], (unsigned)(tid / (kFastThreads / 32)));
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(k) : "r"(a) : "memory");
+    keys[tid] = k;
+  }
+  __syncthreads();
+  if (tid < kFastWarps) {
+    const unsigned k = keys[tid];
+    int rank = 0;                                    // maxima before this one in (larger, earlier) order
+#pragma unroll 8
+    for (int j = 0; j < kFastWarps; j += 4) {
+      const uint4 q = *reinterpret_cast<const uint4*>(keys + j);
+      rank += (q.x > k || (q.x == k && j < tid)) + (q.y > k || (q.y == k && j + 1 < tid)) +
+              (q.z > k || (q.z == k && j + 2 < tid)) + (q.w > k || (q.w == k && j + 3 < tid));
+    }
+    if (rank == f - 1) s_threshold = k;
+  }
+  __syncthreads();
+  const unsigned threshold = s_threshold;
+  if (mine >= threshold) {
+    auto take = [&](int i, unsigned k) {
+      if (k < threshold) return;
+      unsigned at;
+      asm volatile("atom.shared::cluster.add.u32 %0, [%1], 1;" : "=r"(at) : "r"(peer_addr(&s_count, 0u)) : "memory");
+      if (at < (unsigned)kFastList) {
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_addr(&list_key[at], 0u)), "r"(k) : "memory");
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_addr(&list_id[at], 0u)), "r"(i) : "memory");
+      }
+    };
+#pragma unroll 1
+    for (int v = first; v < nvec; v += kStep) {
+      if (special(v)) {
+        for (int i = v * N; i < min(w, (v + 1) * N); ++i) take(i, key_at(i));
+      } else {
+        const uint4 raw = __ldg(reinterpret_cast<const uint4*>(r) + v);
+        if (order_key(vec_max(raw, (const T*)nullptr)) < threshold) continue;
+        float e[N];
+        unpack(raw, e, (const T*)nullptr);
+#pragma unroll
+        for (int q = 0; q < N; ++q) take(v * N + q, order_key(e[q]));
+      }
+    }
+  }
+  cluster_sync();                                    // the list is complete in CTA 0
+  if (crank != 0) return;
+  const int n = (int)min(s_count, (unsigned)(kFastList + 1));
+  if (n > kFastList) {
+    block_topk_by([&](int i) { return i == y ? -INFINITY : cvt(r[i]); }, w, f, false, nullptr, cand + off, nullptr);
+    return;
+  }
+  // the F_j first in (larger key, lower id) order, written by ascending id
+  for (int q = tid; q < kFastList / 32; q += kFastThreads) chosen[q] = 0u;
+  __syncthreads();
+  for (int e = tid; e < n; e += kFastThreads) {
+    const unsigned k = list_key[e];
+    const int id = list_id[e];
+    int rank = 0;
+    for (int j = 0; j < n; ++j) rank += list_key[j] > k || (list_key[j] == k && list_id[j] < id);
+    if (rank < f) atomicOr(&chosen[e >> 5], 1u << (e & 31));
+  }
+  __syncthreads();
+  for (int e = tid; e < n; e += kFastThreads) {
+    if (!(chosen[e >> 5] >> (e & 31) & 1u)) continue;
+    const int id = list_id[e];
+    int pos = 0;
+    for (int j = 0; j < n; ++j) pos += (chosen[j >> 5] >> (j & 31) & 1u) && list_id[j] < id;
+    cand[off + pos] = id;
+  }
+}
+
 }  // namespace corr
 }  // namespace covspec

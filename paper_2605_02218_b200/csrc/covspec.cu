@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -1319,27 +1320,63 @@ int covspec_fanout(int f0, double rho, int j) {
   return (int)ceil((double)f0 * pow(rho, (double)j) - 1e-9);
 }
 
-int covspec_branch_candidates(int logit_dtype, int rows, int vocab, long long ld, const void* z_draft,
-                              const int* drafted, const int* cand_offsets, int max_fanout, int* cand,
-                              void* stream) {
-  if (!z_draft || !cand_offsets || !cand) return COVSPEC_ERR_ARG;
+}  // extern "C"
+
+namespace {
+
+// Offsets on the device or (dev_offsets == nullptr) on the host; see the two entry points.
+int branch_candidates_impl(int logit_dtype, int rows, int vocab, long long ld, const void* z_draft, const int* drafted,
+                           const int* dev_offsets, const int* host_offsets, int max_fanout, int* cand, cudaStream_t s) {
+  if (!z_draft || (!dev_offsets && !host_offsets) || !cand) return COVSPEC_ERR_ARG;
   if (logit_dtype != COVSPEC_F32 && logit_dtype != COVSPEC_BF16 && logit_dtype != COVSPEC_F16)
     return COVSPEC_ERR_ARG;
   int esize = logit_dtype == COVSPEC_F32 ? 4 : 2;
   if (rows < 1 || vocab < 2 || ld < vocab || (ld * esize) % 16 != 0) return COVSPEC_ERR_SHAPE;
   if (max_fanout < 0 || max_fanout > vocab - 1) return COVSPEC_ERR_SHAPE;
-  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (logit_dtype == COVSPEC_F32)
-    corr::branch_candidates_kernel<float><<<rows, 1024, 0, s>>>(static_cast<const float*>(z_draft), ld, vocab,
-                                                                drafted, cand_offsets, cand);
-  else if (logit_dtype == COVSPEC_BF16)
-    corr::branch_candidates_kernel<__nv_bfloat16><<<rows, 1024, 0, s>>>(
-        static_cast<const __nv_bfloat16*>(z_draft), ld, vocab, drafted, cand_offsets, cand);
-  else
-    corr::branch_candidates_kernel<__half><<<rows, 1024, 0, s>>>(static_cast<const __half*>(z_draft), ld, vocab,
-                                                                 drafted, cand_offsets, cand);
-  CUDA_TRY(cudaGetLastError());
-  return COVSPEC_OK;
+  // the cluster kernel reads whole 16-byte vectors; larger fan-outs, short rows and other bases take a
+  // block per row
+  const bool fast = max_fanout <= corr::kFastFanout && (reinterpret_cast<uintptr_t>(z_draft) & 15) == 0 &&
+                    (long long)vocab * esize >= 16ll * corr::kFastMinVec;
+  auto launch = [&](auto* tag) -> int {
+    using T = std::remove_pointer_t<decltype(tag)>;
+    const T* z = static_cast<const T*>(z_draft);
+    if (!fast) {
+      if (!dev_offsets) return COVSPEC_ERR_UNSUPPORTED;
+      corr::branch_candidates_kernel<T><<<rows, 1024, 0, s>>>(z, ld, vocab, drafted, dev_offsets, cand);
+      CUDA_TRY(cudaGetLastError());
+      return COVSPEC_OK;
+    }
+    corr::FanOffsets fo;
+    for (int r0 = 0; r0 < rows; r0 += corr::kFastRows) {
+      const int n = std::min(corr::kFastRows, rows - r0);
+      if (host_offsets) memcpy(fo.v, host_offsets + r0, sizeof(int) * (n + 1));
+      corr::branch_fast_kernel<T><<<n * corr::kFastCtas, corr::kFastThreads, 0, s>>>(
+          z + (size_t)r0 * ld, ld, vocab, drafted ? drafted + r0 : nullptr, dev_offsets ? dev_offsets + r0 : nullptr, fo, cand);
+      CUDA_TRY(cudaGetLastError());
+    }
+    return COVSPEC_OK;
+  };
+  return logit_dtype == COVSPEC_F32 ? launch((float*)nullptr)
+         : logit_dtype == COVSPEC_BF16 ? launch((__nv_bfloat16*)nullptr) : launch((__half*)nullptr);
+}
+
+}  // namespace
+
+extern "C" {
+
+int covspec_branch_candidates(int logit_dtype, int rows, int vocab, long long ld, const void* z_draft,
+                              const int* drafted, const int* cand_offsets, int max_fanout, int* cand,
+                              void* stream) {
+  if (!cand_offsets) return COVSPEC_ERR_ARG;
+  return branch_candidates_impl(logit_dtype, rows, vocab, ld, z_draft, drafted, cand_offsets, nullptr, max_fanout, cand,
+                                reinterpret_cast<cudaStream_t>(stream));
+}
+
+int covspec_branch_candidates_host(int logit_dtype, int rows, int vocab, long long ld, const void* z_draft,
+                                   const int* drafted, const int* cand_offsets, int max_fanout, int* cand,
+                                   void* stream) {
+  return branch_candidates_impl(logit_dtype, rows, vocab, ld, z_draft, drafted, nullptr, cand_offsets, max_fanout, cand,
+                                reinterpret_cast<cudaStream_t>(stream));
 }
 
 int covspec_selftest_wait_timeout(covspec_ctx* ctx, void* stream) {

@@ -107,3 +107,25 @@ def test_branch_candidates(dtype):
         for i in range(rows):
             want = C.bonus_candidates(zd[i], int(ys[i]), min(fan[i], vocab - 1))
             assert np.array_equal(cand[off[i]:off[i + 1]], want), (vocab, i)
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("vocab,rows,fan", [(16384, 3, 64), (16391, 2, 64), (32767, 520, 3), (40961, 5, 1), (151674, 4, 65)])
+def test_branch_candidates_at_the_limits_of_the_cluster_kernel(dtype, vocab, rows, fan):
+    # shortest rows and largest fan-out the cluster kernel takes, ragged ends, more rows than one launch
+    # carries, one past the largest fan-out; mass ties (more entries at the threshold than are ranked
+    # directly), the largest entry drafted, the last entry drafted
+    from paper_2605_02218_b200 import api
+    data = workloads.make_logits(seed=vocab, rows=rows, vocab=vocab, dtype=dtype, device="cuda:0")
+    z, y = data["z_draft"], data["drafted"]
+    y[0] = int(z[0, :vocab].float().argmax())
+    if rows > 1:
+        z[1, :vocab] = z[1, :vocab].clamp(-1, 1)
+        y[1] = vocab - 1
+    fans = [max(0, fan - i % 3) for i in range(rows)]
+    cand, off = api.branch_candidates(z, fans, y, vocab=vocab)
+    torch.cuda.synchronize()
+    cand = cand.cpu().numpy()
+    for i in sorted({0, 1, rows // 2, rows - 1} & set(range(rows))):
+        want = C.bonus_candidates(z[i, :vocab].cpu().double().numpy(), int(y[i]), fans[i])
+        assert np.array_equal(cand[off[i]:off[i + 1]], want), i
