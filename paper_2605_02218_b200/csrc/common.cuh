@@ -59,6 +59,11 @@ struct LayerPtrs {
   const void* h[kMaxLayers];
 };
 
+// Index of the calling warp in its block, handed round by a shuffle so that the compiler knows it to be the
+// same in all lanes.  A branch on threadIdx.x / 32 counts as divergent: every shuffle and vote inside it
+// became a call that gathers the warp first, about 280 cycles each.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

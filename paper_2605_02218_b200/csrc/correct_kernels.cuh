@@ -4,7 +4,7 @@
 // max(p_t - p_d, 0) / mass and a token drawn from it by inverse CDF with a uniform number supplied by
 // the caller.
 //
-// One cluster of two CTAs per position.  Both logit rows (2 * W * elem bytes, ~600 KB at W = 152 k
+// One cluster of CTAs per position.  Both logit rows (2 * W * elem bytes, ~600 KB at W = 152 k
 // in 16 bits) are read from HBM once; the second sweep (residual mass) and the short third one (the
 // cumulative sum inside the one warp segment that contains the sample) find them in L2.  Each warp
 // owns a contiguous segment of the row and reads it with coalesced 16-byte vectors, so the order of
@@ -14,17 +14,18 @@
 #pragma once
 #include <cuda_fp16.h>
 
+#include <atomic>
+
 #include "common.cuh"
 #include "select_kernels.cuh"
 
 namespace covspec {
 namespace corr {
 
-constexpr int kClusterCtas = 2;                       // CTAs that share one position
 constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kCtasPerSm = 2;                         // resident CTAs per SM the register budget allows
-constexpr int kSegs = kClusterCtas * kWarps;         // warp segments of a row
+constexpr int kSegs = 32;                            // segments of a row, one warp's work with two CTAs per position
 constexpr int kMaxChunks = 256;                      // chunks of a segment whose totals fit in shared memory
 
 __device__ __forceinline__ float cvt(float v) { return v; }
@@ -96,9 +97,13 @@ __device__ __forceinline__ void load_vec(const T* __restrict__ row, int i, int w
 // Running (max, sum of exp(z - max)) pair of a softmax denominator.
 struct MaxSum {
   float m, s;
+  // Branch-free: in a reduction by shuffles half of the lanes take either side, and the code for both
+  // sides of five steps, run once per position, was fetched line by line (11 k cycles for four steps).
   __device__ __forceinline__ void merge(const MaxSum& o) {
-    if (o.m > m) { s = s * __expf(m - o.m) + o.s; m = o.m; }
-    else if (o.m > -INFINITY) s += o.s * __expf(o.m - m);
+    const bool up = o.m > m;
+    const float hm = up ? o.m : m, hs = up ? o.s : s, lm = up ? m : o.m, ls = up ? s : o.s;
+    m = hm;
+    s = lm > -INFINITY ? fmaf(ls, __expf(lm - hm), hs) : hs;
   }
 };
 __device__ __forceinline__ MaxSum shfl_xor(const MaxSum& a, int o) {
@@ -119,7 +124,10 @@ struct Top2 {
   __device__ __forceinline__ void add(float z) {
     if (z > a) { b = a; a = z; } else if (z > b) b = z;
   }
-  __device__ __forceinline__ void merge(const Top2& o) { add(o.a); add(o.b); }
+  __device__ __forceinline__ void merge(const Top2& o) {
+    b = fmaxf(fminf(a, o.a), fmaxf(b, o.b));
+    a = fmaxf(a, o.a);
+  }
 };
 
 // Branch-free trackers of the two largest logits of the vectors one thread sees.  The 16-bit types
@@ -166,7 +174,7 @@ template <> struct Top2Run<__nv_bfloat16> {
 // reference: exp(60) ~ 1e26 leaves room for a whole vocabulary of such terms in float32.
 constexpr float kRefSlack = 60.f;
 
-// ---- thread-block cluster helpers (a position is shared by the kClusterCtas CTAs of a cluster) ----
+// ---- thread-block cluster helpers (a position is shared by the CTAs of a cluster) ----
 __device__ __forceinline__ unsigned cluster_rank() {
   unsigned r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -175,44 +183,64 @@ __device__ __forceinline__ unsigned cluster_rank() {
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// A float of the shared memory of CTA `cta` of the cluster, at the address `p` has in this CTA.
-__device__ __forceinline__ float peer_float(const float* p, unsigned cta) {
+// The address `p` (shared memory of this CTA) has in CTA `cta` of the cluster.
+__device__ __forceinline__ unsigned peer_addr(const void* p, unsigned cta) {
   unsigned local = (unsigned)__cvta_generic_to_shared(p), remote;
-  float v;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(cta));
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote) : "memory");
-  return v;
+  return remote;
+}
+// Partial results are pushed into every CTA's shared memory ahead of a cluster barrier: a warp that
+// fetches 32 scattered values of a peer waits 1.5-2 k cycles per load.
+__device__ __forceinline__ void peer_store(unsigned addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ void peer_store(unsigned addr, float2 v) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void peer_store(unsigned addr, float4 v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+               : "memory");
 }
 
 // rows: positions; w: vocabulary size; ldz: elements between consecutive rows (multiple of 16 bytes).
 //
-// One cluster of kClusterCtas CTAs per position, two CTAs resident per SM: the sweep that streams
-// the rows from HBM in one CTA overlaps the sweeps that re-read them from L2 (special-function
-// bound) in the other CTA of the SM, while the positions in flight (one per cluster: 148 x 600 KB)
-// still fit in L2 - with one whole position per CTA and two CTAs per SM they would not.  The row is
-// cut into kSegs contiguous warp segments in row order (CTA rank, warp); partial results cross the
-// cluster through distributed shared memory.
-template <typename T>
-__global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kThreads, kCtasPerSm)
+// The row is cut into kSegs = 32 contiguous segments of whole 16-byte vectors; lane l of a segment owns its
+// vectors l, l + 32, ... and adds their sums up in that order, whatever the number of warps that share the
+// work, so that a result does not depend on how many positions a call has.
+//   CL = 2: one cluster of two CTAs per position, one warp per segment, two CTAs resident per SM: the sweep
+//           that streams the rows from HBM in one CTA overlaps the sweeps that re-read them from L2
+//           (special-function bound) in the other CTA of the SM, while the positions in flight (one per
+//           cluster) still fit in L2.
+//   CL = 4, 8: 2 or 4 warps per segment, for calls with too few positions to fill the SMs: chunks of 32
+//           vectors are dealt over the warps of the segment, the vector sums go through shared memory and
+//           one warp adds them up.
+// Partial results cross the cluster through distributed shared memory.  With `store` the residual sums of
+// the vectors stay in shared memory: the draw then only scans them and evaluates one chunk of 32 vectors
+// again, instead of the whole segment.
+template <typename T, int CL>
+__global__ void __launch_bounds__(kThreads, kCtasPerSm)
 correct_kernel(const T* __restrict__ zd, const T* __restrict__ zt, long long ldz, int w,
                const int* __restrict__ drafted, const float* __restrict__ uniforms, float gamma,
                float* __restrict__ margin, int* __restrict__ gate, float* __restrict__ accept,
-               float* __restrict__ resid_mass, int* __restrict__ token) {
+               float* __restrict__ resid_mass, int* __restrict__ token, int store) {
   constexpr int N = Vec<T>::N;
-  __shared__ MaxSum sh_d[kWarps], sh_t[kWarps];
-  __shared__ Top2 sh_top[kWarps];
-  __shared__ float sh_part[6];                 // this CTA's (max, sum) pairs and two largest draft logits
-  __shared__ float sh_mass[2][kWarps];         // this CTA's warp masses (residual pass, p_t pass)
-  __shared__ float sh_all[kSegs];              // warp masses of the whole cluster, in row order
-  __shared__ float sh_chunk[kMaxChunks];       // totals of the 32-vector chunks of the segment that holds the sample
-  __shared__ float bc[2];
-  __shared__ int sh_token;
+  constexpr int WPS = CL * kWarps / kSegs;         // warps per segment
+  constexpr int SPC = kSegs / CL;                  // segments per CTA
+  extern __shared__ float vec_sums[];              // [SPC][chunks][32] (store), [2][SPC][chunks][32] (WPS > 1)
+  // results of the whole cluster, filled in by every CTA
+  __shared__ float4 sh_seg[kSegs];                 // per segment: (max, sum) pairs of the draft and the target row
+  __shared__ float2 sh_top[CL * kWarps];           // per warp: two largest draft logits
+  __shared__ float sh_mass[2][kSegs];              // segment masses in row order (residual pass, p_t pass)
+  __shared__ float sh_chunk[kMaxChunks];           // totals of the 32-vector chunks of the segment that holds the sample
   const unsigned crank = cluster_rank();
-  const int row = blockIdx.x / kClusterCtas, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int seg_id = (int)crank * kWarps + warp;
+  const int row = blockIdx.x / CL, tid = threadIdx.x, lane = tid & 31, warp = warp_index();
+  const int ls = warp / WPS, sub = warp % WPS;     // segment inside the CTA, warp inside the segment
+  const int seg_id = (int)crank * SPC + ls;
   const T* rd = zd + (size_t)row * ldz;
   const T* rt = zt + (size_t)row * ldz;
   const T* const tag = nullptr;
+  // peers may be written to once they have started: waited for after the first sweep
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   // scalars of the position, requested now so that their latency hides behind the first sweep
   const float x_uniform = __ldg(uniforms + row);
   float zd_y = 0.f, zt_y = 0.f;
@@ -225,10 +253,16 @@ correct_kernel(const T* __restrict__ zd, const T* __restrict__ zt, long long ldz
   // contiguous segment of this warp, in whole vectors
   const int nvec = (w + N - 1) / N;
   const int vec_per_seg = (nvec + kSegs - 1) / kSegs;
+  const int chunks = (vec_per_seg + 31) >> 5;
   const int v0 = min(nvec, seg_id * vec_per_seg), v1 = min(nvec, v0 + vec_per_seg);
+  // vectors that lie wholly inside the row, then the one that straddles its end (if any)
+  const int nfull = w / N, f1 = min(v1, nfull);
+  const bool owns_tail = nfull < nvec && nfull >= v0 && nfull < v1 && ((nfull - v0) & 31) == lane;
+  float* my_sums = vec_sums + (size_t)ls * chunks * 32 + lane;                       // + 32 * chunk
+  float* my_sums2 = my_sums + (size_t)SPC * chunks * 32;
 
   // ---- sweep 1: softmax denominators of both rows (Eq. 2, 4), two largest draft logits (Eq. 16) ----
-  // The sums run relative to a reference logit of this thread, in the base-2 domain:
+  // The sums run relative to a reference logit of this lane, in the base-2 domain:
   // exp(z - m) = 2^(z log2(e) - m log2(e)).  The reference is the largest logit of the first vector
   // and moves only when a logit lies more than kRefSlack above it (any reference gives the same
   // quotient; the slack keeps the terms inside the float32 range), so the branch is rarely taken.
@@ -236,11 +270,8 @@ correct_kernel(const T* __restrict__ zd, const T* __restrict__ zt, long long ldz
   float nd = 0.f, nt = 0.f;                     // -m log2(e) of the two references
   float thr_d = -INFINITY, thr_t = -INFINITY;   // reference + slack
   Top2Run<T> top_run;
-  auto sweep1 = [&](const uint4& ra, const uint4& rb) {
-    // every vector holds at least one element of the vocabulary; 2^(-inf) = 0 takes care of padding
-    const float va = vec_max(ra, tag), vb = vec_max(rb, tag);
-    if (va > thr_d) { md.s *= __expf(md.m - va); md.m = va; nd = -va * kLog2e; thr_d = va + kRefSlack; }
-    if (vb > thr_t) { mt.s *= __expf(mt.m - vb); mt.m = vb; nt = -vb * kLog2e; thr_t = vb + kRefSlack; }
+  // sum of exp over one vector of either row, terms in element order
+  auto exp_sums = [&](const uint4& ra, const uint4& rb) {
     float a[N], b[N];
     unpack(ra, a, tag);
     unpack(rb, b, tag);
@@ -250,100 +281,164 @@ correct_kernel(const T* __restrict__ zd, const T* __restrict__ zt, long long ldz
       sa += ex2(fmaf(a[k], kLog2e, nd));
       sb += ex2(fmaf(b[k], kLog2e, nt));
     }
-    md.s += sa;
-    mt.s += sb;
-    top_run.add(ra);
+    return make_float2(sa, sb);
   };
-  // vectors that lie wholly inside the row, then the one that straddles its end (if any)
-  const int nfull = w / N, f1 = min(v1, nfull);
-  const bool owns_tail = nfull < nvec && nfull >= v0 && nfull < v1 && ((nfull - v0) & 31) == lane;
-  {
+  auto move_reference = [&](float va, float vb) {
+    if (va > thr_d) { md.s *= __expf(md.m - va); md.m = va; nd = -va * kLog2e; thr_d = va + kRefSlack; }
+    if (vb > thr_t) { mt.s *= __expf(mt.m - vb); mt.m = vb; nt = -vb * kLog2e; thr_t = vb + kRefSlack; }
+  };
+  auto sweep1 = [&](const uint4& ra, const uint4& rb) {
+    // every vector holds at least one element of the vocabulary; 2^(-inf) = 0 takes care of padding
+    move_reference(vec_max(ra, tag), vec_max(rb, tag));
+    const float2 s = exp_sums(ra, rb);
+    md.s += s.x;
+    mt.s += s.y;
+  };
+  auto sweep1_segment = [&]() {                 // the whole segment by one warp
     const uint4* pa = reinterpret_cast<const uint4*>(rd) + v0 + lane;
     const uint4* pb = reinterpret_cast<const uint4*>(rt) + v0 + lane;
 #pragma unroll 2
-    for (int v = v0 + lane; v < f1; v += 32, pa += 32, pb += 32) sweep1(__ldg(pa), __ldg(pb));
-    if (owns_tail) sweep1(load_raw(rd, nfull * N, w), load_raw(rt, nfull * N, w));
-  }
-  Top2 top = top_run.result();
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    md.merge(shfl_xor(md, o));
-    mt.merge(shfl_xor(mt, o));
-    Top2 other{__shfl_xor_sync(0xffffffffu, top.a, o), __shfl_xor_sync(0xffffffffu, top.b, o)};
-    top.merge(other);
-  }
-  if (lane == 0) { sh_d[warp] = md; sh_t[warp] = mt; sh_top[warp] = top; }
-  __syncthreads();
-  if (warp == 0) {
-    if (lane < kWarps) { md = sh_d[lane]; mt = sh_t[lane]; top = sh_top[lane]; }
-    else { md = MaxSum{-INFINITY, 0.f}; mt = md; top = Top2{-INFINITY, -INFINITY}; }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      md.merge(shfl_xor(md, o));
-      mt.merge(shfl_xor(mt, o));
-      Top2 other{__shfl_xor_sync(0xffffffffu, top.a, o), __shfl_xor_sync(0xffffffffu, top.b, o)};
-      top.merge(other);
+    for (int v = v0 + lane; v < f1; v += 32, pa += 32, pb += 32) {
+      const uint4 ra = __ldg(pa), rb = __ldg(pb);
+      sweep1(ra, rb);
+      if (WPS == 1) top_run.add(ra);
     }
-    if (lane == 0) {
-      sh_part[0] = md.m; sh_part[1] = md.s; sh_part[2] = mt.m; sh_part[3] = mt.s;
-      sh_part[4] = top.a; sh_part[5] = top.b;
+    if (owns_tail) {
+      const uint4 ra = load_raw(rd, nfull * N, w);
+      sweep1(ra, load_raw(rt, nfull * N, w));
+      if (WPS == 1) top_run.add(ra);
     }
-  }
-  cluster_sync();                               // every CTA's partial results are in its shared memory
-  if (warp == 0) {
-    // the same merge, in rank order, in every CTA of the cluster
-    md = MaxSum{-INFINITY, 0.f}; mt = md; top = Top2{-INFINITY, -INFINITY};
-    // lane 6 c + k fetches value k of CTA c; the values are then handed round by shuffles
-    float mine = 0.f;
-    if (lane < 6 * kClusterCtas) mine = peer_float(&sh_part[lane % 6], (unsigned)(lane / 6));
-    for (int c = 0; c < kClusterCtas; ++c) {
-      MaxSum od{__shfl_sync(0xffffffffu, mine, 6 * c), __shfl_sync(0xffffffffu, mine, 6 * c + 1)};
-      MaxSum ot{__shfl_sync(0xffffffffu, mine, 6 * c + 2), __shfl_sync(0xffffffffu, mine, 6 * c + 3)};
-      Top2 otop{__shfl_sync(0xffffffffu, mine, 6 * c + 4), __shfl_sync(0xffffffffu, mine, 6 * c + 5)};
-      md.merge(od); mt.merge(ot); top.merge(otop);
+  };
+  if constexpr (WPS == 1) {
+    sweep1_segment();
+  } else {
+    // the lane's reference is that of its first vector; a warp that meets a logit too far above it makes
+    // one warp go through the segment again in order
+    const int vref = v0 + lane < v1 ? v0 + lane : -1;
+    if (vref >= 0) move_reference(vec_max(load_raw(rd, vref * N, w), tag), vec_max(load_raw(rt, vref * N, w), tag));
+    bool moved = false;
+#pragma unroll 2
+    for (int c = sub; c < chunks; c += WPS) {
+      const int v = v0 + 32 * c + lane;
+      if (v < v1) {
+        const uint4 ra = load_raw(rd, v * N, w), rb = load_raw(rt, v * N, w);
+        moved |= vec_max(ra, tag) > thr_d || vec_max(rb, tag) > thr_t;
+        const float2 s = exp_sums(ra, rb);
+        my_sums[32 * c] = s.x;
+        my_sums2[32 * c] = s.y;
+        top_run.add(ra);
+      }
     }
-    if (lane == 0) {
-      // exponent offsets of the two distributions: p = 2^(z log2(e) + bc)
-      bc[0] = -(md.m * kLog2e + log2f(md.s));
-      bc[1] = -(mt.m * kLog2e + log2f(mt.s));
-      if (crank == 0) {
-        float m = (1.f - (top.b > -INFINITY ? __expf(top.b - top.a) : 0.f)) * __expf(top.a - md.m) / md.s;
-        margin[row] = m;
-        gate[row] = m < gamma ? 1 : 0;                                       // Eq. 17
-        if (accept != nullptr) {
-          float al = 1.f;
-          if (has_y) {
-            float pd = __expf(zd_y - md.m) / md.s, pt = __expf(zt_y - mt.m) / mt.s;
-            al = pd > 0.f ? fminf(1.f, pt / pd) : 1.f;                       // Eq. 5
-          }
-          accept[row] = al;
-        }
+    const int again = __syncthreads_or(moved);
+    if (sub == 0) {
+      if (again) {
+        md = MaxSum{-INFINITY, 0.f}; mt = md;
+        thr_d = thr_t = -INFINITY;
+        sweep1_segment();
+      } else {
+#pragma unroll 4
+        for (int c = 0; c < chunks; ++c)
+          if (v0 + 32 * c + lane < v1) { md.s += my_sums[32 * c]; mt.s += my_sums2[32 * c]; }
       }
     }
   }
-  __syncthreads();
-  const float cd = bc[0], ct = bc[1];
+  Top2 top = top_run.result();
+#pragma unroll 1
+  for (int o = 16; o > 0; o >>= 1) {
+    if (sub == 0) { md.merge(shfl_xor(md, o)); mt.merge(shfl_xor(mt, o)); }
+    Top2 other{__shfl_xor_sync(0xffffffffu, top.a, o), __shfl_xor_sync(0xffffffffu, top.b, o)};
+    top.merge(other);
+  }
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  if (lane < CL) {
+    if (sub == 0) peer_store(peer_addr(&sh_seg[seg_id], (unsigned)lane), make_float4(md.m, md.s, mt.m, mt.s));
+    peer_store(peer_addr(&sh_top[(int)crank * kWarps + warp], (unsigned)lane), make_float2(top.a, top.b));
+  }
+  cluster_sync();                               // every CTA has all partial results
+  // the same merge in every warp of the cluster: lane q holds segment q; each half of the segments is
+  // merged in a butterfly of its own, then the two halves
+  const float4 mine_seg = sh_seg[lane];
+  MaxSum sd{mine_seg.x, mine_seg.y}, st{mine_seg.z, mine_seg.w};
+  top = Top2{-INFINITY, -INFINITY};
+#pragma unroll
+  for (int q = 0; q < WPS; ++q) {
+    const float2 o = sh_top[lane * WPS + q];
+    top.merge(Top2{o.x, o.y});
+  }
+#pragma unroll 1
+  for (int o = 8; o > 0; o >>= 1) {             // inside the halves
+    sd.merge(shfl_xor(sd, o)); st.merge(shfl_xor(st, o));
+    Top2 other{__shfl_xor_sync(0xffffffffu, top.a, o), __shfl_xor_sync(0xffffffffu, top.b, o)};
+    top.merge(other);
+  }
+  {
+    Top2 other{__shfl_xor_sync(0xffffffffu, top.a, 16), __shfl_xor_sync(0xffffffffu, top.b, 16)};
+    top.merge(other);
+  }
+  // the lower half's result, then the upper half's, in every lane
+  md = MaxSum{__shfl_sync(0xffffffffu, sd.m, 0), __shfl_sync(0xffffffffu, sd.s, 0)};
+  mt = MaxSum{__shfl_sync(0xffffffffu, st.m, 0), __shfl_sync(0xffffffffu, st.s, 0)};
+  md.merge(MaxSum{__shfl_sync(0xffffffffu, sd.m, 16), __shfl_sync(0xffffffffu, sd.s, 16)});
+  mt.merge(MaxSum{__shfl_sync(0xffffffffu, st.m, 16), __shfl_sync(0xffffffffu, st.s, 16)});
+  // exponent offsets of the two distributions: p = 2^(z log2(e) + offset)
+  const float cd = -(md.m * kLog2e + log2f(md.s)), ct = -(mt.m * kLog2e + log2f(mt.s));
+  if (crank == 0 && tid == 0) {                 // off the critical path of the other warps
+    float m = (1.f - (top.b > -INFINITY ? __expf(top.b - top.a) : 0.f)) * __expf(top.a - md.m) / md.s;
+    margin[row] = m;
+    gate[row] = m < gamma ? 1 : 0;                                       // Eq. 17
+    if (accept != nullptr) {
+      float al = 1.f;
+      if (has_y) {
+        float pd = __expf(zd_y - md.m) / md.s, pt = __expf(zt_y - mt.m) / mt.s;
+        al = pd > 0.f ? fminf(1.f, pt / pd) : 1.f;                       // Eq. 5
+      }
+      accept[row] = al;
+    }
+  }
 
-  // ---- sweep 2: residual mass per warp segment (Eq. 6 denominator) ----
+  // ---- sweep 2: residual mass per segment (Eq. 6 denominator) ----
   // use_pt: the residual is identically zero (the two distributions coincide): draw from p_t.
   for (int use_pt = 0; use_pt < 2; ++use_pt) {
     float part = 0.f;
     if (!use_pt) {
-      auto sweep2 = [&](const uint4& ra, const uint4& rb) {
+      auto residual = [&](const uint4& ra, const uint4& rb) {         // summed over one vector, in element order
         float a[N], b[N];
         unpack(ra, a, tag);
         unpack(rb, b, tag);
         float acc = 0.f;
 #pragma unroll
         for (int k = 0; k < N; ++k) acc += fmaxf(prob(b[k], ct) - prob(a[k], cd), 0.f);
-        part += acc;
+        return acc;
       };
-      const uint4* pa = reinterpret_cast<const uint4*>(rd) + v0 + lane;
-      const uint4* pb = reinterpret_cast<const uint4*>(rt) + v0 + lane;
+      if constexpr (WPS == 1) {
+        const uint4* pa = reinterpret_cast<const uint4*>(rd) + v0 + lane;
+        const uint4* pb = reinterpret_cast<const uint4*>(rt) + v0 + lane;
+        float* keep = my_sums;
 #pragma unroll 2
-      for (int v = v0 + lane; v < f1; v += 32, pa += 32, pb += 32) sweep2(__ldg(pa), __ldg(pb));
-      if (owns_tail) sweep2(load_raw(rd, nfull * N, w), load_raw(rt, nfull * N, w));
-    } else {
+        for (int v = v0 + lane; v < f1; v += 32, pa += 32, pb += 32, keep += 32) {
+          const float acc = residual(__ldg(pa), __ldg(pb));
+          if (store) *keep = acc;
+          part += acc;
+        }
+        if (owns_tail) {
+          const float acc = residual(load_raw(rd, nfull * N, w), load_raw(rt, nfull * N, w));
+          if (store) my_sums[nfull - v0 - lane] = acc;
+          part += acc;
+        }
+      } else {
+#pragma unroll 2
+        for (int c = sub; c < chunks; c += WPS) {
+          const int v = v0 + 32 * c + lane;
+          if (v < v1) my_sums[32 * c] = residual(load_raw(rd, v * N, w), load_raw(rt, v * N, w));
+        }
+        __syncthreads();
+        if (sub == 0)
+#pragma unroll 4
+          for (int c = 0; c < chunks; ++c)
+            if (v0 + 32 * c + lane < v1) part += my_sums[32 * c];
+      }
+    } else if (sub == 0) {
       for (int v = v0 + lane; v < v1; v += 32) {
         float b[N];
         load_vec(rt, v * N, w, b);
@@ -352,11 +447,11 @@ correct_kernel(const T* __restrict__ zd, const T* __restrict__ zt, long long ldz
       }
     }
     part = warp_sum(part);
-    if (lane == 0) sh_mass[use_pt][warp] = part;
-    cluster_sync();                             // the masses of every CTA are in its shared memory
-    if (tid < kSegs) sh_all[tid] = peer_float(&sh_mass[use_pt][tid % kWarps], (unsigned)(tid / kWarps));
-    __syncthreads();
+    if (sub == 0 && lane < CL) peer_store(peer_addr(&sh_mass[use_pt][seg_id], (unsigned)lane), part);
+    cluster_sync();                             // every CTA has all segment masses (the last access to a peer)
+    const float* sh_all = sh_mass[use_pt];
     float mass = 0.f;
+#pragma unroll
     for (int q = 0; q < kSegs; ++q) mass += sh_all[q];                    // same order in every thread
     if (!use_pt && crank == 0 && tid == 0 && resid_mass != nullptr) resid_mass[row] = mass;
     if (mass > 0.f || use_pt) {
@@ -364,12 +459,12 @@ correct_kernel(const T* __restrict__ zd, const T* __restrict__ zt, long long ldz
       const float target = x_uniform * mass;
       float before = 0.f;
       int seg = -1;
+#pragma unroll
       for (int q = 0; q < kSegs; ++q) {
-        if (seg < 0 && before + sh_all[q] > target) seg = q;
-        if (seg < 0) before += sh_all[q];
+        const float next = before + sh_all[q];
+        if (seg < 0 && next > target) seg = q;
+        if (seg < 0) before = next;
       }
-      if (tid == 0) sh_token = -2;              // -2: the segment belongs to another CTA
-      __syncthreads();
       float tgt = target;
       if (seg < 0) {
         // rounding left x * mass at or above the total: the last token with positive probability,
@@ -378,13 +473,13 @@ correct_kernel(const T* __restrict__ zd, const T* __restrict__ zt, long long ldz
         while (seg > 0 && !(sh_all[seg] > 0.f)) --seg;
         tgt = INFINITY;
       }
+      if (seg / SPC != (int)crank) break;       // another CTA's segment
       // The segment is walked in chunks of 32 vectors.  The warps of the CTA that owns it first
       // sum the chunks in parallel; the walk then starts at the first chunk whose running total
       // passes the target (running totals added up in chunk order, as the walk itself would).
       const int sv0 = min(nvec, seg * vec_per_seg), sv1 = min(nvec, sv0 + vec_per_seg);
       const int nchunks = (sv1 - sv0 + 31) >> 5;
-      const bool mine_cta = seg / kWarps == (int)crank;
-      const bool skip_ahead = mine_cta && nchunks <= kMaxChunks && tgt != INFINITY;
+      const bool skip_ahead = nchunks <= kMaxChunks && tgt != INFINITY;
       auto chunk_values = [&](int v, float (&r)[N]) -> float {
         float lsum = 0.f;
         if (v < sv1) {
@@ -404,9 +499,11 @@ correct_kernel(const T* __restrict__ zd, const T* __restrict__ zt, long long ldz
         return lsum;
       };
       if (skip_ahead) {
+        const float* kept = vec_sums + (size_t)(seg - (int)crank * SPC) * chunks * 32 + lane;
         for (int c = warp; c < nchunks; c += kWarps) {
-          float r[N];
-          float inc = chunk_values(sv0 + 32 * c + lane, r);
+          float r[N], inc;
+          if (store && !use_pt) inc = sv0 + 32 * c + lane < sv1 ? kept[32 * c] : 0.f;
+          else inc = chunk_values(sv0 + 32 * c + lane, r);
 #pragma unroll
           for (int o = 1; o < 32; o <<= 1) {          // the same inclusive scan the walk uses
             float t = __shfl_up_sync(0xffffffffu, inc, o);
@@ -416,7 +513,7 @@ correct_kernel(const T* __restrict__ zd, const T* __restrict__ zt, long long ldz
         }
       }
       __syncthreads();
-      if (seg_id == seg) {
+      if (seg_id == seg && sub == 0) {
         float run = before;
         int first_chunk = 0;
         if (skip_ahead) {
@@ -449,12 +546,8 @@ correct_kernel(const T* __restrict__ zd, const T* __restrict__ zt, long long ldz
           if (hit) { found = __shfl_sync(0xffffffffu, mine, __ffs(hit) - 1); break; }
           run += __shfl_sync(0xffffffffu, inc, 31);
         }
-        if (lane == 0) sh_token = found >= 0 ? found : last_pos;
-      }
-      __syncthreads();
-      if (tid == 0 && sh_token != -2) {
-        int tk = sh_token;
-        if (tk < 0) {
+        int tk = found >= 0 ? found : last_pos;
+        if (tk < 0 && lane == 0) {
           // the chosen segment held no positive entry at all (possible only through rounding):
           // scan back for the last positive probability in the whole row
           for (int i = w - 1; i >= 0 && tk < 0; --i) {
@@ -462,13 +555,63 @@ correct_kernel(const T* __restrict__ zd, const T* __restrict__ zt, long long ldz
             if ((use_pt ? pt : pt - pd) > 0.f) tk = i;
           }
         }
-        token[row] = tk;
+        if (lane == 0) token[row] = tk;
       }
       break;
     }
     __syncthreads();
   }
-  cluster_sync();                               // no CTA leaves while its shared memory may be read
+}
+
+// CTAs per position.  Two are enough once every SM has its two CTAs (148 positions); fewer positions are
+// spread over up to eight CTAs each, as many as still run at the same time (two CTAs on each of 148
+// SMs), so that a drafted block of eight positions uses 64 SMs instead of 16.
+inline int cluster_ctas(int rows) { return rows > 74 ? 2 : rows > 37 ? 4 : 8; }
+constexpr size_t kSumsMost = 96 * 1024;              // shared memory for the vector sums: two CTAs per SM
+// Dynamic shared memory of a CTA: one sum per vector of its segments, two where several warps share one.
+template <typename T>
+size_t sums_bytes(int cl, int w) {
+  const int nvec = (w + Vec<T>::N - 1) / Vec<T>::N, chunks = ((nvec + kSegs - 1) / kSegs + 31) / 32;
+  return (size_t)(kSegs / cl) * chunks * 32 * sizeof(float) * (cl > 2 ? 2 : 1);
+}
+
+template <typename T, int CL>
+cudaError_t launch_correct_n(int rows, const T* zd, const T* zt, long long ldz, int w, const int* drafted,
+                             const float* uniforms, float gamma, float* margin, int* gate, float* accept,
+                             float* resid_mass, int* token, cudaStream_t s) {
+  static std::atomic<unsigned long long> configured{0};   // bit per device; setting the attribute twice is harmless
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev >= 64 || !(configured.load(std::memory_order_acquire) >> dev & 1ull)) {
+    e = cudaFuncSetAttribute(correct_kernel<T, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSumsMost);
+    if (e != cudaSuccess) return e;
+    if (dev < 64) configured.fetch_or(1ull << dev, std::memory_order_release);
+  }
+  const size_t bytes = sums_bytes<T>(CL, w);
+  const bool store = bytes <= kSumsMost;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)rows * CL);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = store ? bytes : 0;
+  cfg.stream = s;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = CL;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, correct_kernel<T, CL>, zd, zt, ldz, w, drafted, uniforms, gamma, margin, gate, accept,
+                            resid_mass, token, store ? 1 : 0);
+}
+template <typename T>
+cudaError_t launch_correct(int rows, const T* zd, const T* zt, long long ldz, int w, const int* drafted,
+                           const float* uniforms, float gamma, float* margin, int* gate, float* accept,
+                           float* resid_mass, int* token, cudaStream_t s) {
+  int cl = cluster_ctas(rows);
+  if (sums_bytes<T>(cl, w) > kSumsMost) cl = 2;       // a row too long for sums in shared memory: two CTAs need none
+  const auto f = cl == 2 ? launch_correct_n<T, 2> : cl == 4 ? launch_correct_n<T, 4> : launch_correct_n<T, 8>;
+  return f(rows, zd, zt, ldz, w, drafted, uniforms, gamma, margin, gate, accept, resid_mass, token, s);
 }
 
 // Bonus-token candidates of the parallel branching (Sec. III-C.1, Eq. 23): for every position the
@@ -501,12 +644,6 @@ constexpr int kFastMinVec = 32 * kFastFanout;        // shorter rows give fewer 
 constexpr int kFastList = 1024;                      // entries that are ranked directly; more (mass ties): block_topk_by
 constexpr int kFastRows = 512;                       // positions per launch: their offsets travel as kernel arguments
 struct FanOffsets { int v[kFastRows + 1]; };
-
-__device__ __forceinline__ unsigned peer_addr(const void* p, unsigned cta) {
-  unsigned local = (unsigned)__cvta_generic_to_shared(p), remote;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(cta));
-  return remote;
-}
 
 template <typename T>
 __global__ void __cluster_dims__(kFastCtas, 1, 1) __launch_bounds__(kFastThreads)

@@ -1265,19 +1265,13 @@ int covspec_correct(int logit_dtype, int rows, int vocab, long long ld, const vo
   if (rows < 1 || vocab < 2 || ld < vocab || (ld * esize) % 16 != 0) return COVSPEC_ERR_SHAPE;
   if ((reinterpret_cast<uintptr_t>(z_draft) | reinterpret_cast<uintptr_t>(z_target)) & 15) return COVSPEC_ERR_ARG;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (logit_dtype == COVSPEC_F32)
-    corr::correct_kernel<float><<<rows * corr::kClusterCtas, corr::kThreads, 0, s>>>(
-        static_cast<const float*>(z_draft), static_cast<const float*>(z_target), ld, vocab, drafted,
-        uniforms, gamma, margin, gate, accept, resid_mass, token);
-  else if (logit_dtype == COVSPEC_BF16)
-    corr::correct_kernel<__nv_bfloat16><<<rows * corr::kClusterCtas, corr::kThreads, 0, s>>>(
-        static_cast<const __nv_bfloat16*>(z_draft), static_cast<const __nv_bfloat16*>(z_target), ld,
-        vocab, drafted, uniforms, gamma, margin, gate, accept, resid_mass, token);
-  else
-    corr::correct_kernel<__half><<<rows * corr::kClusterCtas, corr::kThreads, 0, s>>>(
-        static_cast<const __half*>(z_draft), static_cast<const __half*>(z_target), ld, vocab, drafted,
-        uniforms, gamma, margin, gate, accept, resid_mass, token);
-  CUDA_TRY(cudaGetLastError());
+  auto launch = [&](auto* tag) {
+    using T = std::remove_pointer_t<decltype(tag)>;
+    return corr::launch_correct<T>(rows, static_cast<const T*>(z_draft), static_cast<const T*>(z_target), ld, vocab, drafted,
+                                   uniforms, gamma, margin, gate, accept, resid_mass, token, s);
+  };
+  CUDA_TRY(logit_dtype == COVSPEC_F32 ? launch((float*)nullptr)
+           : logit_dtype == COVSPEC_BF16 ? launch((__nv_bfloat16*)nullptr) : launch((__half*)nullptr));
   return COVSPEC_OK;
 }
 

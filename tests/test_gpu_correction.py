@@ -129,3 +129,21 @@ def test_branch_candidates_at_the_limits_of_the_cluster_kernel(dtype, vocab, row
     for i in sorted({0, 1, rows // 2, rows - 1} & set(range(rows))):
         want = C.bonus_candidates(z[i, :vocab].cpu().double().numpy(), int(y[i]), fans[i])
         assert np.array_equal(cand[off[i]:off[i + 1]], want), i
+
+
+@pytest.mark.parametrize("rows", [1, 37, 38, 74, 75])
+def test_result_of_a_position_does_not_depend_on_the_call_size(rows):
+    # 8, 4 or 2 CTAs share a position, by the number of positions of the call; every split adds its sums
+    # up in the same order, so a position gives the same bits in a call of 160 positions as in a small one;
+    # a spread-out row makes the running reference of the sums move in the middle of a segment
+    from paper_2605_02218_b200 import api
+    vocab = 40013
+    data = workloads.make_logits(seed=5, rows=160, vocab=vocab, dtype=torch.float32, device="cuda:0")
+    data["z_draft"][0, 20000:vocab] += 200.0
+    data["z_target"][min(36, rows - 1), 30000:vocab] += 150.0
+    args = lambda n: (data["z_draft"][:n], data["z_target"][:n], data["uniforms"][:n], 0.05, data["drafted"][:n])
+    whole = api.correct(*args(160), vocab=vocab)
+    part = api.correct(*args(rows), vocab=vocab)
+    torch.cuda.synchronize()
+    for a, b in zip(whole, part):
+        assert torch.equal(a[:rows], b)
