@@ -7,6 +7,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <string>
 #include <type_traits>
@@ -17,6 +18,7 @@
 #include "eig_kernels.cuh"
 #include "gemm_simt.cuh"
 #include "greedy_kernels.cuh"
+#include "identity_tc.cuh"
 #include "relevance_tc.cuh"
 #include "relevance_pair.cuh"
 #include "subspace_tc.cuh"
@@ -510,6 +512,43 @@ bool tc_supported(const covspec_ctx* ctx) {
          c.head_dim == tc::kHeadDim && c.head_reduce == 0 && c.d >= tc::kBK;
 }
 
+// Eq. 10 with the identity embedding on the tensor cores: bf16 rows whose bases TMA can address, at least one
+// whole k-chunk of features.
+bool identity_tc_usable(int dtype, int d, const void* X, const void* Q) {
+  return dtype == COVSPEC_BF16 && d >= ident::kChunk && d % 8 == 0 &&
+         ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Q)) & 15) == 0;
+}
+// One launch over `tiles` 128-token tiles; plan == nullptr: the requests come with `reqs`.
+int launch_identity_tc(const void* X, const void* Q, long long rows_x, long long rows_q, int d, int t_max,
+                       const ReqPlan* plan, const ident::InlineReqs& reqs, int batch, int tiles, int num_sms,
+                       float* s_query, int* status, cudaStream_t s) {
+  static std::atomic<unsigned long long> configured{0};      // bit per device
+  int dev = 0;
+  CUDA_TRY(cudaGetDevice(&dev));
+  const int most = 224 * 1024;
+  if (dev >= 64 || !(configured.load(std::memory_order_acquire) >> dev & 1ull)) {
+    CUDA_TRY(cudaFuncSetAttribute(ident::identity_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    if (dev < 64) configured.fetch_or(1ull << dev, std::memory_order_release);
+  }
+  ident::IdParams prm{};
+  prm.plan = plan; prm.batch = batch;
+  prm.k_chunks = (d + ident::kChunk - 1) / ident::kChunk;
+  prm.n_cols = std::min(ident::kQueries, (t_max + 15) / 16 * 16);
+  prm.stage_bytes = ident::kBytesX + prm.n_cols * ident::kChunk * 2;
+  // a deep ring when every tile has an SM to itself (latency), else two CTAs share one
+  const int budget = (tiles <= num_sms ? most : 112 * 1024) - ident::kTailBytes - 1024;
+  prm.stages = std::max(2, std::min({ident::kMaxStages, prm.k_chunks, budget / prm.stage_bytes}));
+  prm.s_query = s_query; prm.status = status;
+  CUtensorMap map_x, map_q;
+  int st;
+  if ((st = make_map_bf16(&map_x, X, rows_x, d, ident::kTokens))) return st;
+  if ((st = make_map_bf16(&map_q, Q, rows_q, d, prm.n_cols))) return st;
+  const int smem = prm.stages * prm.stage_bytes + ident::kTailBytes + 1024;
+  ident::identity_tc_kernel<<<tiles, ident::kIdThreads, smem, s>>>(map_x, map_q, reqs, prm);
+  CUDA_TRY(cudaGetLastError());
+  return COVSPEC_OK;
+}
+
 // Eq. 10 on the tensor cores, two-SM form (relevance_pair.cuh): query embedding (MODE 1), -inf fill,
 // fused projection + cosine max over pairs of token tiles.
 int relevance_pair(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cudaStream_t s) {
@@ -648,14 +687,16 @@ int score_impl(covspec_ctx* ctx, const covspec_problem* p, float* s_query, float
   if (!s_act) s_act = ctx->sa;
   bool identity = cfg.n_heads == 0;
   bool use_tc = tc_supported(ctx);
+  bool identity_tc = identity && cfg.relevance_path != 1 && identity_tc_usable(cfg.dtype, cfg.d, X, Q);
   // The tensor-core relevance kernel leaves HBM idle: the activity stream runs beside it on the
   // context's side stream (fork here, join before the scores are fused).
-  bool overlap = use_tc && cfg.act_layers > 0 && cfg.activity_overlap > 0;
+  // The identity kernel reads X once and is done early: the full-rate activity kernel fills the SMs it leaves.
+  bool overlap = (use_tc || identity_tc) && cfg.act_layers > 0 && cfg.activity_overlap > 0;
   if (overlap) {
     CUDA_TRY(cudaEventRecord(ctx->ev_fork, s));
     CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
     prof_mark(ctx, ST_ACTIVITY, 0, ctx->side);
-    int st = launch_activity<T>(ctx, p, s_act, true, ctx->side);
+    int st = launch_activity<T>(ctx, p, s_act, use_tc, ctx->side);
     if (st) return st;
     prof_mark(ctx, ST_ACTIVITY, 1, ctx->side);
     CUDA_TRY(cudaEventRecord(ctx->ev_join, ctx->side));
@@ -675,6 +716,13 @@ int score_impl(covspec_ctx* ctx, const covspec_problem* p, float* s_query, float
     }
     int st = cfg.relevance_path == 2 ? relevance_pair(ctx, p, s_query, s) : relevance_tc(ctx, p, s_query, s);
     if (st) return st;
+  } else if (identity_tc) {
+    prof_mark(ctx, ST_RELEVANCE, 0, s);
+    int st = launch_identity_tc(X, Q, rowsX, rowsQ, cfg.d, pl.t_max, ctx->d_plan, ident::InlineReqs{}, B, pl.n_tiles,
+                                ctx->num_sms, s_query, ctx->status, s);
+    if (st) return st;
+    ++ctx->launches;
+    prof_mark(ctx, ST_RELEVANCE, 1, s);
   } else {
   prof_mark(ctx, ST_QEMBED, 0, s);
   if (identity) {
@@ -1475,6 +1523,28 @@ __global__ void static_plan_kernel(ReqPlan* __restrict__ plan, const StaticPlanC
 template <typename T>
 int query_score_static_impl(int d, int batch, const int* vis_offsets, const int* txt_offsets,
                             const void* X, const void* Q, float* s_query, cudaStream_t s) {
+  if (std::is_same<T, __nv_bfloat16>::value && identity_tc_usable(COVSPEC_BF16, d, X, Q)) {
+    // tensor cores: the requests travel as kernel arguments, no scratch is used
+    int dev = 0, num_sms = 148;
+    CUDA_TRY(cudaGetDevice(&dev));
+    CUDA_TRY(cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev));
+    for (int b0 = 0; b0 < batch; b0 += ident::kInlineReqs) {
+      ident::InlineReqs reqs;
+      const int count = std::min(ident::kInlineReqs, batch - b0);
+      int tiles = 0, t_max = 0;
+      for (int i = 0; i < count; ++i) {
+        const int b = b0 + i, n = vis_offsets[b + 1] - vis_offsets[b], t = txt_offsets[b + 1] - txt_offsets[b];
+        reqs.e[i] = make_int4(vis_offsets[b], n, txt_offsets[b], t);
+        reqs.tile_off[i] = tiles;
+        tiles += (n + ident::kTokens - 1) / ident::kTokens;
+        t_max = std::max(t_max, t);
+      }
+      int st = launch_identity_tc(X, Q, vis_offsets[batch], txt_offsets[batch], d, t_max, nullptr, reqs, count, tiles,
+                                  num_sms, s_query, nullptr, s);
+      if (st) return st;
+    }
+    return COVSPEC_OK;
+  }
   unsigned char* scratch = nullptr;
   int st = static_scratch_ptr(&scratch);
   if (st) return st;
