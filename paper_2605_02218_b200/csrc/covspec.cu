@@ -525,7 +525,7 @@ int launch_identity_tc(const void* X, const void* Q, long long rows_x, long long
   static std::atomic<unsigned long long> configured{0};      // bit per device
   int dev = 0;
   CUDA_TRY(cudaGetDevice(&dev));
-  const int most = 224 * 1024;
+  const int most = 208 * 1024;
   if (dev >= 64 || !(configured.load(std::memory_order_acquire) >> dev & 1ull)) {
     CUDA_TRY(cudaFuncSetAttribute(ident::identity_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     if (dev < 64) configured.fetch_or(1ull << dev, std::memory_order_release);
@@ -534,17 +534,21 @@ int launch_identity_tc(const void* X, const void* Q, long long rows_x, long long
   prm.plan = plan; prm.batch = batch;
   prm.k_chunks = (d + ident::kChunk - 1) / ident::kChunk;
   prm.n_cols = std::min(ident::kQueries, (t_max + 15) / 16 * 16);
-  prm.stage_bytes = ident::kBytesX + prm.n_cols * ident::kChunk * 2;
-  // a deep ring when every tile has an SM to itself (latency), else two CTAs share one
-  const int budget = (tiles <= num_sms ? most : 112 * 1024) - ident::kTailBytes - 1024;
+  prm.tile_rows = tiles <= num_sms ? ident::kTokens / 2 : ident::kTokens;
+  const int blocks = tiles * (ident::kTokens / prm.tile_rows);
+  // a deep ring when every block has an SM to itself, else two share one; what is left serves the blocks of
+  // the activity kernel beside it
+  prm.stage_bytes = (prm.tile_rows + prm.n_cols) * ident::kChunk * 2;
+  const int slack = 64 * 128;               // rows 64-127 of the last stage's X tile, read and dropped
+  const int budget = (blocks <= num_sms ? 208 : 104) * 1024 - ident::kTailBytes - 1024 - slack;
   prm.stages = std::max(2, std::min({ident::kMaxStages, prm.k_chunks, budget / prm.stage_bytes}));
   prm.s_query = s_query; prm.status = status;
   CUtensorMap map_x, map_q;
   int st;
-  if ((st = make_map_bf16(&map_x, X, rows_x, d, ident::kTokens))) return st;
+  if ((st = make_map_bf16(&map_x, X, rows_x, d, prm.tile_rows))) return st;
   if ((st = make_map_bf16(&map_q, Q, rows_q, d, prm.n_cols))) return st;
-  const int smem = prm.stages * prm.stage_bytes + ident::kTailBytes + 1024;
-  ident::identity_tc_kernel<<<tiles, ident::kIdThreads, smem, s>>>(map_x, map_q, reqs, prm);
+  const int smem = prm.stages * prm.stage_bytes + slack + ident::kTailBytes + 1024;
+  ident::identity_tc_kernel<<<blocks, ident::kIdThreads, smem, s>>>(map_x, map_q, reqs, prm);
   CUDA_TRY(cudaGetLastError());
   return COVSPEC_OK;
 }
@@ -692,14 +696,19 @@ int score_impl(covspec_ctx* ctx, const covspec_problem* p, float* s_query, float
   // context's side stream (fork here, join before the scores are fused).
   // The identity kernel reads X once and is done early: the full-rate activity kernel fills the SMs it leaves.
   bool overlap = (use_tc || identity_tc) && cfg.act_layers > 0 && cfg.activity_overlap > 0;
-  if (overlap) {
-    CUDA_TRY(cudaEventRecord(ctx->ev_fork, s));
+  auto fork_activity = [&]() -> int {
     CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
     prof_mark(ctx, ST_ACTIVITY, 0, ctx->side);
     int st = launch_activity<T>(ctx, p, s_act, use_tc, ctx->side);
     if (st) return st;
     prof_mark(ctx, ST_ACTIVITY, 1, ctx->side);
     CUDA_TRY(cudaEventRecord(ctx->ev_join, ctx->side));
+    return COVSPEC_OK;
+  };
+  if (overlap) CUDA_TRY(cudaEventRecord(ctx->ev_fork, s));
+  if (overlap && use_tc) {
+    int st = fork_activity();
+    if (st) return st;
   }
   if (use_tc) {
     if (ctx->split_tc) {
@@ -723,6 +732,8 @@ int score_impl(covspec_ctx* ctx, const covspec_problem* p, float* s_query, float
     if (st) return st;
     ++ctx->launches;
     prof_mark(ctx, ST_RELEVANCE, 1, s);
+    // after the identity kernel, whose few large blocks would otherwise wait for the activity blocks to end
+    if (overlap && (st = fork_activity())) return st;
   } else {
   prof_mark(ctx, ST_QEMBED, 0, s);
   if (identity) {
@@ -1100,7 +1111,7 @@ int covspec_prune_init(const covspec_config* cfg, covspec_ctx** out) {
     ok = ctx->tc_ready;
   }
   if (ok) {
-    // The background activity kernel shares its SMs with the relevance kernel, whose CTA needs the
+    // The activity kernels share their SMs with the relevance kernels, whose CTAs need the
     // largest shared-memory carve-out: ask for the same split, or the two could not be resident on
     // one SM at the same time (an SM changes its L1 / shared-memory split only when it is idle).
     auto max_shared = [](auto* kernel) {
@@ -1109,7 +1120,9 @@ int covspec_prune_init(const covspec_config* cfg, covspec_ctx** out) {
     };
     ok = max_shared(activity_stream_kernel<__nv_bfloat16, 4>) && max_shared(activity_stream_kernel<__nv_bfloat16, 8>) &&
          max_shared(activity_stream_kernel<__nv_bfloat16, 16>) && max_shared(activity_stream_kernel<float, 4>) &&
-         max_shared(activity_stream_kernel<float, 8>) && max_shared(activity_stream_kernel<float, 16>);
+         max_shared(activity_stream_kernel<float, 8>) && max_shared(activity_stream_kernel<float, 16>) &&
+         max_shared(activity_kernel<__nv_bfloat16, 4>) && max_shared(activity_kernel<__nv_bfloat16, 8>) &&
+         max_shared(activity_kernel<__nv_bfloat16, 16>);      // beside the identity kernel
   }
   if (ok) {
     // tensor maps over the workspace arrays of the subspace iteration (fixed for the context)

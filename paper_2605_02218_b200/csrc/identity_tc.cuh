@@ -8,7 +8,8 @@
 // up in registers: the tensor core's sums truncate, and short chains keep that near the rounding of
 // ordinary float32 sums.
 //
-// One CTA per 128-token tile of a request; the request's query elements pass in groups of up to 128.
+// One CTA per 128-token tile of a request (or per 64 tokens, while that leaves at most two CTAs per SM: a
+// block is bound by the latency of its loads and by shared-memory bandwidth); the request's query elements pass in groups of up to 128.
 // Warps 0-3: one token per thread (length of x, epilogue); 4-7: one query element per thread (length of
 // q); warp 8: TMA producer; warp 9: MMA issuer and TMEM owner.  Bound by HBM (X once).  The CUDA-core
 // kernel (cosmax_kernel, one warp per token) read every query element once per token through L1: 16
@@ -24,8 +25,7 @@ using namespace tc;
 constexpr int kTokens = 128;             // tokens per tile (UMMA M)
 constexpr int kQueries = 128;            // query elements per pass (UMMA N at most)
 constexpr int kChunk = 64;               // features per k-chunk (one 128-byte swizzle row)
-constexpr int kBytesX = kTokens * kChunk * 2;          // 16 KB
-constexpr int kMaxStages = 8;
+constexpr int kMaxStages = 12;
 constexpr int kColumns = 256;            // TMEM columns: two CTAs fit on an SM
 constexpr int kIdThreads = 320;
 constexpr int kGroupChunks = 8;          // k-chunks per accumulation group, if TMEM has the columns
@@ -44,24 +44,38 @@ struct IdParams {
   int k_chunks;
   int n_cols;                            // query elements per pass, a multiple of 16
   int stages, stage_bytes;
+  int tile_rows;                         // tokens per block: 128 or 64
   float* s_query;
   int* status;                           // may be nullptr
 };
 
-// Sum of squares of one 128-byte row of a swizzled tile.
-__device__ __forceinline__ void add_row_squares(const uint8_t* tile, int r, float& s0, float& s1) {
+// Sums of squares of one 128-byte row of a swizzled tile, in four pairs of running sums (packed float32
+// multiply-adds; short chains, the loads of a row in flight together).
+__device__ __forceinline__ void add_row_squares(const uint8_t* tile, int r, unsigned long long (&acc)[4]) {
   const uint8_t* row = tile + r * 128;
+  uint4 v[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) v[c] = *reinterpret_cast<const uint4*>(row + ((c ^ (r & 7)) * 16));
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
-    const uint4 v = *reinterpret_cast<const uint4*>(row + ((c ^ (r & 7)) * 16));
-    const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+    const uint32_t u[4] = {v[c].x, v[c].y, v[c].z, v[c].w};
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const float lo = __uint_as_float(u[e] << 16), hi = __uint_as_float(u[e] & 0xffff0000u);
-      s0 = fmaf(lo, lo, s0);
-      s1 = fmaf(hi, hi, s1);
+      unsigned long long x;
+      asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(u[e] << 16), "r"(u[e] & 0xffff0000u));
+      asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(acc[e]) : "l"(x));
     }
   }
+}
+__device__ __forceinline__ float total_squares(const unsigned long long (&acc)[4]) {
+  float s = 0.f;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(acc[e]));
+    s += lo + hi;
+  }
+  return s;
 }
 // 1 / sqrt(ss); 0 for a zero row, NaN for a row that is not finite.
 __device__ __forceinline__ float inverse_length(float ss) {
@@ -99,18 +113,21 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
+  // tile_rows = 64: two blocks share a 128-token tile (the MMA still computes 128 rows: the upper 64 read whatever
+  // follows in the ring and go nowhere)
+  const int R = prm.tile_rows, item = (int)blockIdx.x / (kTokens / R), half = (int)blockIdx.x % (kTokens / R);
   int vis_off, n, txt_off, T, tile;
   if (prm.plan != nullptr) {
-    const int b = find_request((int)blockIdx.x, prm.batch, [&](int q) { return prm.plan[q].tile_off; });
+    const int b = find_request(item, prm.batch, [&](int q) { return prm.plan[q].tile_off; });
     vis_off = prm.plan[b].vis_off; n = prm.plan[b].n; txt_off = prm.plan[b].txt_off; T = prm.plan[b].t;
-    tile = (int)blockIdx.x - prm.plan[b].tile_off;
+    tile = item - prm.plan[b].tile_off;
   } else {
-    const int b = find_request((int)blockIdx.x, prm.batch, [&](int q) { return reqs.tile_off[q]; });
+    const int b = find_request(item, prm.batch, [&](int q) { return reqs.tile_off[q]; });
     vis_off = reqs.e[b].x; n = reqs.e[b].y; txt_off = reqs.e[b].z; T = reqs.e[b].w;
-    tile = (int)blockIdx.x - reqs.tile_off[b];
+    tile = item - reqs.tile_off[b];
   }
-  const int row0 = vis_off + tile * kTokens, nrows = min(kTokens, n - tile * kTokens);
-  const int passes = (T + prm.n_cols - 1) / prm.n_cols;
+  const int at = tile * kTokens + half * R, row0 = vis_off + at, nrows = min(R, n - at);
+  const int passes = nrows > 0 ? (T + prm.n_cols - 1) / prm.n_cols : 0;
   // accumulation groups: contiguous ranges of k-chunks, one set of TMEM columns each
   const int group_cols = (prm.n_cols + 31) & ~31;
   const int n_groups = max(1, min(kColumns / group_cols, (prm.k_chunks + kGroupChunks - 1) / kGroupChunks));
@@ -128,7 +145,7 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
           mbar_expect_tx(&full[s], prm.stage_bytes);
           const uint32_t dst = smem_u32(smem + (size_t)s * prm.stage_bytes);
           tma_load_2d(dst, &map_x, kc * kChunk, row0, &full[s]);
-          tma_load_2d(dst + kBytesX, &map_q, kc * kChunk, txt_off + pass * prm.n_cols, &full[s]);
+          tma_load_2d(dst + R * 128, &map_q, kc * kChunk, txt_off + pass * prm.n_cols, &full[s]);
           if (++s == prm.stages) { s = 0; ph ^= 1u; }
         }
     }
@@ -146,7 +163,7 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
           if (!(ok = mbar_wait(&full[s], ph, abort_flag))) break;
           tc_fence_after();
           const uint32_t x_addr = smem_u32(smem + (size_t)s * prm.stage_bytes);
-          const uint64_t adesc = umma_desc(x_addr), bdesc = umma_desc(x_addr + kBytesX);
+          const uint64_t adesc = umma_desc(x_addr), bdesc = umma_desc(x_addr + R * 128);
           const int g = kc / per_group;
 #pragma unroll
           for (int k = 0; k < kChunk / 16; ++k)
@@ -167,18 +184,18 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     int s = 0;
     uint32_t ph = 0;
     for (int pass = 0; pass < passes; ++pass) {
-      float s0 = 0.f, s1 = 0.f;
-      const bool measure = tokens ? pass == 0 : r < prm.n_cols;
+      unsigned long long sq[4] = {0ull, 0ull, 0ull, 0ull};
+      const bool measure = tokens ? pass == 0 && (warp & 3) * 32 < nrows : r < prm.n_cols;
       for (int kc = 0; kc < prm.k_chunks; ++kc) {
         ok = ok && mbar_wait(&full[s], ph, abort_flag);
-        if (measure) add_row_squares(smem + (size_t)s * prm.stage_bytes + (tokens ? 0 : kBytesX), r, s0, s1);
+        if (measure) add_row_squares(smem + (size_t)s * prm.stage_bytes + (tokens ? 0 : R * 128), r, sq);
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[s]);
         if (++s == prm.stages) { s = 0; ph ^= 1u; }
       }
-      if (tokens && pass == 0) { inv_x = inverse_length(s0 + s1); nonfinite = inv_x != inv_x; }
+      if (tokens && pass == 0) { inv_x = inverse_length(total_squares(sq)); nonfinite = inv_x != inv_x; }
       named_barrier(1, 256);                           // the previous pass no longer reads inv_q
-      if (!tokens && measure) inv_q[r] = inverse_length(s0 + s1);
+      if (!tokens && measure) inv_q[r] = inverse_length(total_squares(sq));
       named_barrier(1, 256);
       if (tokens) {
         ok = ok && mbar_wait(acc_full, pass & 1u, abort_flag);

@@ -234,38 +234,51 @@ __device__ __forceinline__ float block_reduce(float v, Op op, float identity, fl
 
 struct NormParams { float shift, scale; };
 
-// Parameters (shift, scale) such that normalised = (s - shift) * scale, per request.
-__device__ __forceinline__ NormParams norm_params(const float* s, int n, int mode, float* scratch,
-                                                   int* status) {
+// Parameters (shift, scale) such that normalised = (s - shift) * scale, per request.  `at(j)` is the thread's
+// j-th score, that of token threadIdx.x + j * blockDim.x; PER > 0: at most PER per thread, unrolled.
+template <int PER, typename At>
+__device__ __forceinline__ NormParams norm_params_by(At at, int n, int mode, float* scratch, int* status) {
   NormParams np{0.f, 1.f};
   if (mode == 2) return np;
   auto fmin2 = [](float a, float b) { return fminf(a, b); };
   auto fmax2 = [](float a, float b) { return fmaxf(a, b); };
   auto fadd2 = [](float a, float b) { return a + b; };
+  const int mine = (n - (int)threadIdx.x + (int)blockDim.x - 1) / (int)blockDim.x;     // this thread's tokens (<= 0: none)
+  auto each = [&](auto f) {
+    if constexpr (PER > 0) {
+#pragma unroll
+      for (int j = 0; j < PER; ++j)
+        if (j < mine) f(at(j));
+    } else {
+      for (int j = 0; j < mine; ++j) f(at(j));
+    }
+  };
   bool bad = false;
   if (mode == 0) {
     float lo = FLT_MAX, hi = -FLT_MAX;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      float v = s[i];
+    each([&](float v) {
       bad |= !isfinite(v);
       lo = fminf(lo, v); hi = fmaxf(hi, v);
-    }
+    });
     lo = block_reduce(lo, fmin2, FLT_MAX, scratch);
     hi = block_reduce(hi, fmax2, -FLT_MAX, scratch);
     np.shift = lo;
     np.scale = hi > lo ? 1.f / (hi - lo) : 0.f;
   } else {
     float sum = 0.f;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) { float v = s[i]; bad |= !isfinite(v); sum += v; }
+    each([&](float v) { bad |= !isfinite(v); sum += v; });
     float mean = block_reduce(sum, fadd2, 0.f, scratch) / (float)n;
     float sq = 0.f;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) { float df = s[i] - mean; sq += df * df; }
+    each([&](float v) { float df = v - mean; sq += df * df; });
     float var = block_reduce(sq, fadd2, 0.f, scratch) / (float)n;
     np.shift = mean;
     np.scale = var > 0.f ? rsqrtf(var) : 0.f;
   }
   if (bad) atomicOr(status, kStatusNonFinite);
   return np;
+}
+__device__ __forceinline__ NormParams norm_params(const float* s, int n, int mode, float* scratch, int* status) {
+  return norm_params_by<0>([&](int j) { return s[threadIdx.x + j * blockDim.x]; }, n, mode, scratch, status);
 }
 
 // Eq. 12 for one request (whole block): normalise both scores to a common scale, fuse with lambda.

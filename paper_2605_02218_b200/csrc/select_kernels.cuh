@@ -19,7 +19,7 @@ __device__ __forceinline__ unsigned order_key(float v) {
 // Returns the exclusive prefix; *total receives the block sum.
 __device__ __forceinline__ unsigned block_exclusive_scan(unsigned v, unsigned* warp_tot,
                                                          unsigned* total) {
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int lane = threadIdx.x & 31, w = warp_index(), nw = blockDim.x >> 5;
   unsigned inc = v;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -44,12 +44,97 @@ __device__ __forceinline__ unsigned block_exclusive_scan(unsigned v, unsigned* w
   return warp_tot[w] + inc - v;
 }
 
-// Top-k of keys[0..n) by an 8-bit-per-pass radix select on the ordered keys, then an ordered
-// emission: every element above the k-th value, plus the lowest-index elements equal to it until k
-// are taken.  out[0..k) receives the selected positions in ascending order, mapped through `remap`
-// when given.  `all_equal` treats every key as equal (selects the first k positions).
-constexpr int kRankSelectMax = 1024;   // up to this many keys the selection ranks every key directly
-constexpr int kRegKeys = 16;           // keys per thread the radix select keeps in registers
+// Top-k of n keys: larger key first, then lower index; out[0..k) receives the selected positions in ascending
+// order, mapped through `remap` when given.  Two forms:
+//   up to kRegKeys keys per thread: the keys stay in registers (thread t holds the positions t,
+//   t + blockDim, ...) and the k-th largest key is found bit by bit, one block-wide count per bit below the
+//   prefix that all keys share, ending as soon as a count equals k (about 15 counts of 150-300 cycles for
+//   scores).  A radix select through shared-memory histograms took 12 us at 768 keys (scores
+//   crowd into a few digit values, whose updates queue up) and ranking every key 18 us.
+//   longer segments: an 8-bit-per-pass radix select that re-reads its keys, then an ordered emission.
+constexpr int kRegKeys = 16;           // keys per thread the select keeps in registers
+
+// One value per thread -> its block-wide reduction, one barrier.  `slots`: two rows used in turn.
+struct CountSlots { unsigned v[2][32]; };
+
+template <int PER>
+__device__ __forceinline__ void block_select_regs(const unsigned (&key)[PER], int n, int k, const int* __restrict__ remap,
+                                                  int* __restrict__ out, int* status) {
+  __shared__ CountSlots slots, slots2;
+  __shared__ unsigned counts[PER * 32];
+  __shared__ unsigned s_total;
+  const int lane = threadIdx.x & 31, warp = warp_index(), nw = blockDim.x >> 5, nt = blockDim.x, tid = threadIdx.x;
+  unsigned all_and = 0xffffffffu, all_or = 0u;
+#pragma unroll
+  for (int j = 0; j < PER; ++j)
+    if (tid + j * nt < n) { all_and &= key[j]; all_or |= key[j]; }
+  all_and = __reduce_and_sync(0xffffffffu, all_and);
+  all_or = __reduce_or_sync(0xffffffffu, all_or);
+  if (lane == 0) { slots.v[0][warp] = all_and; slots2.v[0][warp] = all_or; }
+  __syncthreads();
+  all_and = __reduce_and_sync(0xffffffffu, lane < nw ? slots.v[0][lane] : 0xffffffffu);
+  all_or = __reduce_or_sync(0xffffffffu, lane < nw ? slots2.v[0][lane] : 0u);
+  const unsigned diff = all_and ^ all_or;
+  const int top = 31 - __clz((int)diff);                     // -1: all keys are equal
+  unsigned thr = all_and & ~((2u << top) - 1u);              // shared prefix (top = 31: nothing)
+  if (top < 0) thr = all_and;
+  bool exact = false;                                        // keys >= thr are the answer, no ties
+  int buf = 1;
+  for (int bit = top; bit >= 0 && !exact; --bit, buf ^= 1) {
+    const unsigned cand = thr | (1u << bit);
+    unsigned c = 0u;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) c += key[j] >= cand;       // positions beyond n hold key 0 < cand
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (lane == 0) slots.v[buf][warp] = c;
+    __syncthreads();
+    c = __reduce_add_sync(0xffffffffu, lane < nw ? slots.v[buf][lane] : 0u);
+    if (c >= (unsigned)k) { thr = cand; exact = c == (unsigned)k; }
+  }
+  // ordered emission: counts per (j, warp), which is position order, then one scan
+  unsigned mg[PER], me[PER];
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const bool in = tid + j * nt < n;
+    mg[j] = __ballot_sync(0xffffffffu, in && (exact ? key[j] >= thr : key[j] > thr));
+    me[j] = __ballot_sync(0xffffffffu, in && !exact && key[j] == thr);
+    if (lane == 0) counts[j * nw + warp] = (unsigned)__popc(mg[j]) | (unsigned)__popc(me[j]) << 16;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    unsigned v[PER], sum = 0u;                               // PER consecutive entries per lane (nw <= 32)
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      v[j] = sum;
+      if (lane * PER + j < PER * nw) sum += counts[lane * PER + j];
+    }
+    unsigned inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      unsigned t = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += t;
+    }
+#pragma unroll
+    for (int j = 0; j < PER; ++j)
+      if (lane * PER + j < PER * nw) counts[lane * PER + j] = inc - sum + v[j];
+    if (lane == 31) s_total = inc;
+  }
+  __syncthreads();
+  const unsigned kk = (unsigned)k - (s_total & 0xffffu);     // how many keys equal to the threshold are taken
+  const unsigned below = (1u << lane) - 1u;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const bool g = mg[j] >> lane & 1u, e = me[j] >> lane & 1u;
+    if (!g && !e) continue;
+    const unsigned before = counts[j * nw + warp];
+    const unsigned gt_before = (before & 0xffffu) + __popc(mg[j] & below), eq_before = (before >> 16) + __popc(me[j] & below);
+    const unsigned pos = gt_before + min(eq_before, kk);
+    if ((g || eq_before < kk) && COVSPEC_IN_BOUNDS(pos, k, status)) {
+      const int i = tid + j * nt;
+      out[pos] = remap ? remap[i] : i;
+    }
+  }
+}
 
 // One digit of the radix select, by the first warp: with `kk` keys still to take among those that
 // match the digits fixed so far, the largest digit value d such that the keys with a larger digit
@@ -90,109 +175,39 @@ __device__ __forceinline__ void select_digit(const unsigned* hist, unsigned kk, 
   }
 }
 
+// The select on up to PER keys per thread; `load(i)` returns key i as a float.
+template <int PER, typename LoadF>
+__device__ __forceinline__ void block_topk_regs(LoadF load, int n, int k, bool all_equal, const int* __restrict__ remap,
+                                                int* __restrict__ out, int* status) {
+  unsigned key[PER];
+  bool bad = false;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const int i = (int)threadIdx.x + j * (int)blockDim.x;
+    key[j] = 0u;
+    if (i < n && !all_equal) {
+      const float v = load(i);
+      bad |= !(fabsf(v) <= 3.402823466e38f);
+      key[j] = order_key(v);
+    }
+  }
+  if (bad && status != nullptr) atomicOr(status, kStatusNonFinite);
+  block_select_regs<PER>(key, n, k, remap, out, status);
+}
+
 // `load(i)` returns key i as a float; `status` may be nullptr (non-finite keys are then not reported).
+// `all_equal` treats every key as equal (selects the first k positions).
 template <typename LoadF>
 __device__ void block_topk_by(LoadF load, int n, int k, bool all_equal,
                               const int* __restrict__ remap, int* __restrict__ out, int* status) {
+  const int per = (n + (int)blockDim.x - 1) / (int)blockDim.x;
+  if (per <= 1) { block_topk_regs<1>(load, n, k, all_equal, remap, out, status); return; }
+  if (per <= 4) { block_topk_regs<4>(load, n, k, all_equal, remap, out, status); return; }
+  if (per <= kRegKeys) { block_topk_regs<kRegKeys>(load, n, k, all_equal, remap, out, status); return; }
   __shared__ unsigned hist[256];
-  __shared__ unsigned whist[8][256];
   __shared__ unsigned sel_prefix, sel_k;
   __shared__ unsigned warp_tot[33];
-  __shared__ unsigned skeys[kRankSelectMax];
-  if (n <= kRankSelectMax) {
-    // Small segments: rank of key i = number of keys that precede it in (larger value, lower index)
-    // order, counted against the whole segment held in shared memory (every thread reads the same
-    // key at the same time: a broadcast); key i is selected when its rank is below k.  Positions
-    // are emitted in ascending order through a block scan of the selection flags.
-    bool bad = false;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      float v = load(i);
-      bad |= !all_equal && !(fabsf(v) <= 3.402823466e38f);
-      skeys[i] = all_equal ? 0u : order_key(v);
-    }
-    if (bad && status != nullptr) atomicOr(status, kStatusNonFinite);
-    __syncthreads();
-    unsigned run = 0u;
-    for (int base = 0; base < n; base += blockDim.x) {
-      int i = base + threadIdx.x;
-      unsigned sel = 0u;
-      if (i < n) {
-        unsigned ki = skeys[i];
-        int rank = 0;
-        for (int j = 0; j < i; ++j) rank += skeys[j] >= ki;       // equal keys with a lower index come first
-        for (int j = i + 1; j < n; ++j) rank += skeys[j] > ki;
-        sel = rank < k;
-      }
-      unsigned tot;
-      unsigned ex = block_exclusive_scan(sel, warp_tot, &tot);
-      if (sel && COVSPEC_IN_BOUNDS(run + ex, k, status)) out[run + ex] = remap ? remap[i] : i;
-      run += tot;
-    }
-    return;
-  }
   unsigned prefix = 0u, mask = 0u, kk = (unsigned)k;
-  const int per = (n + (int)blockDim.x - 1) / (int)blockDim.x;
-  if (per <= kRegKeys) {
-    // Medium segments: every thread keeps a contiguous run of `per` keys in registers, so the four
-    // digit passes read nothing from memory and the ordered emission needs one block scan.
-    unsigned kreg[kRegKeys];
-    const int i0 = (int)threadIdx.x * per;
-    const int cnt = max(0, min(per, n - i0));
-    bool bad = false;
-#pragma unroll
-    for (int j = 0; j < kRegKeys; ++j) {
-      kreg[j] = 0u;
-      if (j < cnt && !all_equal) {
-        float v = load(i0 + j);
-        bad |= !(fabsf(v) <= 3.402823466e38f);
-        kreg[j] = order_key(v);
-      }
-    }
-    if (bad && status != nullptr) atomicOr(status, kStatusNonFinite);
-    if (!all_equal) {
-      for (int shift = 24; shift >= 0; shift -= 8) {
-        // scores of one request crowd into a few digit values: eight copies of the histogram
-        // (one per warp modulo 8) spread the same-address updates
-        for (int i = threadIdx.x; i < 8 * 256; i += blockDim.x) (&whist[0][0])[i] = 0u;
-        __syncthreads();
-        unsigned* myhist = whist[(threadIdx.x >> 5) & 7];
-#pragma unroll
-        for (int j = 0; j < kRegKeys; ++j)
-          if (j < cnt && (kreg[j] & mask) == prefix) atomicAdd(&myhist[(kreg[j] >> shift) & 255u], 1u);
-        __syncthreads();
-        for (int i = threadIdx.x; i < 256; i += blockDim.x) {
-          unsigned c = 0u;
-#pragma unroll
-          for (int q = 0; q < 8; ++q) c += whist[q][i];
-          hist[i] = c;
-        }
-        __syncthreads();
-        if (threadIdx.x < 32) select_digit(hist, kk, prefix, shift, &sel_prefix, &sel_k);
-        __syncthreads();
-        prefix = sel_prefix;
-        kk = sel_k;
-        mask |= 255u << shift;
-      }
-    }
-    unsigned gt = 0u, eq = 0u;
-#pragma unroll
-    for (int j = 0; j < kRegKeys; ++j)
-      if (j < cnt) { gt += kreg[j] > prefix; eq += kreg[j] == prefix; }
-    unsigned tot;
-    unsigned ex = block_exclusive_scan(gt | (eq << 16), warp_tot, &tot);
-    unsigned gt_before = ex & 0xffffu, eq_before = ex >> 16;
-#pragma unroll
-    for (int j = 0; j < kRegKeys; ++j) {
-      if (j < cnt) {
-        const bool g = kreg[j] > prefix, e = kreg[j] == prefix;
-        if ((g || (e && eq_before < kk)) && COVSPEC_IN_BOUNDS(gt_before + min(eq_before, kk), k, status))
-          out[gt_before + min(eq_before, kk)] = remap ? remap[i0 + j] : i0 + j;
-        gt_before += g;
-        eq_before += e;
-      }
-    }
-    return;
-  }
   if (!all_equal) {
     bool bad = false;
     for (int shift = 24; shift >= 0; shift -= 8) {
@@ -205,7 +220,7 @@ __device__ void block_topk_by(LoadF load, int n, int k, bool all_equal,
         if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
       }
       __syncthreads();
-      if (threadIdx.x < 32) select_digit(hist, kk, prefix, shift, &sel_prefix, &sel_k);
+      if (warp_index() == 0) select_digit(hist, kk, prefix, shift, &sel_prefix, &sel_k);
       __syncthreads();
       prefix = sel_prefix;
       kk = sel_k;
@@ -250,17 +265,57 @@ preselect_kernel(const float* __restrict__ s_fused, const ReqPlan* __restrict__ 
   block_topk(s_fused + rp.vis_off, rp.n, rp.m, false, nullptr, presel + rp.presel_off, status);
 }
 
-// Eq. 12 and the preselection in one launch (the fused call): the block that fused a request's
-// scores selects its M best right away.
+// Eq. 12 and the preselection in one launch (the fused call): the block that fused a request's scores selects
+// its M best right away.  Up to kRegKeys tokens per thread both scores, the fused score and its keys stay in
+// registers from the one read of the scores to the selection; longer requests go through memory.
+template <int PER>
+__device__ __forceinline__ void fuse_select_regs(const ReqPlan& rp, const float* __restrict__ s_query,
+                                                 const float* __restrict__ s_act, float lambda, int mode,
+                                                 float* __restrict__ s_fused, int* __restrict__ presel, float* scratch,
+                                                 int* status) {
+  const int n = rp.n, tid = threadIdx.x, nt = blockDim.x;
+  float q[PER], a[PER];
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const int i = tid + j * nt;
+    q[j] = i < n ? s_query[rp.vis_off + i] : 0.f;
+    a[j] = i < n && s_act != nullptr ? s_act[rp.vis_off + i] : 0.f;
+  }
+  const NormParams nq = norm_params_by<PER>([&](int j) { return q[j]; }, n, mode, scratch, status);
+  NormParams na{0.f, 1.f};
+  if (s_act != nullptr) na = norm_params_by<PER>([&](int j) { return a[j]; }, n, mode, scratch, status);
+  unsigned key[PER];
+  bool bad = false;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const int i = tid + j * nt;
+    key[j] = 0u;
+    if (i < n) {
+      const float f = s_act == nullptr ? (q[j] - nq.shift) * nq.scale
+                                       : lambda * ((q[j] - nq.shift) * nq.scale) + (1.f - lambda) * ((a[j] - na.shift) * na.scale);
+      s_fused[rp.vis_off + i] = f;
+      bad |= !(fabsf(f) <= 3.402823466e38f);
+      key[j] = order_key(f);
+    }
+  }
+  if (bad) atomicOr(status, kStatusNonFinite);
+  block_select_regs<PER>(key, n, rp.m, nullptr, presel + rp.presel_off, status);
+}
+
 __global__ void __launch_bounds__(1024)
 fuse_preselect_kernel(const float* __restrict__ s_query, const float* __restrict__ s_act,
                       const ReqPlan* __restrict__ plan, float lambda, int mode,
                       float* __restrict__ s_fused, int* __restrict__ presel, int* status) {
   __shared__ float scratch[32];
-  ReqPlan rp = plan[blockIdx.x];
-  fuse_request(rp, s_query, s_act, lambda, mode, s_fused, scratch, status);
-  __syncthreads();                                  // the block's own global writes are visible to it
-  block_topk(s_fused + rp.vis_off, rp.n, rp.m, false, nullptr, presel + rp.presel_off, status);
+  const ReqPlan rp = plan[blockIdx.x];
+  if (rp.n <= 1024) fuse_select_regs<1>(rp, s_query, s_act, lambda, mode, s_fused, presel, scratch, status);
+  else if (rp.n <= 4 * 1024) fuse_select_regs<4>(rp, s_query, s_act, lambda, mode, s_fused, presel, scratch, status);
+  else if (rp.n <= kRegKeys * 1024) fuse_select_regs<kRegKeys>(rp, s_query, s_act, lambda, mode, s_fused, presel, scratch, status);
+  else {
+    fuse_request(rp, s_query, s_act, lambda, mode, s_fused, scratch, status);
+    __syncthreads();                                  // the block's own global writes are visible to it
+    block_topk(s_fused + rp.vis_off, rp.n, rp.m, false, nullptr, presel + rp.presel_off, status);
+  }
 }
 
 // Final selection: one block per request, the B_vis largest energies among the M preselected
