@@ -116,7 +116,7 @@ struct covspec_ctx {
   bool split_tc = false;
   int dp = 0, d3 = 0;                    // d rounded up to 64; 3 * dp
   __nv_bfloat16 *X3 = nullptr, *Q3 = nullptr, *Wq3 = nullptr, *Wk3 = nullptr, *Za3 = nullptr, *Zb3 = nullptr;
-  CUtensorMap map_za3, map_zb3w;
+  CUtensorMap map_za3, map_zb3w, map_zb3;
   // pinned staging for the plan upload
   char* h_stage = nullptr;
   long long stage_bytes = 0, stage_sched_off = 0;
@@ -804,9 +804,18 @@ int select_impl(covspec_ctx* ctx, const covspec_problem* p, const float* s_fused
     prof_mark(ctx, ST_PRESELECT, 1, s);
   }
   if (pl.n_stage2 > 0) {
-    prof_mark(ctx, ST_GRAM, 0, s);
     int st;
-    dim3 gb(std::min(64, (pl.p_max * pl.m_max + 255) / 256 + 1), B);
+    if (cfg.lowrank_mode != 1) {
+      // the start block needs the plan only: it is written beside the gather and the Gram matrix
+      CUDA_TRY(cudaEventRecord(ctx->ev_fork, s));
+      CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
+      dim3 gb(std::min(64, (pl.p_max * pl.m_max + 255) / 256 + 1), B);
+      sub::basis_init_kernel<<<gb, 256, 0, ctx->side>>>(ctx->d_plan, ctx->Yp[0][0], ctx->Yp[0][1], ctx->Yp[1][0],
+                                                        ctx->Yp[1][1], ctx->ld, energy, ctx->sync, B, cfg.eig_iters);
+      LAUNCH_CHECK(ctx);
+      CUDA_TRY(cudaEventRecord(ctx->ev_join, ctx->side));
+    }
+    prof_mark(ctx, ST_GRAM, 0, s);
     if (ctx->split_tc) {
       // float32 inputs on the tensor cores: the preselected rows are gathered and split in one pass
       SplitJobs jobs{};
@@ -819,7 +828,7 @@ int select_impl(covspec_ctx* ctx, const covspec_problem* p, const float* s_fused
       gp.k_chunks = ctx->d3 / sub::kBK;
       gp.g_hi = ctx->Ghi; gp.g_lo = ctx->Glo; gp.ld = ctx->ld; gp.status = ctx->status;
       int grid_g = std::min(pl.n_gram_tiles, ctx->num_sms);
-      sub::gram_tc_kernel<<<grid_g, 192, sub::kGramSmem, s>>>(ctx->map_za3, ctx->map_zb3w, gp);
+      sub::gram_tc_kernel<<<grid_g, 192, sub::kGramSmem, s>>>(ctx->map_za3, ctx->map_zb3w, ctx->map_zb3, gp);
       LAUNCH_CHECK(ctx);
       prof_mark(ctx, ST_GRAM, 1, s);
     } else {
@@ -832,9 +841,10 @@ int select_impl(covspec_ctx* ctx, const covspec_problem* p, const float* s_fused
       sub::GramParams gp{};
       gp.plan = ctx->d_plan; gp.batch = B; gp.n_items = pl.n_gram_tiles;
       gp.k_chunks = (cfg.d + sub::kBK - 1) / sub::kBK;
+      gp.same = 1;
       gp.g_hi = ctx->Ghi; gp.g_lo = ctx->Glo; gp.ld = ctx->ld; gp.status = ctx->status;
       int grid = std::min(pl.n_gram_tiles, ctx->num_sms);
-      sub::gram_tc_kernel<<<grid, 192, sub::kGramSmem, s>>>(ctx->map_zg, ctx->map_zgw, gp);
+      sub::gram_tc_kernel<<<grid, 192, sub::kGramSmem, s>>>(ctx->map_zg, ctx->map_zgw, ctx->map_zg, gp);
       LAUNCH_CHECK(ctx);
     } else {
       if ((st = launch_table<T, T, float, float, false>(ctx, T_GRAM_G, 1, s))) return st;
@@ -855,9 +865,7 @@ int select_impl(covspec_ctx* ctx, const covspec_problem* p, const float* s_fused
       LAUNCH_CHECK(ctx);
       return COVSPEC_OK;
     }
-    sub::basis_init_kernel<<<gb, 256, 0, s>>>(ctx->d_plan, ctx->Yp[0][0], ctx->Yp[0][1], ctx->Yp[1][0],
-                                              ctx->Yp[1][1], ctx->ld, energy, ctx->sync, B, cfg.eig_iters);
-    LAUNCH_CHECK(ctx);
+    CUDA_TRY(cudaStreamWaitEvent(s, ctx->ev_join, 0));
     // every multiplication by G, the factorisations between them, the Rayleigh-Ritz solve and the
     // energies: one cooperative launch (its CTAs wait on one another through global counters)
     sub::FusedParams fp{};
@@ -1130,6 +1138,7 @@ int covspec_prune_init(const covspec_config* cfg, covspec_ctx** out) {
     if (!f32) st = make_map_bf16(&ctx->map_zg, ctx->Zg, c.max_total_presel, c.d, sub::kTile);
     if (!f32 && !st) st = make_map_bf16(&ctx->map_zgw, ctx->Zg, c.max_total_presel, c.d, sub::kGramN);
     if (ctx->split_tc && !st) st = make_map_bf16(&ctx->map_za3, ctx->Za3, c.max_total_presel, ctx->d3, sub::kTile);
+    if (ctx->split_tc && !st) st = make_map_bf16(&ctx->map_zb3, ctx->Zb3, c.max_total_presel, ctx->d3, sub::kTile);
     if (ctx->split_tc && !st) st = make_map_bf16(&ctx->map_zb3w, ctx->Zb3, c.max_total_presel, ctx->d3, sub::kGramN);
     if (!st) st = make_map_bf16(&ctx->map_gh, ctx->Ghi, ctx->cap_rows, ctx->ld, sub::kTile);
     if (!st) st = make_map_bf16(&ctx->map_gl, ctx->Glo, ctx->cap_rows, ctx->ld, sub::kTile);

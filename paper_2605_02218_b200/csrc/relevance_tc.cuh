@@ -204,13 +204,15 @@ relevance_tc_kernel(const __grid_constant__ CUtensorMap map_a,   // X (MODE 0) o
         for (int hp = hp_begin; hp < hp_end && ok; ++hp, ++acc_it) {
           if (!(ok = mbar_wait(acc_empty, (acc_it & 1u) ^ 1u, abort_flag))) break;
           tc_fence_after();
+          bool ready = false;
           for (int kc = 0; kc < prm.k_chunks; ++kc, ++it) {
             int s = it % kStages;
             uint32_t ph = (it / kStages) & 1u;
-            if (!(ok = mbar_wait(&full[s], ph, abort_flag))) break;
+            if (!ready && !(ok = mbar_wait(&full[s], ph, abort_flag))) break;
             tc_fence_after();
             uint32_t a_addr = smem_u32(stage_base + s * kBytesStage);
             uint64_t adesc = umma_desc(a_addr), bdesc = umma_desc(a_addr + kBytesA);
+            ready = kc + 1 < prm.k_chunks && mbar_peek(&full[(it + 1) % kStages], ((it + 1) / kStages) & 1u);
 #pragma unroll
             for (int k = 0; k < kBK / 16; ++k)
               umma_bf16(tmem_base, adesc + 2 * k, bdesc + 2 * k, idesc1, (kc | k) != 0);

@@ -794,11 +794,13 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
           if (!(ok = mbar_wait(acc_empty, (n & 1u) ^ 1u, abort_flag))) break;
           tc_fence_after();
           int k_chunks = (rp.m + kBK - 1) / kBK;
+          bool ready = false;
           for (int kc = 0; kc < k_chunks; ++kc, ++it) {
             int s = it % kPowStages;
-            if (!(ok = mbar_wait(&full[s], (it / kPowStages) & 1u, abort_flag))) break;
+            if (!ready && !(ok = mbar_wait(&full[s], (it / kPowStages) & 1u, abort_flag))) break;
             tc_fence_after();
             uint32_t base = smem_u32(smem + s * kPowStageBytes);
+            ready = kc + 1 < k_chunks && mbar_peek(&full[(it + 1) % kPowStages], ((it + 1) / kPowStages) & 1u);
             // T += G_hi Y_hi + G_lo Y_hi + G_hi Y_lo
 #pragma unroll
             for (int term = 0; term < 3; ++term) {
