@@ -64,6 +64,13 @@ struct LayerPtrs {
 // became a call that gathers the warp first, about 280 cycles each.
 __device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
 
+// Programmatic dependent launch.  A kernel launched that way (launch_dependent in the host runtime) may start
+// while the kernel before it on the stream still runs: it waits here before it touches anything that
+// kernel, or one before it, writes or reads.  launch_dependents_now lets the next kernel start; without it that
+// happens when this one ends.
+__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void launch_dependents_now() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

@@ -439,6 +439,24 @@ int get_plan(covspec_ctx* ctx, const covspec_problem* p, cudaStream_t stream) {
     CUDA_TRY(cudaGetLastError());                       \
   } while (0)
 
+// Launch that may overlap the end of the kernel before it on the stream; the kernel calls
+// wait_for_previous_kernel (common.cuh) before it uses anything of that kernel's.  About 2 us less between two
+// short kernels.
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Records the begin (edge 0) or end (edge 1) event of a stage for the current profiled call.
 inline void prof_mark(covspec_ctx* ctx, int stage, int edge, cudaStream_t s) {
   if (ctx->prof_cap == 0 || ctx->prof_calls >= ctx->prof_cap) return;
@@ -637,7 +655,7 @@ int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cud
   prm.n_items = pl.n_tiles * prm.n_groups;
   prm.qn_out = nullptr; prm.s_query = s_query; prm.fill = nullptr;
   grid = prm.n_items < ctx->num_sms ? prm.n_items : ctx->num_sms;
-  tc::relevance_tc_kernel<0><<<grid, 192, tc::kSmemBytes, s>>>(map_x, map_wk, map_qn, map_qnl, prm);
+  CUDA_TRY(launch_dependent(tc::relevance_tc_kernel<0>, dim3(grid), 192, tc::kSmemBytes, s, map_x, map_wk, map_qn, map_qnl, prm));
   LAUNCH_CHECK(ctx);
   prof_mark(ctx, ST_RELEVANCE, 1, s);
   return COVSPEC_OK;
@@ -821,21 +839,21 @@ int select_impl(covspec_ctx* ctx, const covspec_problem* p, const float* s_fused
       SplitJobs jobs{};
       jobs.j[0] = SplitJob{reinterpret_cast<const float*>(p->X), presel, ctx->Za3, ctx->Zb3, pl.total_presel};
       dim3 grid((unsigned)std::min<long long>(pl.total_presel, 8ll * ctx->num_sms), 1);
-      split3_kernel<<<grid, 256, 0, s>>>(jobs, ctx->d_plan, B, cfg.d, ctx->dp);
+      CUDA_TRY(launch_dependent(split3_kernel, grid, 256, 0, s, jobs, ctx->d_plan, B, cfg.d, ctx->dp));
       LAUNCH_CHECK(ctx);
       sub::GramParams gp{};
       gp.plan = ctx->d_plan; gp.batch = B; gp.n_items = pl.n_gram_tiles;
       gp.k_chunks = ctx->d3 / sub::kBK;
       gp.g_hi = ctx->Ghi; gp.g_lo = ctx->Glo; gp.ld = ctx->ld; gp.status = ctx->status;
       int grid_g = std::min(pl.n_gram_tiles, ctx->num_sms);
-      sub::gram_tc_kernel<<<grid_g, 192, sub::kGramSmem, s>>>(ctx->map_za3, ctx->map_zb3w, ctx->map_zb3, gp);
+      CUDA_TRY(launch_dependent(sub::gram_tc_kernel, dim3(grid_g), 192, sub::kGramSmem, s, ctx->map_za3, ctx->map_zb3w, ctx->map_zb3, gp));
       LAUNCH_CHECK(ctx);
       prof_mark(ctx, ST_GRAM, 1, s);
     } else {
     int vec16 = cfg.d * ctx->esize / 16;
-    gather_rows_kernel<<<gather_grid(pl.total_presel), kGatherWarps * 32, 0, s>>>(
+    CUDA_TRY(launch_dependent(gather_rows_kernel, dim3(gather_grid(pl.total_presel)), kGatherWarps * 32, 0, s,
         reinterpret_cast<const uint4*>(p->X), presel, ctx->d_plan, B, 1, vec16, (int)pl.total_presel,
-        reinterpret_cast<uint4*>(ctx->Zg), nullptr, ctx->status);
+        reinterpret_cast<uint4*>(ctx->Zg), nullptr, ctx->status));
     LAUNCH_CHECK(ctx);
     if (cfg.dtype == COVSPEC_BF16) {
       sub::GramParams gp{};
@@ -844,7 +862,7 @@ int select_impl(covspec_ctx* ctx, const covspec_problem* p, const float* s_fused
       gp.same = 1;
       gp.g_hi = ctx->Ghi; gp.g_lo = ctx->Glo; gp.ld = ctx->ld; gp.status = ctx->status;
       int grid = std::min(pl.n_gram_tiles, ctx->num_sms);
-      sub::gram_tc_kernel<<<grid, 192, sub::kGramSmem, s>>>(ctx->map_zg, ctx->map_zgw, ctx->map_zg, gp);
+      CUDA_TRY(launch_dependent(sub::gram_tc_kernel, dim3(grid), 192, sub::kGramSmem, s, ctx->map_zg, ctx->map_zgw, ctx->map_zg, gp));
       LAUNCH_CHECK(ctx);
     } else {
       if ((st = launch_table<T, T, float, float, false>(ctx, T_GRAM_G, 1, s))) return st;
@@ -894,7 +912,7 @@ int select_impl(covspec_ctx* ctx, const covspec_problem* p, const float* s_fused
   }
   if (pl.n_stage2 > 0) prof_mark(ctx, ST_EIG, 1, s);
   prof_mark(ctx, ST_FINAL, 0, s);
-  final_select_kernel<<<B, 1024, 0, s>>>(energy, presel, ctx->d_plan, keep_idx, ctx->status);
+  CUDA_TRY(launch_dependent(final_select_kernel, dim3(B), 1024, 0, s, energy, presel, ctx->d_plan, keep_idx, ctx->status));
   LAUNCH_CHECK(ctx);
   return COVSPEC_OK;
 }
@@ -903,9 +921,9 @@ int compact_impl(covspec_ctx* ctx, const covspec_problem* p, const int* keep_idx
                  int* out_pos, cudaStream_t s) {
   const Plan& pl = ctx->plan;
   int vec16 = ctx->cfg.d * ctx->esize / 16;
-  gather_rows_kernel<<<gather_grid(pl.total_keep), kGatherWarps * 32, 0, s>>>(
+  CUDA_TRY(launch_dependent(gather_rows_kernel, dim3(gather_grid(pl.total_keep)), kGatherWarps * 32, 0, s,
       reinterpret_cast<const uint4*>(p->X), keep_idx, ctx->d_plan, p->batch, 0, vec16, (int)pl.total_keep,
-      reinterpret_cast<uint4*>(out), out_pos, ctx->status);
+      reinterpret_cast<uint4*>(out), out_pos, ctx->status));
   LAUNCH_CHECK(ctx);
   prof_mark(ctx, ST_FINAL, 1, s);
   return COVSPEC_OK;

@@ -118,6 +118,9 @@ relevance_tc_kernel(const __grid_constant__ CUtensorMap map_a,   // X (MODE 0) o
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // The visual side starts while the query side still runs, on the SMs that it leaves: its main loops need
+  // nothing of it; what it fills in is waited for before the first query tile and the first maximum.
+  if (MODE == 1) launch_dependents_now();
   if (MODE == 1 && prm.fill != nullptr) {
     // the visual-side launch combines head groups with an atomic max: its score array starts at -inf
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < prm.fill_n;
@@ -152,7 +155,7 @@ relevance_tc_kernel(const __grid_constant__ CUtensorMap map_a,   // X (MODE 0) o
     // ---------------------------------------------------------------- TMA producer
     if (lane == 0) {
       uint32_t it = 0;
-      bool ok = true;
+      bool ok = true, waited = false;
       for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x) {
         int row0, nrows, txt0, T, hp_begin, hp_end;
         decode(item, row0, nrows, txt0, T, hp_begin, hp_end);
@@ -167,6 +170,7 @@ relevance_tc_kernel(const __grid_constant__ CUtensorMap map_a,   // X (MODE 0) o
             tma_load_2d(dst + kBytesA, &map_b, kc * kBK, hp * kTileN, &full[s]);
           }
           if (MODE == 0 && ok) {
+            if (!waited) { wait_for_previous_kernel(); waited = true; }
             // query sub-tiles of this head pair use the next ring slots, in the order the MMA issuer
             // consumes them: head, group of up to kLogitSlots tiles, half, tile; one slot holds the
             // [64 x 64] hi block followed by the lo block
@@ -377,6 +381,7 @@ relevance_tc_kernel(const __grid_constant__ CUtensorMap map_a,   // X (MODE 0) o
           }
         }
       }
+      if (MODE == 0 && item == (int)blockIdx.x) wait_for_previous_kernel();      // the scores are filled with -inf
       if (MODE == 0 && ok && r < nrows) {
         if (nonfinite) atomicOr(prm.status, kStatusNonFinite);
         else atomic_max_float(prm.s_query + row0 + r, best);

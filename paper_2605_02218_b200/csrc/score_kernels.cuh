@@ -186,6 +186,7 @@ struct SplitJobs { SplitJob j[4]; };
 
 __global__ void __launch_bounds__(256)
 split3_kernel(SplitJobs jobs, const ReqPlan* __restrict__ plan, int batch, int d, int dp) {
+  wait_for_previous_kernel();
   const SplitJob job = jobs.j[blockIdx.y];
   for (long long row = blockIdx.x; row < job.rows; row += gridDim.x) {
     long long src_row = row;

@@ -324,6 +324,7 @@ fuse_preselect_kernel(const float* __restrict__ s_query, const float* __restrict
 __global__ void __launch_bounds__(1024)
 final_select_kernel(const float* __restrict__ energy, const int* __restrict__ presel,
                     const ReqPlan* __restrict__ plan, int* __restrict__ keep_idx, int* status) {
+  wait_for_previous_kernel();
   ReqPlan rp = plan[blockIdx.x];
   block_topk(energy + rp.presel_off, rp.m, rp.b_vis, rp.stage2 == 0, presel + rp.presel_off,
              keep_idx + rp.keep_off, status);
@@ -339,6 +340,7 @@ gather_rows_kernel(const uint4* __restrict__ src, const int* __restrict__ idx,
                    uint4* __restrict__ dst, int* __restrict__ out_pos, int* status) {
   const int lane = threadIdx.x & 31;
   const int row = blockIdx.x * kGatherWarps + (threadIdx.x >> 5);
+  wait_for_previous_kernel();
   if (row >= rows) return;
   long long first = 0;
   int tok = 0;

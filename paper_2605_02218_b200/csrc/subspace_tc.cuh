@@ -127,6 +127,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_z,   // row operand [sum 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  wait_for_previous_kernel();
 
   auto decode = [&](int item, ReqPlan& rp, int& ti, int& tjp) {
     int b = find_request(item, prm.batch, [&](int q) { return prm.plan[q].gram_tile_off; });
