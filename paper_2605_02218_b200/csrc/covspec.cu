@@ -20,6 +20,7 @@
 #include "greedy_kernels.cuh"
 #include "identity_tc.cuh"
 #include "relevance_tc.cuh"
+#include "relevance_vis.cuh"
 #include "relevance_pair.cuh"
 #include "subspace_tc.cuh"
 #include "subspace_fused.cuh"
@@ -655,7 +656,7 @@ int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cud
   prm.n_items = pl.n_tiles * prm.n_groups;
   prm.qn_out = nullptr; prm.s_query = s_query; prm.fill = nullptr;
   grid = prm.n_items < ctx->num_sms ? prm.n_items : ctx->num_sms;
-  CUDA_TRY(launch_dependent(tc::relevance_tc_kernel<0>, dim3(grid), 192, tc::kSmemBytes, s, map_x, map_wk, map_qn, map_qnl, prm));
+  CUDA_TRY(launch_dependent(tc::relevance_vis_kernel, dim3(grid), tc::kVisThreads, tc::kVisSmem, s, map_x, map_wk, map_qn, map_qnl, prm));
   LAUNCH_CHECK(ctx);
   prof_mark(ctx, ST_RELEVANCE, 1, s);
   return COVSPEC_OK;
@@ -1122,8 +1123,8 @@ int covspec_prune_init(const covspec_config* cfg, covspec_ctx** out) {
   }
   if (ok) {
     ctx->tc_ready =
-        cudaFuncSetAttribute(tc::relevance_tc_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             tc::kSmemBytes) == cudaSuccess &&
+        cudaFuncSetAttribute(tc::relevance_vis_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             tc::kVisSmem) == cudaSuccess &&
         cudaFuncSetAttribute(tc::relevance_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              tc::kSmemBytes) == cudaSuccess &&
         cudaFuncSetAttribute(tc2::relevance_pair_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
