@@ -90,8 +90,9 @@ typedef struct {
   int ritz_window;     /* basis vectors above the cut at r that take part in the final Rayleigh-Ritz
                           step together with the eig_oversample ones below it (default 16; >= p: all) */
   int activity_overlap; /* > 0: while Eq. 10 runs on the tensor cores (which leaves HBM idle), Eq. 11
-                          streams the snapshot stack on a second stream of the context with this many
-                          512-thread blocks per SM (1 or 2; default 1), joined before Eq. 12; 0: the two
+                          streams the snapshot stack on a second stream of the context with at least this
+                          many 512-thread blocks per SM (1 or 2; default 1: two where one would take longer
+                          than Eq. 10), joined before Eq. 12; 0: the two
                           scores are computed one after the other on the caller's stream           */
   float conv_tol;      /* the subspace iteration behind Eq. 14 runs a fixed number of steps; after the
                           last one the library estimates, from the Ritz values, how far the energies

@@ -675,6 +675,12 @@ int launch_activity(covspec_ctx* ctx, const covspec_problem* p, float* s_act, bo
   if (background) {
     // beside the two-SM relevance kernel only one block per SM fits (shared-memory reserve)
     int per_sm = cfg.relevance_path == 2 ? 1 : cfg.activity_overlap;
+    // One block per SM reads about 1.8 TB/s beside the relevance kernel; where that would end after the
+    // kernel (about 1.1 PFLOP/s) a second one is added (batch of 16 x 576 tokens, d = 2048: 115 -> 71 us).
+    // Where it ends before, a second block only slows the kernel down (video: 3570 -> 3940 us a call).
+    const double stream_s = (double)(cfg.act_layers + 1) * rowsX * cfg.d * ctx->esize / 1.8e12;
+    const double kernel_s = 2.0 * rowsX * (ctx->split_tc ? ctx->d3 : cfg.d) * ctx->P / 1.1e15;
+    if (per_sm == 1 && cfg.relevance_path != 2 && stream_s > kernel_s) per_sm = 2;
     unsigned grid = (unsigned)std::min<long long>((rowsX + 15) / 16, (long long)ctx->num_sms * per_sm);
     if (cfg.act_layers <= 4)
       activity_stream_kernel<T, 4><<<grid, 512, 0, s>>>(lp, cfg.act_layers, rowsX, cfg.d, s_act);
