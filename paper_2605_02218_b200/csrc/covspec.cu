@@ -638,7 +638,7 @@ int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cud
   int n_hp = (cfg.n_heads + 1) / 2;
   tc::Params prm{};
   prm.plan = ctx->d_plan; prm.batch = p->batch;
-  prm.n_groups = n_hp; prm.hp_per_group = 1;
+  prm.n_groups = n_hp;
   prm.n_heads = cfg.n_heads; prm.k_chunks = (d + tc::kBK - 1) / tc::kBK; prm.P = P;
   prm.status = ctx->status;
   // query side
@@ -648,7 +648,7 @@ int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cud
   prm.qn_out = qn; prm.qn_lo_off = lo_off; prm.s_query = nullptr;
   prm.fill = s_query; prm.fill_n = pl.total_vis;          // -inf for the visual-side launch below
   int grid = prm.n_items < ctx->num_sms ? prm.n_items : ctx->num_sms;
-  tc::relevance_tc_kernel<1><<<grid, 192, tc::kSmemBytes, s>>>(map_q, map_wq, map_qn, map_qnl, prm);
+  tc::query_embed_kernel<<<grid, 192, tc::kQuerySmem, s>>>(map_q, map_wq, prm);
   LAUNCH_CHECK(ctx);
   prof_mark(ctx, ST_QEMBED, 1, s);
   // visual side
@@ -1131,8 +1131,8 @@ int covspec_prune_init(const covspec_config* cfg, covspec_ctx** out) {
     ctx->tc_ready =
         cudaFuncSetAttribute(tc::relevance_vis_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              tc::kVisSmem) == cudaSuccess &&
-        cudaFuncSetAttribute(tc::relevance_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             tc::kSmemBytes) == cudaSuccess &&
+        cudaFuncSetAttribute(tc::query_embed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             tc::kQuerySmem) == cudaSuccess &&
         cudaFuncSetAttribute(tc2::relevance_pair_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              tc2::kSmemBytes2) == cudaSuccess &&
         cudaFuncSetAttribute(tc2::relevance_pair_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,

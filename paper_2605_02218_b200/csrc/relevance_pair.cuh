@@ -32,6 +32,9 @@ namespace tc2 {
 
 using namespace tc;
 
+constexpr int kLogitSlots = 4;         // logits tiles that accumulate across the two halves
+constexpr int kLogitCol = 256;         // logits tiles live at columns 256 + 64 * slot
+
 constexpr int kStages2 = 5;
 constexpr int kBytesBh = (kTileN / 2) * kBK * 2;          // 16 KB: this CTA's half of the weight chunk
 constexpr int kBytesStage2 = kBytesA + kBytesBh;          // 32 KB

@@ -33,6 +33,7 @@ constexpr int kVisStages = 3;
 constexpr int kVisThreads = 256;
 constexpr int kQueryBlock = kTT * kHalf * 2;              // 8 KB
 constexpr int kVisSmem = kVisStages * kBytesStage + 4 * kBytesKp + 2 * kQueryBlock + 1024 /*barriers*/;
+static_assert(kVisSmem == kQuerySmem, "see kQuerySmem");
 constexpr int kLogitTiles = kHeadDim / kTT;               // logits tiles in the columns of one head
 
 __global__ void __launch_bounds__(kVisThreads, 1)
