@@ -345,7 +345,7 @@ template <int N> struct IntTag { static constexpr int value = N; };
 // from L2, and the window's factorisation finds this code where the steps before it left it.
 __device__ __noinline__ void cholesky_team(int n, int t_off, float* out) {
   double* T = reinterpret_cast<double*>(pow_smem()) + t_off;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = warp_index();
   auto sync = [&]() { named_barrier(1, kEpiThreads); };
   const int nb = (n + 7) >> 3;
   double* aux = T + nb * (nb + 1) / 2 * 64;
@@ -525,7 +525,7 @@ __device__ __noinline__ bool team_cholesky(const double* pbase, int nt, int p, i
   double* Tm = reinterpret_cast<double*>(pow_smem());
   float* dg = pow_tail().dinv;
   volatile int* s_word = pow_tail().s_word;
-  const int et = threadIdx.x, warp = et >> 5, lane = et & 31;
+  const int et = threadIdx.x, warp = warp_index(), lane = et & 31;
   const int P = (p + 7) & ~7, nb = (p + 7) >> 3;
   auto epi_sync = [&]() { named_barrier(1, kEpiThreads); };
   // identity padding of the layout rows / columns p .. P-1 and the entries left of the diagonal
@@ -569,7 +569,7 @@ __device__ __noinline__ void team_ritz(const double* pbase, int nt, int p, int w
   float* dg = pow_tail().lt;
   float* s_scale = pow_tail().s_scale;
   int* s_flag = pow_tail().s_flag;
-  const int et = threadIdx.x, warp = et >> 5, lane = et & 31;
+  const int et = threadIdx.x, warp = warp_index(), lane = et & 31;
   auto epi_sync = [&]() { named_barrier(1, kEpiThreads); };
   const int w0 = p - w, nbot = p - r;
   const bool small = w <= 32;            // the usual window: see jacobi_warp32 for the row order of a column
@@ -689,7 +689,7 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
   uint32_t* tmem_slot = tail.tmem_slot;
   volatile int* abort_flag = tail.abort_flag;
   volatile int* s_word = tail.s_word;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   unsigned* gabort = prm.sync + (size_t)prm.batch * kSyncStride;
 
   if (threadIdx.x == 0) {

@@ -508,7 +508,7 @@ __device__ __noinline__ void solve_team(int x_off, int P, int tile_rows, bool sp
   float* x = reinterpret_cast<float*>(pow_smem()) + x_off;
   const float* lt = reinterpret_cast<float*>(pow_smem() + kPowRegion);
   const float* dinv = lt + kLtFloats;
-  const int et = threadIdx.x, warp = et >> 5, lane = et & 31, nS = (P + 31) >> 5;
+  const int et = threadIdx.x, warp = warp_index(), lane = et & 31, nS = (P + 31) >> 5;
 #pragma unroll 1
   for (int S = 0; S < nS; ++S) {
     if (S > 0) {
