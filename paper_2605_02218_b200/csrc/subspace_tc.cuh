@@ -357,8 +357,10 @@ __device__ __forceinline__ uint8_t* pow_smem() {
 // solve_gemm takes the contributions of the columns before super-block S off its 32 columns: a product
 // of (rows) x (32 S) with (32 S) x 32, by the eight warps, RT rows x 4 columns per thread.  A warp
 // covers 16 RT rows x 8 columns, so that a column step reads 16 RT + 8 words of shared memory for
-// 128 RT products (three wavefronts for sixteen multiply-adds per thread when RT = 4): bound by the FP32
-// pipe, where one thread per row needed a word for every product and was bound by shared memory.
+// 128 RT products: sixteen multiply-adds per thread when RT = 4, as many cycles as the two loads take.
+// Neighbouring lanes share a row group and take different columns: a 16-byte load takes two cycles where neighbours
+// read the same address and four where the two halves of the warp read the same addresses (measured), which made
+// the first form of this mapping (lane & 15) bound by shared memory.
 // solve_diag then solves inside the super-block, one thread per row, the row's 32 values in
 // registers.  p = 144, 128 rows: 40 -> 14 k cycles.
 // The products enter every sum in ascending column order; `split` (steps before the last one): the
@@ -366,10 +368,10 @@ __device__ __forceinline__ uint8_t* pow_smem() {
 template <int RT, int RG>
 __device__ __forceinline__ void solve_gemm(float* x, const float* lt, int P, int S, bool split, int nrows, int warp,
                                            int lane) {
-  const int rg = warp % RG, row0 = 16 * RT * rg + RT * (lane & 15);
+  const int rg = warp % RG, row0 = 16 * RT * rg + RT * (lane >> 1);
   const int j0 = 32 * S + 8 * (warp / RG);
   if (16 * RT * rg >= ((nrows + 31) & ~31) || j0 >= P) return;       // whole warp
-  const int j = j0 + 4 * (lane >> 4);
+  const int j = j0 + 4 * (lane & 1);
   float acc[4][RT];
   auto t_at = [&](int c) { return x + (j + c) * kXsLd + row0; };
   auto rows_load = [&](const float* src, float (&v)[RT]) {
