@@ -109,13 +109,14 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
   } else if (warp == 5) {
     // ---------------------------------------------------------------- MMA issuer
     if (lane == 0) {
-      const uint32_t idesc = umma_idesc(kTileM, kTileN);
       uint32_t it = 0, n = 0;
       bool ok = true;
       for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x, ++n) {
         const uint32_t buf = n & 1u;
         if (!(ok = mbar_wait(&acc_empty[buf], ((n >> 1) & 1u) ^ 1u, abort_flag))) break;
         tc_fence_after();
+        // a lone last head takes half the columns (see relevance_vis_kernel)
+        const uint32_t idesc = umma_idesc(kTileM, item % prm.n_groups * 2 + 1 < prm.n_heads ? kTileN : kHeadDim);
         for (int kc = 0; kc < prm.k_chunks; ++kc, ++it) {
           const int s = it % kQueryStages;
           if (!(ok = mbar_wait(&full[s], (it / kQueryStages) & 1u, abort_flag))) break;

@@ -120,7 +120,6 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
   } else if (warp == 5) {
     // ---------------------------------------------------------------- MMA issuer, main loop
     if (lane == 0) {
-      const uint32_t idesc = umma_idesc(kTileM, kTileN);
       int s = 0;
       uint32_t ph = 0, n = 0;
       bool ok = true;
@@ -128,6 +127,9 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
         const uint32_t buf = n & 1u;
         if (!(ok = mbar_wait(&acc_empty[buf], ((n >> 1) & 1u) ^ 1u, abort_flag))) break;
         tc_fence_after();
+        // a lone last head takes half the columns and half the tensor time (576 tokens, one float32 head, d = 1024: a
+        // call 171.0 -> 169.0 us; fetching half the weight tile as well gained nothing)
+        const uint32_t idesc = umma_idesc(kTileM, item % prm.n_groups * 2 + 1 < prm.n_heads ? kTileN : kHeadDim);
         for (int kc = 0; kc < prm.k_chunks; ++kc) {
           if (!(ok = mbar_wait(&full[s], ph, abort_flag))) break;
           tc_fence_after();
