@@ -626,13 +626,18 @@ int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cud
   const void *X = p->X, *Q = p->Q, *Wk = p->Wk, *Wq = p->Wq;
   if (ctx->split_tc) { X = ctx->X3; Q = ctx->Q3; Wk = ctx->Wk3; Wq = ctx->Wq3; d = ctx->d3; }
   __nv_bfloat16* qn = reinterpret_cast<__nv_bfloat16*>(ctx->Qn);
+  // Query side: one head per item while that leaves items for at most half the SMs (the visual side starts on the
+  // others): its main loop is the shorter of the two then, and the logits wait for it (one request, 16 heads, d = 2048:
+  // 20.4 -> 18.4 us; five float32 requests with 3 heads stage by stage: 296.7 -> 292.1 us).
+  const int q_tiles = (int)((pl.total_txt + tc::kTileM - 1) / tc::kTileM);
+  const int group_heads = q_tiles * cfg.n_heads <= ctx->num_sms / 2 ? 1 : 2;
   CUtensorMap map_x, map_wk, map_q, map_wq, map_qn, map_qnl;
   long long lo_off = (long long)cfg.max_total_txt * P;   // lo parts follow the hi parts
   int st;
   if ((st = make_map_bf16(&map_x, X, pl.total_vis, d, tc::kTileM))) return st;
   if ((st = make_map_bf16(&map_wk, Wk, P, d, tc::kTileN))) return st;
   if ((st = make_map_bf16(&map_q, Q, pl.total_txt, d, tc::kTileM))) return st;
-  if ((st = make_map_bf16(&map_wq, Wq, P, d, tc::kTileN))) return st;
+  if ((st = make_map_bf16(&map_wq, Wq, P, d, group_heads * tc::kHeadDim))) return st;
   if ((st = make_map_bf16(&map_qn, qn, pl.total_txt, P, tc::kTT))) return st;
   if ((st = make_map_bf16(&map_qnl, qn + lo_off, pl.total_txt, P, tc::kTT))) return st;
   int n_hp = (cfg.n_heads + 1) / 2;
@@ -644,7 +649,9 @@ int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cud
   // query side
   prof_mark(ctx, ST_QEMBED, 0, s);
   prm.rows_total = pl.total_txt;
-  prm.n_items = (int)((pl.total_txt + tc::kTileM - 1) / tc::kTileM) * prm.n_groups;
+  prm.group_heads = group_heads;
+  prm.n_groups = (cfg.n_heads + group_heads - 1) / group_heads;
+  prm.n_items = q_tiles * prm.n_groups;
   prm.qn_out = qn; prm.qn_lo_off = lo_off; prm.s_query = nullptr;
   prm.fill = s_query; prm.fill_n = pl.total_vis;          // -inf for the visual-side launch below
   int grid = prm.n_items < ctx->num_sms ? prm.n_items : ctx->num_sms;
@@ -653,6 +660,7 @@ int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cud
   prof_mark(ctx, ST_QEMBED, 1, s);
   // visual side
   prof_mark(ctx, ST_RELEVANCE, 0, s);
+  prm.n_groups = n_hp;
   prm.n_items = pl.n_tiles * prm.n_groups;
   prm.qn_out = nullptr; prm.s_query = s_query; prm.fill = nullptr;
   grid = prm.n_items < ctx->num_sms ? prm.n_items : ctx->num_sms;

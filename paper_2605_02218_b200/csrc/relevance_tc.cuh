@@ -35,7 +35,8 @@ struct Params {
   const ReqPlan* plan;
   int batch;
   int n_items;          // (tile, pair of heads) pairs
-  int n_groups;         // pairs of heads
+  int n_groups;         // pairs of heads (query side: groups of group_heads)
+  int group_heads;      // query side: heads per item, 2 or 1
   int n_heads;
   int k_chunks;         // ceil(d / 64)
   int P;                // n_heads * 128
@@ -94,14 +95,14 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
       uint32_t it = 0;
       bool ok = true;
       for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x) {
-        const int row0 = item / prm.n_groups * kTileM, hp = item % prm.n_groups;
+        const int row0 = item / prm.n_groups * kTileM, head0 = item % prm.n_groups * prm.group_heads;
         for (int kc = 0; kc < prm.k_chunks; ++kc, ++it) {
           const int s = it % kQueryStages;
           if (!(ok = mbar_wait(&empty[s], ((it / kQueryStages) & 1u) ^ 1u, abort_flag))) break;
-          mbar_expect_tx(&full[s], kBytesStage);
+          mbar_expect_tx(&full[s], kBytesA + prm.group_heads * kHeadDim * kBK * 2);
           const uint32_t dst = smem_u32(smem + s * kBytesStage);
           tma_load_2d(dst, &map_a, kc * kBK, row0, &full[s]);
-          tma_load_2d(dst + kBytesA, &map_b, kc * kBK, hp * kTileN, &full[s]);
+          tma_load_2d(dst + kBytesA, &map_b, kc * kBK, head0 * kHeadDim, &full[s]);
         }
       }
     }
@@ -116,7 +117,8 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
         if (!(ok = mbar_wait(&acc_empty[buf], ((n >> 1) & 1u) ^ 1u, abort_flag))) break;
         tc_fence_after();
         // a lone last head takes half the columns (see relevance_vis_kernel)
-        const uint32_t idesc = umma_idesc(kTileM, item % prm.n_groups * 2 + 1 < prm.n_heads ? kTileN : kHeadDim);
+        const int head0 = item % prm.n_groups * prm.group_heads;
+        const uint32_t idesc = umma_idesc(kTileM, min(prm.group_heads, prm.n_heads - head0) * kHeadDim);
         for (int kc = 0; kc < prm.k_chunks; ++kc, ++it) {
           const int s = it % kQueryStages;
           if (!(ok = mbar_wait(&full[s], (it / kQueryStages) & 1u, abort_flag))) break;
@@ -138,14 +140,14 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
     uint32_t n = 0;
     bool ok = true;
     for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x, ++n) {
-      const int row0 = item / prm.n_groups * kTileM, hp = item % prm.n_groups;
+      const int row0 = item / prm.n_groups * kTileM, head0 = item % prm.n_groups * prm.group_heads;
       const long long rem = prm.rows_total - row0;
       const int nrows = rem < kTileM ? (int)rem : kTileM;
       const uint32_t buf = n & 1u;
       if (!(ok = mbar_wait(&acc_full[buf], (n >> 1) & 1u, abort_flag))) break;
       tc_fence_after();
       const uint32_t t_lane = tmem_base + ((uint32_t)(warp * 32) << 16) + buf * kTileN;
-      const int heads = min(2, prm.n_heads - 2 * hp);
+      const int heads = min(prm.group_heads, prm.n_heads - head0);
       for (int h = 0; h < heads; ++h) {
         // unit-length bf16 head slice of the projected query element to global memory
         float ss = 0.f;
@@ -165,7 +167,7 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
           tmem_ld32(t_lane + h * kHeadDim + c4 * 32, v);
           if (r < nrows) {
             __nv_bfloat16* dst = prm.qn_out + (size_t)(row0 + r) * prm.P +
-                                 (size_t)(2 * hp + h) * kHeadDim + c4 * 32;
+                                 (size_t)(head0 + h) * kHeadDim + c4 * 32;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
               uint32_t ph[4], pw[4];
