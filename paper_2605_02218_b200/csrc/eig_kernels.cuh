@@ -40,8 +40,8 @@ __host__ __device__ inline size_t cholesky_smem_bytes(int n) {
 // they are mutually orthogonal.  Round-robin ordering, w/2 disjoint pairs per round, one 4-lane
 // group per pair with the two columns held in registers between the inner products and the
 // rotation, so that a round is a short instruction stream on few warps and the barrier between
-// rounds spans only those warps (named barrier 1 over `nact` threads; the caller guarantees that
-// exactly the threads tid < nact enter).  A pair is left alone when its inner product g is
+// rounds spans only those warps (named barrier 1 over `nact` threads, a multiple of 32; the caller guarantees
+// that exactly the threads tid < nact enter).  A pair is left alone when its inner product g is
 // negligible against the two norms (g^2 <= 1e-12 |a|^2 |b|^2) or so small that the energies move by
 // less than ~2e-5 of the problem's scale s1 (g^2 <= (2e-5 s1)^2 min(|a|^2, |b|^2)).  Returns false
 // when max_sweeps sweeps did not reach a sweep without rotations.
@@ -56,50 +56,55 @@ __device__ __forceinline__ bool jacobi_sweeps(float* C, int ldc, int w, float s1
   for (int sweep = 0; sweep < max_sweeps && !converged; ++sweep) {
     int rotated = 0;
     for (int round = 0; round < np - 1; ++round) {
-      int a = 0, b = 0;
-      bool active = g < half;
-      if (active) {
-        a = round + g; if (a >= np - 1) a -= np - 1;
-        b = round - g; if (b < 0) b += np - 1;
-        if (g == 0) { a = round; b = np - 1; }
-        if (a > b) { int t = a; a = b; b = t; }
-        active = b < w;
-      }
-      float* ca = C + a * ldc;
-      float* cb = C + b * ldc;
-      float xa[ROWS], xb[ROWS];
-      float al = 0.f, be = 0.f, ga = 0.f;
-#pragma unroll
-      for (int q = 0; q < ROWS; ++q) {
-        int row = gl + 4 * q;
-        bool in = active && row < w;
-        xa[q] = in ? ca[row] : 0.f;
-        xb[q] = in ? cb[row] : 0.f;
-        al += xa[q] * xa[q]; be += xb[q] * xb[q]; ga += xa[q] * xb[q];
-      }
-#pragma unroll
-      for (int o = 2; o > 0; o >>= 1) {
-        al += __shfl_xor_sync(0xffffffffu, al, o);
-        be += __shfl_xor_sync(0xffffffffu, be, o);
-        ga += __shfl_xor_sync(0xffffffffu, ga, o);
-      }
-      float g2 = ga * ga;
-      float thr2 = fmaxf(1e-12f * al * be, abs2 * fminf(al, be));
-      if (active && g2 > thr2 && g2 > 1e-37f) {
-        // tan of the rotation angle: t = sign(d g) 2|g| / (|d| + sqrt(d^2 + 4 g^2)), d = |b|^2 - |a|^2
-        float d = be - al;
-        float t = __fdividef(2.f * ga, fabsf(d) + __fsqrt_rn(d * d + 4.f * g2));
-        if (d < 0.f) t = -t;
-        float c = rsqrtf(t * t + 1.f), sn = t * c;
+      // windows of more than nact / 2 columns have more pairs than groups: the groups go round again (the pairs of
+      // a round are disjoint, so their order does not matter)
+      for (int g0 = 0; g0 < half; g0 += nact >> 2) {
+        const int pair = g0 + g;
+        int a = 0, b = 0;
+        bool active = pair < half;
+        if (active) {
+          a = round + pair; if (a >= np - 1) a -= np - 1;
+          b = round - pair; if (b < 0) b += np - 1;
+          if (pair == 0) { a = round; b = np - 1; }
+          if (a > b) { int t = a; a = b; b = t; }
+          active = b < w;
+        }
+        float* ca = C + a * ldc;
+        float* cb = C + b * ldc;
+        float xa[ROWS], xb[ROWS];
+        float al = 0.f, be = 0.f, ga = 0.f;
 #pragma unroll
         for (int q = 0; q < ROWS; ++q) {
           int row = gl + 4 * q;
-          if (row < w) {
-            ca[row] = c * xa[q] - sn * xb[q];
-            cb[row] = sn * xa[q] + c * xb[q];
-          }
+          bool in = active && row < w;
+          xa[q] = in ? ca[row] : 0.f;
+          xb[q] = in ? cb[row] : 0.f;
+          al += xa[q] * xa[q]; be += xb[q] * xb[q]; ga += xa[q] * xb[q];
         }
-        rotated = 1;
+#pragma unroll
+        for (int o = 2; o > 0; o >>= 1) {
+          al += __shfl_xor_sync(0xffffffffu, al, o);
+          be += __shfl_xor_sync(0xffffffffu, be, o);
+          ga += __shfl_xor_sync(0xffffffffu, ga, o);
+        }
+        float g2 = ga * ga;
+        float thr2 = fmaxf(1e-12f * al * be, abs2 * fminf(al, be));
+        if (active && g2 > thr2 && g2 > 1e-37f) {
+          // tan of the rotation angle: t = sign(d g) 2|g| / (|d| + sqrt(d^2 + 4 g^2)), d = |b|^2 - |a|^2
+          float d = be - al;
+          float t = __fdividef(2.f * ga, fabsf(d) + __fsqrt_rn(d * d + 4.f * g2));
+          if (d < 0.f) t = -t;
+          float c = rsqrtf(t * t + 1.f), sn = t * c;
+#pragma unroll
+          for (int q = 0; q < ROWS; ++q) {
+            int row = gl + 4 * q;
+            if (row < w) {
+              ca[row] = c * xa[q] - sn * xb[q];
+              cb[row] = sn * xa[q] + c * xb[q];
+            }
+          }
+          rotated = 1;
+        }
       }
       sub::named_barrier(1, nact);
     }

@@ -465,3 +465,12 @@ def test_poisoned_scratch_changes_nothing_at_full_size(name):
         assert pr.device_status() == 0
         assert torch.equal(keep2, keep) and torch.equal(out2, out), hex(byte)
     pr.close()
+
+
+def test_ritz_window_with_more_pairs_than_lane_groups():
+    # a window of 132 vectors has 66 column pairs for the 64 lane groups of the eigen-solve; after two
+    # multiplications the window is still far from diagonal, and with pairs left out the sweeps ended at
+    # their limit (status -7)
+    wl = workloads.make_workload("pairs", seed=296, dtype=torch.bfloat16, batch=1, n_vis=600, n_txt=9, d=384, n_heads=1,
+                                 rank=64, keep=232)
+    parity.run_gpu(wl, pruner_kw=dict(ritz_window=1000, eig_iters=1, eig_early_stop=0, conv_tol=0.0))
