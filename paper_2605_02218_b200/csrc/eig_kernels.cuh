@@ -31,7 +31,7 @@ using sub::tri_index;
 
 // Bytes of shared memory the blocked Cholesky factorisation needs for an n x n matrix (8 x 8 tiles
 // of the lower triangle in float64, the original diagonal and the reciprocal pivots).
-__host__ __device__ inline size_t cholesky_smem_bytes(int n) {
+__host__ __device__ constexpr size_t cholesky_smem_bytes(int n) {
   int nb = (n + 7) / 8;
   return ((size_t)nb * (nb + 1) / 2 * 64 + 16 * nb) * sizeof(double);
 }
@@ -204,9 +204,9 @@ __device__ __noinline__ bool jacobi_warp32(int c_off, int w, float s1, int max_s
 
 // Column stride of the window factor in shared memory: >= w and congruent to 4 modulo 32, so that
 // the eight 4-lane groups of a warp, which hold consecutive columns, hit distinct banks.
-__host__ __device__ inline int ritz_ldc(int w) { return (w + 27) / 32 * 32 + 4; }
-// Bytes of dynamic shared memory of ritz_kernel for a window of w vectors.
-__host__ __device__ inline size_t ritz_smem_bytes(int w) {
+__host__ __device__ constexpr int ritz_ldc(int w) { return (w + 27) / 32 * 32 + 4; }
+// Bytes of shared memory the Rayleigh-Ritz step takes for a window of w vectors.
+__host__ __device__ constexpr size_t ritz_smem_bytes(int w) {
   return ((((size_t)w * ritz_ldc(w) + w + 1) & ~(size_t)1)) * sizeof(float) + cholesky_smem_bytes(w);
 }
 

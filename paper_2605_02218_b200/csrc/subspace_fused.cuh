@@ -718,6 +718,13 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
     tile = item - rp.ptile_off;
   };
 
+  // request of the factor server with this index: the index-th one that has a stage 2
+  auto server_request = [&](int index) -> int {
+    for (int q = 0; q < prm.batch; ++q)
+      if (prm.plan[q].stage2 && index-- == 0) return q;
+    return -1;
+  };
+
   if (warp == 8) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
@@ -764,15 +771,21 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
     // A server has nothing to multiply.  While it waits for the tiles this warp runs the eigenvalue
     // rotations of the Ritz window once on a made-up matrix, in the part of the ring that the team
     // does not use: the code is then in the SM's instruction cache when the last step needs it, instead of
-    // being fetched line by line from L2 in the middle of the request's critical path.
+    // being fetched line by line from L2 in the middle of the request's critical path.  Nothing orders the team behind
+    // this warp, so the place must be one that no phase of the team's work reaches: the factorisation and windows of
+    // up to 32 end below it; wider windows do not take this code.
     constexpr int kOff = (kPowRegion - 32 * kRitzLd32 * 4) / 4;
-    float* C = reinterpret_cast<float*>(smem) + kOff;
-    for (int e = lane; e < 32 * kRitzLd32; e += 32) C[e] = 0.f;
-    __syncwarp();
-    C[lane * kRitzLd32 + ritz_row(lane)] = 1.f;
-    if (lane == 0) C[ritz_row(1)] = 0.5f;
-    __syncwarp();
-    jacobi_warp32(kOff, 32, 1.f, 1);
+    static_assert(cholesky_smem_bytes(kPMax) <= kOff * 4 && ritz_smem_bytes(32) <= kOff * 4, "place of the rehearsal");
+    const int served = server_request((int)blockIdx.x - prm.n_tile_ctas);
+    if (served >= 0 && prm.plan[served].win <= 32) {
+      float* C = reinterpret_cast<float*>(smem) + kOff;
+      for (int e = lane; e < 32 * kRitzLd32; e += 32) C[e] = 0.f;
+      __syncwarp();
+      C[lane * kRitzLd32 + ritz_row(lane)] = 1.f;
+      if (lane == 0) C[ritz_row(1)] = 0.5f;
+      __syncwarp();
+      jacobi_warp32(kOff, 32, 1.f, 1);
+    }
   } else if (warp == 9) {
     // ------------------------------------------------------------ MMA issuer
     if (lane == 0) {
@@ -876,10 +889,7 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
       // This CTA carries no tile.  It factors for one request: on a CTA that also carries a tile the
       // factorisation, which needs the operand ring as scratch, would delay that tile's next
       // multiplication, and with it the request's next step.
-      const int mine = (int)blockIdx.x - prm.n_tile_ctas;
-      int b = -1, seen = 0;
-      for (int q = 0; q < prm.batch && b < 0; ++q)
-        if (prm.plan[q].stage2) { if (seen == mine) b = q; ++seen; }
+      const int b = server_request((int)blockIdx.x - prm.n_tile_ctas);
       if (b >= 0) {
         const ReqPlan rp = prm.plan[b];
         unsigned* sync_b = prm.sync + (size_t)b * kSyncStride;
