@@ -562,11 +562,14 @@ __device__ __noinline__ bool team_cholesky(const double* pbase, int nt, int p, i
 }
 
 // Rayleigh-Ritz on the window next to the cut (see eig_kernels.cuh) and the convergence estimate.
-// Uses the operand ring and the factor's place behind it as scratch.
+// Uses the operand ring and the factor's place behind it as scratch: the window factor C, the float64 window block
+// and its two diagonals end before the reciprocal diagonal, which serves as `dg`, for every window.  (At the
+// start of the factor's place `dg` lay inside the float64 block of windows of 136 and more.)
+static_assert(ritz_smem_bytes(kPMax) + 16 <= kPowRegion + kLtFloats * sizeof(float), "scratch of team_ritz");
 __device__ __noinline__ void team_ritz(const double* pbase, int nt, int p, int w, int r, int m, float* out_u,
                                        int max_sweeps, float conv_tol, int steps, int* status) {
   float* C = reinterpret_cast<float*>(pow_smem());
-  float* dg = pow_tail().lt;
+  float* dg = pow_tail().dinv;
   float* s_scale = pow_tail().s_scale;
   int* s_flag = pow_tail().s_flag;
   const int et = threadIdx.x, warp = warp_index(), lane = et & 31;

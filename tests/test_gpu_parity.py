@@ -474,3 +474,22 @@ def test_ritz_window_with_more_pairs_than_lane_groups():
     wl = workloads.make_workload("pairs", seed=296, dtype=torch.bfloat16, batch=1, n_vis=600, n_txt=9, d=384, n_heads=1,
                                  rank=64, keep=232)
     parity.run_gpu(wl, pruner_kw=dict(ritz_window=1000, eig_iters=1, eig_early_stop=0, conv_tol=0.0))
+
+
+@pytest.mark.parametrize("keep,oversample,window", [(256, 16, 40), (256, 16, 64), (256, 16, 100), (256, 16, 112),
+                                                    (240, 16, 1000), (256, 16, 1000), (256, 32, 1000)])
+def test_wide_ritz_windows(keep, oversample, window):
+    # windows of 56, 80, 116, 128 and all of p = 136, 144, 160 basis vectors: the scratch of the Rayleigh-Ritz step
+    # grows with the window (at p >= 136 its float64 block used to reach the diagonal kept beside it)
+    wl = workloads.make_workload("window", seed=keep + oversample + window, dtype=torch.bfloat16, batch=2, n_vis=(600, 700),
+                                 n_txt=9, d=384, n_heads=1, rank=64, keep=keep)
+    kw = dict(ritz_window=window, eig_oversample=oversample)
+    _report(wl.name, parity.run_gpu(wl, pruner_kw=kw))
+    from paper_2605_02218_b200 import api
+    dev = wl.to("cuda:0")
+    pr = api.Pruner.for_workload(dev, **kw)
+    m = pr.marshal(dev)
+    _, _, sf = pr.score(m)
+    energies = [pr.select(m, sf)[4] for _ in range(4)]
+    assert all(torch.equal(energies[0], e) for e in energies[1:])
+    pr.close()
