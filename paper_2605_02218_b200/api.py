@@ -423,7 +423,8 @@ def correct(z_draft: torch.Tensor, z_target: torch.Tensor, uniforms: torch.Tenso
     margin, accept, mass = torch.empty((3, rows), dtype=torch.float32, device=dev).unbind(0)
     gate, token = torch.empty((2, rows), dtype=torch.int32, device=dev).unbind(0)
     st = lib.covspec_correct(_LOGIT_DTYPES[z_draft.dtype], rows, ld if vocab is None else vocab, ld, z_draft.data_ptr(),
-                             z_target.data_ptr(), None if drafted is None else drafted.data_ptr(), uniforms.data_ptr(), gamma,
+                             z_target.data_ptr(), None if drafted is None else drafted.data_ptr(),
+                             None if uniforms is None else uniforms.data_ptr(), gamma,
                              margin.data_ptr(), gate.data_ptr(), accept.data_ptr(), mass.data_ptr(), token.data_ptr(),
                              _raw_stream())
     if st:

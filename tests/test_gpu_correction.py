@@ -90,6 +90,14 @@ def test_argument_errors():
     assert e.value.status == -2
 
 
+def test_missing_random_numbers_are_an_argument_error():
+    from paper_2605_02218_b200 import api
+    z = torch.zeros(2, 16, dtype=torch.float16, device="cuda:0")
+    with pytest.raises(api.CovspecError) as e:
+        api.correct(z, z, None, 0.1)
+    assert e.value.status == -1
+
+
 @pytest.mark.parametrize("dtype", [torch.float16, torch.float32])
 def test_branch_candidates(dtype):
     from paper_2605_02218_b200 import api
