@@ -98,6 +98,16 @@ def test_missing_random_numbers_are_an_argument_error():
     assert e.value.status == -1
 
 
+def test_every_result_of_a_correction_has_memory_of_its_own():
+    # kept or passed on by itself: no result holds another one's memory, each base is aligned for vector loads
+    from paper_2605_02218_b200 import api
+    data = workloads.make_logits(seed=6, rows=3, vocab=1000, dtype=torch.float16, device="cuda:0")
+    got = api.correct(data["z_draft"], data["z_target"], data["uniforms"], 0.05, data["drafted"], vocab=1000)
+    assert len({t.untyped_storage().data_ptr() for t in got}) == len(got)
+    for t in got:
+        assert t.untyped_storage().nbytes() == 4 * 3 and t._base is None and t.data_ptr() % 16 == 0
+
+
 @pytest.mark.parametrize("dtype", [torch.float16, torch.float32])
 def test_branch_candidates(dtype):
     from paper_2605_02218_b200 import api
