@@ -186,9 +186,17 @@ class _Marshalled:
                                keep_p, float(keep_ratio))
 
 
+# torch's own accessors of the current stream's address; a build without them takes the public route
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+_raw_of_device = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _raw_stream() -> int:
-    """The address torch.cuda.current_stream().cuda_stream gives, without making the Stream object (2-3 us)."""
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    """The address torch.cuda.current_stream().cuda_stream gives, without making the Stream object (0.2 us
+    against 3.2)."""
+    if _raw_device is None or _raw_of_device is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_of_device(_raw_device())
 
 
 def _stream():

@@ -138,3 +138,17 @@ def test_checked_build_exports_the_same_interface(lib):
     assert lib.covspec_build_has_bounds_checks() == 0
     dbg.covspec_strerror.restype = C.c_char_p
     assert b"out of range" in dbg.covspec_strerror(-10)
+
+
+def test_current_stream_without_torch_internals(monkeypatch):
+    # the binding reads the stream's address through two internals of torch; without them it takes the public way
+    import importlib.util
+    from types import SimpleNamespace
+    import torch
+    for name in ("_cuda_getDevice", "_cuda_getCurrentRawStream"):
+        monkeypatch.delattr(torch._C, name, raising=False)
+    spec = importlib.util.spec_from_file_location("covspec_api_again", api.__file__)
+    again = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(again)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: SimpleNamespace(cuda_stream=4711))
+    assert again._raw_stream() == 4711 and again._stream().value == 4711
