@@ -563,10 +563,14 @@ correct_kernel(const T* __restrict__ zd, const T* __restrict__ zt, long long ldz
   }
 }
 
-// CTAs per position.  Two are enough once every SM has its two CTAs (148 positions); fewer positions are
-// spread over up to eight CTAs each, as many as still run at the same time (two CTAs on each of 148
-// SMs), so that a drafted block of eight positions uses 64 SMs instead of 16.
-inline int cluster_ctas(int rows) { return rows > 74 ? 2 : rows > 37 ? 4 : 8; }
+// CTAs per position.  Few positions are spread over up to eight CTAs each, so that a drafted block of eight positions uses
+// 64 SMs instead of 16, for as long as every CTA gets an SM to itself: 128 CTAs of clusters of 4 or 8 do on 148 SMs
+// (a cluster stays inside one GPC, so not every SM can be had); beyond that two CTAs of one SM take their
+// sweeps in turn and splitting costs more than it gives.  151,674 float16 logits, calls back to back in a graph,
+// clusters of 8 / 4 / 2: 8 positions 13.0 / 16.8 / 19.1 us, 16: 16.8 / 17.0 / 19.1, 32: 19.7 / 17.4 / 19.4,
+// 38: 27.3 / 23.3 / 19.3, 74: 41.5 / 34.9 / 19.7.
+constexpr int kSpreadCtas = 128;
+inline int cluster_ctas(int rows) { return 8 * rows <= kSpreadCtas ? 8 : 4 * rows <= kSpreadCtas ? 4 : 2; }
 constexpr size_t kSumsMost = 96 * 1024;              // shared memory for the vector sums: two CTAs per SM
 // Dynamic shared memory of a CTA: one sum per vector of its segments, two where several warps share one.
 template <typename T>

@@ -165,3 +165,19 @@ def test_result_of_a_position_does_not_depend_on_the_call_size(rows):
     torch.cuda.synchronize()
     for a, b in zip(whole, part):
         assert torch.equal(a[:rows], b)
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("rows", [1, 16, 17, 32, 33])
+def test_call_size_at_the_limits_of_the_cluster_sizes(rows, dtype):
+    # the same for all logit types at the limits of the 8, 4 and 2 CTAs per position, a vocabulary that ends inside a vector
+    from paper_2605_02218_b200 import api
+    vocab = 40013
+    data = workloads.make_logits(seed=9, rows=160, vocab=vocab, dtype=dtype, device="cuda:0")
+    data["z_draft"][rows - 1, 20000:vocab] += 200.0
+    args = lambda n: (data["z_draft"][:n], data["z_target"][:n], data["uniforms"][:n], 0.05, data["drafted"][:n])
+    whole = api.correct(*args(160), vocab=vocab)
+    part = api.correct(*args(rows), vocab=vocab)
+    torch.cuda.synchronize()
+    for a, b in zip(whole, part):
+        assert torch.equal(a[:rows], b)
