@@ -173,6 +173,11 @@ template <> struct Top2Run<__nv_bfloat16> {
 // How far above the reference of a running sum a logit may lie before the sum is moved to a new
 // reference: exp(60) ~ 1e26 leaves room for a whole vocabulary of such terms in float32.
 constexpr float kRefSlack = 60.f;
+// Lowest reference.  Masked entries (the type's lowest value, -1e30, ...) may open a lane's share of the row; relative
+// to such a reference the exponent's rounding alone is beyond the range (1.44e9, for a reference of -1e9, is
+// rounded by up to 64), the sum becomes infinite and the next move of the reference makes it NaN.  Entries this low
+// weigh nothing beside an ordinary logit.
+constexpr float kRefFloor = -1e9f;
 
 // ---- thread-block cluster helpers (a position is shared by the CTAs of a cluster) ----
 __device__ __forceinline__ unsigned cluster_rank() {
@@ -284,8 +289,14 @@ correct_kernel(const T* __restrict__ zd, const T* __restrict__ zt, long long ldz
     return make_float2(sa, sb);
   };
   auto move_reference = [&](float va, float vb) {
-    if (va > thr_d) { md.s *= __expf(md.m - va); md.m = va; nd = -va * kLog2e; thr_d = va + kRefSlack; }
-    if (vb > thr_t) { mt.s *= __expf(mt.m - vb); mt.m = vb; nt = -vb * kLog2e; thr_t = vb + kRefSlack; }
+    if (va > thr_d) {
+      const float m = fmaxf(va, kRefFloor);
+      md.s *= __expf(md.m - m); md.m = m; nd = -m * kLog2e; thr_d = m + kRefSlack;
+    }
+    if (vb > thr_t) {
+      const float m = fmaxf(vb, kRefFloor);
+      mt.s *= __expf(mt.m - m); mt.m = m; nt = -m * kLog2e; thr_t = m + kRefSlack;
+    }
   };
   auto sweep1 = [&](const uint4& ra, const uint4& rb) {
     // every vector holds at least one element of the vocabulary; 2^(-inf) = 0 takes care of padding

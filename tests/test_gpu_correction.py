@@ -181,3 +181,28 @@ def test_call_size_at_the_limits_of_the_cluster_sizes(rows, dtype):
     torch.cuda.synchronize()
     for a, b in zip(whole, part):
         assert torch.equal(a[:rows], b)
+
+
+@pytest.mark.parametrize("dtype,value", [(torch.float16, None), (torch.bfloat16, None), (torch.float32, None),
+                                         (torch.float32, -1e30), (torch.float32, -1e9), (torch.float16, -np.inf)])
+@pytest.mark.parametrize("rows", [2, 24, 40])
+def test_masked_logits(dtype, value, rows):
+    # most of the vocabulary masked in both rows (None: the type's lowest value), the beginning of the row included;
+    # one row unmasked in the draft with the drafted token masked in the target
+    from paper_2605_02218_b200 import api
+    vocab = 20011
+    value = torch.finfo(dtype).min if value is None else value
+    data = workloads.make_logits(seed=11, rows=rows, vocab=vocab, dtype=dtype, device="cuda:0")
+    zd, zt = data["z_draft"], data["z_target"]
+    allowed = torch.zeros(vocab, dtype=torch.bool, device="cuda:0")
+    allowed[torch.arange(50, vocab, 701)] = True
+    plain = zd[1].clone()
+    zd[:, :vocab][:, ~allowed] = value
+    zt[:, :vocab][:, ~allowed] = value
+    zd[1] = plain
+    data["drafted"][:] = 50 + 701 * 3
+    data["drafted"][1] = 7
+    got = api.correct(zd, zt, data["uniforms"], 0.05, data["drafted"], vocab=vocab)
+    torch.cuda.synchronize()
+    _check(data, 0.05, got)
+    assert all(bool(allowed[t]) for t in got[4].tolist())
