@@ -579,9 +579,14 @@ correct_kernel(const T* __restrict__ zd, const T* __restrict__ zt, long long ldz
 // (a cluster stays inside one GPC, so not every SM can be had); beyond that two CTAs of one SM take their
 // sweeps in turn and splitting costs more than it gives.  151,674 float16 logits, calls back to back in a graph,
 // clusters of 8 / 4 / 2: 8 positions 13.0 / 16.8 / 19.1 us, 16: 16.8 / 17.0 / 19.1, 32: 19.7 / 17.4 / 19.4,
-// 38: 27.3 / 23.3 / 19.3, 74: 41.5 / 34.9 / 19.7.
+// 38: 27.3 / 23.3 / 19.3, 74: 41.5 / 34.9 / 19.7.  float32 rows (twice the bytes): 8: 16.1 / 21.8 / 22.8,
+// 24: 20.7 / 22.0 / 22.9, 32: 22.3 / 22.4 / 23.4, 38: 33.0 / 28.4 / 23.4; clusters of 8 all the way.
 constexpr int kSpreadCtas = 128;
-inline int cluster_ctas(int rows) { return 8 * rows <= kSpreadCtas ? 8 : 4 * rows <= kSpreadCtas ? 4 : 2; }
+template <typename T>
+int cluster_ctas(int rows) {
+  if (4 * rows > kSpreadCtas) return 2;
+  return 8 * rows <= kSpreadCtas || sizeof(T) == 4 ? 8 : 4;
+}
 constexpr size_t kSumsMost = 96 * 1024;              // shared memory for the vector sums: two CTAs per SM
 // Dynamic shared memory of a CTA: one sum per vector of its segments, two where several warps share one.
 template <typename T>
@@ -623,7 +628,7 @@ template <typename T>
 cudaError_t launch_correct(int rows, const T* zd, const T* zt, long long ldz, int w, const int* drafted,
                            const float* uniforms, float gamma, float* margin, int* gate, float* accept,
                            float* resid_mass, int* token, cudaStream_t s) {
-  int cl = cluster_ctas(rows);
+  int cl = cluster_ctas<T>(rows);
   if (sums_bytes<T>(cl, w) > kSumsMost) cl = 2;       // a row too long for sums in shared memory: two CTAs need none
   const auto f = cl == 2 ? launch_correct_n<T, 2> : cl == 4 ? launch_correct_n<T, 4> : launch_correct_n<T, 8>;
   return f(rows, zd, zt, ldz, w, drafted, uniforms, gamma, margin, gate, accept, resid_mass, token, s);
