@@ -226,13 +226,15 @@ int covspec_fanout(int f0, double rho, int j);
  *  z_draft       device [rows, ld], layout and alignment as in covspec_correct
  *  drafted       device [rows] int32 drafted token ids, or NULL (nothing excluded)
  *  cand_offsets  device [rows+1] int32 prefix sums of the fan-outs F_j (built by the caller)
- *  max_fanout    largest F_j (host); must be <= vocab - 1
+ *  max_fanout    largest F_j (host); must be <= vocab - 1.  A hint for the choice of the kernel: a position whose
+ *                offsets ask for more still gets its F_j candidates
  *  cand          device [cand_offsets[rows]] int32 (out): candidate token ids, ascending per position */
 int covspec_branch_candidates(int logit_dtype, int rows, int vocab, long long ld, const void* z_draft,
                               const int* drafted, const int* cand_offsets, int max_fanout, int* cand,
                               void* stream);
 
 /* The same with cand_offsets on the host (read before the call returns; no copy to the device is made).
+ * Offsets that fall, start below zero or ask for more than max_fanout at a position: COVSPEC_ERR_SHAPE.
  * Fan-outs up to 64, rows of at least 32 KB and a 16-byte aligned z_draft; else COVSPEC_ERR_UNSUPPORTED and
  * nothing is launched. */
 int covspec_branch_candidates_host(int logit_dtype, int rows, int vocab, long long ld, const void* z_draft,

@@ -684,6 +684,11 @@ branch_fast_kernel(const T* __restrict__ zd, long long ldz, int w, const int* __
   if (f <= 0) return;                                // the whole cluster
   const T* r = zd + (size_t)row * ldz;
   const int y = drafted != nullptr ? __ldg(drafted + row) : -1;
+  if (f > kFastFanout) {                             // offsets that ask for more than max_fanout said (again the whole cluster)
+    if (crank == 0)
+      block_topk_by([&](int i) { return i == y ? -INFINITY : cvt(r[i]); }, w, f, false, nullptr, cand + off, nullptr);
+    return;
+  }
   const int nvec = (w + N - 1) / N, first = (int)crank * kFastThreads + tid;
   constexpr int kStep = kFastCtas * kFastThreads;
   if (tid == 0) s_count = 0u;

@@ -1430,6 +1430,12 @@ int branch_candidates_impl(int logit_dtype, int rows, int vocab, long long ld, c
   int esize = logit_dtype == COVSPEC_F32 ? 4 : 2;
   if (rows < 1 || vocab < 2 || ld < vocab || (ld * esize) % 16 != 0) return COVSPEC_ERR_SHAPE;
   if (max_fanout < 0 || max_fanout > vocab - 1) return COVSPEC_ERR_SHAPE;
+  if (host_offsets) {
+    if (host_offsets[0] < 0) return COVSPEC_ERR_SHAPE;
+    for (int r = 0; r < rows; ++r)
+      if (host_offsets[r + 1] < host_offsets[r] || (long long)host_offsets[r + 1] - host_offsets[r] > max_fanout)
+        return COVSPEC_ERR_SHAPE;
+  }
   // the cluster kernel reads whole 16-byte vectors; larger fan-outs, short rows and other bases take a
   // block per row
   const bool fast = max_fanout <= corr::kFastFanout && (reinterpret_cast<uintptr_t>(z_draft) & 15) == 0 &&

@@ -206,3 +206,24 @@ def test_masked_logits(dtype, value, rows):
     torch.cuda.synchronize()
     _check(data, 0.05, got)
     assert all(bool(allowed[t]) for t in got[4].tolist())
+
+
+def test_branch_candidates_beyond_the_stated_fan_out():
+    # device offsets that ask one position for more than max_fanout says: every position gets what its offsets ask for
+    from paper_2605_02218_b200 import api
+    lib, vocab, fans = api.load_library(), 40000, [4, 65, 200, 0, 1500, 8]
+    data = workloads.make_logits(seed=13, rows=len(fans), vocab=vocab, dtype=torch.float16, device="cuda:0")
+    off = np.concatenate([[0], np.cumsum(fans)]).astype(np.int32)
+    d_off = torch.from_numpy(off).cuda()
+    cand = torch.full((int(off[-1]),), -1, dtype=torch.int32, device="cuda:0")
+    st = lib.covspec_branch_candidates(api.COVSPEC_F16, len(fans), vocab, data["ld"], data["z_draft"].data_ptr(),
+                                       data["drafted"].data_ptr(), d_off.data_ptr(), 8, cand.data_ptr(), api._raw_stream())
+    assert st == 0
+    torch.cuda.synchronize()
+    cand = cand.cpu().numpy()
+    for i, f in enumerate(fans):
+        want = C.bonus_candidates(data["z_draft"][i, :vocab].cpu().double().numpy(), int(data["drafted"][i]), f)
+        assert np.array_equal(cand[off[i]:off[i + 1]], want), i
+    with pytest.raises(api.CovspecError) as e:
+        api.branch_candidates(data["z_draft"], [2, -1, 3, 0, 1, 1], data["drafted"], vocab=vocab)
+    assert e.value.status == -2

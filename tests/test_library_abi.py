@@ -152,3 +152,12 @@ def test_current_stream_without_torch_internals(monkeypatch):
     spec.loader.exec_module(again)
     monkeypatch.setattr(torch.cuda, "current_stream", lambda: SimpleNamespace(cuda_stream=4711))
     assert again._raw_stream() == 4711 and again._stream().value == 4711
+
+
+@pytest.mark.parametrize("offsets,most", [([0, 3, 2, 4], 8), ([-1, 2, 4, 6], 8), ([0, 4, 13, 15], 8), ([0, 1, 2, 3], -1)])
+def test_branch_candidate_offsets_are_tested_on_the_host(lib, offsets, most):
+    # a falling offset would send a position's candidates over its neighbour's or past the end of the buffer; the call ends
+    # before anything is launched (the addresses are never used)
+    off = np.array(offsets, dtype=np.int32)
+    assert lib.covspec_branch_candidates_host(api.COVSPEC_F16, 3, 40000, 40000, C.c_void_p(1 << 20), None,
+                                              off.ctypes.data_as(C.c_void_p), most, C.c_void_p(1 << 20), None) == -2
