@@ -634,6 +634,13 @@ cudaError_t launch_correct(int rows, const T* zd, const T* zt, long long ldz, in
   return f(rows, zd, zt, ldz, w, drafted, uniforms, gamma, margin, gate, accept, resid_mass, token, s);
 }
 
+// Logit i of a row as the candidate selections see it: the drafted token `y` comes last, behind entries masked with -inf
+// (NaN has the smallest key).
+template <typename T>
+__device__ __forceinline__ float entry(const T* __restrict__ r, int i, int y) {
+  return i == y ? __int_as_float(0x7fc00000) : cvt(r[i]);
+}
+
 // Bonus-token candidates of the parallel branching (Sec. III-C.1, Eq. 23): for every position the
 // F_j largest draft logits, the token drafted at that position excluded; ties go to the lower
 // token id; ids are written in ascending order at cand[cand_offsets[row] ...].  One block per
@@ -647,7 +654,7 @@ branch_candidates_kernel(const T* __restrict__ zd, long long ldz, int w, const i
   if (f <= 0) return;
   const T* r = zd + (size_t)row * ldz;
   const int y = drafted != nullptr ? drafted[row] : -1;
-  block_topk_by([&](int i) { return i == y ? -INFINITY : cvt(r[i]); }, w, min(f, w), false, nullptr,
+  block_topk_by([&](int i) { return entry(r, i, y); }, w, min(f, w), false, nullptr,
                 cand + off, nullptr);
 }
 
@@ -686,13 +693,13 @@ branch_fast_kernel(const T* __restrict__ zd, long long ldz, int w, const int* __
   const int y = drafted != nullptr ? __ldg(drafted + row) : -1;
   if (f > kFastFanout) {                             // offsets that ask for more than max_fanout said (again the whole cluster)
     if (crank == 0)
-      block_topk_by([&](int i) { return i == y ? -INFINITY : cvt(r[i]); }, w, f, false, nullptr, cand + off, nullptr);
+      block_topk_by([&](int i) { return entry(r, i, y); }, w, f, false, nullptr, cand + off, nullptr);
     return;
   }
   const int nvec = (w + N - 1) / N, first = (int)crank * kFastThreads + tid;
   constexpr int kStep = kFastCtas * kFastThreads;
   if (tid == 0) s_count = 0u;
-  auto key_at = [&](int i) { return order_key(i == y ? -INFINITY : cvt(r[i])); };
+  auto key_at = [&](int i) { return order_key(entry(r, i, y)); };
   auto special = [&](int v) { return (v + 1) * N > w || (y >= v * N && y < (v + 1) * N); };   // row end, drafted token
   unsigned mine = 0u;
 #pragma unroll 4
@@ -756,7 +763,7 @@ branch_fast_kernel(const T* __restrict__ zd, long long ldz, int w, const int* __
   if (crank != 0) return;
   const int n = (int)min(s_count, (unsigned)(kFastList + 1));
   if (n > kFastList) {
-    block_topk_by([&](int i) { return i == y ? -INFINITY : cvt(r[i]); }, w, f, false, nullptr, cand + off, nullptr);
+    block_topk_by([&](int i) { return entry(r, i, y); }, w, f, false, nullptr, cand + off, nullptr);
     return;
   }
   // the F_j first in (larger key, lower id) order, written by ascending id

@@ -227,3 +227,18 @@ def test_branch_candidates_beyond_the_stated_fan_out():
     with pytest.raises(api.CovspecError) as e:
         api.branch_candidates(data["z_draft"], [2, -1, 3, 0, 1, 1], data["drafted"], vocab=vocab)
     assert e.value.status == -2
+
+
+@pytest.mark.parametrize("vocab", [5003, 40013])
+def test_drafted_token_is_no_candidate_among_masked_ones(vocab):
+    # fewer unmasked tokens than candidates: the rest are masked ones by their ids, never the drafted token
+    from paper_2605_02218_b200 import api
+    data = workloads.make_logits(seed=15, rows=2, vocab=vocab, dtype=torch.float16, device="cuda:0")
+    z, y = data["z_draft"], data["drafted"]
+    z[:, 4:vocab] = -np.inf
+    y[0], y[1] = 6, 2
+    cand, off = api.branch_candidates(z, [9, 9], y, vocab=vocab)
+    torch.cuda.synchronize()
+    for i in range(2):
+        want = C.bonus_candidates(z[i, :vocab].cpu().double().numpy(), int(y[i]), 9)
+        assert np.array_equal(cand.cpu().numpy()[off[i]:off[i + 1]], want), i
