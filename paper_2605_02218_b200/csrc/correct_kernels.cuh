@@ -668,9 +668,83 @@ constexpr int kFastFanout = 64;                      // largest fan-out of this 
 constexpr int kFastCtas = 8, kFastThreads = 512;
 constexpr int kFastWarps = kFastCtas * kFastThreads / 32;
 constexpr int kFastMinVec = 32 * kFastFanout;        // shorter rows give fewer warps with a vector than F_j may ask for
-constexpr int kFastList = 1024;                      // entries that are ranked directly; more (mass ties): block_topk_by
+constexpr int kFastList = 1024;                      // entries that are ranked directly
 constexpr int kFastRows = 512;                       // positions per launch: their offsets travel as kernel arguments
 struct FanOffsets { int v[kFastRows + 1]; };
+
+// Mass ties: a row masked down to fewer tokens than F_j, say, whose F_j-th largest key (the threshold) is the mask, so
+// that more entries reach it than are ranked directly.  One CTA lists what lies above the threshold (raising it while
+// that is more than the list holds), then takes ties in the order of their ids until it has F_j; returns the length of
+// the list, or -1 when the list was too short to the end: the candidates are then selected and written here.  A row
+// of 151,674 float16 logits with 15 of them unmasked, F_j = 32, eight rows: 26 us (499 with every thread that saw a tie
+// at the counter and the general selection behind it).  Out of line: rare.
+template <typename T>
+__device__ __noinline__ int list_ties(const T* __restrict__ r, int w, int y, int f, unsigned threshold, unsigned* count,
+                                      unsigned* list_key, int* list_id, int* __restrict__ cand) {
+  constexpr int N = Vec<T>::N;
+  __shared__ unsigned scan_totals[33];
+  __shared__ unsigned raised;
+  const int tid = threadIdx.x, nvec = (w + N - 1) / N;
+  __syncthreads();                                   // everybody has read the count
+  if (tid == 0) *count = 0u;
+  __syncthreads();
+  auto special = [&](int v) { return (v + 1) * N > w || (y >= v * N && y < (v + 1) * N); };
+  auto each = [&](int v, auto take) {                // (id, key) of every entry of vector v
+    if (special(v)) {
+      for (int i = v * N; i < min(w, (v + 1) * N); ++i) take(i, order_key(entry(r, i, y)));
+    } else {
+      float e[N];
+      unpack(__ldg(reinterpret_cast<const uint4*>(r) + v), e, (const T*)nullptr);
+#pragma unroll
+      for (int q = 0; q < N; ++q) take(v * N + q, order_key(e[q]));
+    }
+  };
+  int n = 0;
+  for (int round = 0;; ++round) {
+#pragma unroll 4
+    for (int v = tid; v < nvec; v += kFastThreads) {
+      if (!special(v) && order_key(vec_max(__ldg(reinterpret_cast<const uint4*>(r) + v), (const T*)nullptr)) <= threshold) continue;
+      each(v, [&](int i, unsigned k) {
+        if (k <= threshold) return;
+        const unsigned at = atomicAdd(count, 1u);
+        if (at < (unsigned)kFastList) { list_key[at] = k; list_id[at] = i; }
+      });
+    }
+    __syncthreads();
+    n = (int)min(*count, (unsigned)(kFastList + 1));
+    if (n <= kFastList) break;
+    if (round == 3) {
+      block_topk_by([&](int i) { return entry(r, i, y); }, w, f, false, nullptr, cand, nullptr);
+      return -1;
+    }
+    // more than the list holds: the F_j-th largest of those it holds is a higher threshold that F_j entries reach
+    for (int e = tid; e < kFastList; e += kFastThreads) {
+      const unsigned k = list_key[e];
+      int above = 0, reach = 0;
+      for (int j = 0; j < kFastList; ++j) { above += list_key[j] > k; reach += list_key[j] >= k; }
+      if (above < f && f <= reach) raised = k;
+    }
+    __syncthreads();
+    threshold = raised;
+    if (tid == 0) *count = 0u;
+    __syncthreads();
+  }
+  for (int v0 = 0; n < f && v0 < nvec; v0 += kFastThreads) {         // n: the same in all threads
+    const int v = v0 + tid;
+    unsigned ties = 0u, total;
+    if (v < nvec) each(v, [&](int, unsigned k) { ties += k == threshold; });
+    int at = n + (int)block_exclusive_scan(ties, scan_totals, &total);
+    if (ties != 0u)
+      each(v, [&](int i, unsigned k) {
+        if (k != threshold) return;
+        if (at < f) { list_key[at] = k; list_id[at] = i; }
+        ++at;
+      });
+    n = min(f, n + (int)total);
+  }
+  __syncthreads();
+  return n;
+}
 
 template <typename T>
 __global__ void __cluster_dims__(kFastCtas, 1, 1) __launch_bounds__(kFastThreads)
@@ -735,7 +809,10 @@ branch_fast_kernel(const T* __restrict__ zd, long long ldz, int w, const int* __
   }
   __syncthreads();
   const unsigned threshold = s_threshold;
-  if (mine >= threshold) {
+  // far more warps at the threshold than F_j: mass ties, which CTA 0 takes up by itself (thousands of threads would
+  // queue up at its counter)
+  const bool push = __syncthreads_count(tid < kFastWarps && keys[tid & (kFastWarps - 1)] >= threshold) <= f + kFastWarps / 4;
+  if (push && mine >= threshold) {
     auto take = [&](int i, unsigned k) {
       if (k < threshold) return;
       unsigned at;
@@ -761,10 +838,10 @@ branch_fast_kernel(const T* __restrict__ zd, long long ldz, int w, const int* __
   }
   cluster_sync();                                    // the list is complete in CTA 0
   if (crank != 0) return;
-  const int n = (int)min(s_count, (unsigned)(kFastList + 1));
+  int n = push ? (int)min(s_count, (unsigned)(kFastList + 1)) : kFastList + 1;
   if (n > kFastList) {
-    block_topk_by([&](int i) { return entry(r, i, y); }, w, f, false, nullptr, cand + off, nullptr);
-    return;
+    n = list_ties<T>(r, w, y, f, threshold, &s_count, list_key, list_id, cand + off);
+    if (n < 0) return;
   }
   // the F_j first in (larger key, lower id) order, written by ascending id
   for (int q = tid; q < kFastList / 32; q += kFastThreads) chosen[q] = 0u;

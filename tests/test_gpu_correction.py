@@ -242,3 +242,38 @@ def test_drafted_token_is_no_candidate_among_masked_ones(vocab):
     for i in range(2):
         want = C.bonus_candidates(z[i, :vocab].cpu().double().numpy(), int(y[i]), 9)
         assert np.array_equal(cand.cpu().numpy()[off[i]:off[i + 1]], want), i
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("vocab", [16390, 40013])
+def test_branch_candidates_among_mass_ties(dtype, vocab):
+    # rows whose F_j-th largest logit is shared by most of the row: masked down to a few tokens (-inf and the type's lowest
+    # value; the drafted token among them or among the masked ones), one value throughout, ties only at the end,
+    # and more entries above the ties than are ranked directly (bunched, and rising to the end of the row)
+    from paper_2605_02218_b200 import api
+    rows = 8
+    data = workloads.make_logits(seed=14, rows=rows, vocab=vocab, dtype=dtype, device="cuda:0")
+    z, y = data["z_draft"], data["drafted"]
+    allowed = torch.zeros(vocab, dtype=torch.bool, device="cuda:0")
+    allowed[[3, 9000, 9001, vocab - 1]] = True
+    for i, value in enumerate((-np.inf, torch.finfo(dtype).min, -np.inf)):
+        z[i, :vocab][~allowed] = value
+    y[0], y[1], y[2] = 9000, 5, 0
+    z[3, :vocab] = 1.5
+    y[3] = 0
+    z[4, :vocab] = -2.0
+    z[4, vocab - 3000:vocab] = 4.0
+    z[4, 17] = 5.0
+    z[5, :vocab] = 0.0
+    z[5, 100:2500] = torch.linspace(1, 9, 2400, device="cuda:0").to(dtype)
+    stride = torch.arange(vocab, device="cuda:0") % 32768 < (256 if dtype != torch.float32 else 128)
+    z[6, :vocab] = torch.where(stride, 2.0 + torch.rand(vocab, device="cuda:0"), torch.zeros(vocab, device="cuda:0")).to(dtype)
+    z[7, :vocab] = 0.0
+    z[7, vocab - 9000:vocab] = torch.linspace(1, 9, 9000, device="cuda:0").to(dtype)
+    for fan in (1, 3, 4, 32, 64):
+        cand, off = api.branch_candidates(z, [fan] * rows, y, vocab=vocab)
+        torch.cuda.synchronize()
+        cand = cand.cpu().numpy()
+        for i in range(rows):
+            want = C.bonus_candidates(z[i, :vocab].cpu().double().numpy(), int(y[i]), fan)
+            assert np.array_equal(cand[off[i]:off[i + 1]], want), (i, fan)
