@@ -672,15 +672,43 @@ constexpr int kFastList = 1024;                      // entries that are ranked 
 constexpr int kFastRows = 512;                       // positions per launch: their offsets travel as kernel arguments
 struct FanOffsets { int v[kFastRows + 1]; };
 
+// The F_j first of the n listed entries in (larger key, lower id) order, written by ascending id.
+__device__ __forceinline__ void write_ranked(const unsigned* list_key, const int* list_id, int n, int f, unsigned* chosen,
+                                             int* __restrict__ cand) {
+  for (int q = (int)threadIdx.x; q < kFastList / 32; q += kFastThreads) chosen[q] = 0u;
+  __syncthreads();
+  for (int e = (int)threadIdx.x; e < n; e += kFastThreads) {
+    const unsigned k = list_key[e];
+    const int id = list_id[e];
+    int rank = 0;
+    for (int j = 0; j < n; ++j) rank += list_key[j] > k || (list_key[j] == k && list_id[j] < id);
+    if (rank < f) atomicOr(&chosen[e >> 5], 1u << (e & 31));
+  }
+  __syncthreads();
+  for (int e = (int)threadIdx.x; e < n; e += kFastThreads) {
+    if (!(chosen[e >> 5] >> (e & 31) & 1u)) continue;
+    const int id = list_id[e];
+    int pos = 0;
+    for (int j = 0; j < n; ++j) pos += (chosen[j >> 5] >> (j & 31) & 1u) && list_id[j] < id;
+    cand[pos] = id;
+  }
+}
+
+// The general selection.
+template <typename T>
+__device__ __forceinline__ void select_row(const T* __restrict__ r, int w, int y, int f, int* __restrict__ cand) {
+  block_topk_by([&](int i) { return entry(r, i, y); }, w, f, false, nullptr, cand, nullptr);
+}
+
 // Mass ties: a row masked down to fewer tokens than F_j, say, whose F_j-th largest key (the threshold) is the mask, so
 // that more entries reach it than are ranked directly.  One CTA lists what lies above the threshold (raising it while
-// that is more than the list holds), then takes ties in the order of their ids until it has F_j; returns the length of
-// the list, or -1 when the list was too short to the end: the candidates are then selected and written here.  A row
+// that is more than the list holds), takes ties in the order of their ids until it has F_j, and writes the candidates.  A row
 // of 151,674 float16 logits with 15 of them unmasked, F_j = 32, eight rows: 26 us (499 with every thread that saw a tie
-// at the counter and the general selection behind it).  Out of line: rare.
+// at the counter and the general selection behind it).  In line: a call, although hardly ever taken, made the
+// usual path 4 % longer.
 template <typename T>
-__device__ __noinline__ int list_ties(const T* __restrict__ r, int w, int y, int f, unsigned threshold, unsigned* count,
-                                      unsigned* list_key, int* list_id, int* __restrict__ cand) {
+__device__ __forceinline__ void list_ties(const T* __restrict__ r, int w, int y, int f, unsigned threshold, unsigned* count,
+                                          unsigned* list_key, int* list_id, unsigned* chosen, int* __restrict__ cand) {
   constexpr int N = Vec<T>::N;
   __shared__ unsigned scan_totals[33];
   __shared__ unsigned raised;
@@ -714,8 +742,8 @@ __device__ __noinline__ int list_ties(const T* __restrict__ r, int w, int y, int
     n = (int)min(*count, (unsigned)(kFastList + 1));
     if (n <= kFastList) break;
     if (round == 3) {
-      block_topk_by([&](int i) { return entry(r, i, y); }, w, f, false, nullptr, cand, nullptr);
-      return -1;
+      select_row<T>(r, w, y, f, cand);
+      return;
     }
     // more than the list holds: the F_j-th largest of those it holds is a higher threshold that F_j entries reach
     for (int e = tid; e < kFastList; e += kFastThreads) {
@@ -743,7 +771,7 @@ __device__ __noinline__ int list_ties(const T* __restrict__ r, int w, int y, int
     n = min(f, n + (int)total);
   }
   __syncthreads();
-  return n;
+  write_ranked(list_key, list_id, n, f, chosen, cand);
 }
 
 template <typename T>
@@ -766,8 +794,7 @@ branch_fast_kernel(const T* __restrict__ zd, long long ldz, int w, const int* __
   const T* r = zd + (size_t)row * ldz;
   const int y = drafted != nullptr ? __ldg(drafted + row) : -1;
   if (f > kFastFanout) {                             // offsets that ask for more than max_fanout said (again the whole cluster)
-    if (crank == 0)
-      block_topk_by([&](int i) { return entry(r, i, y); }, w, f, false, nullptr, cand + off, nullptr);
+    if (crank == 0) select_row<T>(r, w, y, f, cand + off);
     return;
   }
   const int nvec = (w + N - 1) / N, first = (int)crank * kFastThreads + tid;
@@ -811,7 +838,12 @@ branch_fast_kernel(const T* __restrict__ zd, long long ldz, int w, const int* __
   const unsigned threshold = s_threshold;
   // far more warps at the threshold than F_j: mass ties, which CTA 0 takes up by itself (thousands of threads would
   // queue up at its counter)
-  const bool push = __syncthreads_count(tid < kFastWarps && keys[tid & (kFastWarps - 1)] >= threshold) <= f + kFastWarps / 4;
+  bool push = __any_sync(0xffffffffu, mine >= threshold);
+  if (push) {
+    const uint4 q = *reinterpret_cast<const uint4*>(keys + 4 * (tid & 31));
+    push = __reduce_add_sync(0xffffffffu, (q.x >= threshold) + (q.y >= threshold) + (q.z >= threshold) + (q.w >= threshold)) <=
+           f + kFastWarps / 4;
+  }
   if (push && mine >= threshold) {
     auto take = [&](int i, unsigned k) {
       if (k < threshold) return;
@@ -838,29 +870,12 @@ branch_fast_kernel(const T* __restrict__ zd, long long ldz, int w, const int* __
   }
   cluster_sync();                                    // the list is complete in CTA 0
   if (crank != 0) return;
-  int n = push ? (int)min(s_count, (unsigned)(kFastList + 1)) : kFastList + 1;
-  if (n > kFastList) {
-    n = list_ties<T>(r, w, y, f, threshold, &s_count, list_key, list_id, cand + off);
-    if (n < 0) return;
+  const int n = (int)min(s_count, (unsigned)(kFastList + 1));
+  if (n < f || n > kFastList) {                      // nothing was pushed, or too much
+    list_ties<T>(r, w, y, f, threshold, &s_count, list_key, list_id, chosen, cand + off);
+    return;
   }
-  // the F_j first in (larger key, lower id) order, written by ascending id
-  for (int q = tid; q < kFastList / 32; q += kFastThreads) chosen[q] = 0u;
-  __syncthreads();
-  for (int e = tid; e < n; e += kFastThreads) {
-    const unsigned k = list_key[e];
-    const int id = list_id[e];
-    int rank = 0;
-    for (int j = 0; j < n; ++j) rank += list_key[j] > k || (list_key[j] == k && list_id[j] < id);
-    if (rank < f) atomicOr(&chosen[e >> 5], 1u << (e & 31));
-  }
-  __syncthreads();
-  for (int e = tid; e < n; e += kFastThreads) {
-    if (!(chosen[e >> 5] >> (e & 31) & 1u)) continue;
-    const int id = list_id[e];
-    int pos = 0;
-    for (int j = 0; j < n; ++j) pos += (chosen[j >> 5] >> (j & 31) & 1u) && list_id[j] < id;
-    cand[off + pos] = id;
-  }
+  write_ranked(list_key, list_id, n, f, chosen, cand + off);
 }
 
 }  // namespace corr
