@@ -291,7 +291,8 @@ const char* covspec_profile_stage_name(int stage);
  *
  *  dtype, d      as in covspec_config (d a multiple of 8); identity embedding, max over elements
  *  X, Q          device, laid out as in covspec_problem; vis_offsets, txt_offsets host [batch+1]
- *  s_query       device [vis_offsets[batch]] float32 (out): Eq. 10 per visual token
+ *  s_query       device [vis_offsets[batch]] float32 (out): Eq. 10 per visual token; NaN for a token whose row, or
+ *                a query element of whose request, is not finite, and where a bounded wait gave up
  * Limits: batch <= COVSPEC_STATIC_MAX_BATCH and txt_offsets[batch] * d <=
  * COVSPEC_STATIC_MAX_QUERY_ELEMS; larger problems are rejected with COVSPEC_ERR_STATIC_CAPACITY
  * and nothing is launched.
@@ -304,6 +305,12 @@ const char* covspec_profile_stage_name(int stage);
 #define COVSPEC_STATIC_MAX_QUERY_ELEMS (1 << 20)   /* 4 MiB of float32 scratch */
 int covspec_query_score_static(int dtype, int d, int batch, const void* X, const int* vis_offsets,
                                const void* Q, const int* txt_offsets, float* s_query, void* stream);
+
+/* Self-test of the same entry point (bf16 rows that it takes to the tensor cores, else
+ * COVSPEC_ERR_UNSUPPORTED): the call with waits that give up at once.  There is no context and so no
+ * status word; every score is NaN instead.  Nothing waits and no copy is in flight when it ends. */
+int covspec_selftest_static_timeout(int d, int batch, const void* X, const int* vis_offsets,
+                                    const void* Q, const int* txt_offsets, float* s_query, void* stream);
 
 /* Number of kernels the last call on this context launched. */
 int covspec_last_launch_count(const covspec_ctx* ctx);

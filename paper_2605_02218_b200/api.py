@@ -31,7 +31,7 @@ EXPORTS = [
     "covspec_correct", "covspec_fanout", "covspec_branch_candidates", "covspec_branch_candidates_host",
     "covspec_uplink_bits", "covspec_downlink_bits", "covspec_comm_latency", "covspec_ema_update",
     "covspec_draft_length", "covspec_get_iteration_counts", "covspec_build_has_bounds_checks",
-    "covspec_selftest_fill_workspace",
+    "covspec_selftest_fill_workspace", "covspec_selftest_static_timeout",
 ]
 STATIC_MAX_BATCH = 256
 STATIC_MAX_QUERY_ELEMS = 1 << 20
@@ -121,6 +121,7 @@ def load_library():
     lib.covspec_last_cuda_error.argtypes = []
     lib.covspec_last_cuda_error.restype = C.c_char_p
     lib.covspec_query_score_static.argtypes = [C.c_int, C.c_int, C.c_int, vp, ip, vp, ip, fp, vp]
+    lib.covspec_selftest_static_timeout.argtypes = [C.c_int, C.c_int, vp, ip, vp, ip, fp, vp]
     lib.covspec_profile_begin.argtypes = [vp, C.c_int]
     lib.covspec_profile_end.argtypes = [vp, C.POINTER(C.c_double), C.c_int, ip]
     lib.covspec_profile_stage_count.argtypes = []

@@ -540,7 +540,7 @@ bool identity_tc_usable(int dtype, int d, const void* X, const void* Q) {
 // One launch over `tiles` 128-token tiles; plan == nullptr: the requests come with `reqs`.
 int launch_identity_tc(const void* X, const void* Q, long long rows_x, long long rows_q, int d, int t_max,
                        const ReqPlan* plan, const ident::InlineReqs& reqs, int batch, int tiles, int num_sms,
-                       float* s_query, int* status, cudaStream_t s) {
+                       float* s_query, int* status, uint32_t spin_limit, cudaStream_t s) {
   static std::atomic<unsigned long long> configured{0};      // bit per device
   int dev = 0;
   CUDA_TRY(cudaGetDevice(&dev));
@@ -561,7 +561,7 @@ int launch_identity_tc(const void* X, const void* Q, long long rows_x, long long
   const int slack = 64 * 128;               // rows 64-127 of the last stage's X tile, read and dropped
   const int budget = (blocks <= num_sms ? 208 : 104) * 1024 - ident::kTailBytes - 1024 - slack;
   prm.stages = std::max(2, std::min({ident::kMaxStages, prm.k_chunks, budget / prm.stage_bytes}));
-  prm.s_query = s_query; prm.status = status;
+  prm.s_query = s_query; prm.status = status; prm.spin_limit = spin_limit;
   CUtensorMap map_x, map_q;
   int st;
   if ((st = make_map_bf16(&map_x, X, rows_x, d, prm.tile_rows))) return st;
@@ -761,7 +761,7 @@ int score_impl(covspec_ctx* ctx, const covspec_problem* p, float* s_query, float
   } else if (identity_tc) {
     prof_mark(ctx, ST_RELEVANCE, 0, s);
     int st = launch_identity_tc(X, Q, rowsX, rowsQ, cfg.d, pl.t_max, ctx->d_plan, ident::InlineReqs{}, B, pl.n_tiles,
-                                ctx->num_sms, s_query, ctx->status, s);
+                                ctx->num_sms, s_query, ctx->status, tc::kSpinLimit, s);
     if (st) return st;
     ++ctx->launches;
     prof_mark(ctx, ST_RELEVANCE, 1, s);
@@ -1583,7 +1583,7 @@ __global__ void static_plan_kernel(ReqPlan* __restrict__ plan, const StaticPlanC
 
 template <typename T>
 int query_score_static_impl(int d, int batch, const int* vis_offsets, const int* txt_offsets,
-                            const void* X, const void* Q, float* s_query, cudaStream_t s) {
+                            const void* X, const void* Q, float* s_query, uint32_t spin_limit, cudaStream_t s) {
   if (std::is_same<T, __nv_bfloat16>::value && identity_tc_usable(COVSPEC_BF16, d, X, Q)) {
     // tensor cores: the requests travel as kernel arguments, no scratch is used
     int dev = 0, num_sms = 148;
@@ -1601,7 +1601,7 @@ int query_score_static_impl(int d, int batch, const int* vis_offsets, const int*
         t_max = std::max(t_max, t);
       }
       int st = launch_identity_tc(X, Q, vis_offsets[batch], txt_offsets[batch], d, t_max, nullptr, reqs, count, tiles,
-                                  num_sms, s_query, nullptr, s);
+                                  num_sms, s_query, nullptr, spin_limit, s);
       if (st) return st;
     }
     return COVSPEC_OK;
@@ -1634,9 +1634,8 @@ int query_score_static_impl(int d, int batch, const int* vis_offsets, const int*
 
 }  // namespace
 
-extern "C" int covspec_query_score_static(int dtype, int d, int batch, const void* X,
-                                          const int* vis_offsets, const void* Q,
-                                          const int* txt_offsets, float* s_query, void* stream) {
+static int query_score_static(int dtype, int d, int batch, const void* X, const int* vis_offsets, const void* Q,
+                              const int* txt_offsets, float* s_query, uint32_t spin_limit, void* stream) {
   if (!X || !Q || !vis_offsets || !txt_offsets || !s_query || batch < 1) return COVSPEC_ERR_ARG;
   if (dtype != COVSPEC_F32 && dtype != COVSPEC_BF16) return COVSPEC_ERR_ARG;
   if (d < 8 || d % 8) return COVSPEC_ERR_UNSUPPORTED;
@@ -1648,6 +1647,19 @@ extern "C" int covspec_query_score_static(int dtype, int d, int batch, const voi
   if ((long long)txt_offsets[batch] * d > kStaticMaxQueryElems) return COVSPEC_ERR_STATIC_CAPACITY;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   return dtype == COVSPEC_BF16
-             ? query_score_static_impl<__nv_bfloat16>(d, batch, vis_offsets, txt_offsets, X, Q, s_query, s)
-             : query_score_static_impl<float>(d, batch, vis_offsets, txt_offsets, X, Q, s_query, s);
+             ? query_score_static_impl<__nv_bfloat16>(d, batch, vis_offsets, txt_offsets, X, Q, s_query, spin_limit, s)
+             : query_score_static_impl<float>(d, batch, vis_offsets, txt_offsets, X, Q, s_query, spin_limit, s);
+}
+
+extern "C" int covspec_query_score_static(int dtype, int d, int batch, const void* X,
+                                          const int* vis_offsets, const void* Q,
+                                          const int* txt_offsets, float* s_query, void* stream) {
+  return query_score_static(dtype, d, batch, X, vis_offsets, Q, txt_offsets, s_query, tc::kSpinLimit, stream);
+}
+
+extern "C" int covspec_selftest_static_timeout(int d, int batch, const void* X, const int* vis_offsets,
+                                               const void* Q, const int* txt_offsets, float* s_query,
+                                               void* stream) {
+  if (!identity_tc_usable(COVSPEC_BF16, d, X, Q)) return COVSPEC_ERR_UNSUPPORTED;
+  return query_score_static(COVSPEC_BF16, d, batch, X, vis_offsets, Q, txt_offsets, s_query, 0u, stream);
 }

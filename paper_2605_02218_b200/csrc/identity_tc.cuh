@@ -47,6 +47,7 @@ struct IdParams {
   int tile_rows;                         // tokens per block: 128 or 64
   float* s_query;
   int* status;                           // may be nullptr
+  uint32_t spin_limit;                   // polls after which a wait gives up
 };
 
 // Sums of squares of one 128-byte row of a swizzled tile, in four pairs of running sums (packed float32
@@ -99,6 +100,7 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   float* inv_q = reinterpret_cast<float*>(tail + 512);     // [kQueries]
   const int warp = warp_index(), lane = threadIdx.x & 31;
+  auto wait = [&](uint64_t* bar, uint32_t parity) { return mbar_wait_limited(bar, parity, abort_flag, prm.spin_limit); };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < prm.stages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 9); }
@@ -141,7 +143,7 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
       bool ok = true;
       for (int pass = 0; pass < passes && ok; ++pass)
         for (int kc = 0; kc < prm.k_chunks; ++kc) {
-          if (!(ok = mbar_wait(&empty[s], ph, abort_flag))) break;
+          if (!(ok = wait(&empty[s], ph))) break;
           mbar_expect_tx(&full[s], prm.stage_bytes);
           const uint32_t dst = smem_u32(smem + (size_t)s * prm.stage_bytes);
           tma_load_2d(dst, &map_x, kc * kChunk, row0, &full[s]);
@@ -157,10 +159,10 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
       uint32_t ph = 0;
       bool ok = true;
       for (int pass = 0; pass < passes && ok; ++pass) {
-        if (!(ok = mbar_wait(acc_empty, (pass & 1u) ^ 1u, abort_flag))) break;
+        if (!(ok = wait(acc_empty, (pass & 1u) ^ 1u))) break;
         tc_fence_after();
         for (int kc = 0; kc < prm.k_chunks; ++kc) {
-          if (!(ok = mbar_wait(&full[s], ph, abort_flag))) break;
+          if (!(ok = wait(&full[s], ph))) break;
           tc_fence_after();
           const uint32_t x_addr = smem_u32(smem + (size_t)s * prm.stage_bytes);
           const uint64_t adesc = umma_desc(x_addr), bdesc = umma_desc(x_addr + R * 128);
@@ -187,7 +189,7 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
       unsigned long long sq[4] = {0ull, 0ull, 0ull, 0ull};
       const bool measure = tokens ? pass == 0 && (warp & 3) * 32 < nrows : r < prm.n_cols;
       for (int kc = 0; kc < prm.k_chunks; ++kc) {
-        ok = ok && mbar_wait(&full[s], ph, abort_flag);
+        ok = ok && wait(&full[s], ph);
         if (measure) add_row_squares(smem + (size_t)s * prm.stage_bytes + (tokens ? 0 : R * 128), r, sq);
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[s]);
@@ -198,7 +200,7 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
       if (!tokens && measure) inv_q[r] = inverse_length(total_squares(sq));
       named_barrier(1, 256);
       if (tokens) {
-        ok = ok && mbar_wait(acc_full, pass & 1u, abort_flag);
+        ok = ok && wait(acc_full, pass & 1u);
         tc_fence_after();
         const int cols = min(prm.n_cols, T - pass * prm.n_cols);
 #pragma unroll 1
@@ -224,7 +226,8 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         if (lane == 0) mbar_arrive(acc_empty);
       }
     }
-    if (tokens && ok && r < nrows) prm.s_query[row0 + r] = nonfinite ? __int_as_float(0x7fc00000) : best * inv_x;
+    // a wait that gave up leaves NaN, for callers that have no status word to look at
+    if (tokens && r < nrows) prm.s_query[row0 + r] = nonfinite || !ok ? __int_as_float(0x7fc00000) : best * inv_x;
   }
 
   tc_fence_before();

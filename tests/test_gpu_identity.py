@@ -58,3 +58,22 @@ def test_more_requests_than_one_launch_carries():
     assert torch.equal(sq, st)
     assert (sq - simt).abs().max().item() <= 2 * TOL
     pr.close()
+
+
+def test_static_scores_are_nan_where_a_wait_gave_up():
+    # the allocation-free entry point has no status word: a kernel that gave up must not leave the old contents behind
+    import ctypes as C
+    from paper_2605_02218_b200 import api, build
+    build.build()
+    wl = workloads.make_workload("timeout", seed=8, dtype=torch.bfloat16, batch=3, n_vis=(60, 300), n_txt=(1, 140), d=256,
+                                 n_heads=0, rank=4, keep=1, act_layers=0).to("cuda:0")
+    out = torch.full((wl.total_vis,), 7.0, device="cuda:0")
+    ip = lambda a: a.ctypes.data_as(C.POINTER(C.c_int))
+    vis, txt = (np.ascontiguousarray(a, dtype=np.int32) for a in (wl.vis_offsets, wl.txt_offsets))
+    st = api.load_library().covspec_selftest_static_timeout(wl.d, wl.batch, wl.X.data_ptr(), ip(vis), wl.Q.data_ptr(), ip(txt),
+                                                            out.data_ptr(), api._raw_stream())
+    assert st == 0
+    torch.cuda.synchronize()
+    assert torch.isnan(out).all()
+    again = api.query_score_static(wl.X, wl.Q, wl.vis_offsets, wl.txt_offsets)
+    assert torch.isfinite(again).all()
