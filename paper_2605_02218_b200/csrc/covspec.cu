@@ -562,6 +562,10 @@ int launch_identity_tc(const void* X, const void* Q, long long rows_x, long long
   const int budget = (blocks <= num_sms ? 208 : 104) * 1024 - ident::kTailBytes - 1024 - slack;
   prm.stages = std::max(2, std::min({ident::kMaxStages, prm.k_chunks, budget / prm.stage_bytes}));
   prm.s_query = s_query; prm.status = status; prm.spin_limit = spin_limit;
+  prm.x = static_cast<const __nv_bfloat16*>(X); prm.q = static_cast<const __nv_bfloat16*>(Q); prm.d = d;
+  // twice a bound on the error of a product, relative to |x| |q|: one truncation per accumulation step of 16 features
+  // (2^-22 each is twice what they lose) and what the lengths and the float32 form of the score add
+  prm.margin = 2.f * (float)(4 * prm.k_chunks + 16) * 0x1p-22f;
   CUtensorMap map_x, map_q;
   int st;
   if ((st = make_map_bf16(&map_x, X, rows_x, d, prm.tile_rows))) return st;

@@ -1,20 +1,26 @@
 // Eq. 10 with the identity embedding (e(x) = x, no projection heads) on the tensor cores, bf16 inputs.
 //
 //   S^query_i = max_j (x_i . q_j) / (|x_i| |q_j|)
-// bf16 inputs enter the products exactly: one tcgen05.mma per 16 features on the raw rows, float32
-// accumulators in TMEM, and the two lengths in float32 from the same tiles while they lie in shared
-// memory, so that X is read once and nothing is converted or staged in between.  The accumulation is cut
-// into up to four column groups of TMEM, each over a contiguous range of features, that the epilogue adds
-// up in registers: the tensor core's sums truncate, and short chains keep that near the rounding of
-// ordinary float32 sums.
+// The tensor cores find the query elements that can attain the maximum, ordinary float32 arithmetic computes the score:
+//   1. products of all tokens of a tile with the request's query elements by tcgen05.mma on the raw bf16 rows, float32
+//      accumulators in TMEM, and the lengths in float32 from the same tiles while they lie in shared memory; X is read
+//      from HBM once and nothing is converted or staged in between.
+//   2. the accumulators truncate: a sum over d features may be off by about (d / 16) 2^-23 |x| |q|.  Every query element
+//      that comes within twice a bound on that of the largest value is a candidate; nearly always there is one.
+//   3. the cosine of every candidate is computed again by one warp per token, with the arithmetic of cosmax_kernel in its
+//      order (score_kernels.cuh), and the largest is the score: the bits are those of that kernel, whatever the
+//      batch a request comes in.  (Tensor-core sums as scores were off by 2.5e-7 to 2.1e-6 relative, d = 1024-4096,
+//      against 6e-8 to 1e-7, and depended on the longest query of the call.)
 //
 // One CTA per 128-token tile of a request (or per 64 tokens, while that leaves at most two CTAs per SM: a
 // block is bound by the latency of its loads and by shared-memory bandwidth); the request's query elements pass in groups of up to 128.
-// Warps 0-3: one token per thread (length of x, epilogue); 4-7: one query element per thread (length of
-// q); warp 8: TMA producer; warp 9: MMA issuer and TMEM owner.  Bound by HBM (X once).  The CUDA-core
-// kernel (cosmax_kernel, one warp per token) read every query element once per token through L1: 16
-// requests of 400-729 tokens, d = 2048, 210 us for 37 MB.
+// Warps 0-3: one token per thread (length of x, candidates); 4-7: one query element per thread (length of
+// q); 0-7: step 3; warp 8: TMA producer; warp 9: MMA issuer and TMEM owner.  Bound by HBM (X once).  cosmax_kernel (one warp
+// per token) reads every query element once per token through L1: 16 requests of 400-729 tokens, d = 2048, 210 us
+// for 37 MB.
 #pragma once
+#include <float.h>
+
 #include "tc_common.cuh"
 
 namespace covspec {
@@ -26,10 +32,10 @@ constexpr int kTokens = 128;             // tokens per tile (UMMA M)
 constexpr int kQueries = 128;            // query elements per pass (UMMA N at most)
 constexpr int kChunk = 64;               // features per k-chunk (one 128-byte swizzle row)
 constexpr int kMaxStages = 12;
-constexpr int kColumns = 256;            // TMEM columns: two CTAs fit on an SM
+constexpr int kColumns = 128;            // TMEM columns
 constexpr int kIdThreads = 320;
-constexpr int kGroupChunks = 8;          // k-chunks per accumulation group, if TMEM has the columns
-constexpr int kTailBytes = 2048;         // barriers, reciprocal query lengths
+// barriers (512), reciprocal query lengths [kQueries], best exact cosine [kTokens], candidate bits [kTokens][kQueries]
+constexpr int kTailBytes = 512 + kQueries * 4 + kTokens * 4 + kTokens * kQueries / 8;
 
 // Requests handed over by value (the allocation-free entry point, which has no plan on the device).
 constexpr int kInlineReqs = 64;
@@ -39,6 +45,10 @@ struct InlineReqs {
 };
 
 struct IdParams {
+  const __nv_bfloat16* x;                // the arrays behind the tensor maps
+  const __nv_bfloat16* q;
+  int d;
+  float margin;                          // candidates: within margin |x| |q| of the largest product
   const ReqPlan* plan;                   // or nullptr: the inline requests
   int batch;
   int k_chunks;
@@ -78,12 +88,74 @@ __device__ __forceinline__ float total_squares(const unsigned long long (&acc)[4
   }
   return s;
 }
+// The same for the 32 sums in which qnorm_kernel's lanes take a row: feature k goes to sum k % 32, in ascending order.
+__device__ __forceinline__ void add_row_squares_by_lane(const uint8_t* tile, int r, unsigned long long (&acc)[16]) {
+  const uint8_t* row = tile + r * 128;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const uint4 v = *reinterpret_cast<const uint4*>(row + ((c ^ (r & 7)) * 16));
+    const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      unsigned long long x;
+      asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(u[e] << 16), "r"(u[e] & 0xffff0000u));
+      asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(acc[(4 * c + e) & 15]) : "l"(x));
+    }
+  }
+}
+// Their total as warp_sum adds the lanes up.
+__device__ __forceinline__ float total_by_lane(const unsigned long long (&acc)[16]) {
+  float s[32];
+#pragma unroll
+  for (int e = 0; e < 16; ++e) asm("mov.b64 {%0, %1}, %2;" : "=f"(s[2 * e]), "=f"(s[2 * e + 1]) : "l"(acc[e]));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int l = 0; l < o; ++l) s[l] += s[l + o];
+  return s[0];
+}
 // 1 / sqrt(ss); 0 for a zero row, NaN for a row that is not finite.
 __device__ __forceinline__ float inverse_length(float ss) {
   if (!(ss <= 3.402823466e38f)) return __int_as_float(0x7fc00000);
   if (!(ss > 1.17549435e-38f)) return 0.f;
   float inv = rsqrtf(ss);
   return inv * (1.5f - 0.5f * ss * inv * inv);
+}
+
+// Takes the lowest set bit out of a set of 128; -1: none left.
+__device__ __forceinline__ int next_candidate(uint4& m) {
+  if (m.x) { const int b = __ffs((int)m.x) - 1; m.x &= m.x - 1u; return b; }
+  if (m.y) { const int b = __ffs((int)m.y) - 1; m.y &= m.y - 1u; return 32 + b; }
+  if (m.z) { const int b = __ffs((int)m.z) - 1; m.z &= m.z - 1u; return 64 + b; }
+  if (m.w) { const int b = __ffs((int)m.w) - 1; m.w &= m.w - 1u; return 96 + b; }
+  return -1;
+}
+
+// Cosines of two tokens with a query element each, by one warp, as cosmax_kernel computes them; *inv: the tokens'
+// reciprocal lengths.  Two at a time: a row is a handful of loads per lane, whose latency is all there is.
+__device__ __forceinline__ void exact_cosines(const __nv_bfloat16* const (&x)[2], const __nv_bfloat16* const (&q)[2],
+                                              const float (&inv_q)[2], int d, int lane, float (&inv)[2], float (&dot)[2]) {
+  float ss[2] = {0.f, 0.f};
+  dot[0] = dot[1] = 0.f;
+#pragma unroll 4
+  for (int k = lane * 4; k < d; k += 128) {
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      float v[4], u[4];
+      load4(x[p] + k, v);
+      load4(q[p] + k, u);
+      const float4 w = make_float4(u[0] * inv_q[p], u[1] * inv_q[p], u[2] * inv_q[p], u[3] * inv_q[p]);
+      ss[p] += v[0] * v[0] + v[1] * v[1] + v[2] * v[2] + v[3] * v[3];
+      dot[p] += v[0] * w.x + v[1] * w.y + v[2] * w.z + v[3] * w.w;
+    }
+  }
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    ss[p] = warp_sum(ss[p]);
+    inv[p] = 0.f;
+    if (ss[p] > FLT_MIN) { inv[p] = rsqrtf(ss[p]); inv[p] = inv[p] * (1.5f - 0.5f * ss[p] * inv[p] * inv[p]); }
+    dot[p] = warp_sum(dot[p]) * inv[p];
+  }
 }
 
 __global__ void __launch_bounds__(kIdThreads, 2)
@@ -99,6 +171,8 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   float* inv_q = reinterpret_cast<float*>(tail + 512);     // [kQueries]
+  float* exact = inv_q + kQueries;                         // [kTokens]
+  uint16_t* candidates = reinterpret_cast<uint16_t*>(exact + kTokens);      // [kTokens][kQueries / 16]
   const int warp = warp_index(), lane = threadIdx.x & 31;
   auto wait = [&](uint64_t* bar, uint32_t parity) { return mbar_wait_limited(bar, parity, abort_flag, prm.spin_limit); };
 
@@ -130,12 +204,6 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
   }
   const int at = tile * kTokens + half * R, row0 = vis_off + at, nrows = min(R, n - at);
   const int passes = nrows > 0 ? (T + prm.n_cols - 1) / prm.n_cols : 0;
-  // accumulation groups: contiguous ranges of k-chunks, one set of TMEM columns each
-  const int group_cols = (prm.n_cols + 31) & ~31;
-  const int n_groups = max(1, min(kColumns / group_cols, (prm.k_chunks + kGroupChunks - 1) / kGroupChunks));
-  const int per_group = (prm.k_chunks + n_groups - 1) / n_groups;
-  const int groups_used = (prm.k_chunks + per_group - 1) / per_group;
-
   if (warp == 8) {
     if (lane == 0) {
       int s = 0;
@@ -166,10 +234,9 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
           tc_fence_after();
           const uint32_t x_addr = smem_u32(smem + (size_t)s * prm.stage_bytes);
           const uint64_t adesc = umma_desc(x_addr), bdesc = umma_desc(x_addr + R * 128);
-          const int g = kc / per_group;
 #pragma unroll
           for (int k = 0; k < kChunk / 16; ++k)
-            umma_bf16(tmem_base + g * group_cols, adesc + 2 * k, bdesc + 2 * k, idesc, (kc - g * per_group + k) != 0);
+            umma_bf16(tmem_base, adesc + 2 * k, bdesc + 2 * k, idesc, (kc | k) != 0);
           umma_commit(&empty[s]);
           if (++s == prm.stages) { s = 0; ph ^= 1u; }
         }
@@ -181,53 +248,119 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     const int r = (warp & 3) * 32 + lane;              // token (warps 0-3) or query element (4-7) of the tile
     const bool tokens = warp < 4;
     const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-    float best = -INFINITY, inv_x = 0.f;
+    float best = -INFINITY, len_x = 0.f, inv_x = 0.f;    // best: largest product so far, divided by the query length
     bool nonfinite = false, ok = true;
     int s = 0;
     uint32_t ph = 0;
+    if (tokens) exact[r] = -FLT_MAX;
     for (int pass = 0; pass < passes; ++pass) {
-      unsigned long long sq[4] = {0ull, 0ull, 0ull, 0ull};
-      const bool measure = tokens ? pass == 0 && (warp & 3) * 32 < nrows : r < prm.n_cols;
-      for (int kc = 0; kc < prm.k_chunks; ++kc) {
-        ok = ok && wait(&full[s], ph);
-        if (measure) add_row_squares(smem + (size_t)s * prm.stage_bytes + (tokens ? 0 : R * 128), r, sq);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[s]);
-        if (++s == prm.stages) { s = 0; ph ^= 1u; }
+      if (tokens) {
+        unsigned long long sq[4] = {0ull, 0ull, 0ull, 0ull};
+        const bool measure = pass == 0 && (warp & 3) * 32 < nrows;
+        for (int kc = 0; kc < prm.k_chunks; ++kc) {
+          ok = ok && wait(&full[s], ph);
+          if (measure) add_row_squares(smem + (size_t)s * prm.stage_bytes, r, sq);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&empty[s]);
+          if (++s == prm.stages) { s = 0; ph ^= 1u; }
+        }
+        if (pass == 0) {
+          const float ss = total_squares(sq);
+          inv_x = inverse_length(ss);
+          len_x = ss * inv_x;
+          nonfinite = inv_x != inv_x;
+        }
+        named_barrier(1, 256);                           // the previous pass no longer reads inv_q and the candidates
+      } else {
+        unsigned long long sq[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) sq[e] = 0ull;
+        const bool measure = r < prm.n_cols;
+        for (int kc = 0; kc < prm.k_chunks; ++kc) {
+          ok = ok && wait(&full[s], ph);
+          if (measure) add_row_squares_by_lane(smem + (size_t)s * prm.stage_bytes + R * 128, r, sq);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&empty[s]);
+          if (++s == prm.stages) { s = 0; ph ^= 1u; }
+        }
+        named_barrier(1, 256);
+        if (measure) inv_q[r] = inverse_length(total_by_lane(sq));
       }
-      if (tokens && pass == 0) { inv_x = inverse_length(total_squares(sq)); nonfinite = inv_x != inv_x; }
-      named_barrier(1, 256);                           // the previous pass no longer reads inv_q
-      if (!tokens && measure) inv_q[r] = inverse_length(total_squares(sq));
       named_barrier(1, 256);
       if (tokens) {
         ok = ok && wait(acc_full, pass & 1u);
         tc_fence_after();
         const int cols = min(prm.n_cols, T - pass * prm.n_cols);
+        float top = -INFINITY, most = 0.f;
 #pragma unroll 1
         for (int c0 = 0; c0 < cols; c0 += 16) {
           float v[16];
           tmem_ld16(t_lane + c0, v);
-          for (int g = 1; g < groups_used; ++g) {
-            float u[16];
-            tmem_ld16(t_lane + g * group_cols + c0, u);
-#pragma unroll
-            for (int e = 0; e < 16; ++e) v[e] += u[e];
-          }
 #pragma unroll
           for (int e = 0; e < 16; ++e)
             if (c0 + e < cols) {
               const float c = v[e] * inv_q[c0 + e];
               nonfinite |= c != c;
-              best = fmaxf(best, c);
+              top = fmaxf(top, c);
+              most = fmaxf(most, inv_q[c0 + e]);
             }
+        }
+        // |x| |q| so small that the products themselves may be lost below the float32 range: every element is a candidate
+        const bool tiny = inv_x == 0.f || !(most * inv_x <= 1.2e24f);
+        if (!tiny) best = fmaxf(best, top);
+        const float limit = tiny ? -INFINITY : best - prm.margin * len_x;
+#pragma unroll 1
+        for (int c0 = 0; c0 < kQueries; c0 += 16) {
+          uint32_t bits = 0u;
+          if (c0 < cols) {
+            float v[16];
+            tmem_ld16(t_lane + c0, v);
+#pragma unroll
+            for (int e = 0; e < 16; ++e)
+              if (c0 + e < cols && v[e] * inv_q[c0 + e] >= limit) bits |= 1u << e;
+          }
+          candidates[r * (kQueries / 16) + (c0 >> 4)] = (uint16_t)(nonfinite || !ok ? 0u : bits);
         }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(acc_empty);
       }
+      named_barrier(1, 256);                             // the candidates of the pass are known
+      for (int t0 = warp; t0 < nrows; t0 += 16) {
+        const int t[2] = {t0, min(t0 + 8, nrows - 1)};
+        uint4 m[2];
+        m[0] = reinterpret_cast<const uint4*>(candidates)[t[0]];
+        m[1] = t0 + 8 < nrows ? reinterpret_cast<const uint4*>(candidates)[t[1]] : make_uint4(0u, 0u, 0u, 0u);
+        float high[2] = {exact[t[0]], exact[t[1]]};
+        for (;;) {
+          const int j[2] = {next_candidate(m[0]), next_candidate(m[1])};
+          if (j[0] < 0 && j[1] < 0) break;
+          const __nv_bfloat16 *xr[2], *qr[2];
+          float iq[2], inv[2], dot[2];
+#pragma unroll
+          for (int p = 0; p < 2; ++p) {                  // a token without one shares the other's loads
+            const int tp = j[p] >= 0 ? t[p] : t[1 - p], jp = j[p] >= 0 ? j[p] : j[1 - p];
+            xr[p] = prm.x + (size_t)(row0 + tp) * prm.d;
+            qr[p] = prm.q + (size_t)(txt_off + pass * prm.n_cols + jp) * prm.d;
+            iq[p] = inv_q[jp];
+          }
+          exact_cosines(xr, qr, iq, prm.d, lane, inv, dot);
+#pragma unroll
+          for (int p = 0; p < 2; ++p)
+            if (j[p] >= 0) {
+              high[p] = fmaxf(high[p], dot[p]);
+              if (inv[p] == 0.f) m[p] = make_uint4(0u, 0u, 0u, 0u);        // a zero token: 0 with every element
+            }
+        }
+        if (lane == 0) {
+          exact[t[0]] = high[0];
+          if (t0 + 8 < nrows) exact[t[1]] = high[1];
+        }
+      }
     }
+    named_barrier(1, 256);
     // a wait that gave up leaves NaN, for callers that have no status word to look at
-    if (tokens && r < nrows) prm.s_query[row0 + r] = nonfinite || !ok ? __int_as_float(0x7fc00000) : best * inv_x;
+    if (tokens && r < nrows) prm.s_query[row0 + r] = nonfinite || !ok ? __int_as_float(0x7fc00000) : exact[r];
   }
 
   tc_fence_before();

@@ -77,3 +77,77 @@ def test_static_scores_are_nan_where_a_wait_gave_up():
     assert torch.isnan(out).all()
     again = api.query_score_static(wl.X, wl.Q, wl.vis_offsets, wl.txt_offsets)
     assert torch.isfinite(again).all()
+
+
+def _both_routes(wl):
+    """Query scores on the tensor cores and on the CUDA cores (relevance_path = 1)."""
+    from paper_2605_02218_b200 import api
+    out = []
+    for path in (0, 1):
+        pr = api.Pruner.for_workload(wl, relevance_path=path)
+        out.append(pr.score(pr.marshal(wl))[0])
+        pr.device_status()                               # scores that are not finite are reported there as well
+        pr.close()
+    return out
+
+
+@pytest.mark.parametrize("d", [64, 72, 520, 1032, 2048, 4096])
+@pytest.mark.parametrize("n_txt", [1, 17, 100, 128, 129, 300])
+def test_identity_scores_have_the_bits_of_the_cuda_core_kernel(d, n_txt):
+    # candidates come from truncating sums, the scores from float32 sums in one fixed order: no less precise than the
+    # CUDA-core kernel, at any width and query length
+    from paper_2605_02218_b200 import api, build
+    build.build()
+    ns = [1, 127, 128, 129, 1100]
+    ts = [max(1, n_txt - i) for i in range(len(ns))]
+    wl = workloads.make_workload("identity", seed=d + n_txt, dtype=torch.bfloat16, batch=len(ns), sizes=(ns, ts), d=d,
+                                 n_heads=0, rank=8, keep=1, act_layers=0).to("cuda:0")
+    tc, simt = _both_routes(wl)
+    assert torch.equal(tc, simt)
+    if int(wl.txt_offsets[-1]) * d <= api.STATIC_MAX_QUERY_ELEMS:
+        assert torch.equal(api.query_score_static(wl.X, wl.Q, wl.vis_offsets, wl.txt_offsets), simt)
+
+
+def test_identity_scores_of_unusual_rows():
+    # many candidates (repeated query elements, all of them alike, tokens along a query element), zero and tiny rows on either
+    # side (products below the float32 range), rows that are not finite or whose length is not
+    from paper_2605_02218_b200 import build
+    build.build()
+    d, ns, ts = 1024, [300, 200, 260, 200, 130, 140], [40, 200, 9, 64, 30, 150]
+    wl = workloads.make_workload("unusual", seed=3, dtype=torch.bfloat16, batch=len(ns), sizes=(ns, ts), d=d, n_heads=0,
+                                 rank=8, keep=1, act_layers=0).to("cuda:0")
+    v, t = [int(a) for a in wl.vis_offsets], [int(a) for a in wl.txt_offsets]
+    X, Q = wl.X, wl.Q
+    Q[t[0] + 5:t[0] + 12] = Q[t[0] + 4]                  # repeated
+    X[v[0]:v[0] + 50] = Q[t[0] + 4] * 3
+    Q[t[1]:t[2]] = Q[t[1]]                               # all alike, over two passes
+    X[v[2] + 3] = 0
+    X[v[2] + 4] *= 1e-21
+    X[v[2] + 5:v[2] + 9] *= 2e-20
+    X[v[2] + 9:v[2] + 40] *= 1e-18
+    Q[t[2]] = 0
+    Q[t[2] + 1] *= 1e-21
+    Q[t[2] + 2:t[2] + 9] *= 1e-18
+    X[v[3] + 7, 11] = float("nan")
+    X[v[3] + 8, 0] = float("inf")
+    X[v[3] + 9] = 3e38
+    X[v[3] + 10:v[3] + 20] *= 1e16
+    Q[t[3]:t[3] + 4] *= 1e16
+    Q[t[4] + 3, 5] = float("nan")                        # the whole request
+    Q[t[5] + 140, 9] = float("-inf")
+    tc, simt = _both_routes(wl)
+    assert torch.equal(torch.isnan(tc), torch.isnan(simt))
+    assert int(torch.isnan(tc).sum()) == 3 + ns[4] + ns[5]
+    assert torch.equal(torch.nan_to_num(tc), torch.nan_to_num(simt))
+
+
+def test_identity_scores_do_not_depend_on_the_batch():
+    # a request alone, and beside one with a much longer query and with enough tokens for whole 128-token tiles
+    from paper_2605_02218_b200 import api, build
+    build.build()
+    d, ns, ts = 4096, [333, 20000], [30, 250]
+    wl = workloads.make_workload("batch", seed=4, dtype=torch.bfloat16, batch=2, sizes=(ns, ts), d=d, n_heads=0, rank=8,
+                                 keep=1, act_layers=0).to("cuda:0")
+    both = _both_routes(wl)[0][:ns[0]]
+    alone = api.query_score_static(wl.X[:ns[0]], wl.Q[:ts[0]], wl.vis_offsets[:2], wl.txt_offsets[:2])
+    assert torch.equal(both, alone)
