@@ -537,10 +537,12 @@ bool identity_tc_usable(int dtype, int d, const void* X, const void* Q) {
   return dtype == COVSPEC_BF16 && d >= ident::kChunk && d % 8 == 0 &&
          ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Q)) & 15) == 0;
 }
-// One launch over `tiles` 128-token tiles; plan == nullptr: the requests come with `reqs`.
+// One or two launches over `tiles` 128-token tiles of the rows from `first` on; plan == nullptr: the requests come with `reqs`.
+// inv_q: scratch of one float per query row.
 int launch_identity_tc(const void* X, const void* Q, long long rows_x, long long rows_q, int d, int t_max,
                        const ReqPlan* plan, const ident::InlineReqs& reqs, int batch, int tiles, int num_sms,
-                       float* s_query, int* status, uint32_t spin_limit, cudaStream_t s) {
+                       long long first, long long rows, float* s_query, float* inv_q, int* status, uint32_t spin_limit,
+                       cudaStream_t s) {
   static std::atomic<unsigned long long> configured{0};      // bit per device
   int dev = 0;
   CUDA_TRY(cudaGetDevice(&dev));
@@ -562,10 +564,16 @@ int launch_identity_tc(const void* X, const void* Q, long long rows_x, long long
   const int budget = (blocks <= num_sms ? 208 : 104) * 1024 - ident::kTailBytes - 1024 - slack;
   prm.stages = std::max(2, std::min({ident::kMaxStages, prm.k_chunks, budget / prm.stage_bytes}));
   prm.s_query = s_query; prm.status = status; prm.spin_limit = spin_limit;
+  prm.inv_q = inv_q;
+  prm.defer = rows_q <= ident::kPairRows ? 2 : rows_q <= ident::kDeferredRows ? 1 : 0;
   prm.x = static_cast<const __nv_bfloat16*>(X); prm.q = static_cast<const __nv_bfloat16*>(Q); prm.d = d;
-  // twice a bound on the error of a product, relative to |x| |q|: one truncation per accumulation step of 16 features
-  // (2^-22 each is twice what they lose) and what the lengths and the float32 form of the score add
-  prm.margin = 2.f * (float)(4 * prm.k_chunks + 16) * 0x1p-22f;
+  const int columns = (prm.n_cols + 31) / 32 * 32;
+  const int want = std::max(1, std::min(ident::kColumns / columns, (prm.k_chunks + ident::kGroupChunks - 1) / ident::kGroupChunks));
+  prm.per_group = (prm.k_chunks + want - 1) / want;
+  prm.groups = (prm.k_chunks + prm.per_group - 1) / prm.per_group;
+  // twice the bound on the error of a product, relative to |x| |q|: 2^-23 per accumulation step of a group (four to a
+  // chunk); 16 more for the sums of the groups, the lengths and the float32 form of the score
+  prm.margin = 2.f * (float)(4 * prm.per_group + 16) * 0x1p-23f;
   CUtensorMap map_x, map_q;
   int st;
   if ((st = make_map_bf16(&map_x, X, rows_x, d, prm.tile_rows))) return st;
@@ -573,6 +581,9 @@ int launch_identity_tc(const void* X, const void* Q, long long rows_x, long long
   const int smem = prm.stages * prm.stage_bytes + slack + ident::kTailBytes + 1024;
   ident::identity_tc_kernel<<<blocks, ident::kIdThreads, smem, s>>>(map_x, map_q, reqs, prm);
   CUDA_TRY(cudaGetLastError());
+  if (prm.defer)
+    CUDA_TRY(launch_dependent(ident::identity_exact_kernel, dim3((unsigned)((rows + 7) / 8)), 256, 0, s, prm.x, prm.q, inv_q, d,
+                              prm.defer == 2 ? 1 : 0, (int)first, (int)rows, s_query));
   return COVSPEC_OK;
 }
 
@@ -765,9 +776,9 @@ int score_impl(covspec_ctx* ctx, const covspec_problem* p, float* s_query, float
   } else if (identity_tc) {
     prof_mark(ctx, ST_RELEVANCE, 0, s);
     int st = launch_identity_tc(X, Q, rowsX, rowsQ, cfg.d, pl.t_max, ctx->d_plan, ident::InlineReqs{}, B, pl.n_tiles,
-                                ctx->num_sms, s_query, ctx->status, tc::kSpinLimit, s);
+                                ctx->num_sms, 0, rowsX, s_query, ctx->Qn, ctx->status, tc::kSpinLimit, s);
     if (st) return st;
-    ++ctx->launches;
+    ctx->launches += rowsQ <= ident::kDeferredRows ? 2 : 1;
     prof_mark(ctx, ST_RELEVANCE, 1, s);
     // after the identity kernel, whose few large blocks would otherwise wait for the activity blocks to end
     if (overlap && (st = fork_activity())) return st;
@@ -1589,7 +1600,11 @@ template <typename T>
 int query_score_static_impl(int d, int batch, const int* vis_offsets, const int* txt_offsets,
                             const void* X, const void* Q, float* s_query, uint32_t spin_limit, cudaStream_t s) {
   if (std::is_same<T, __nv_bfloat16>::value && identity_tc_usable(COVSPEC_BF16, d, X, Q)) {
-    // tensor cores: the requests travel as kernel arguments, no scratch is used
+    // tensor cores: the requests travel as kernel arguments, the scratch takes the reciprocal query lengths
+    unsigned char* scratch = nullptr;
+    int got = static_scratch_ptr(&scratch);
+    if (got) return got;
+    float* inv_q = reinterpret_cast<float*>(scratch + kStaticPlanBytes);
     int dev = 0, num_sms = 148;
     CUDA_TRY(cudaGetDevice(&dev));
     CUDA_TRY(cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1605,7 +1620,8 @@ int query_score_static_impl(int d, int batch, const int* vis_offsets, const int*
         t_max = std::max(t_max, t);
       }
       int st = launch_identity_tc(X, Q, vis_offsets[batch], txt_offsets[batch], d, t_max, nullptr, reqs, count, tiles,
-                                  num_sms, s_query, nullptr, spin_limit, s);
+                                  num_sms, vis_offsets[b0], vis_offsets[b0 + count] - vis_offsets[b0], s_query,
+                                  inv_q, nullptr, spin_limit, s);
       if (st) return st;
     }
     return COVSPEC_OK;

@@ -5,12 +5,18 @@
 //   1. products of all tokens of a tile with the request's query elements by tcgen05.mma on the raw bf16 rows, float32
 //      accumulators in TMEM, and the lengths in float32 from the same tiles while they lie in shared memory; X is read
 //      from HBM once and nothing is converted or staged in between.
-//   2. the accumulators truncate: a sum over d features may be off by about (d / 16) 2^-23 |x| |q|.  Every query element
-//      that comes within twice a bound on that of the largest value is a candidate; nearly always there is one.
+//   2. the accumulators truncate, by less than 2^-23 |x| |q| a step of 16 features (a fifth of that was measured).  A sum is
+//      cut into as many groups of contiguous features as TMEM has columns for, up to eight, added up in float32: the
+//      bound falls with their number.  Every query element within twice the bound of the largest value is a
+//      candidate; nearly always there is one.
 //   3. the cosine of every candidate is computed again by one warp per token, with the arithmetic of cosmax_kernel in its
 //      order (score_kernels.cuh), and the largest is the score: the bits are those of that kernel, whatever the
 //      batch a request comes in.  (Tensor-core sums as scores were off by 2.5e-7 to 2.1e-6 relative, d = 1024-4096,
-//      against 6e-8 to 1e-7, and depended on the longest query of the call.)
+//      against 6e-8 to 1e-7, and depended on the longest query of the call.)  One or two candidates
+//      of a token go to identity_exact_kernel, which has the whole chip's warps to wait for the rows; more of them, and
+//      requests of more than one pass, are seen to here.  (All of it here: 4 requests of 576 tokens, d = 1024, 32 query
+//      elements 19.1 us, so 17.2; 16 of 400-729 at d = 2048 beside the activity stream 66.8 and 61.2; 2 of 16384 at
+//      d = 3584 121.7 and 93.5: a single token with two candidates held a tile up for 3 to 18 us.)
 //
 // One CTA per 128-token tile of a request (or per 64 tokens, while that leaves at most two CTAs per SM: a
 // block is bound by the latency of its loads and by shared-memory bandwidth); the request's query elements pass in groups of up to 128.
@@ -32,8 +38,9 @@ constexpr int kTokens = 128;             // tokens per tile (UMMA M)
 constexpr int kQueries = 128;            // query elements per pass (UMMA N at most)
 constexpr int kChunk = 64;               // features per k-chunk (one 128-byte swizzle row)
 constexpr int kMaxStages = 12;
-constexpr int kColumns = 128;            // TMEM columns
+constexpr int kColumns = 256;            // TMEM columns: two CTAs fit on an SM
 constexpr int kIdThreads = 320;
+constexpr int kGroupChunks = 4;          // k-chunks per accumulation group, if TMEM has the columns
 // barriers (512), reciprocal query lengths [kQueries], best exact cosine [kTokens], candidate bits [kTokens][kQueries]
 constexpr int kTailBytes = 512 + kQueries * 4 + kTokens * 4 + kTokens * kQueries / 8;
 
@@ -48,7 +55,10 @@ struct IdParams {
   const __nv_bfloat16* x;                // the arrays behind the tensor maps
   const __nv_bfloat16* q;
   int d;
+  float* inv_q;                          // reciprocal query lengths for identity_exact_kernel
   float margin;                          // candidates: within margin |x| |q| of the largest product
+  int per_group, groups;                 // accumulation groups: k-chunks each, their number
+  int defer;                             // candidates that may be left to identity_exact_kernel: 0, 1 or 2
   const ReqPlan* plan;                   // or nullptr: the inline requests
   int batch;
   int k_chunks;
@@ -131,32 +141,60 @@ __device__ __forceinline__ int next_candidate(uint4& m) {
   return -1;
 }
 
-// Cosines of two tokens with a query element each, by one warp, as cosmax_kernel computes them; *inv: the tokens'
-// reciprocal lengths.  Two at a time: a row is a handful of loads per lane, whose latency is all there is.
-__device__ __forceinline__ void exact_cosines(const __nv_bfloat16* const (&x)[2], const __nv_bfloat16* const (&q)[2],
-                                              const float (&inv_q)[2], int d, int lane, float (&inv)[2], float (&dot)[2]) {
-  float ss[2] = {0.f, 0.f};
-  dot[0] = dot[1] = 0.f;
-#pragma unroll 4
-  for (int k = lane * 4; k < d; k += 128) {
+// Cosines of PT tokens with a query element each, by one warp, as cosmax_kernel computes them; *inv: the tokens'
+// reciprocal lengths.  A row is a handful of loads per lane, whose latency is all there is: several at a time.
+template <int PT, int UNROLL>
+__device__ __forceinline__ void exact_cosines(const __nv_bfloat16* const (&x)[PT], const __nv_bfloat16* const (&q)[PT],
+                                              const float (&inv_q)[PT], int d, int lane, float (&inv)[PT], float (&dot)[PT]) {
+  float ss[PT];
 #pragma unroll
-    for (int p = 0; p < 2; ++p) {
-      float v[4], u[4];
-      load4(x[p] + k, v);
-      load4(q[p] + k, u);
-      const float4 w = make_float4(u[0] * inv_q[p], u[1] * inv_q[p], u[2] * inv_q[p], u[3] * inv_q[p]);
-      ss[p] += v[0] * v[0] + v[1] * v[1] + v[2] * v[2] + v[3] * v[3];
-      dot[p] += v[0] * w.x + v[1] * w.y + v[2] * w.z + v[3] * w.w;
-    }
+  for (int p = 0; p < PT; ++p) ss[p] = dot[p] = 0.f;
+  auto add = [&](int p, const uint2& xr, const uint2& qr) {
+    const float v[4] = {__uint_as_float(xr.x << 16), __uint_as_float(xr.x & 0xffff0000u), __uint_as_float(xr.y << 16), __uint_as_float(xr.y & 0xffff0000u)};
+    const float u[4] = {__uint_as_float(qr.x << 16), __uint_as_float(qr.x & 0xffff0000u), __uint_as_float(qr.y << 16), __uint_as_float(qr.y & 0xffff0000u)};
+    const float4 w = make_float4(u[0] * inv_q[p], u[1] * inv_q[p], u[2] * inv_q[p], u[3] * inv_q[p]);
+    ss[p] += v[0] * v[0] + v[1] * v[1] + v[2] * v[2] + v[3] * v[3];
+    dot[p] += v[0] * w.x + v[1] * w.y + v[2] * w.z + v[3] * w.w;
+  };
+  int k = lane * 4;
+  for (int left = d >> 7; left > 0; left -= UNROLL) {    // 128 features an iteration, UNROLL of them in flight
+    uint2 vx[UNROLL][PT], vq[UNROLL][PT];
+#pragma unroll
+    for (int i = 0; i < UNROLL; ++i)
+#pragma unroll
+      for (int p = 0; p < PT; ++p)
+        if (i < left) {
+          vx[i][p] = __ldg(reinterpret_cast<const uint2*>(x[p] + k + 128 * i));
+          vq[i][p] = __ldg(reinterpret_cast<const uint2*>(q[p] + k + 128 * i));
+        }
+#pragma unroll
+    for (int i = 0; i < UNROLL; ++i)
+#pragma unroll
+      for (int p = 0; p < PT; ++p)
+        if (i < left) add(p, vx[i][p], vq[i][p]);
+    k += 128 * min(left, UNROLL);
+  }
+  if (k < d) {
+#pragma unroll
+    for (int p = 0; p < PT; ++p)
+      add(p, __ldg(reinterpret_cast<const uint2*>(x[p] + k)), __ldg(reinterpret_cast<const uint2*>(q[p] + k)));
   }
 #pragma unroll
-  for (int p = 0; p < 2; ++p) {
+  for (int p = 0; p < PT; ++p) {
     ss[p] = warp_sum(ss[p]);
     inv[p] = 0.f;
     if (ss[p] > FLT_MIN) { inv[p] = rsqrtf(ss[p]); inv[p] = inv[p] * (1.5f - 0.5f * ss[p] * inv[p] * inv[p]); }
     dot[p] = warp_sum(dot[p]) * inv[p];
   }
 }
+
+// A token left to identity_exact_kernel: a NaN that no score has (scores that are not finite are the positive one) with the
+// row of its only candidate in the query array; or, in arrays of up to kPairRows rows, with the row of the first of two
+// and the distance to the second.
+constexpr uint32_t kDeferred = 0xffc00000u;
+constexpr long long kDeferredRows = 1ll << 22;
+constexpr int kPairBits = 14;
+constexpr long long kPairRows = 1ll << kPairBits;
 
 __global__ void __launch_bounds__(kIdThreads, 2)
 identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_q,
@@ -204,6 +242,18 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
   }
   const int at = tile * kTokens + half * R, row0 = vis_off + at, nrows = min(R, n - at);
   const int passes = nrows > 0 ? (T + prm.n_cols - 1) / prm.n_cols : 0;
+  const int group_cols = (prm.n_cols + 31) & ~31;
+  // 16 columns of the products: the groups added up in their order
+  auto products16 = [&](uint32_t t_col, float (&v)[16]) {
+    tmem_ld16(t_col, v);
+    for (int g = 1; g < prm.groups; ++g) {
+      float u[16];
+      tmem_ld16(t_col + g * group_cols, u);
+#pragma unroll
+      for (int e = 0; e < 16; ++e) v[e] += u[e];
+    }
+  };
+
   if (warp == 8) {
     if (lane == 0) {
       int s = 0;
@@ -234,9 +284,10 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
           tc_fence_after();
           const uint32_t x_addr = smem_u32(smem + (size_t)s * prm.stage_bytes);
           const uint64_t adesc = umma_desc(x_addr), bdesc = umma_desc(x_addr + R * 128);
+          const int g = kc / prm.per_group;
 #pragma unroll
           for (int k = 0; k < kChunk / 16; ++k)
-            umma_bf16(tmem_base, adesc + 2 * k, bdesc + 2 * k, idesc, (kc | k) != 0);
+            umma_bf16(tmem_base + g * group_cols, adesc + 2 * k, bdesc + 2 * k, idesc, (kc - g * prm.per_group + k) != 0);
           umma_commit(&empty[s]);
           if (++s == prm.stages) { s = 0; ph ^= 1u; }
         }
@@ -251,6 +302,7 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     float best = -INFINITY, len_x = 0.f, inv_x = 0.f;    // best: largest product so far, divided by the query length
     bool nonfinite = false, ok = true;
     int s = 0;
+    uint32_t deferred = 0u;                              // left to identity_exact_kernel
     uint32_t ph = 0;
     if (tokens) exact[r] = -FLT_MAX;
     for (int pass = 0; pass < passes; ++pass) {
@@ -284,7 +336,11 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
           if (++s == prm.stages) { s = 0; ph ^= 1u; }
         }
         named_barrier(1, 256);
-        if (measure) inv_q[r] = inverse_length(total_by_lane(sq));
+        if (measure) {
+          const float inv = ok ? inverse_length(total_by_lane(sq)) : __int_as_float(0x7fc00000);
+          inv_q[r] = inv;
+          if (prm.defer && passes == 1 && at == 0 && r < T) prm.inv_q[txt_off + r] = inv;
+        }
       }
       named_barrier(1, 256);
       if (tokens) {
@@ -295,7 +351,7 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
 #pragma unroll 1
         for (int c0 = 0; c0 < cols; c0 += 16) {
           float v[16];
-          tmem_ld16(t_lane + c0, v);
+          products16(t_lane + c0, v);
 #pragma unroll
           for (int e = 0; e < 16; ++e)
             if (c0 + e < cols) {
@@ -309,18 +365,26 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         const bool tiny = inv_x == 0.f || !(most * inv_x <= 1.2e24f);
         if (!tiny) best = fmaxf(best, top);
         const float limit = tiny ? -INFINITY : best - prm.margin * len_x;
+        int found = 0, low = 0, high = 0;                // candidates of the pass, the first and the last of them
 #pragma unroll 1
         for (int c0 = 0; c0 < kQueries; c0 += 16) {
           uint32_t bits = 0u;
           if (c0 < cols) {
             float v[16];
-            tmem_ld16(t_lane + c0, v);
+            products16(t_lane + c0, v);
 #pragma unroll
             for (int e = 0; e < 16; ++e)
               if (c0 + e < cols && v[e] * inv_q[c0 + e] >= limit) bits |= 1u << e;
           }
-          candidates[r * (kQueries / 16) + (c0 >> 4)] = (uint16_t)(nonfinite || !ok ? 0u : bits);
+          if (nonfinite || !ok) bits = 0u;
+          if (bits && found == 0) low = c0 + __ffs((int)bits) - 1;
+          if (bits) high = c0 + 31 - __clz((int)bits);
+          found += __popc(bits);
+          candidates[r * (kQueries / 16) + (c0 >> 4)] = (uint16_t)bits;
         }
+        if (passes == 1 && found >= 1 && found <= prm.defer)
+          deferred = kDeferred | (uint32_t)(txt_off + low) | (uint32_t)(high - low) << kPairBits;
+        if (deferred) reinterpret_cast<uint4*>(candidates)[r] = make_uint4(0u, 0u, 0u, 0u);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(acc_empty);
@@ -344,7 +408,7 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             qr[p] = prm.q + (size_t)(txt_off + pass * prm.n_cols + jp) * prm.d;
             iq[p] = inv_q[jp];
           }
-          exact_cosines(xr, qr, iq, prm.d, lane, inv, dot);
+          exact_cosines<2, 4>(xr, qr, iq, prm.d, lane, inv, dot);
 #pragma unroll
           for (int p = 0; p < 2; ++p)
             if (j[p] >= 0) {
@@ -360,13 +424,43 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     }
     named_barrier(1, 256);
     // a wait that gave up leaves NaN, for callers that have no status word to look at
-    if (tokens && r < nrows) prm.s_query[row0 + r] = nonfinite || !ok ? __int_as_float(0x7fc00000) : exact[r];
+    if (tokens && r < nrows) {
+      const uint32_t score = nonfinite || !ok ? 0x7fc00000u : deferred ? deferred : __float_as_uint(exact[r]);
+      reinterpret_cast<uint32_t*>(prm.s_query)[row0 + r] = score;
+    }
   }
 
   tc_fence_before();
   __syncthreads();
   if (warp == 9) tmem_dealloc(tmem_base, kColumns);
   if (threadIdx.x == 0 && *abort_flag && prm.status != nullptr) atomicOr(prm.status, kStatusTimeout);
+}
+
+// The scores of the tokens that identity_tc_kernel left with one or two candidates; one warp per token, bound by the
+// latency and issue of a row's loads and sums (32,768 tokens, d = 3584: about 45 us, 36 of them HBM).
+__global__ void __launch_bounds__(256, 4)
+identity_exact_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ q,
+                      const float* __restrict__ inv_q, int d, int pairs, int first, int rows, float* __restrict__ s_query) {
+  const int row = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
+  wait_for_previous_kernel();
+  if (row >= rows) return;
+  const uint32_t code = __float_as_uint(s_query[first + row]);
+  if ((code & kDeferred) != kDeferred) return;
+  const uint32_t low = code & (pairs ? (uint32_t)kPairRows - 1u : ~kDeferred);
+  const uint32_t high = low + (pairs ? (code & ~kDeferred) >> kPairBits : 0u);
+  const __nv_bfloat16* const xr[1] = {x + (size_t)(first + row) * d};
+  float best = -FLT_MAX;
+  bool nonfinite = false;
+  for (uint32_t j = low;; j = high) {
+    const __nv_bfloat16* const qr[1] = {q + (size_t)j * d};
+    const float iq[1] = {inv_q[j]};
+    float inv[1], dot[1];
+    exact_cosines<1, 8>(xr, qr, iq, d, lane, inv, dot);
+    best = fmaxf(best, dot[0]);
+    nonfinite |= iq[0] != iq[0];
+    if (j == high) break;
+  }
+  if (lane == 0) s_query[first + row] = nonfinite ? __int_as_float(0x7fc00000) : best;
 }
 
 }  // namespace ident

@@ -151,3 +151,22 @@ def test_identity_scores_do_not_depend_on_the_batch():
     both = _both_routes(wl)[0][:ns[0]]
     alone = api.query_score_static(wl.X[:ns[0]], wl.Q[:ts[0]], wl.vis_offsets[:2], wl.txt_offsets[:2])
     assert torch.equal(both, alone)
+
+
+def test_identity_scores_with_more_query_rows_than_a_pair_code_holds():
+    # up to 16384 query rows a token hands on two candidates, beyond only one; three and more stay where they were found
+    from paper_2605_02218_b200 import build
+    build.build()
+    batch, t, d = 129, 128, 64
+    wl = workloads.make_workload("many-queries", seed=5, dtype=torch.bfloat16, batch=batch, sizes=([40] * batch, [t] * batch),
+                                 d=d, n_heads=0, rank=4, keep=1, act_layers=0).to("cuda:0")
+    for b in range(0, batch, 3):
+        q0, x0 = int(wl.txt_offsets[b]), int(wl.vis_offsets[b])
+        wl.Q[q0 + 100:q0 + 100 + b % 4] = wl.Q[q0 + 3]       # none, one, two or three repetitions
+        wl.X[x0:x0 + 20] = wl.Q[q0 + 3] * 2
+    assert int(wl.txt_offsets[-1]) > 1 << 14
+    for n in (batch, 128):                                    # 16512 and 16384 rows
+        part = workloads.Workload(**{**wl.__dict__, "vis_offsets": wl.vis_offsets[:n + 1], "txt_offsets": wl.txt_offsets[:n + 1],
+                                     "keep": wl.keep[:n], "X": wl.X[:40 * n], "Q": wl.Q[:t * n]})
+        tc, simt = _both_routes(part)
+        assert torch.equal(tc, simt)
