@@ -277,3 +277,17 @@ def test_branch_candidates_among_mass_ties(dtype, vocab):
         for i in range(rows):
             want = C.bonus_candidates(z[i, :vocab].cpu().double().numpy(), int(y[i]), fan)
             assert np.array_equal(cand[off[i]:off[i + 1]], want), (i, fan)
+
+
+@pytest.mark.parametrize("dtype,vocab", [(torch.float32, 200003), (torch.float32, 420001), (torch.float16, 420001)])
+def test_rows_too_long_for_sums_in_shared_memory(dtype, vocab):
+    # the largest rows of the cluster sizes: fewer CTAs per position than the call's size asks for, and no kept sums
+    from paper_2605_02218_b200 import api
+    data = workloads.make_logits(seed=17, rows=160, vocab=vocab, dtype=dtype, device="cuda:0")
+    args = lambda n: (data["z_draft"][:n], data["z_target"][:n], data["uniforms"][:n], 0.05, data["drafted"][:n])
+    whole = api.correct(*args(160), vocab=vocab)
+    for rows in (1, 24):
+        for a, b in zip(whole, api.correct(*args(rows), vocab=vocab)):
+            assert torch.equal(a[:rows], b)
+    torch.cuda.synchronize()
+    _check(data, 0.05, whole, rows=[0, 1, 159])
