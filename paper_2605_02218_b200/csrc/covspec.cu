@@ -537,7 +537,7 @@ bool identity_tc_usable(int dtype, int d, const void* X, const void* Q) {
   return dtype == COVSPEC_BF16 && d >= ident::kChunk && d % 8 == 0 &&
          ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Q)) & 15) == 0;
 }
-// One or two launches over `tiles` 128-token tiles of the rows from `first` on; plan == nullptr: the requests come with `reqs`.
+// Two launches over `tiles` 128-token tiles of the rows from `first` on; plan == nullptr: the requests come with `reqs`.
 // inv_q: scratch of one float per query row.
 int launch_identity_tc(const void* X, const void* Q, long long rows_x, long long rows_q, int d, int t_max,
                        const ReqPlan* plan, const ident::InlineReqs& reqs, int batch, int tiles, int num_sms,
@@ -565,8 +565,7 @@ int launch_identity_tc(const void* X, const void* Q, long long rows_x, long long
   prm.stages = std::max(2, std::min({ident::kMaxStages, prm.k_chunks, budget / prm.stage_bytes}));
   prm.s_query = s_query; prm.status = status; prm.spin_limit = spin_limit;
   prm.inv_q = inv_q;
-  prm.defer = rows_q <= ident::kPairRows ? 2 : rows_q <= ident::kDeferredRows ? 1 : 0;
-  prm.x = static_cast<const __nv_bfloat16*>(X); prm.q = static_cast<const __nv_bfloat16*>(Q); prm.d = d;
+  prm.pairs = rows_q <= ident::kPairRows ? 1 : 0;
   const int columns = (prm.n_cols + 31) / 32 * 32;
   const int want = std::max(1, std::min(ident::kColumns / columns, (prm.k_chunks + ident::kGroupChunks - 1) / ident::kGroupChunks));
   prm.per_group = (prm.k_chunks + want - 1) / want;
@@ -581,9 +580,9 @@ int launch_identity_tc(const void* X, const void* Q, long long rows_x, long long
   const int smem = prm.stages * prm.stage_bytes + slack + ident::kTailBytes + 1024;
   ident::identity_tc_kernel<<<blocks, ident::kIdThreads, smem, s>>>(map_x, map_q, reqs, prm);
   CUDA_TRY(cudaGetLastError());
-  if (prm.defer)
-    CUDA_TRY(launch_dependent(ident::identity_exact_kernel, dim3((unsigned)((rows + 7) / 8)), 256, 0, s, prm.x, prm.q, inv_q, d,
-                              prm.defer == 2 ? 1 : 0, (int)first, (int)rows, s_query));
+  CUDA_TRY(launch_dependent(ident::identity_exact_kernel, dim3((unsigned)((rows + 7) / 8)), 256, 0, s,
+                            static_cast<const __nv_bfloat16*>(X), static_cast<const __nv_bfloat16*>(Q), inv_q, reqs, prm, d,
+                            (int)first, (int)rows));
   return COVSPEC_OK;
 }
 
@@ -739,7 +738,7 @@ int score_impl(covspec_ctx* ctx, const covspec_problem* p, float* s_query, float
   if (!s_act) s_act = ctx->sa;
   bool identity = cfg.n_heads == 0;
   bool use_tc = tc_supported(ctx);
-  bool identity_tc = identity && cfg.relevance_path != 1 && identity_tc_usable(cfg.dtype, cfg.d, X, Q);
+  bool identity_tc = identity && cfg.relevance_path != 1 && identity_tc_usable(cfg.dtype, cfg.d, X, Q) && rowsQ <= ident::kCodeRows;
   // The tensor-core relevance kernel leaves HBM idle: the activity stream runs beside it on the
   // context's side stream (fork here, join before the scores are fused).
   // The identity kernel reads X once and is done early: the full-rate activity kernel fills the SMs it leaves.
@@ -778,7 +777,7 @@ int score_impl(covspec_ctx* ctx, const covspec_problem* p, float* s_query, float
     int st = launch_identity_tc(X, Q, rowsX, rowsQ, cfg.d, pl.t_max, ctx->d_plan, ident::InlineReqs{}, B, pl.n_tiles,
                                 ctx->num_sms, 0, rowsX, s_query, ctx->Qn, ctx->status, tc::kSpinLimit, s);
     if (st) return st;
-    ctx->launches += rowsQ <= ident::kDeferredRows ? 2 : 1;
+    ctx->launches += 2;
     prof_mark(ctx, ST_RELEVANCE, 1, s);
     // after the identity kernel, whose few large blocks would otherwise wait for the activity blocks to end
     if (overlap && (st = fork_activity())) return st;

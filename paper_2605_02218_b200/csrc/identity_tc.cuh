@@ -9,21 +9,19 @@
 //      cut into as many groups of contiguous features as TMEM has columns for, up to eight, added up in float32: the
 //      bound falls with their number.  Every query element within twice the bound of the largest value is a
 //      candidate; nearly always there is one.
-//   3. the cosine of every candidate is computed again by one warp per token, with the arithmetic of cosmax_kernel in its
-//      order (score_kernels.cuh), and the largest is the score: the bits are those of that kernel, whatever the
-//      batch a request comes in.  (Tensor-core sums as scores were off by 2.5e-7 to 2.1e-6 relative, d = 1024-4096,
-//      against 6e-8 to 1e-7, and depended on the longest query of the call.)  One or two candidates
-//      of a token go to identity_exact_kernel, which has the whole chip's warps to wait for the rows; more of them, and
-//      requests of more than one pass, are seen to here.  (All of it here: 4 requests of 576 tokens, d = 1024, 32 query
-//      elements 19.1 us, so 17.2; 16 of 400-729 at d = 2048 beside the activity stream 66.8 and 61.2; 2 of 16384 at
-//      d = 3584 121.7 and 93.5: a single token with two candidates held a tile up for 3 to 18 us.)
+//   3. identity_exact_kernel computes the cosine of every candidate again, one warp per token, with the arithmetic of
+//      cosmax_kernel in its order (score_kernels.cuh), and the largest is the score: the bits are those of that kernel,
+//      whatever the batch a request comes in.  (Tensor-core sums as scores were off by 2.5e-7 to 2.1e-6 relative,
+//      d = 1024-4096, against 6e-8 to 1e-7, and depended on the longest query of the call.)  A second launch because
+//      a row is a handful of loads whose latency is all there is: it takes the whole chip's warps to wait for them.  With
+//      step 3 in the first kernel, by eight warps a tile, 2 x 16384 tokens at d = 3584 took 121.7 us instead of 89.1 and 4 x 576 at
+//      d = 1024 19.1 instead of 16.1 (the sums themselves as scores: 43.4 and 11.2; cosmax_kernel 1093 and 48.9).
 //
 // One CTA per 128-token tile of a request (or per 64 tokens, while that leaves at most two CTAs per SM: a
 // block is bound by the latency of its loads and by shared-memory bandwidth); the request's query elements pass in groups of up to 128.
 // Warps 0-3: one token per thread (length of x, candidates); 4-7: one query element per thread (length of
-// q); 0-7: step 3; warp 8: TMA producer; warp 9: MMA issuer and TMEM owner.  Bound by HBM (X once).  cosmax_kernel (one warp
-// per token) reads every query element once per token through L1: 16 requests of 400-729 tokens, d = 2048, 210 us
-// for 37 MB.
+// q); warp 8: TMA producer; warp 9: MMA issuer and TMEM owner.  Bound by HBM (X once).  cosmax_kernel (one warp per token)
+// reads every query element once per token through L1: 16 requests of 400-729 tokens, d = 2048, 210 us for 37 MB.
 #pragma once
 #include <float.h>
 
@@ -41,8 +39,7 @@ constexpr int kMaxStages = 12;
 constexpr int kColumns = 256;            // TMEM columns: two CTAs fit on an SM
 constexpr int kIdThreads = 320;
 constexpr int kGroupChunks = 4;          // k-chunks per accumulation group, if TMEM has the columns
-// barriers (512), reciprocal query lengths [kQueries], best exact cosine [kTokens], candidate bits [kTokens][kQueries]
-constexpr int kTailBytes = 512 + kQueries * 4 + kTokens * 4 + kTokens * kQueries / 8;
+constexpr int kTailBytes = 2048;         // barriers, reciprocal query lengths
 
 // Requests handed over by value (the allocation-free entry point, which has no plan on the device).
 constexpr int kInlineReqs = 64;
@@ -52,13 +49,10 @@ struct InlineReqs {
 };
 
 struct IdParams {
-  const __nv_bfloat16* x;                // the arrays behind the tensor maps
-  const __nv_bfloat16* q;
-  int d;
   float* inv_q;                          // reciprocal query lengths for identity_exact_kernel
   float margin;                          // candidates: within margin |x| |q| of the largest product
   int per_group, groups;                 // accumulation groups: k-chunks each, their number
-  int defer;                             // candidates that may be left to identity_exact_kernel: 0, 1 or 2
+  int pairs;                             // 1: codes of two candidates fit (see kPairRows)
   const ReqPlan* plan;                   // or nullptr: the inline requests
   int batch;
   int k_chunks;
@@ -132,68 +126,46 @@ __device__ __forceinline__ float inverse_length(float ss) {
   return inv * (1.5f - 0.5f * ss * inv * inv);
 }
 
-// Takes the lowest set bit out of a set of 128; -1: none left.
-__device__ __forceinline__ int next_candidate(uint4& m) {
-  if (m.x) { const int b = __ffs((int)m.x) - 1; m.x &= m.x - 1u; return b; }
-  if (m.y) { const int b = __ffs((int)m.y) - 1; m.y &= m.y - 1u; return 32 + b; }
-  if (m.z) { const int b = __ffs((int)m.z) - 1; m.z &= m.z - 1u; return 64 + b; }
-  if (m.w) { const int b = __ffs((int)m.w) - 1; m.w &= m.w - 1u; return 96 + b; }
-  return -1;
-}
-
-// Cosines of PT tokens with a query element each, by one warp, as cosmax_kernel computes them; *inv: the tokens'
-// reciprocal lengths.  A row is a handful of loads per lane, whose latency is all there is: several at a time.
-template <int PT, int UNROLL>
-__device__ __forceinline__ void exact_cosines(const __nv_bfloat16* const (&x)[PT], const __nv_bfloat16* const (&q)[PT],
-                                              const float (&inv_q)[PT], int d, int lane, float (&inv)[PT], float (&dot)[PT]) {
-  float ss[PT];
-#pragma unroll
-  for (int p = 0; p < PT; ++p) ss[p] = dot[p] = 0.f;
-  auto add = [&](int p, const uint2& xr, const uint2& qr) {
+// Cosine of a token with a query element, by one warp, as cosmax_kernel computes it; inv: the token's reciprocal length.
+__device__ __forceinline__ float exact_cosine(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ q,
+                                              float inv_q, int d, int lane, float& inv) {
+  constexpr int kFlight = 8;                             // iterations of 128 features whose loads are in flight together
+  float ss = 0.f, dot = 0.f;
+  auto add = [&](const uint2& xr, const uint2& qr) {
     const float v[4] = {__uint_as_float(xr.x << 16), __uint_as_float(xr.x & 0xffff0000u), __uint_as_float(xr.y << 16), __uint_as_float(xr.y & 0xffff0000u)};
     const float u[4] = {__uint_as_float(qr.x << 16), __uint_as_float(qr.x & 0xffff0000u), __uint_as_float(qr.y << 16), __uint_as_float(qr.y & 0xffff0000u)};
-    const float4 w = make_float4(u[0] * inv_q[p], u[1] * inv_q[p], u[2] * inv_q[p], u[3] * inv_q[p]);
-    ss[p] += v[0] * v[0] + v[1] * v[1] + v[2] * v[2] + v[3] * v[3];
-    dot[p] += v[0] * w.x + v[1] * w.y + v[2] * w.z + v[3] * w.w;
+    const float4 w = make_float4(u[0] * inv_q, u[1] * inv_q, u[2] * inv_q, u[3] * inv_q);
+    ss += v[0] * v[0] + v[1] * v[1] + v[2] * v[2] + v[3] * v[3];
+    dot += v[0] * w.x + v[1] * w.y + v[2] * w.z + v[3] * w.w;
   };
   int k = lane * 4;
-  for (int left = d >> 7; left > 0; left -= UNROLL) {    // 128 features an iteration, UNROLL of them in flight
-    uint2 vx[UNROLL][PT], vq[UNROLL][PT];
+  for (int left = d >> 7; left > 0; left -= kFlight) {
+    uint2 vx[kFlight], vq[kFlight];
 #pragma unroll
-    for (int i = 0; i < UNROLL; ++i)
+    for (int i = 0; i < kFlight; ++i)
+      if (i < left) {
+        vx[i] = __ldg(reinterpret_cast<const uint2*>(x + k + 128 * i));
+        vq[i] = __ldg(reinterpret_cast<const uint2*>(q + k + 128 * i));
+      }
 #pragma unroll
-      for (int p = 0; p < PT; ++p)
-        if (i < left) {
-          vx[i][p] = __ldg(reinterpret_cast<const uint2*>(x[p] + k + 128 * i));
-          vq[i][p] = __ldg(reinterpret_cast<const uint2*>(q[p] + k + 128 * i));
-        }
-#pragma unroll
-    for (int i = 0; i < UNROLL; ++i)
-#pragma unroll
-      for (int p = 0; p < PT; ++p)
-        if (i < left) add(p, vx[i][p], vq[i][p]);
-    k += 128 * min(left, UNROLL);
+    for (int i = 0; i < kFlight; ++i)
+      if (i < left) add(vx[i], vq[i]);
+    k += 128 * min(left, kFlight);
   }
-  if (k < d) {
-#pragma unroll
-    for (int p = 0; p < PT; ++p)
-      add(p, __ldg(reinterpret_cast<const uint2*>(x[p] + k)), __ldg(reinterpret_cast<const uint2*>(q[p] + k)));
-  }
-#pragma unroll
-  for (int p = 0; p < PT; ++p) {
-    ss[p] = warp_sum(ss[p]);
-    inv[p] = 0.f;
-    if (ss[p] > FLT_MIN) { inv[p] = rsqrtf(ss[p]); inv[p] = inv[p] * (1.5f - 0.5f * ss[p] * inv[p] * inv[p]); }
-    dot[p] = warp_sum(dot[p]) * inv[p];
-  }
+  if (k < d) add(__ldg(reinterpret_cast<const uint2*>(x + k)), __ldg(reinterpret_cast<const uint2*>(q + k)));
+  ss = warp_sum(ss);
+  inv = 0.f;
+  if (ss > FLT_MIN) { inv = rsqrtf(ss); inv = inv * (1.5f - 0.5f * ss * inv * inv); }
+  return warp_sum(dot) * inv;
 }
 
-// A token left to identity_exact_kernel: a NaN that no score has (scores that are not finite are the positive one) with the
-// row of its only candidate in the query array; or, in arrays of up to kPairRows rows, with the row of the first of two
-// and the distance to the second.
-constexpr uint32_t kDeferred = 0xffc00000u;
-constexpr long long kDeferredRows = 1ll << 22;
-constexpr int kPairBits = 14;
+// What the first kernel leaves in a token's place for identity_exact_kernel: a NaN that no score has (scores that are not
+// finite are the positive one) with the row of its only candidate in the query array; in arrays of up to kPairRows
+// rows, with the row of the first of two and the distance to the second; or kAll: every query element of the request (three
+// candidates and more, lengths near the float32 range's lower end).
+constexpr uint32_t kCode = 0xffc00000u, kAll = 0x3fffffu;
+constexpr long long kCodeRows = (1ll << 22) - 1;
+constexpr int kPairBits = 14, kPairReach = 254;
 constexpr long long kPairRows = 1ll << kPairBits;
 
 __global__ void __launch_bounds__(kIdThreads, 2)
@@ -209,8 +181,6 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   float* inv_q = reinterpret_cast<float*>(tail + 512);     // [kQueries]
-  float* exact = inv_q + kQueries;                         // [kTokens]
-  uint16_t* candidates = reinterpret_cast<uint16_t*>(exact + kTokens);      // [kTokens][kQueries / 16]
   const int warp = warp_index(), lane = threadIdx.x & 31;
   auto wait = [&](uint64_t* bar, uint32_t parity) { return mbar_wait_limited(bar, parity, abort_flag, prm.spin_limit); };
 
@@ -302,9 +272,11 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     float best = -INFINITY, len_x = 0.f, inv_x = 0.f;    // best: largest product so far, divided by the query length
     bool nonfinite = false, ok = true;
     int s = 0;
-    uint32_t deferred = 0u;                              // left to identity_exact_kernel
+    // up to two candidates so far (product and query row; a row of -1: none), and the largest product of those beyond
+    float c1 = 0.f, c2 = 0.f, beyond = -INFINITY;
+    int q1 = -1, q2 = -1;
+    bool all = false;
     uint32_t ph = 0;
-    if (tokens) exact[r] = -FLT_MAX;
     for (int pass = 0; pass < passes; ++pass) {
       if (tokens) {
         unsigned long long sq[4] = {0ull, 0ull, 0ull, 0ull};
@@ -322,7 +294,7 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
           len_x = ss * inv_x;
           nonfinite = inv_x != inv_x;
         }
-        named_barrier(1, 256);                           // the previous pass no longer reads inv_q and the candidates
+        named_barrier(1, 256);                           // the previous pass no longer reads inv_q
       } else {
         unsigned long long sq[16];
 #pragma unroll
@@ -339,7 +311,7 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         if (measure) {
           const float inv = ok ? inverse_length(total_by_lane(sq)) : __int_as_float(0x7fc00000);
           inv_q[r] = inv;
-          if (prm.defer && passes == 1 && at == 0 && r < T) prm.inv_q[txt_off + r] = inv;
+          if (at == 0 && pass * prm.n_cols + r < T) prm.inv_q[txt_off + pass * prm.n_cols + r] = inv;
         }
       }
       named_barrier(1, 256);
@@ -362,71 +334,38 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             }
         }
         // |x| |q| so small that the products themselves may be lost below the float32 range: every element is a candidate
-        const bool tiny = inv_x == 0.f || !(most * inv_x <= 1.2e24f);
-        if (!tiny) best = fmaxf(best, top);
-        const float limit = tiny ? -INFINITY : best - prm.margin * len_x;
-        int found = 0, low = 0, high = 0;                // candidates of the pass, the first and the last of them
+        all |= inv_x == 0.f || !(most * inv_x <= 1.2e24f);
+        best = fmaxf(best, top);
+        const float limit = best - prm.margin * len_x;
+        if (q2 >= 0 && c2 < limit) q2 = -1;
+        if (q1 >= 0 && c1 < limit) { c1 = c2; q1 = q2; q2 = -1; }
 #pragma unroll 1
-        for (int c0 = 0; c0 < kQueries; c0 += 16) {
-          uint32_t bits = 0u;
-          if (c0 < cols) {
-            float v[16];
-            products16(t_lane + c0, v);
+        for (int c0 = 0; c0 < cols; c0 += 16) {
+          float v[16];
+          products16(t_lane + c0, v);
 #pragma unroll
-            for (int e = 0; e < 16; ++e)
-              if (c0 + e < cols && v[e] * inv_q[c0 + e] >= limit) bits |= 1u << e;
+          for (int e = 0; e < 16; ++e) {
+            const float c = c0 + e < cols ? v[e] * inv_q[c0 + e] : -INFINITY;
+            if (c >= limit) {
+              const int row = txt_off + pass * prm.n_cols + c0 + e;
+              if (q1 < 0) { c1 = c; q1 = row; }
+              else if (q2 < 0) { c2 = c; q2 = row; }
+              else beyond = fmaxf(beyond, c);
+            }
           }
-          if (nonfinite || !ok) bits = 0u;
-          if (bits && found == 0) low = c0 + __ffs((int)bits) - 1;
-          if (bits) high = c0 + 31 - __clz((int)bits);
-          found += __popc(bits);
-          candidates[r * (kQueries / 16) + (c0 >> 4)] = (uint16_t)bits;
         }
-        if (passes == 1 && found >= 1 && found <= prm.defer)
-          deferred = kDeferred | (uint32_t)(txt_off + low) | (uint32_t)(high - low) << kPairBits;
-        if (deferred) reinterpret_cast<uint4*>(candidates)[r] = make_uint4(0u, 0u, 0u, 0u);
+        if (beyond < limit) beyond = -INFINITY;
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(acc_empty);
       }
-      named_barrier(1, 256);                             // the candidates of the pass are known
-      for (int t0 = warp; t0 < nrows; t0 += 16) {
-        const int t[2] = {t0, min(t0 + 8, nrows - 1)};
-        uint4 m[2];
-        m[0] = reinterpret_cast<const uint4*>(candidates)[t[0]];
-        m[1] = t0 + 8 < nrows ? reinterpret_cast<const uint4*>(candidates)[t[1]] : make_uint4(0u, 0u, 0u, 0u);
-        float high[2] = {exact[t[0]], exact[t[1]]};
-        for (;;) {
-          const int j[2] = {next_candidate(m[0]), next_candidate(m[1])};
-          if (j[0] < 0 && j[1] < 0) break;
-          const __nv_bfloat16 *xr[2], *qr[2];
-          float iq[2], inv[2], dot[2];
-#pragma unroll
-          for (int p = 0; p < 2; ++p) {                  // a token without one shares the other's loads
-            const int tp = j[p] >= 0 ? t[p] : t[1 - p], jp = j[p] >= 0 ? j[p] : j[1 - p];
-            xr[p] = prm.x + (size_t)(row0 + tp) * prm.d;
-            qr[p] = prm.q + (size_t)(txt_off + pass * prm.n_cols + jp) * prm.d;
-            iq[p] = inv_q[jp];
-          }
-          exact_cosines<2, 4>(xr, qr, iq, prm.d, lane, inv, dot);
-#pragma unroll
-          for (int p = 0; p < 2; ++p)
-            if (j[p] >= 0) {
-              high[p] = fmaxf(high[p], dot[p]);
-              if (inv[p] == 0.f) m[p] = make_uint4(0u, 0u, 0u, 0u);        // a zero token: 0 with every element
-            }
-        }
-        if (lane == 0) {
-          exact[t[0]] = high[0];
-          if (t0 + 8 < nrows) exact[t[1]] = high[1];
-        }
-      }
     }
-    named_barrier(1, 256);
     // a wait that gave up leaves NaN, for callers that have no status word to look at
     if (tokens && r < nrows) {
-      const uint32_t score = nonfinite || !ok ? 0x7fc00000u : deferred ? deferred : __float_as_uint(exact[r]);
-      reinterpret_cast<uint32_t*>(prm.s_query)[row0 + r] = score;
+      uint32_t code = (uint32_t)q1;
+      if (q2 >= 0) code |= (uint32_t)(q2 - q1) << kPairBits;
+      if (all || q1 < 0 || beyond > -INFINITY || (q2 >= 0 && (!prm.pairs || q2 - q1 > kPairReach))) code = kAll;
+      reinterpret_cast<uint32_t*>(prm.s_query)[row0 + r] = nonfinite || !ok ? 0x7fc00000u : kCode | code;
     }
   }
 
@@ -436,31 +375,42 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
   if (threadIdx.x == 0 && *abort_flag && prm.status != nullptr) atomicOr(prm.status, kStatusTimeout);
 }
 
-// The scores of the tokens that identity_tc_kernel left with one or two candidates; one warp per token, bound by the
-// latency and issue of a row's loads and sums (32,768 tokens, d = 3584: about 45 us, 36 of them HBM).
+// The scores from the candidates that identity_tc_kernel found; one warp per token, bound by the latency and issue of a
+// row's loads and sums (32,768 tokens, d = 3584: about 45 us, 36 of them HBM).
 __global__ void __launch_bounds__(256, 4)
 identity_exact_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ q,
-                      const float* __restrict__ inv_q, int d, int pairs, int first, int rows, float* __restrict__ s_query) {
-  const int row = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
+                      const float* __restrict__ inv_q, const __grid_constant__ InlineReqs reqs, const IdParams prm, int d,
+                      int first, int rows) {
+  const int row = first + (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
   wait_for_previous_kernel();
-  if (row >= rows) return;
-  const uint32_t code = __float_as_uint(s_query[first + row]);
-  if ((code & kDeferred) != kDeferred) return;
-  const uint32_t low = code & (pairs ? (uint32_t)kPairRows - 1u : ~kDeferred);
-  const uint32_t high = low + (pairs ? (code & ~kDeferred) >> kPairBits : 0u);
-  const __nv_bfloat16* const xr[1] = {x + (size_t)(first + row) * d};
+  if (row >= first + rows) return;
+  const uint32_t code = __float_as_uint(prm.s_query[row]);
+  if ((code & kCode) != kCode) return;                   // not finite
+  int low, high, step;                                   // candidates low, low + step, .. high
+  if ((code & kAll) == kAll) {
+    if (prm.plan != nullptr) {
+      const int b = find_request(row, prm.batch, [&](int i) { return prm.plan[i].vis_off; });
+      low = prm.plan[b].txt_off; high = low + prm.plan[b].t - 1;
+    } else {
+      const int b = find_request(row, prm.batch, [&](int i) { return reqs.e[i].x; });
+      low = reqs.e[b].z; high = low + reqs.e[b].w - 1;
+    }
+    step = 1;
+  } else {
+    low = (int)(code & (prm.pairs ? (uint32_t)kPairRows - 1u : kAll));
+    step = max(1, prm.pairs ? (int)((code & kAll) >> kPairBits) : 0);
+    high = prm.pairs ? low + (int)((code & kAll) >> kPairBits) : low;
+  }
   float best = -FLT_MAX;
   bool nonfinite = false;
-  for (uint32_t j = low;; j = high) {
-    const __nv_bfloat16* const qr[1] = {q + (size_t)j * d};
-    const float iq[1] = {inv_q[j]};
-    float inv[1], dot[1];
-    exact_cosines<1, 8>(xr, qr, iq, d, lane, inv, dot);
-    best = fmaxf(best, dot[0]);
-    nonfinite |= iq[0] != iq[0];
-    if (j == high) break;
+  for (int j = low; j <= high; j += step) {
+    const float iq = inv_q[j];
+    float inv;
+    best = fmaxf(best, exact_cosine(x + (size_t)row * d, q + (size_t)j * d, iq, d, lane, inv));
+    nonfinite |= iq != iq;
+    if (inv == 0.f) break;                               // a zero token: 0 with every element
   }
-  if (lane == 0) s_query[first + row] = nonfinite ? __int_as_float(0x7fc00000) : best;
+  if (lane == 0) prm.s_query[row] = nonfinite ? __int_as_float(0x7fc00000) : best;
 }
 
 }  // namespace ident
