@@ -285,8 +285,9 @@ const char* covspec_profile_stage_name(int stage);
  * framework and must not see foreign cudaMalloc calls, or in a latency path where an allocation's
  * implicit device synchronisation is unacceptable.  Such callers cannot create a covspec_ctx
  * (covspec_prune_init allocates the workspace).  This entry point needs no context: its scratch
- * (the unit-length query elements and the per-request plan) lives in a fixed device array inside
- * the library, which every GPU that loads the library holds until the process exits.  The call
+ * (the unit-length query elements and the per-request plan; for bf16 rows on the tensor cores the
+ * query elements' reciprocal lengths alone) lives in a fixed device array inside the library, which
+ * every GPU that loads the library holds until the process exits.  The call
  * issues no cudaMalloc, cudaFree or other allocating routine.
  *
  *  dtype, d      as in covspec_config (d a multiple of 8); identity embedding, max over elements

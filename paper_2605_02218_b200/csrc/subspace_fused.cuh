@@ -849,7 +849,7 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
     };
     // Do the CTAs of a request with nt tiles add up its partial matrices slice by slice?  One CTA reads
     // about 64 bytes a cycle, the two more rounds through L2 that sharing takes cost 5-6 k cycles: worth it
-    // from 48 k entries over all tiles on (11 tiles at p = 88, 4 at p = 144), and only if there is somebody
+    // from 48 k entries over all tiles on (12 tiles at p = 88, 5 at p = 144), and only if there is somebody
     // to share with (a server's request has one CTA per tile).
     auto spread_of = [&](int nt, int P) {
       return prm.spread_sum && nt * ((P >> 3) * ((P >> 3) + 1) / 2 * 64) > 48000 && (prm.n_servers > 0 || n_groups > 1);
