@@ -265,6 +265,15 @@ __device__ __forceinline__ void factor_diag_thread(double* D, const double* d0, 
 
 constexpr int kEpiThreads = 256;         // warps 0-7
 
+// What the kernel needs to know of a tile.  Every role looks its tiles up once per step; the search through the requests is a
+// chain of loads that the acquiring loads of the counters send to L2 each time (64 requests: 5 k cycles a tile and step
+// in the epilogue alone), so a CTA's first kCachedTiles tiles are looked up once per launch.
+struct TileItem {
+  int b, tile;              // request, tile of the request
+  int m, p, r, win, presel_off, ptile_off;
+};
+constexpr int kCachedTiles = 16;
+
 // The part behind the ring: the triangular factor, its reciprocal diagonal (a scratch array of p floats
 // while a factor is being made), barriers, then single words.
 struct PowTail {
@@ -274,6 +283,7 @@ struct PowTail {
   volatile int *abort_flag, *s_word;     // s_word: [2] broadcast slots of the epilogue
   int* s_flag;                           // Jacobi rotation flag
   float* s_scale;
+  TileItem* tiles;                       // [kCachedTiles]
 };
 __device__ __forceinline__ PowTail pow_tail() {
   PowTail t;
@@ -285,6 +295,7 @@ __device__ __forceinline__ PowTail pow_tail() {
   t.s_word = reinterpret_cast<volatile int*>(t.tmem_slot + 2);
   t.s_flag = reinterpret_cast<int*>(t.tmem_slot + 4);
   t.s_scale = reinterpret_cast<float*>(t.tmem_slot + 6);
+  t.tiles = reinterpret_cast<TileItem*>(t.tmem_slot + 8);
   return t;
 }
 
@@ -703,23 +714,25 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 9) tmem_alloc(tmem_slot, kPowTmemCols);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
-
   const int s_begin = prm.sched[blockIdx.x], s_end = prm.sched[blockIdx.x + 1];
   const int* s_items = prm.sched + gridDim.x + 1;
   const int my_group = prm.sched[gridDim.x + 1 + prm.n_items + blockIdx.x] & 0xffff;
   const int n_groups = prm.sched[gridDim.x + 1 + prm.n_items + blockIdx.x] >> 16;
   const int last_step = prm.steps - 1;
   const int R = prm.tile_rows;
-  auto decode = [&](int item, int& b, ReqPlan& rp, int& tile) {
-    b = find_request(item, prm.batch, [&](int q) { return prm.plan[q].ptile_off; });
-    rp = prm.plan[b];
-    tile = item - rp.ptile_off;
+  auto look_up = [&](int item) {
+    const int b = find_request(item, prm.batch, [&](int q) { return prm.plan[q].ptile_off; });
+    const ReqPlan& rp = prm.plan[b];
+    return TileItem{b, item - rp.ptile_off, rp.m, rp.p, rp.r, rp.win, rp.presel_off, rp.ptile_off};
   };
+  if (threadIdx.x < min(kCachedTiles, s_end - s_begin)) tail.tiles[threadIdx.x] = look_up(s_items[s_begin + threadIdx.x]);
+  if (warp == 9) tmem_alloc(tmem_slot, kPowTmemCols);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  // the CTA's si-th tile
+  auto tile_at = [&](int si) { return si - s_begin < kCachedTiles ? tail.tiles[si - s_begin] : look_up(s_items[si]); };
 
   // request of the factor server with this index: the index-th one that has a stage 2
   auto server_request = [&](int index) -> int {
@@ -737,9 +750,8 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
         const CUtensorMap* myh = (step & 1) ? &map_y1h : &map_y0h;
         const CUtensorMap* myl = (step & 1) ? &map_y1l : &map_y0l;
         for (int si = s_begin; si < s_end && ok; ++si, ++n) {
-          const int item = s_items[si];
-          int b, tile; ReqPlan rp;
-          decode(item, b, rp, tile);
+          const TileItem rp = tile_at(si);
+          const int b = rp.b;
           if (step > 0) {
             // every tile of the request has written its slab of the block this step multiplies,
             // unless the request has already had its last step
@@ -759,7 +771,7 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
             if (!(ok = mbar_wait(&empty[s], ((it / kPowStages) & 1u) ^ 1u, abort_flag))) break;
             mbar_expect_tx(&full[s], kPowStageBytes);
             uint32_t dst = smem_u32(smem + s * kPowStageBytes);
-            int grow = rp.presel_off + tile * R;
+            int grow = rp.presel_off + rp.tile * R;
             tma_load_2d(dst, &map_gh, kc * kBK, grow, &full[s]);
             tma_load_2d(dst + kPowBytesA, &map_gl, kc * kBK, grow, &full[s]);
             tma_load_2d(dst + 2 * kPowBytesA, myh, kc * kBK, b * kPMax, &full[s]);
@@ -796,9 +808,8 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
       bool ok = true;
       for (int step = 0; step <= last_step && ok; ++step) {
         for (int si = s_begin; si < s_end && ok; ++si, ++n) {
-          const int item = s_items[si];
-          int b, tile; ReqPlan rp;
-          decode(item, b, rp, tile);
+          const TileItem rp = tile_at(si);
+          const int b = rp.b;
           const uint32_t idesc = umma_idesc(kTile, (rp.p + 15) & ~15);
           if (step > 0) {
             const unsigned nt = (unsigned)((rp.m + R - 1) / R);
@@ -860,7 +871,7 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
     // Factors the summed Gram matrix of request b after step `step` (Cholesky, or the Rayleigh-Ritz
     // solve after the last step) and publishes the result; returns whether the next step was
     // declared the last one.  Uses the operand ring as scratch.
-    auto factor_request = [&](int b, const ReqPlan& rp, unsigned* sync_b, int step, bool is_last, int last_b,
+    auto factor_request = [&](int b, const auto& rp, unsigned* sync_b, int step, bool is_last, int last_b,
                               int nt_sum) -> bool {
       const int p = rp.p;
       const double* pbase = prm.partial + (size_t)rp.ptile_off * kTileDoubles;
@@ -910,9 +921,8 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
       __nv_bfloat16* y_hi = prm.y_hi[(step & 1) ^ 1];
       __nv_bfloat16* y_lo = prm.y_lo[(step & 1) ^ 1];
       for (int si = s_begin; si < s_end; ++si, ++n) {
-        const int item = s_items[si];
-        int b, tile; ReqPlan rp;
-        decode(item, b, rp, tile);
+        const TileItem rp = tile_at(si);
+        const int b = rp.b, tile = rp.tile;
         const int p = rp.p, P = (p + 7) & ~7;
         unsigned* sync_b = prm.sync + (size_t)b * kSyncStride;
         const unsigned nt = (unsigned)((rp.m + R - 1) / R);
@@ -1078,7 +1088,7 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
         {
           // The last step only feeds the Rayleigh-Ritz window: the trailing block of columns from
           // coff on, plus the diagonal of the leading columns (the scale of the problem).
-          double* out = prm.partial + (size_t)item * kTileDoubles;
+          double* out = prm.partial + (size_t)(rp.ptile_off + tile) * kTileDoubles;
           for (int c = et; c < coff; c += kEpiThreads) {
             double sq = 0.0;
             for (int rr = 0; rr < nrows; ++rr) { double x = (double)xs[c * kXsLd + rr]; sq += x * x; }
@@ -1164,9 +1174,8 @@ subspace_kernel(const __grid_constant__ CUtensorMap map_gh, const __grid_constan
       float* part = us + kPMax * kPMax;                                // [128] running sums
       int cached_u = -1;
       for (int si = s_begin; si < s_end; ++si) {
-        const int item = s_items[si];
-        int b, tile; ReqPlan rp;
-        decode(item, b, rp, tile);
+        const TileItem rp = tile_at(si);
+        const int b = rp.b, tile = rp.tile;
         const int p = rp.p, w = rp.win, nbot = p - rp.r, nb8 = (nbot + 7) & ~7;
         const int nrows = min(R, rp.m - tile * R);
         const int rr = et & 127, second = et >> 7;
