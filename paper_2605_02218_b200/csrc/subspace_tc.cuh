@@ -460,40 +460,57 @@ __device__ __forceinline__ void solve_gemm_any(int tile_rows, float* x, const fl
     else solve_gemm<2, 2>(x, lt, P, S, split, nrows, warp, lane);
   }
 }
-// NG: groups of eight columns in the super-block (four but for the last one of a width that is not a multiple of 32)
+// NG: groups of eight columns in the super-block (four but for the last one of a width that is not a multiple of 32).
+// One warp per scheduler and a chain from column to column: a column's factor row is loaded while the column before it is
+// applied, and two columns are updated by one packed multiply-add.
 template <int NG>
 __device__ __forceinline__ void solve_diag_n(float* xr, const float* lt, const float* dinv, int P, int S, bool keep) {
-  float acc[8 * NG];
+  constexpr int W = 8 * NG;
+  float acc[W];
   float* xb = xr + 32 * S * kXsLd;
-#pragma unroll
-  for (int e = 0; e < 8 * NG; ++e) acc[e] = xb[e * kXsLd];
   const int a0 = 8 * S;
   const float* lp = lt + 4 * a0 * P - 8 * a0 * (a0 - 1);      // row 32 S of the layout, at its first column 32 S
-  int stride = P - 32 * S;
+  const int stride = P - 32 * S;
+  // row i of the factor from the group of four columns that holds i on: P - 32 S - 4 (i / 4) entries a row
+  auto row_at = [&](int i) { const int a = i >> 2; return lp + 4 * a * stride - 8 * a * (a - 1) + (i & 3) * (stride - 4 * a); };
+  float4 l[2][2 * NG];
+  auto load_row = [&](int i, float4 (&dst)[2 * NG]) {
 #pragma unroll
-  for (int a = 0; a < 2 * NG; ++a) {
-    const float4 d4 = *reinterpret_cast<const float4*>(dinv + 32 * S + 4 * a);
-    const float dv[4] = {d4.x, d4.y, d4.z, d4.w};
+    for (int v = 0; v < 2 * NG; ++v)
+      if (4 * v + 3 > i) dst[v] = *reinterpret_cast<const float4*>(row_at(i) + 4 * (v - (i >> 2)));
+  };
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int i = 4 * a + q;
-      const float xi = acc[i] * dv[q];
-      acc[i] = xi;
+  for (int e = 0; e < W; ++e) acc[e] = xb[e * kXsLd];
+  float4 d4 = *reinterpret_cast<const float4*>(dinv + 32 * S);
+  load_row(0, l[0]);
 #pragma unroll
-      for (int v = a; v < 2 * NG; ++v) {
-        if (v == a && q == 3) continue;
-        const float4 l = *reinterpret_cast<const float4*>(lp + q * stride + 4 * (v - a));
-        const float lv[4] = {l.x, l.y, l.z, l.w};
+  for (int i = 0; i < W; ++i) {
+    const float dv = (i & 3) == 0 ? d4.x : (i & 3) == 1 ? d4.y : (i & 3) == 2 ? d4.z : d4.w;
+    const float xi = acc[i] * dv;
+    acc[i] = xi;
+    if (i + 1 < W) {
+      if ((i & 3) == 3) d4 = *reinterpret_cast<const float4*>(dinv + 32 * S + i + 1);
+      load_row(i + 1, l[(i + 1) & 1]);
+    }
+    const f32x2 nx = pack2(-xi, -xi);
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-          if (4 * v + e > i) acc[4 * v + e] -= xi * lv[e];
+    for (int v = 0; v < 2 * NG; ++v) {
+      if (4 * v + 3 <= i) continue;
+      const float lv[4] = {l[i & 1][v].x, l[i & 1][v].y, l[i & 1][v].z, l[i & 1][v].w};
+#pragma unroll
+      for (int e = 0; e < 4; e += 2) {
+        const int j = 4 * v + e;
+        if (j > i) {
+          const float2 t = unpack2(fma2(nx, pack2(lv[e], lv[e + 1]), pack2(acc[j], acc[j + 1])));
+          acc[j] = t.x; acc[j + 1] = t.y;
+        } else if (j + 1 > i) {
+          acc[j + 1] = fmaf(-xi, lv[e + 1], acc[j + 1]);
+        }
       }
     }
-    lp += 4 * stride;
-    stride -= 4;
   }
 #pragma unroll
-  for (int e = 0; e < 8 * NG; ++e) xb[e * kXsLd] = keep ? acc[e] : 0.f;
+  for (int e = 0; e < W; ++e) xb[e * kXsLd] = keep ? acc[e] : 0.f;
 }
 __device__ __forceinline__ void solve_diag(float* xr, const float* lt, const float* dinv, int P, int S, bool keep) {
   const int ng = (P - 32 * S) >> 3;
