@@ -941,7 +941,9 @@ int select_impl(covspec_ctx* ctx, const covspec_problem* p, const float* s_fused
   }
   if (pl.n_stage2 > 0) prof_mark(ctx, ST_EIG, 1, s);
   prof_mark(ctx, ST_FINAL, 0, s);
-  CUDA_TRY(launch_dependent(final_select_kernel, dim3(B), 1024, 0, s, energy, presel, ctx->d_plan, keep_idx, ctx->status));
+  // one key per thread: a barrier of few warps is the shorter one
+  const int select_threads = (int)std::min<long long>(1024, round_up(std::max(pl.m_max, 128), 32));
+  CUDA_TRY(launch_dependent(final_select_kernel, dim3(B), select_threads, 0, s, energy, presel, ctx->d_plan, keep_idx, ctx->status));
   LAUNCH_CHECK(ctx);
   return COVSPEC_OK;
 }

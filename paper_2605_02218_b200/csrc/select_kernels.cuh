@@ -47,8 +47,8 @@ __device__ __forceinline__ unsigned block_exclusive_scan(unsigned v, unsigned* w
 // Top-k of n keys: larger key first, then lower index; out[0..k) receives the selected positions in ascending
 // order, mapped through `remap` when given.  Two forms:
 //   up to kRegKeys keys per thread: the keys stay in registers (thread t holds the positions t,
-//   t + blockDim, ...) and the k-th largest key is found bit by bit, one block-wide count per bit below the
-//   prefix that all keys share, ending as soon as a count equals k (about 15 counts of 150-300 cycles for
+//   t + blockDim, ...) and the k-th largest key is found two bits at a time, one block-wide count per pair of bits
+//   below the prefix that all keys share, ending as soon as a count equals k (about 8 counts of 150-300 cycles for
 //   scores).  A radix select through shared-memory histograms took 12 us at 768 keys (scores
 //   crowd into a few digit values, whose updates queue up) and ranking every key 18 us.
 //   longer segments: an 8-bit-per-pass radix select that re-reads its keys, then an ordered emission.
@@ -80,16 +80,26 @@ __device__ __forceinline__ void block_select_regs(const unsigned (&key)[PER], in
   if (top < 0) thr = all_and;
   bool exact = false;                                        // keys >= thr are the answer, no ties
   int buf = 1;
-  for (int bit = top; bit >= 0 && !exact; --bit, buf ^= 1) {
-    const unsigned cand = thr | (1u << bit);
-    unsigned c = 0u;
+  for (int bit = top; bit >= 0 && !exact; bit -= 2, buf ^= 1) {
+    // two bits per round: the largest of three candidates that at least k keys reach (the last round of an odd number of
+    // bits has one)
+    const int low = max(bit - 1, 0);
+    const unsigned step = 1u << low;
+    unsigned c12 = 0u, c3 = 0u;                              // keys >= thr + step, >= thr + 2 step (upper half), >= thr + 3 step
 #pragma unroll
-    for (int j = 0; j < PER; ++j) c += key[j] >= cand;       // positions beyond n hold key 0 < cand
-    c = __reduce_add_sync(0xffffffffu, c);
-    if (lane == 0) slots.v[buf][warp] = c;
+    for (int j = 0; j < PER; ++j) {                          // positions beyond n hold key 0 < thr + step
+      c12 += (key[j] >= thr + step ? 1u : 0u) + (bit > 0 && key[j] >= thr + 2u * step ? 1u << 16 : 0u);
+      c3 += bit > 0 && key[j] >= thr + 3u * step;
+    }
+    c12 = __reduce_add_sync(0xffffffffu, c12);
+    c3 = __reduce_add_sync(0xffffffffu, c3);
+    if (lane == 0) { slots.v[buf][warp] = c12; slots2.v[buf][warp] = c3; }
     __syncthreads();
-    c = __reduce_add_sync(0xffffffffu, lane < nw ? slots.v[buf][lane] : 0u);
-    if (c >= (unsigned)k) { thr = cand; exact = c == (unsigned)k; }
+    c12 = __reduce_add_sync(0xffffffffu, lane < nw ? slots.v[buf][lane] : 0u);
+    c3 = __reduce_add_sync(0xffffffffu, lane < nw ? slots2.v[buf][lane] : 0u);
+    const unsigned c1 = c12 & 0xffffu, c2 = c12 >> 16;
+    const unsigned take = c3 >= (unsigned)k ? 3u : c2 >= (unsigned)k ? 2u : c1 >= (unsigned)k ? 1u : 0u;
+    if (take) { thr += take * step; exact = (take == 3u ? c3 : take == 2u ? c2 : c1) == (unsigned)k; }
   }
   // ordered emission: counts per (j, warp), which is position order, then one scan
   unsigned mg[PER], me[PER];
