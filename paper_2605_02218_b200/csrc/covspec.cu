@@ -111,16 +111,17 @@ struct covspec_ctx {
   unsigned* sync = nullptr;              // per-request counters of the fused subspace kernel + abort word
   float* Cg = nullptr;                   // factor columns of the greedy low-rank mode
   long long cg_cap = 0;
-  CUtensorMap map_zg, map_zgw, map_gh, map_gl, map_y[2][2];
+  CUtensorMap map_gh, map_gl, map_y[2][2];
+  CUtensorMap map_gram_col[4];           // column operand of the Gram kernel: boxes of 256, 128, 64 and 32 rows
   // float32 inputs on the tensor cores: operands split into bf16 rows three times as wide
   // (split3_kernel); nullptr / 0 when the configuration does not take that route
   bool split_tc = false;
   int dp = 0, d3 = 0;                    // d rounded up to 64; 3 * dp
   __nv_bfloat16 *X3 = nullptr, *Q3 = nullptr, *Wq3 = nullptr, *Wk3 = nullptr, *Za3 = nullptr, *Zb3 = nullptr;
-  CUtensorMap map_za3, map_zb3w, map_zb3;
+  CUtensorMap map_za3;
   // pinned staging for the plan upload
   char* h_stage = nullptr;
-  long long stage_bytes = 0, stage_sched_off = 0;
+  long long stage_bytes = 0, stage_tiles_off = 0;
   cudaEvent_t stage_free = nullptr;      // the previous upload has been consumed
   // the fused call streams the snapshot stack (Eq. 11) beside the relevance kernel on this stream
   cudaStream_t side = nullptr;
@@ -442,20 +443,42 @@ int get_plan(covspec_ctx* ctx, const covspec_problem* p, cudaStream_t stream) {
 
 // Launch that may overlap the end of the kernel before it on the stream; the kernel calls
 // wait_for_previous_kernel (common.cuh) before it uses anything of that kernel's.  About 2 us less between two
-// short kernels.
+// short kernels.  cluster > 1: CTAs per cluster (kernels without a size of their own).
 template <typename... P, typename... A>
-cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args) {
+cudaError_t launch_clusters(int cluster, bool dependent, void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                            A... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute attr[2]{};
+  cfg.attrs = attr;
+  if (dependent) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs].val.clusterDim.x = (unsigned)cluster;
+    attr[cfg.numAttrs].val.clusterDim.y = attr[cfg.numAttrs].val.clusterDim.z = 1;
+    ++cfg.numAttrs;
+  }
   return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args) {
+  return launch_clusters(1, true, kernel, grid, threads, smem, s, args...);
+}
+
+// Gram matrices of the stage-2 requests: `row` is the map of the row operand.  2 or 4 CTAs per item while that leaves every
+// CTA a single one.
+cudaError_t launch_gram(const covspec_ctx* ctx, const CUtensorMap& row, sub::GramParams gp, cudaStream_t s) {
+  const int shift = 4 * gp.n_items <= ctx->num_sms ? 2 : 2 * gp.n_items <= ctx->num_sms ? 1 : 0;
+  gp.split = 1 << shift;
+  const int grid = shift ? gp.n_items * gp.split : std::min(gp.n_items, ctx->num_sms);
+  return launch_dependent(sub::gram_tc_kernel, dim3((unsigned)grid), 192, sub::kGramSmem, s, row, ctx->map_gram_col[shift],
+                          ctx->map_gram_col[shift + 1], gp);
 }
 
 // Records the begin (edge 0) or end (edge 1) event of a stage for the current profiled call.
@@ -874,8 +897,7 @@ int select_impl(covspec_ctx* ctx, const covspec_problem* p, const float* s_fused
       gp.plan = ctx->d_plan; gp.batch = B; gp.n_items = pl.n_gram_tiles;
       gp.k_chunks = ctx->d3 / sub::kBK;
       gp.g_hi = ctx->Ghi; gp.g_lo = ctx->Glo; gp.ld = ctx->ld; gp.status = ctx->status;
-      int grid_g = std::min(pl.n_gram_tiles, ctx->num_sms);
-      CUDA_TRY(launch_dependent(sub::gram_tc_kernel, dim3(grid_g), 192, sub::kGramSmem, s, ctx->map_za3, ctx->map_zb3w, ctx->map_zb3, gp));
+      CUDA_TRY(launch_gram(ctx, ctx->map_za3, gp, s));
       LAUNCH_CHECK(ctx);
       prof_mark(ctx, ST_GRAM, 1, s);
     } else {
@@ -890,8 +912,7 @@ int select_impl(covspec_ctx* ctx, const covspec_problem* p, const float* s_fused
       gp.k_chunks = (cfg.d + sub::kBK - 1) / sub::kBK;
       gp.same = 1;
       gp.g_hi = ctx->Ghi; gp.g_lo = ctx->Glo; gp.ld = ctx->ld; gp.status = ctx->status;
-      int grid = std::min(pl.n_gram_tiles, ctx->num_sms);
-      CUDA_TRY(launch_dependent(sub::gram_tc_kernel, dim3(grid), 192, sub::kGramSmem, s, ctx->map_zg, ctx->map_zgw, ctx->map_zg, gp));
+      CUDA_TRY(launch_gram(ctx, ctx->map_gram_col[1], gp, s));
       LAUNCH_CHECK(ctx);
     } else {
       if ((st = launch_table<T, T, float, float, false>(ctx, T_GRAM_G, 1, s))) return st;
@@ -1184,11 +1205,10 @@ int covspec_prune_init(const covspec_config* cfg, covspec_ctx** out) {
   if (ok) {
     // tensor maps over the workspace arrays of the subspace iteration (fixed for the context)
     int st = COVSPEC_OK;
-    if (!f32) st = make_map_bf16(&ctx->map_zg, ctx->Zg, c.max_total_presel, c.d, sub::kTile);
-    if (!f32 && !st) st = make_map_bf16(&ctx->map_zgw, ctx->Zg, c.max_total_presel, c.d, sub::kGramN);
+    if (!f32 || ctx->split_tc)
+      for (int i = 0; i < 4 && !st; ++i)
+        st = make_map_bf16(&ctx->map_gram_col[i], f32 ? ctx->Zb3 : ctx->Zg, c.max_total_presel, f32 ? ctx->d3 : c.d, sub::kGramN >> i);
     if (ctx->split_tc && !st) st = make_map_bf16(&ctx->map_za3, ctx->Za3, c.max_total_presel, ctx->d3, sub::kTile);
-    if (ctx->split_tc && !st) st = make_map_bf16(&ctx->map_zb3, ctx->Zb3, c.max_total_presel, ctx->d3, sub::kTile);
-    if (ctx->split_tc && !st) st = make_map_bf16(&ctx->map_zb3w, ctx->Zb3, c.max_total_presel, ctx->d3, sub::kGramN);
     if (!st) st = make_map_bf16(&ctx->map_gh, ctx->Ghi, ctx->cap_rows, ctx->ld, sub::kTile);
     if (!st) st = make_map_bf16(&ctx->map_gl, ctx->Glo, ctx->cap_rows, ctx->ld, sub::kTile);
     for (int i = 0; i < 2 && !st; ++i)

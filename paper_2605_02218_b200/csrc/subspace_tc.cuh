@@ -101,13 +101,18 @@ struct GramParams {
   __nv_bfloat16* g_lo;
   int ld;
   int same;             // 1: the row and the column operand are the same rows
+  int split;            // CTAs that share an item's columns (1, 2 or 4; more than 1: one item per CTA)
   int* status;
 };
+// Shared memory bounds the main loop: a chunk is written once and its operands are read once per product, 128 bytes a cycle.
+// Where a call has few items, 2 or 4 CTAs take the columns of one between them, each with the whole row tile: 64 and 48
+// KB of traffic per chunk instead of 96 (a 128 x 256 block), so that the chain of chunks is the shorter.  Every element is
+// still summed by one accumulator in the order of the inner dimension.
 
 __global__ void __launch_bounds__(192, 1)
 gram_tc_kernel(const __grid_constant__ CUtensorMap map_z,   // row operand [sum M_b, d] bf16, 128-row boxes
-               const __grid_constant__ CUtensorMap map_zw,  // column operand, 256-row boxes
-               const __grid_constant__ CUtensorMap map_zd,  // column operand, 128-row boxes
+               const __grid_constant__ CUtensorMap map_zw,  // column operand, boxes of 256 / split rows
+               const __grid_constant__ CUtensorMap map_zd,  // column operand, boxes of 128 / split rows
                const GramParams prm) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -134,6 +139,8 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_z,   // row operand [sum 
   const uint32_t tmem_base = *tmem_slot;
   wait_for_previous_kernel();
 
+  const int first_item = blockIdx.x / prm.split, stride = gridDim.x / prm.split, sub = blockIdx.x % prm.split;
+  const int same = prm.split == 1 ? prm.same : 0;          // part of the columns holds no whole row tile
   auto decode = [&](int item, ReqPlan& rp, int& ti, int& tjp) {
     int b = find_request(item, prm.batch, [&](int q) { return prm.plan[q].gram_tile_off; });
     rp = prm.plan[b];
@@ -144,12 +151,13 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_z,   // row operand [sum 
     if (lane == 0) {
       uint32_t it = 0;
       bool ok = true;
-      for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x) {
+      for (int item = first_item; item < prm.n_items && ok; item += stride) {
         ReqPlan rp; int ti, tj;
         decode(item, rp, ti, tj);
         // a chunk: row tile, then the pair of column tiles (its first one only where ti = 2 tj)
-        const bool first = ti == 2 * tj, load_a = !prm.same || !(first || ti == 2 * tj + 1);
-        const int bytes = (load_a ? kGramBytesA : 0) + (first ? kGramBytesA : 2 * kGramBytesA);
+        const bool first = ti == 2 * tj, load_a = !same || !(first || ti == 2 * tj + 1);
+        const int width = (first ? kTile : kGramN) / prm.split, col_row = rp.presel_off + tj * kGramN + sub * width;
+        const int bytes = (load_a ? kGramBytesA : 0) + width * kBK * 2;
         for (int kc = 0; kc < prm.k_chunks; kc += kGramChunks, ++it) {
           const int s = it % kGramStages, chunks = min(kGramChunks, prm.k_chunks - kc);
           if (!(ok = mbar_wait(&empty[s], ((it / kGramStages) & 1u) ^ 1u, abort_flag))) break;
@@ -157,7 +165,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_z,   // row operand [sum 
           uint32_t dst = smem_u32(smem + s * kGramStageBytes);
           for (int c = 0; c < chunks; ++c, dst += kGramChunkBytes) {
             if (load_a) tma_load_2d(dst, &map_z, (kc + c) * kBK, rp.presel_off + ti * kTile, &full[s]);
-            tma_load_2d(dst + kGramBytesA, first ? &map_zd : &map_zw, (kc + c) * kBK, rp.presel_off + tj * kGramN, &full[s]);
+            tma_load_2d(dst + kGramBytesA, first ? &map_zd : &map_zw, (kc + c) * kBK, col_row, &full[s]);
           }
         }
       }
@@ -167,12 +175,12 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_z,   // row operand [sum 
     if (lane == 0) {
       uint32_t it = 0, n = 0;
       bool ok = true;
-      for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x, ++n) {
+      for (int item = first_item; item < prm.n_items && ok; item += stride, ++n) {
         ReqPlan rp; int ti, tj;
         decode(item, rp, ti, tj);
-        const uint32_t idesc = umma_idesc(kTile, ti == 2 * tj ? kTile : kGramN);
+        const uint32_t idesc = umma_idesc(kTile, (ti == 2 * tj ? kTile : kGramN) / prm.split);
         // where the row tile lies (see the producer)
-        const int a_off = !prm.same ? 0 : ti == 2 * tj ? kGramBytesA : ti == 2 * tj + 1 ? 2 * kGramBytesA : 0;
+        const int a_off = !same ? 0 : ti == 2 * tj ? kGramBytesA : ti == 2 * tj + 1 ? 2 * kGramBytesA : 0;
         int buf = n & 1;
         if (!(ok = mbar_wait(&acc_empty[buf], ((n >> 1) & 1u) ^ 1u, abort_flag))) break;
         tc_fence_after();
@@ -201,7 +209,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_z,   // row operand [sum 
     const uint32_t t_lane = tmem_base + ((uint32_t)(warp * 32) << 16);
     uint32_t n = 0, rounds = 0;
     bool ok = true;
-    for (int item = blockIdx.x; item < prm.n_items; item += gridDim.x, ++n) {
+    for (int item = first_item; item < prm.n_items; item += stride, ++n) {
       ReqPlan rp; int ti, tj;
       decode(item, rp, ti, tj);
       int buf = n & 1;
@@ -210,12 +218,12 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap map_z,   // row operand [sum 
       const int row = ti * kTile + r;                 // row of G inside the request
       const bool row_ok = row < rp.m;
       const size_t ld = (size_t)prm.ld;
+      const int groups = (ti == 2 * tj ? kTile : kGramN) / 32 / prm.split, first_group = sub * groups;
 #pragma unroll 1
-      for (int c4 = 0; c4 < 8; ++c4) {
+      for (int c4 = first_group; c4 < first_group + groups; ++c4) {
         const int tc = 2 * tj + (c4 >> 2);            // column tile of this group of 32 columns
-        if (tc > ti) break;                           // above the diagonal: dropped
         float v[32];
-        tmem_ld32(t_lane + buf * kGramN + c4 * 32, v);
+        tmem_ld32(t_lane + buf * kGramN + (c4 - first_group) * 32, v);
         const int col0 = tj * kGramN + c4 * 32;
         // entries outside the request's M x M block are stored as zeros: the power step multiplies
         // whole 64-wide k-chunks and must not meet stale non-finite values in the padding
