@@ -72,6 +72,7 @@ struct Plan {
   int tile_rows = 128;                        // rows of a subspace-block tile: 64 when that still gives every tile a CTA
   int tile_ctas = 0, servers = 0;             // CTAs of the subspace kernel that carry tiles / that only factor
   int pow_grid = 0;                           // CTAs of the power step
+  std::vector<int4> tile_list;                // 128-token tiles: first row of X, rows, first query row, query elements
   std::vector<int> sched;                     // [pow_grid + 1] offsets + item lists (longest first) + places (see FusedParams)
   bool one_request_ctas = false;              // no CTA of the subspace kernel carries tiles of two requests
   long long total_vis = 0, total_txt = 0, total_keep = 0, total_presel = 0;
@@ -89,7 +90,8 @@ struct covspec_ctx {
   // carved regions
   int* status = nullptr;
   ReqPlan* d_plan = nullptr;
-  int* d_sched = nullptr;                // power-step schedule: [grid + 1] offsets + item lists
+  int4* d_tiles = nullptr;               // the plan's 128-token tiles (see VisParams), then the power-step schedule:
+                                         // [grid + 1] offsets + item lists
   GemmProb* d_tables = nullptr;          // [T_COUNT][max_batch]
   float* Qn = nullptr;
   float* Kp = nullptr;
@@ -216,6 +218,7 @@ int get_plan(covspec_ctx* ctx, const covspec_problem* p, cudaStream_t stream) {
   pl.keep_ratio = p->keep_ratio;
   pl.req.assign(B, ReqPlan{});
   pl.keep_offsets.assign(B + 1, 0);
+  pl.tile_list.clear();
   pl.presel_offsets.assign(B + 1, 0);
   pl.n_stage2 = 0; pl.t_max = 0; pl.p_max = 0; pl.m_max = 0; pl.n_tiles = 0; pl.n_pairs = 0;
   pl.n_gram_tiles = 0; pl.n_ptiles = 0;
@@ -233,6 +236,8 @@ int get_plan(covspec_ctx* ctx, const covspec_problem* p, cudaStream_t stream) {
     r.p = 0;
     r.ldm = (int)round_up(r.m, 4);
     r.tile_off = pl.n_tiles;
+    for (int i = 0; i < r.n; i += tc::kTileM)
+      pl.tile_list.push_back(make_int4(r.vis_off + i, std::min(tc::kTileM, r.n - i), r.txt_off, r.t));
     pl.n_tiles += (r.n + tc::kTileM - 1) / tc::kTileM;
     r.pair_off = pl.n_pairs;
     pl.n_pairs += ((r.n + tc::kTileM - 1) / tc::kTileM + 1) / 2;
@@ -425,10 +430,12 @@ int get_plan(covspec_ctx* ctx, const covspec_problem* p, cudaStream_t stream) {
   if (s2 > 0)
     CUDA_TRY(cudaMemcpyAsync(ctx->d_tables, h_tab, sizeof(GemmProb) * (size_t)T_COUNT * mb,
                              cudaMemcpyHostToDevice, stream));
-  if (pl.n_ptiles > 0) {
-    int* h_sched = reinterpret_cast<int*>(ctx->h_stage + ctx->stage_sched_off);
-    memcpy(h_sched, pl.sched.data(), sizeof(int) * pl.sched.size());
-    CUDA_TRY(cudaMemcpyAsync(ctx->d_sched, h_sched, sizeof(int) * pl.sched.size(), cudaMemcpyHostToDevice, stream));
+  {
+    char* h_tiles = ctx->h_stage + ctx->stage_tiles_off;
+    const size_t tile_bytes = sizeof(int4) * pl.tile_list.size(), sched_bytes = pl.n_ptiles > 0 ? sizeof(int) * pl.sched.size() : 0;
+    memcpy(h_tiles, pl.tile_list.data(), tile_bytes);
+    memcpy(h_tiles + tile_bytes, pl.sched.data(), sched_bytes);
+    CUDA_TRY(cudaMemcpyAsync(ctx->d_tiles, h_tiles, tile_bytes + sched_bytes, cudaMemcpyHostToDevice, stream));
   }
   CUDA_TRY(cudaEventRecord(ctx->stage_free, stream));
   pl.valid = true;
@@ -672,15 +679,16 @@ int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cud
   long long lo_off = (long long)cfg.max_total_txt * P;   // lo parts follow the hi parts
   int st;
   if ((st = make_map_bf16(&map_x, X, pl.total_vis, d, tc::kTileM))) return st;
-  if ((st = make_map_bf16(&map_wk, Wk, P, d, tc::kTileN))) return st;
+  // Visual side: one head per item while the items with one head leave no cluster more than one.
+  const int n_pairs = (pl.n_tiles + 1) / 2, n_clusters = ctx->num_sms / 2;
+  const int vis_heads = cfg.n_heads == 1 || n_pairs * cfg.n_heads <= n_clusters ? 1 : 2;
+  const int query_rows = std::min(tc::kLogitN, (pl.t_max + 31) / 32 * 32) / 2;      // per CTA of a pair
+  if ((st = make_map_bf16(&map_wk, Wk, P, d, vis_heads * tc::kHeadDim / 2))) return st;
   if ((st = make_map_bf16(&map_q, Q, pl.total_txt, d, tc::kTileM))) return st;
   if ((st = make_map_bf16(&map_wq, Wq, P, d, group_heads * tc::kHeadDim))) return st;
-  if ((st = make_map_bf16(&map_qn, qn, pl.total_txt, P, tc::kTT))) return st;
-  if ((st = make_map_bf16(&map_qnl, qn + lo_off, pl.total_txt, P, tc::kTT))) return st;
-  int n_hp = (cfg.n_heads + 1) / 2;
+  if ((st = make_map_bf16(&map_qn, qn, pl.total_txt, P, query_rows))) return st;
+  if ((st = make_map_bf16(&map_qnl, qn + lo_off, pl.total_txt, P, query_rows))) return st;
   tc::Params prm{};
-  prm.plan = ctx->d_plan; prm.batch = p->batch;
-  prm.n_groups = n_hp;
   prm.n_heads = cfg.n_heads; prm.k_chunks = (d + tc::kBK - 1) / tc::kBK; prm.P = P;
   prm.status = ctx->status;
   // query side
@@ -689,19 +697,35 @@ int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cud
   prm.group_heads = group_heads;
   prm.n_groups = (cfg.n_heads + group_heads - 1) / group_heads;
   prm.n_items = q_tiles * prm.n_groups;
-  prm.qn_out = qn; prm.qn_lo_off = lo_off; prm.s_query = nullptr;
+  prm.qn_out = qn; prm.qn_lo_off = lo_off;
   prm.fill = s_query; prm.fill_n = pl.total_vis;          // -inf for the visual-side launch below
-  int grid = prm.n_items < ctx->num_sms ? prm.n_items : ctx->num_sms;
-  tc::query_embed_kernel<<<grid, 192, tc::kQuerySmem, s>>>(map_q, map_wq, prm);
+  // few items share their inner dimension among the CTAs of a cluster, as long as that leaves half the SMs
+  prm.split = 1;
+  if (group_heads == 1)
+    for (int sp = tc::kQuerySplitMax; sp > 1 && prm.split == 1; sp /= 2)
+      if (prm.n_items * sp <= ctx->num_sms / 2 && prm.k_chunks >= 4 * sp) prm.split = sp;
+  // In clusters of two where nothing is shared: they take both SMs of a pair, so that the other pairs are free for the visual
+  // side's clusters.
+  const int q_cluster = prm.split > 1 ? prm.split : 2;
+  int grid = prm.split > 1 ? prm.n_items * prm.split : 2 * std::min((prm.n_items + 1) / 2, n_clusters);
+  CUDA_TRY(launch_clusters(q_cluster, false, tc::query_embed_kernel, dim3(grid), 192, tc::kQuerySmem, s, map_q, map_wq, prm));
   LAUNCH_CHECK(ctx);
   prof_mark(ctx, ST_QEMBED, 1, s);
   // visual side
   prof_mark(ctx, ST_RELEVANCE, 0, s);
-  prm.n_groups = n_hp;
-  prm.n_items = pl.n_tiles * prm.n_groups;
-  prm.qn_out = nullptr; prm.s_query = s_query; prm.fill = nullptr;
-  grid = prm.n_items < ctx->num_sms ? prm.n_items : ctx->num_sms;
-  CUDA_TRY(launch_dependent(tc::relevance_vis_kernel, dim3(grid), tc::kVisThreads, tc::kVisSmem, s, map_x, map_wk, map_qn, map_qnl, prm));
+  tc::VisParams vis{};
+  vis.tiles = ctx->d_tiles; vis.n_tiles = pl.n_tiles;
+  vis.group_heads = vis_heads;
+  vis.n_groups = (cfg.n_heads + vis_heads - 1) / vis_heads;
+  vis.n_items = n_pairs * vis.n_groups;
+  vis.n_heads = cfg.n_heads; vis.k_chunks = prm.k_chunks;
+  vis.stages = std::min(tc::kVisMaxStages, (tc::kVisRing + (vis.n_items <= n_clusters ? 4 * tc::kBytesKp : 0)) /
+                                               (tc::kBytesA + vis_heads * tc::kVisHeadBytes));
+  vis.rows_total = (int)pl.total_vis;
+  vis.query_rows = query_rows;
+  vis.s_query = s_query; vis.status = ctx->status;
+  grid = 2 * std::min(vis.n_items, n_clusters);
+  CUDA_TRY(launch_dependent(tc::relevance_vis_kernel, dim3(grid), tc::kVisThreads, tc::kVisSmem, s, map_x, map_wk, map_qn, map_qnl, vis));
   LAUNCH_CHECK(ctx);
   prof_mark(ctx, ST_RELEVANCE, 1, s);
   return COVSPEC_OK;
@@ -937,7 +961,7 @@ int select_impl(covspec_ctx* ctx, const covspec_problem* p, const float* s_fused
     // every multiplication by G, the factorisations between them, the Rayleigh-Ritz solve and the
     // energies: one cooperative launch (its CTAs wait on one another through global counters)
     sub::FusedParams fp{};
-    fp.plan = ctx->d_plan; fp.batch = B; fp.n_items = pl.n_ptiles; fp.sched = ctx->d_sched;
+    fp.plan = ctx->d_plan; fp.batch = B; fp.n_items = pl.n_ptiles; fp.sched = reinterpret_cast<const int*>(ctx->d_tiles + pl.n_tiles);
     fp.tile_rows = pl.tile_rows;
     fp.spread_sum = pl.one_request_ctas ? 1 : 0;
     fp.n_tile_ctas = pl.tile_ctas; fp.n_servers = pl.servers;
@@ -1079,7 +1103,8 @@ int covspec_prune_init(const covspec_config* cfg, covspec_ctx** out) {
   long long o_plan = carve(sizeof(ReqPlan) * c.max_batch);
   long long o_tab = carve(sizeof(GemmProb) * (long long)T_COUNT * c.max_batch);
   long long sched_ints = 1024 + ctx->cap_ptiles;   // offsets and places of up to 511 CTAs + one entry per tile
-  long long o_sched = carve(4 * sched_ints);
+  const long long tiles_bytes = 16 * (c.max_total_vis / tc::kTileM + c.max_batch) + 4 * sched_ints;
+  long long o_tiles = carve(tiles_bytes);
   long long o_qn = carve(4ll * c.max_total_txt * ctx->P);
   long long o_kp = carve(4ll * ctx->kp_rows * ctx->P);
   long long o_sq = carve(4ll * c.max_total_vis), o_sa = carve(4ll * c.max_total_vis);
@@ -1123,7 +1148,7 @@ int covspec_prune_init(const covspec_config* cfg, covspec_ctx** out) {
   ctx->status = reinterpret_cast<int*>(w + o_status);
   ctx->d_plan = reinterpret_cast<ReqPlan*>(w + o_plan);
   ctx->d_tables = reinterpret_cast<GemmProb*>(w + o_tab);
-  ctx->d_sched = reinterpret_cast<int*>(w + o_sched);
+  ctx->d_tiles = reinterpret_cast<int4*>(w + o_tiles);
   ctx->Qn = reinterpret_cast<float*>(w + o_qn);
   ctx->Kp = reinterpret_cast<float*>(w + o_kp);
   ctx->sq = reinterpret_cast<float*>(w + o_sq);
@@ -1154,8 +1179,8 @@ int covspec_prune_init(const covspec_config* cfg, covspec_ctx** out) {
   ctx->Cg = reinterpret_cast<float*>(w + o_cg);
   ctx->stage_bytes = round_up(sizeof(ReqPlan) * c.max_batch, 256) +
                      sizeof(GemmProb) * (long long)T_COUNT * c.max_batch;
-  ctx->stage_sched_off = round_up(ctx->stage_bytes, 256);
-  ctx->stage_bytes = ctx->stage_sched_off + 4 * sched_ints;
+  ctx->stage_tiles_off = round_up(ctx->stage_bytes, 256);
+  ctx->stage_bytes = ctx->stage_tiles_off + tiles_bytes;
   bool ok = cudaMemset(ctx->status, 0, 256) == cudaSuccess &&
             cudaMallocHost(&ctx->h_stage, (size_t)ctx->stage_bytes) == cudaSuccess &&
             cudaEventCreateWithFlags(&ctx->stage_free, cudaEventDisableTiming) == cudaSuccess &&

@@ -25,11 +25,16 @@ constexpr int kBytesB = kTileN * kBK * 2;          // 32 KB
 constexpr int kBytesStage = kBytesA + kBytesB;
 constexpr int kBytesKp = kTileM * kHalf * 2;       // 16 KB: [128 x 64] of one half head; hi and lo
 constexpr int kTmemCols = 512;
-constexpr int kQueryStages = 4;
+constexpr int kQueryStages = 4;        // of two heads (48 KB); six of one
+constexpr int kQueryMaxStages = kQueryStages * kBytesStage / (kBytesA + kHeadDim * kBK * 2);
 // As much shared memory as the visual side takes, although 193 KB would do: with more room the blocks of the
 // activity stream gather on few SMs, and the visual side's CTAs do not fit there until the stream has ended.
 constexpr int kQuerySmem = 225 * 1024;
 static_assert(kQueryStages * kBytesStage + 1024 <= kQuerySmem, "ring and barriers");
+// An item's first CTA receives the other CTAs' sums in its ring: [CTA - 1][group of 32 features][8 vectors of 4][128 rows].
+constexpr int kQuerySplitMax = 4;
+constexpr int kQueryPartBytes = kTileM * 32 * 4;
+static_assert((kQuerySplitMax - 1) * (kHeadDim / 32) * kQueryPartBytes <= kQueryStages * kBytesStage, "partial sums in the ring");
 
 struct Params {
   const ReqPlan* plan;
@@ -37,6 +42,8 @@ struct Params {
   int n_items;          // (tile, pair of heads) pairs
   int n_groups;         // pairs of heads (query side: groups of group_heads)
   int group_heads;      // query side: heads per item, 2 or 1
+  int split;            // query side: CTAs (one cluster) that share an item's inner dimension; more than 1: one item of
+                        // one head per cluster
   int n_heads;
   int k_chunks;         // ceil(d / 64)
   int P;                // n_heads * 128
@@ -60,16 +67,16 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
     return;
   }
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kQueryStages * kBytesStage);
-  uint64_t* full = bars;                     // [kQueryStages]
-  uint64_t* empty = bars + kQueryStages;     // [kQueryStages]
-  uint64_t* acc_full = bars + 2 * kQueryStages;   // [2]
+  uint64_t* full = bars;                     // [kQueryMaxStages]
+  uint64_t* empty = full + kQueryMaxStages;  // [kQueryMaxStages]
+  uint64_t* acc_full = empty + kQueryMaxStages;   // [2]
   uint64_t* acc_empty = acc_full + 2;             // [2]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 4);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = warp_index(), lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kQueryStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+    for (int s = 0; s < kQueryMaxStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 128); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -89,18 +96,62 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
       prm.fill[i] = -INFINITY;
   }
 
+  // Epilogue of one head: unit-length bf16 slices (hi and lo) of the tile's projected query elements; load gives 32
+  // features of the thread's row.
+  const int r = (warp & 3) * 32 + lane;                    // row inside the tile = TMEM lane
+  const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+  auto store_head = [&](int row0, int nrows, int head, auto&& load) {
+    float ss = 0.f;
+#pragma unroll 1
+    for (int c4 = 0; c4 < 4; ++c4) {
+      float v[32];
+      load(c4, v);
+#pragma unroll
+      for (int e = 0; e < 32; ++e) ss += v[e] * v[e];
+    }
+    float inv = 0.f;
+    if (ss > 1.17549435e-38f) { inv = rsqrtf(ss); inv = inv * (1.5f - 0.5f * ss * inv * inv); }
+    if (!(ss <= 3.402823466e38f)) inv = __int_as_float(0x7fc00000);
+#pragma unroll 1
+    for (int c4 = 0; c4 < 4; ++c4) {
+      float v[32];
+      load(c4, v);
+      if (r < nrows) {
+        __nv_bfloat16* dst = prm.qn_out + (size_t)(row0 + r) * prm.P + (size_t)head * kHeadDim + c4 * 32;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          uint32_t ph[4], pw[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            float a = v[8 * q + 2 * e] * inv, b = v[8 * q + 2 * e + 1] * inv;
+            __nv_bfloat162 hi = __floats2bfloat162_rn(a, b);
+            ph[e] = *reinterpret_cast<uint32_t*>(&hi);
+            pw[e] = pack_bf16(a - __low2float(hi), b - __high2float(hi));
+          }
+          *reinterpret_cast<uint4*>(dst + q * 8) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
+          *reinterpret_cast<uint4*>(dst + prm.qn_lo_off + q * 8) = make_uint4(pw[0], pw[1], pw[2], pw[3]);
+        }
+      }
+    }
+  };
+
+  const int first_item = blockIdx.x / prm.split, stride = gridDim.x / prm.split, part = blockIdx.x % prm.split;
+  const int stage_bytes = kBytesA + prm.group_heads * kHeadDim * kBK * 2, stages = kQueryStages * kBytesStage / stage_bytes;
+  const int per = (prm.k_chunks + prm.split - 1) / prm.split;
+  const int kc0 = part * per, kc1 = min(prm.k_chunks, kc0 + per);
+
   if (warp == 4) {
     // ---------------------------------------------------------------- TMA producer
     if (lane == 0) {
       uint32_t it = 0;
       bool ok = true;
-      for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x) {
+      for (int item = first_item; item < prm.n_items && ok; item += stride) {
         const int row0 = item / prm.n_groups * kTileM, head0 = item % prm.n_groups * prm.group_heads;
-        for (int kc = 0; kc < prm.k_chunks; ++kc, ++it) {
-          const int s = it % kQueryStages;
-          if (!(ok = mbar_wait(&empty[s], ((it / kQueryStages) & 1u) ^ 1u, abort_flag))) break;
-          mbar_expect_tx(&full[s], kBytesA + prm.group_heads * kHeadDim * kBK * 2);
-          const uint32_t dst = smem_u32(smem + s * kBytesStage);
+        for (int kc = kc0; kc < kc1; ++kc, ++it) {
+          const int s = it % stages;
+          if (!(ok = mbar_wait(&empty[s], ((it / stages) & 1u) ^ 1u, abort_flag))) break;
+          mbar_expect_tx(&full[s], stage_bytes);
+          const uint32_t dst = smem_u32(smem + s * stage_bytes);
           tma_load_2d(dst, &map_a, kc * kBK, row0, &full[s]);
           tma_load_2d(dst + kBytesA, &map_b, kc * kBK, head0 * kHeadDim, &full[s]);
         }
@@ -112,82 +163,82 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
     if (lane == 0) {
       uint32_t it = 0, n = 0;
       bool ok = true;
-      for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x, ++n) {
+      for (int item = first_item; item < prm.n_items && ok; item += stride, ++n) {
         const uint32_t buf = n & 1u;
         if (!(ok = mbar_wait(&acc_empty[buf], ((n >> 1) & 1u) ^ 1u, abort_flag))) break;
         tc_fence_after();
         // a lone last head takes half the columns (see relevance_vis_kernel)
         const int head0 = item % prm.n_groups * prm.group_heads;
         const uint32_t idesc = umma_idesc(kTileM, min(prm.group_heads, prm.n_heads - head0) * kHeadDim);
-        for (int kc = 0; kc < prm.k_chunks; ++kc, ++it) {
-          const int s = it % kQueryStages;
-          if (!(ok = mbar_wait(&full[s], (it / kQueryStages) & 1u, abort_flag))) break;
+        for (int kc = kc0; kc < kc1; ++kc, ++it) {
+          const int s = it % stages;
+          if (!(ok = mbar_wait(&full[s], (it / stages) & 1u, abort_flag))) break;
           tc_fence_after();
-          const uint32_t addr = smem_u32(smem + s * kBytesStage);
+          const uint32_t addr = smem_u32(smem + s * stage_bytes);
           const uint64_t adesc = umma_desc(addr), bdesc = umma_desc(addr + kBytesA);
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k)
-            umma_bf16(tmem_base + buf * kTileN, adesc + 2 * k, bdesc + 2 * k, idesc, (kc | k) != 0);
+            umma_bf16(tmem_base + buf * kTileN, adesc + 2 * k, bdesc + 2 * k, idesc, (kc - kc0) | k);
           umma_commit(&empty[s]);
         }
         if (ok) umma_commit(&acc_full[buf]);
       }
     }
     __syncwarp();
-  } else {
+  } else if (prm.split == 1) {
     // ---------------------------------------------------------------- epilogue (warps 0-3)
-    const int r = warp * 32 + lane;                        // row inside the tile = TMEM lane
     uint32_t n = 0;
     bool ok = true;
-    for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x, ++n) {
+    for (int item = first_item; item < prm.n_items && ok; item += stride, ++n) {
       const int row0 = item / prm.n_groups * kTileM, head0 = item % prm.n_groups * prm.group_heads;
       const long long rem = prm.rows_total - row0;
-      const int nrows = rem < kTileM ? (int)rem : kTileM;
       const uint32_t buf = n & 1u;
       if (!(ok = mbar_wait(&acc_full[buf], (n >> 1) & 1u, abort_flag))) break;
       tc_fence_after();
-      const uint32_t t_lane = tmem_base + ((uint32_t)(warp * 32) << 16) + buf * kTileN;
       const int heads = min(prm.group_heads, prm.n_heads - head0);
-      for (int h = 0; h < heads; ++h) {
-        // unit-length bf16 head slice of the projected query element to global memory
-        float ss = 0.f;
-#pragma unroll 1
-        for (int c4 = 0; c4 < 4; ++c4) {
-          float v[32];
-          tmem_ld32(t_lane + h * kHeadDim + c4 * 32, v);
-#pragma unroll
-          for (int e = 0; e < 32; ++e) ss += v[e] * v[e];
-        }
-        float inv = 0.f;
-        if (ss > 1.17549435e-38f) { inv = rsqrtf(ss); inv = inv * (1.5f - 0.5f * ss * inv * inv); }
-        if (!(ss <= 3.402823466e38f)) inv = __int_as_float(0x7fc00000);
-#pragma unroll 1
-        for (int c4 = 0; c4 < 4; ++c4) {
-          float v[32];
-          tmem_ld32(t_lane + h * kHeadDim + c4 * 32, v);
-          if (r < nrows) {
-            __nv_bfloat16* dst = prm.qn_out + (size_t)(row0 + r) * prm.P +
-                                 (size_t)(head0 + h) * kHeadDim + c4 * 32;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              uint32_t ph[4], pw[4];
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                float a = v[8 * q + 2 * e] * inv, b = v[8 * q + 2 * e + 1] * inv;
-                __nv_bfloat162 hi = __floats2bfloat162_rn(a, b);
-                ph[e] = *reinterpret_cast<uint32_t*>(&hi);
-                pw[e] = pack_bf16(a - __low2float(hi), b - __high2float(hi));
-              }
-              *reinterpret_cast<uint4*>(dst + q * 8) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
-              *reinterpret_cast<uint4*>(dst + prm.qn_lo_off + q * 8) =
-                  make_uint4(pw[0], pw[1], pw[2], pw[3]);
-            }
-          }
-        }
-      }
+      for (int h = 0; h < heads; ++h)
+        store_head(row0, rem < kTileM ? (int)rem : kTileM, head0 + h,
+                   [&](int c4, float (&v)[32]) { tmem_ld32(t_lane + buf * kTileN + h * kHeadDim + c4 * 32, v); });
       tc_fence_before();
       mbar_arrive(&acc_empty[buf]);
     }
+  } else {
+    if (!mbar_wait(&acc_full[0], 0, abort_flag)) atomicOr(prm.status, kStatusTimeout);
+    tc_fence_after();
+  }
+  if (prm.split > 1) {
+    // every CTA's products are complete and its ring is idle: the other CTAs push their sums to the first one, which adds
+    // them up in the order of the inner dimension
+    const int row0 = first_item / prm.n_groups * kTileM, head = first_item % prm.n_groups;
+    const long long rem = prm.rows_total - row0;
+    const int nrows = rem < kTileM ? (int)rem : kTileM;
+    const bool work = warp < 4 && warp * 32 < nrows;         // whole warps
+    __syncwarp();
+    cluster_sync_all();
+    if (work && part != 0) {
+#pragma unroll 1
+      for (int c4 = 0; c4 < kHeadDim / 32; ++c4) {
+        float v[32];
+        tmem_ld32(t_lane + c4 * 32, v);
+        const uint32_t dst = map_to_cta(smem + ((part - 1) * (kHeadDim / 32) + c4) * kQueryPartBytes + r * 16, 0);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) store_at(dst + q * kTileM * 16, v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      }
+    }
+    __syncwarp();
+    cluster_sync_all();
+    if (work && part == 0 && *abort_flag == 0)
+      store_head(row0, nrows, head, [&](int c4, float (&v)[32]) {
+        tmem_ld32(t_lane + c4 * 32, v);
+        for (int c = 1; c < prm.split; ++c) {
+          const float4* src = reinterpret_cast<const float4*>(smem + ((c - 1) * (kHeadDim / 32) + c4) * kQueryPartBytes) + r;
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const float4 w = src[q * kTileM];
+            v[4 * q] += w.x; v[4 * q + 1] += w.y; v[4 * q + 2] += w.z; v[4 * q + 3] += w.w;
+          }
+        }
+      });
   }
 
   tc_fence_before();

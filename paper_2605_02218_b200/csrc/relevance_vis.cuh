@@ -1,240 +1,393 @@
 // The visual side of the query-aware score (Eq. 10) with per-head linear embeddings, bf16 operands.
 //
-// Per work item (one 128-token tile of one request, one pair of heads) the kernel computes
-//   Kp = X_tile * Wk[heads]^T           tcgen05.mma kind::f16, 128 x 256 accumulator in TMEM, operands
-//                                       streamed by TMA through a shared-memory ring
+// A cluster of two CTAs owns a pair of neighbouring 128-token tiles and multiplies with
+// tcgen05.mma.cta_group::2 (M = 256 across the pair).  Per work item (one pair of tiles, one group of one or two
+// heads) it computes
+//   Kp = X_tile * Wk[heads]^T           256 x 256 over the pair, 256 accumulator columns in each SM's TMEM
 //   per token and head: ||Kp||^2        epilogue warps read TMEM, keep the norm in float32 and restage the
 //                                       head as bf16 hi + lo K-major tiles in shared memory
-//   logits = Kp * Qn[head]^T            second product against the unit-length query elements, 64 of them at a
-//                                       time, as hi*hi + lo*hi + hi*lo so that bf16 staging costs ~2^-16
+//   logits = Kp * Qn[head]^T            second product against the unit-length query elements, up to 128 of them
+//                                       at a time, as hi*hi + lo*hi + hi*lo so that bf16 staging costs ~2^-16
 //   S^query = max_j,h logits / ||Kp||   row max in registers, atomic max into the score array
 // so the projected embeddings never leave the SM.
+//
+// Why two SMs: a CTA fetches its own tokens and only its half of the weights, 32 KB per 64 features and 512 tensor
+// cycles.  One SM alone needs 48 KB for its 128 x 256 products, 96 bytes a cycle, and an SM gets about 64 from L2:
+// its main loop ran at two thirds of the tensor rate.  The query elements are shared the same way.
 //
 // The second product and the epilogue of one item run beside the main loop of the next: TMEM holds two
 // accumulators of 256 columns, and the logits of a head take the place of that head's own columns, which have
 // been read by then.  The main loop, the logits and their operands have issuing threads of their own, so
-// nothing interleaves them but the tensor pipe.  With one accumulator the pipe waited for the restaging,
-// the query tiles and the small products of every item: 18 % of the launch at d = 3584 with 64 query
-// elements, 24 % at d = 4096 with 128 and 57 % at d = 1536 with 16-256.
+// nothing interleaves them but the tensor pipe; a head is restaged while the logits of the one before are read.
+// The tiles of a pair may belong to two requests (tiles are paired across the whole batch): such a pair goes
+// through the query elements of both, and each CTA looks at its own request's logits.
 //
-// Warp roles (256 threads): 0-3 epilogue (one TMEM lane = one token each), 4 TMA producer of the main ring,
-// 5 MMA issuer of the main loop and TMEM owner, 6 MMA issuer of the logits, 7 TMA producer of the query
-// tiles.  Every mbarrier wait is bounded; on expiry the CTA raises a status bit, leaves its loops, frees
-// TMEM and exits.
+// Warp roles per CTA (384 threads): 0-7 epilogue (a TMEM lane = a token; warps w and w + 4 share 32 tokens, each
+// taking half of the columns), 8 TMA producer of the main ring, 9 TMEM owner and, in the leader CTA, MMA issuer of
+// the main loop, 10 (leader) MMA issuer of the logits, 11 TMA producer of the query blocks.  Loads are plain
+// per-CTA tile loads whose bytes are counted on the leader's barriers; tcgen05.commit signals the barriers of both
+// CTAs; barriers that the issuers wait on live in the leader.  Every wait is bounded; on expiry the CTA raises
+// a status bit and stops working, and both CTAs meet at a cluster barrier before they exit.
 #pragma once
 #include "relevance_tc.cuh"
 
 namespace covspec {
 namespace tc {
 
-// Shared memory: three ring stages (a fourth bought nothing), one restaged head (hi and lo, two halves of 64
-// features each), a ring of two query blocks [64 elements x 64 features] (hi and lo blocks alternate).
-constexpr int kVisStages = 3;
-constexpr int kVisThreads = 256;
-constexpr int kQueryBlock = kTT * kHalf * 2;              // 8 KB
-constexpr int kVisSmem = kVisStages * kBytesStage + 4 * kBytesKp + 2 * kQueryBlock + 1024 /*barriers*/;
-static_assert(kVisSmem == kQuerySmem, "see kQuerySmem");
-constexpr int kLogitTiles = kHeadDim / kTT;               // logits tiles in the columns of one head
+// Shared memory: the ring of the main loop (four stages of two heads, five of one), one restaged head (hi and lo, two
+// halves of 64 features each), a ring of query
+// blocks [kq query elements x 64 features] (hi and lo blocks alternate; kq is half of the widest logits tile of
+// the call), barriers, the exchange between the two threads of a token.
+// A cluster with a single item restages its heads when the main loop is over: its ring takes their place as well (six
+// stages of two heads, eight of one).  With few items the main loop is bound by the time a stage takes to come round.
+constexpr int kVisRing = 128 * 1024;
+constexpr int kVisMaxStages = 8;
+constexpr int kVisThreads = 384;
+constexpr int kVisEpiWarps = 8;
+constexpr int kVisHeadBytes = kHeadDim / 2 * kBK * 2;      // 8 KB: this CTA's half of a head's weight chunk
+constexpr int kLogitN = 128;                              // query elements per logits tile (UMMA N of the 2nd product)
+constexpr int kQueryRing = 28 * 1024;
+constexpr int kMaxQuerySlots = 8;
+constexpr int kVisSmem = kVisRing + 4 * kBytesKp + kQueryRing + 1024 /*barriers*/ + 2048 /*exchange*/;
+static_assert(kVisSmem <= kQuerySmem, "see kQuerySmem");
 
-__global__ void __launch_bounds__(kVisThreads, 1)
+// ---- two-CTA forms of the building blocks of tc_common.cuh ----
+// TMA tile load into this CTA's shared memory whose bytes are counted on a barrier of the pair's
+// leader CTA (bar_cluster_addr: see map_to_cta).  No multicast.
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t smem_dst, const CUtensorMap* map, int x, int y,
+                                                 uint32_t bar_cluster_addr) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+      ::"r"(smem_dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar_cluster_addr)
+      : "memory");
+}
+__device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                               uint32_t accumulate) {
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "setp.ne.b32 p, %4, 0;\n"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n"
+      "}\n" ::"r"(d_tmem),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// Arrives (once the MMAs issued so far have completed) on the barrier at this offset in both CTAs.
+__device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+          smem_u32(bar)),
+      "h"((unsigned short)3)
+      : "memory");
+}
+
+// One poll that never suspends the thread (try_wait may, while the current chunk's products are still to be issued).
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
+struct VisParams {
+  const int4* tiles;    // [n_tiles] 128-token tiles over all requests: first row of X, rows, first query row, query elements
+  int n_tiles;
+  int n_items;          // (pair of tiles, group of heads) pairs
+  int n_groups;         // groups of heads
+  int group_heads;      // heads per group, 2 or 1 (1: the weight map's boxes are 64 rows high instead of 128)
+  int stages;           // of the main ring, kBytesA + group_heads * kVisHeadBytes each
+  int n_heads;
+  int k_chunks;         // ceil(d / 64)
+  int rows_total;       // rows of X
+  int query_rows;       // kq: query elements of a block, per CTA (the boxes of the query maps)
+  float* s_query;       // out (pre-filled with -inf)
+  int* status;
+};
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kVisThreads, 2)   // (80 registers: see kVisThreads)
 relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d]
                      const __grid_constant__ CUtensorMap map_w,   // Wk: [P, d]
                      const __grid_constant__ CUtensorMap map_q,   // Qn hi: [sum T, P]
                      const __grid_constant__ CUtensorMap map_ql,  // Qn lo
-                     const Params prm) {
+                     const VisParams prm) {
   extern __shared__ __align__(1024) uint8_t rel_smem_raw[];
   uint8_t* smem = rel_smem_raw;
-  if (smem_u32(smem) & 1023u) {          // the swizzled tiles need a 1024-byte aligned base
-    if (threadIdx.x == 0) atomicOr(prm.status, kStatusTimeout);
-    return;
-  }
-  uint8_t* kp_smem = smem + kVisStages * kBytesStage;    // hi half 0, hi half 1, lo half 0, lo half 1
-  uint8_t* q_smem = kp_smem + 4 * kBytesKp;              // [2][kQueryBlock]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(q_smem + 2 * kQueryBlock);
-  uint64_t* full = bars;                                 // [kVisStages]
-  uint64_t* empty = bars + kVisStages;                   // [kVisStages]
-  uint64_t* acc_full = bars + 2 * kVisStages;            // [2]
-  uint64_t* acc_empty = acc_full + 2;                    // [2]
-  uint64_t* kp_ready = acc_full + 4;
-  uint64_t* kp_free = acc_full + 5;
-  uint64_t* logit_full = acc_full + 6;                   // [kLogitTiles]
-  uint64_t* logit_empty = acc_full + 8;                  // [kLogitTiles]
-  uint64_t* q_full = acc_full + 10;                      // [2]
-  uint64_t* q_empty = acc_full + 12;                     // [2]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 14);
+  uint8_t* kp_smem = smem + kVisRing;                      // hi half 0, hi half 1, lo half 0, lo half 1
+  uint8_t* q_smem = kp_smem + 4 * kBytesKp;                // [slots][kq x 64]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(q_smem + kQueryRing);
+  uint64_t* full = bars;                                 // [kVisMaxStages] leader: bytes of both CTAs' loads
+  uint64_t* empty = full + kVisMaxStages;                // [kVisMaxStages] both
+  uint64_t* q_full = empty + kVisMaxStages;                // [kMaxQuerySlots] leader: bytes of both CTAs' loads
+  uint64_t* q_empty = q_full + kMaxQuerySlots;           // [kMaxQuerySlots] both
+  uint64_t* acc_full = q_empty + kMaxQuerySlots;         // [2] both
+  uint64_t* acc_empty = acc_full + 2;                    // [2] leader, one arrival per epilogue warp of both CTAs
+  uint64_t* logit_full = acc_empty + 2;                  // [2] both
+  uint64_t* logit_empty = logit_full + 2;                // [2] leader, epilogue warps
+  uint64_t* kp_ready = logit_empty + 2;                  // leader, epilogue warps
+  uint64_t* kp_free = kp_ready + 1;                      // both
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(kp_free + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  float* exchange = reinterpret_cast<float*>(q_smem + kQueryRing + 1024);      // [2][norm, largest logit][128]
   const int warp = warp_index(), lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();
+  const bool leader = rank == 0;
+  const bool aligned = (smem_u32(smem) & 1023u) == 0;      // the swizzled tiles need a 1024-byte aligned base
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kVisStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+    for (int s = 0; s < kVisMaxStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+    for (int s = 0; s < kMaxQuerySlots; ++s) { mbar_init(&q_full[s], 1); mbar_init(&q_empty[s], 1); }
     for (int i = 0; i < 2; ++i) {
-      mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 128);
-      mbar_init(&logit_full[i], 1); mbar_init(&logit_empty[i], 128);
-      mbar_init(&q_full[i], 1); mbar_init(&q_empty[i], 1);
+      mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 2 * kVisEpiWarps);
+      mbar_init(&logit_full[i], 1); mbar_init(&logit_empty[i], 2 * kVisEpiWarps);
     }
-    mbar_init(kp_ready, 128);
+    mbar_init(kp_ready, 2 * kVisEpiWarps);
     mbar_init(kp_free, 1);
-    *abort_flag = 0;
+    *abort_flag = aligned ? 0 : 1;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 5) tmem_alloc(tmem_slot, kTmemCols);
+  if (warp == 9) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
   tc_fence_before();
   __syncthreads();
+  cluster_sync_all();                      // both CTAs' barriers exist before anything arrives on them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  const int n_clusters = gridDim.x >> 1, cluster_id = blockIdx.x >> 1;
 
-  // Item -> tile rows, query rows, first head; every role walks the same list.
-  auto decode = [&](int item, int& row0, int& nrows, int& txt0, int& T, int& hp, int& heads) {
-    const int tile = item / prm.n_groups;
-    hp = item % prm.n_groups;
-    heads = min(2, prm.n_heads - 2 * hp);
-    const int b = find_request(tile, prm.batch, [&](int q) { return prm.plan[q].tile_off; });
-    const ReqPlan rp = prm.plan[b];
-    const int t = tile - rp.tile_off;
-    row0 = rp.vis_off + t * kTileM;
-    nrows = min(kTileM, rp.n - t * kTileM);
-    txt0 = rp.txt_off;
-    T = rp.t;
+  // Item -> this CTA's tile rows, first head and heads of the group, and the query rows of the pair's requests (one
+  // segment, or two where the tiles belong to different requests); every role walks the same list.
+  struct Item {
+    int row0, nrows, head0, heads;
+    int txt0, T0, tiles0, txt1, T1, tiles1;    // per segment: first query row, query elements, logits tiles (0: no segment)
+    int mine;                              // this CTA's segment
   };
+  auto decode = [&](int item) {
+    Item it;
+    const int pair = item / prm.n_groups, g = item - pair * prm.n_groups;
+    it.head0 = g * prm.group_heads;
+    it.heads = min(prm.group_heads, prm.n_heads - it.head0);
+    const int4 a = prm.tiles[2 * pair], b = prm.tiles[min(2 * pair + 1, prm.n_tiles - 1)];
+    const bool two = a.z != b.z;           // requests (each has query rows of its own)
+    it.txt0 = a.z; it.T0 = a.w; it.tiles0 = (a.w + kLogitN - 1) / kLogitN;
+    it.txt1 = b.z; it.T1 = b.w; it.tiles1 = two ? (b.w + kLogitN - 1) / kLogitN : 0;
+    it.mine = rank != 0 && two ? 1 : 0;
+    const bool exists = 2 * pair + (int)rank < prm.n_tiles;      // no tile: all rows read as zeros
+    it.row0 = exists ? (rank != 0 ? b.x : a.x) : prm.rows_total;
+    it.nrows = exists ? (rank != 0 ? b.y : a.y) : 0;
+    return it;
+  };
+  // Logits tile i of an item: its segment, first query element in it and width (a multiple of 32)
+  auto logits_tile = [&](const Item& it, int i, int& seg, int& j0, int& width) {
+    seg = i >= it.tiles0 ? 1 : 0;
+    j0 = (seg ? i - it.tiles0 : i) * kLogitN;
+    width = min(kLogitN, ((seg ? it.T1 : it.T0) - j0 + 31) & ~31);
+  };
+  const int stage_bytes = kBytesA + prm.group_heads * kVisHeadBytes;
+  const int q_bytes = prm.query_rows * kHalf * 2, q_slots = min(kMaxQuerySlots, kQueryRing / q_bytes);
 
-  if (warp == 4) {
-    // ---------------------------------------------------------------- TMA producer, main ring
-    if (lane == 0) {
+  if (warp == 8) {
+    // ---------------------------------------------------------------- TMA producer, main ring (both CTAs)
+    if (lane == 0 && aligned) {
       int s = 0;
       uint32_t ph = 1;
       bool ok = true;
-      for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x) {
-        int row0, nrows, txt0, T, hp, heads;
-        decode(item, row0, nrows, txt0, T, hp, heads);
+            for (int item = cluster_id; item < prm.n_items && ok; item += n_clusters) {
+        const Item it = decode(item);
+        // the CTA's half of the group's features (a lone last head: 64 of the 128 rows are used)
+        const int wrow = it.head0 * kHeadDim + (int)rank * it.heads * (kHeadDim / 2);
         for (int kc = 0; kc < prm.k_chunks; ++kc) {
           if (!(ok = mbar_wait(&empty[s], ph, abort_flag))) break;
-          mbar_expect_tx(&full[s], kBytesStage);
-          const uint32_t dst = smem_u32(smem + s * kBytesStage);
-          tma_load_2d(dst, &map_x, kc * kBK, row0, &full[s]);
-          tma_load_2d(dst + kBytesA, &map_w, kc * kBK, hp * kTileN, &full[s]);
-          if (++s == kVisStages) { s = 0; ph ^= 1u; }
+          if (leader) mbar_expect_tx(&full[s], 2 * stage_bytes);
+          const uint32_t dst = smem_u32(smem + s * stage_bytes), bar = map_to_cta(&full[s], 0);
+          tma_load_2d_pair(dst, &map_x, kc * kBK, it.row0, bar);
+          tma_load_2d_pair(dst + kBytesA, &map_w, kc * kBK, wrow, bar);
+          if (++s == prm.stages) { s = 0; ph ^= 1u; }
         }
       }
     }
     __syncwarp();
-  } else if (warp == 5) {
-    // ---------------------------------------------------------------- MMA issuer, main loop
-    if (lane == 0) {
+  } else if (warp == 9) {
+    // ---------------------------------------------------------------- MMA issuer, main loop (leader)
+    if (lane == 0 && leader && aligned) {
       int s = 0;
       uint32_t ph = 0, n = 0;
-      bool ok = true;
-      for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x, ++n) {
+      bool ok = true, ready = false;
+      for (int item = cluster_id; item < prm.n_items && ok; item += n_clusters, ++n) {
         const uint32_t buf = n & 1u;
         if (!(ok = mbar_wait(&acc_empty[buf], ((n >> 1) & 1u) ^ 1u, abort_flag))) break;
         tc_fence_after();
-        // a lone last head takes half the columns and half the tensor time (576 tokens, one float32 head, d = 1024: a
-        // call 171.0 -> 169.0 us; fetching half the weight tile as well gained nothing)
-        const uint32_t idesc = umma_idesc(kTileM, item % prm.n_groups * 2 + 1 < prm.n_heads ? kTileN : kHeadDim);
+        const int head0 = item % prm.n_groups * prm.group_heads;
+        const uint32_t idesc = umma_idesc(2 * kTileM, min(prm.group_heads, prm.n_heads - head0) * kHeadDim);
         for (int kc = 0; kc < prm.k_chunks; ++kc) {
-          if (!(ok = mbar_wait(&full[s], ph, abort_flag))) break;
+          if (!ready && !(ok = mbar_wait(&full[s], ph, abort_flag))) break;
           tc_fence_after();
-          const uint32_t a_addr = smem_u32(smem + s * kBytesStage);
+          const uint32_t a_addr = smem_u32(smem + s * stage_bytes);
           const uint64_t adesc = umma_desc(a_addr), bdesc = umma_desc(a_addr + kBytesA);
+          const int cur = s;
+          if (++s == prm.stages) { s = 0; ph ^= 1u; }
+          ready = mbar_test(&full[s], ph);
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k)
-            umma_bf16(tmem_base + buf * kTileN, adesc + 2 * k, bdesc + 2 * k, idesc, (kc | k) != 0);
-          umma_commit(&empty[s]);
-          if (++s == kVisStages) { s = 0; ph ^= 1u; }
+            umma_bf16_pair(tmem_base + buf * kTileN, adesc + 2 * k, bdesc + 2 * k, idesc, (kc | k) != 0);
+          umma_commit_pair(&empty[cur]);
         }
-        if (ok) umma_commit(&acc_full[buf]);
+        if (ok) umma_commit_pair(&acc_full[buf]);
       }
     }
     __syncwarp();
-  } else if (warp == 6) {
-    // ---------------------------------------------------------------- MMA issuer, logits
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc(kTileM, kTT);
-      uint32_t n = 0, head_it = 0, q_it = 0, uses[kLogitTiles] = {0u, 0u};
+  } else if (warp == 10) {
+    // ---------------------------------------------------------------- MMA issuer, logits (leader)
+    if (lane == 0 && leader && aligned) {
+      uint32_t n = 0, head_it = 0, lt = 0, q_ph = 0;
+      int qs = 0;
       bool ok = true;
-      for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x, ++n) {
-        int row0, nrows, txt0, T, hp, heads;
-        decode(item, row0, nrows, txt0, T, hp, heads);
-        const int ntt = (T + kTT - 1) / kTT;
-        for (int h = 0; h < heads && ok; ++h, ++head_it) {
-          if (!(ok = mbar_wait(kp_ready, head_it & 1u, abort_flag))) break;      // this head is restaged
+      for (int item = cluster_id; item < prm.n_items && ok; item += n_clusters, ++n) {
+        const Item it = decode(item);
+        const int ntt = it.tiles0 + it.tiles1;
+        for (int h = 0; h < it.heads && ok; ++h, ++head_it) {
+          if (!(ok = mbar_wait(kp_ready, head_it & 1u, abort_flag))) break;      // both CTAs have restaged this head
           const uint32_t kp_addr = smem_u32(kp_smem);
-          for (int t = 0; t < ntt && ok; ++t) {
-            const int slot = t & 1;
-            if (!(ok = mbar_wait(&logit_empty[slot], (uses[slot] & 1u) ^ 1u, abort_flag))) break;
-            ++uses[slot];
-            const uint32_t d_col = tmem_base + (n & 1u) * kTileN + h * kHeadDim + slot * kTT;
+          const uint32_t d_col = tmem_base + (n & 1u) * kTileN + h * kHeadDim;
+          for (int i = 0; i < ntt && ok; ++i, ++lt) {
+            int seg, j0, width;
+            logits_tile(it, i, seg, j0, width);
+            // the tile before the last has been read (its barrier is used again), and within a head the last one
+            // too: it lies in the same columns
+            if (lt >= 2 && !(ok = mbar_wait(&logit_empty[lt & 1u], ((lt - 2) >> 1) & 1u, abort_flag))) break;
+            if (i > 0 && !(ok = mbar_wait(&logit_empty[(lt - 1) & 1u], ((lt - 1) >> 1) & 1u, abort_flag))) break;
+            const uint32_t idesc = umma_idesc(2 * kTileM, width);
             // logits = sum over the two halves of Kp_hi Qn_hi^T + Kp_lo Qn_hi^T + Kp_hi Qn_lo^T
             for (int half = 0; half < 2 && ok; ++half) {
               const uint64_t hi = umma_desc(kp_addr + half * kBytesKp), lo = umma_desc(kp_addr + (2 + half) * kBytesKp);
 #pragma unroll 1
-              for (int part = 0; part < 2; ++part, ++q_it) {
-                const uint32_t qs = q_it & 1u;
-                if (!(ok = mbar_wait(&q_full[qs], (q_it >> 1) & 1u, abort_flag))) break;
+              for (int part = 0; part < 2; ++part) {
+                if (!(ok = mbar_wait(&q_full[qs], q_ph, abort_flag))) break;
                 tc_fence_after();
-                const uint64_t q = umma_desc(smem_u32(q_smem + qs * kQueryBlock));
+                const uint64_t q = umma_desc(smem_u32(q_smem + qs * q_bytes));
 #pragma unroll
-                for (int ks = 0; ks < kHalf / 16; ++ks) umma_bf16(d_col, hi + 2 * ks, q + 2 * ks, idesc, (half | part | ks) != 0);
+                for (int ks = 0; ks < kHalf / 16; ++ks) umma_bf16_pair(d_col, hi + 2 * ks, q + 2 * ks, idesc, (half | part | ks) != 0);
                 if (part == 0) {
 #pragma unroll
-                  for (int ks = 0; ks < kHalf / 16; ++ks) umma_bf16(d_col, lo + 2 * ks, q + 2 * ks, idesc, 1u);
+                  for (int ks = 0; ks < kHalf / 16; ++ks) umma_bf16_pair(d_col, lo + 2 * ks, q + 2 * ks, idesc, 1u);
                 }
-                umma_commit(&q_empty[qs]);
+                umma_commit_pair(&q_empty[qs]);
+                if (++qs == q_slots) { qs = 0; q_ph ^= 1u; }
               }
             }
-            if (ok) umma_commit(&logit_full[slot]);
+            if (ok) umma_commit_pair(&logit_full[lt & 1u]);
           }
-          if (ok) umma_commit(kp_free);
+          if (ok) umma_commit_pair(kp_free);
         }
       }
     }
     __syncwarp();
-  } else if (warp == 7) {
-    // ---------------------------------------------------------------- TMA producer, query blocks
-    if (lane == 0) {
-      uint32_t q_it = 0;
+  } else if (warp == 11) {
+    // ---------------------------------------------------------------- TMA producer, query blocks (both CTAs)
+    if (lane == 0 && aligned) {
+      int qs = 0;
+      uint32_t ph = 1;
       bool ok = true;
       wait_for_previous_kernel();              // the unit query elements are complete
-      for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x) {
-        int row0, nrows, txt0, T, hp, heads;
-        decode(item, row0, nrows, txt0, T, hp, heads);
-        const int blocks = heads * ((T + kTT - 1) / kTT) * 4;
-        for (int i = 0; i < blocks; ++i, ++q_it) {
-          // head, tile, half, hi / lo: the order in which the logits issuer uses them
-          const int part = i & 1, half = (i >> 1) & 1, ht = i >> 2, ntt = (T + kTT - 1) / kTT;
-          const int h = ht / ntt, t = ht - h * ntt;
-          const uint32_t qs = q_it & 1u;
-          if (!(ok = mbar_wait(&q_empty[qs], ((q_it >> 1) & 1u) ^ 1u, abort_flag))) break;
-          mbar_expect_tx(&q_full[qs], kQueryBlock);
-          tma_load_2d(smem_u32(q_smem + qs * kQueryBlock), part ? &map_ql : &map_q,
-                      (2 * hp + h) * kHeadDim + half * kHalf, txt0 + t * kTT, &q_full[qs]);
-        }
+      for (int item = cluster_id; item < prm.n_items && ok; item += n_clusters) {
+        const Item it = decode(item);
+        const int ntt = it.tiles0 + it.tiles1;
+        for (int h = 0; h < it.heads && ok; ++h)
+          for (int i = 0; i < ntt && ok; ++i) {
+            int seg, j0, width;
+            logits_tile(it, i, seg, j0, width);
+            const int y = (seg ? it.txt1 : it.txt0) + j0 + (int)rank * (width >> 1);
+            for (int p = 0; p < 4; ++p) {      // half, hi / lo: the order in which the logits issuer uses them
+              if (!(ok = mbar_wait(&q_empty[qs], ph, abort_flag))) break;
+              if (leader) mbar_expect_tx(&q_full[qs], 2 * q_bytes);
+              tma_load_2d_pair(smem_u32(q_smem + qs * q_bytes), (p & 1) ? &map_ql : &map_q,
+                               (it.head0 + h) * kHeadDim + (p >> 1) * kHalf, y, map_to_cta(&q_full[qs], 0));
+              if (++qs == q_slots) { qs = 0; ph ^= 1u; }
+            }
+          }
       }
     }
     __syncwarp();
   } else {
-    // ---------------------------------------------------------------- epilogue (warps 0-3)
-    const int r = warp * 32 + lane;                        // token row inside the tile = TMEM lane
-    const uint32_t t_lane = tmem_base + ((uint32_t)(warp * 32) << 16);
-    uint32_t n = 0, head_it = 0, uses[kLogitTiles] = {0u, 0u};
-    bool ok = true;
-    for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x, ++n) {
-      int row0, nrows, txt0, T, hp, heads;
-      decode(item, row0, nrows, txt0, T, hp, heads);
+    // ---------------------------------------------------------------- epilogue (warps 0-7, both CTAs)
+    const int r = (warp & 3) * 32 + lane;                  // token row inside the tile = TMEM lane
+    const int part = warp >> 2;                            // which half of the columns this thread takes
+    const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+    const uint32_t l_kp_ready = map_to_cta(kp_ready, 0), l_acc_empty = map_to_cta(acc_empty, 0),
+                   l_logit_empty = map_to_cta(logit_empty, 0);       // [2] each: 8 bytes apart
+    uint32_t n = 0, head_it = 0, lt = 0;
+    bool ok = aligned;                                     // a thread that gave up stays for the barriers
+    for (int item = cluster_id; item < prm.n_items; item += n_clusters, ++n) {
+      const Item it = decode(item);
       const uint32_t buf = n & 1u;
-      const int ntt = (T + kTT - 1) / kTT;
-      float best = -INFINITY;
+      const int ntt = it.tiles0 + it.tiles1;
+      float best = -INFINITY, top = -INFINITY, ss = 0.f;    // top: largest product of the head so far
       bool nonfinite = false;
-      if (!(ok = mbar_wait(&acc_full[buf], (n >> 1) & 1u, abort_flag))) break;
+      ok = ok && mbar_wait(&acc_full[buf], (n >> 1) & 1u, abort_flag);
       tc_fence_after();
-      for (int h = 0; h < heads && ok; ++h, ++head_it) {
-        const uint32_t cols = t_lane + buf * kTileN + h * kHeadDim;
-        float ss = 0.f;
-        // restage the head as bf16 hi + lo, 32 features at a time, once the previous head's products have read theirs
-        if (!(ok = mbar_wait(kp_free, (head_it & 1u) ^ 1u, abort_flag))) break;
+      // logits tile i of head h: this thread's half of the columns
+      auto read_logits = [&](int h, int i) {
+        int seg, j0, width;
+        logits_tile(it, i, seg, j0, width);
+        ok = ok && mbar_wait(&logit_full[lt & 1u], (lt >> 1) & 1u, abort_flag);
+        tc_fence_after();
+        const int T = seg ? it.T1 : it.T0;
+        if (seg == it.mine) {
+          const uint32_t cols = t_lane + buf * kTileN + h * kHeadDim;
+          const int c_end = (part + 1) * (width >> 1);
 #pragma unroll 1
-        for (int c4 = 0; c4 < 4; ++c4) {
+          for (int c = part * (width >> 1); c < c_end; c += 16) {
+            float v[16];
+            tmem_ld16(cols + c, v);
+#pragma unroll
+            for (int e = 0; e < 16; ++e)
+              if (j0 + c + e < T) {
+                nonfinite |= v[e] != v[e];
+                top = fmaxf(top, v[e]);
+              }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_at(l_logit_empty + 8 * (lt & 1u));
+        ++lt;
+      };
+      // last logits tile of a head, then the two threads of a token put their halves together: a cosine is the
+      // largest product over the length (rounding keeps the order, so scaling after the maximum changes nothing)
+      auto finish_head = [&](int h, float ss_h) {
+        read_logits(h, ntt - 1);
+        float* x = exchange + ((head_it + (uint32_t)h) & 1u) * 256 + r;
+        if (part == 1) { x[0] = ss_h; x[128] = nonfinite ? __int_as_float(0x7fc00000) : top; }
+        named_barrier(1, kVisEpiWarps * 32);
+        if (part == 0) {
+          const float s = ss_h + x[0], o = x[128];
+          nonfinite |= o != o || !(s <= 3.402823466e38f);
+          float inv = 0.f;
+          if (s > 1.17549435e-38f) { inv = rsqrtf(s); inv = inv * (1.5f - 0.5f * s * inv * inv); }
+          best = fmaxf(best, fmaxf(top, o) * inv);
+        }
+        top = -INFINITY;
+      };
+      for (int h = 0; h < it.heads; ++h) {
+        // restage this thread's 64 features of the head as bf16 hi + lo, once the previous head's products have read theirs
+        const uint32_t cols = t_lane + buf * kTileN + h * kHeadDim + part * kHalf;
+        const float ss_before = ss;
+        ss = 0.f;
+        ok = ok && mbar_wait(kp_free, ((head_it + (uint32_t)h) & 1u) ^ 1u, abort_flag);
+#pragma unroll 1
+        for (int c2 = 0; c2 < 2; ++c2) {
           float v[32];
-          tmem_ld32(cols + c4 * 32, v);
+          tmem_ld32(cols + c2 * 32, v);
           uint32_t pk[16], pl[16];
 #pragma unroll
           for (int e = 0; e < 16; ++e) {
@@ -244,10 +397,10 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
             pk[e] = *reinterpret_cast<uint32_t*>(&hi);
             pl[e] = pack_bf16(a - __low2float(hi), b - __high2float(hi));
           }
-          uint8_t* rowp = kp_smem + (c4 >> 1) * kBytesKp + r * 128;
+          uint8_t* rowp = kp_smem + part * kBytesKp + r * 128;
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            int chunk = ((c4 & 1) * 4 + q) ^ (r & 7);
+            int chunk = (c2 * 4 + q) ^ (r & 7);
             *reinterpret_cast<uint4*>(rowp + chunk * 16) =
                 make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
             *reinterpret_cast<uint4*>(rowp + 2 * kBytesKp + chunk * 16) =
@@ -256,45 +409,31 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         tc_fence_before();
-        mbar_arrive(kp_ready);
-        nonfinite |= !(ss <= 3.402823466e38f);
-        float inv = 0.f;
-        if (ss > 1.17549435e-38f) { inv = rsqrtf(ss); inv = inv * (1.5f - 0.5f * ss * inv * inv); }
-        for (int t = 0; t < ntt; ++t) {
-          const int slot = t & 1;
-          if (!(ok = mbar_wait(&logit_full[slot], uses[slot] & 1u, abort_flag))) break;
-          ++uses[slot];
-          tc_fence_after();
-#pragma unroll 1
-          for (int c2 = 0; c2 < 2; ++c2) {
-            const int jbase = t * kTT + c2 * 32;
-            if (jbase >= T) break;
-            float v[32];
-            tmem_ld32(cols + slot * kTT + c2 * 32, v);
-#pragma unroll
-            for (int e = 0; e < 32; ++e)
-              if (jbase + e < T) {
-                nonfinite |= v[e] != v[e];
-                best = fmaxf(best, v[e] * inv);
-              }
-          }
-          tc_fence_before();
-          mbar_arrive(&logit_empty[slot]);
-        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive_at(l_kp_ready);
+        if (h > 0) finish_head(h - 1, ss_before);
+        for (int i = 0; i + 1 < ntt; ++i) read_logits(h, i);
       }
-      if (!ok) break;
-      mbar_arrive(&acc_empty[buf]);            // projections and logits of the item have been read
-      if (item == (int)blockIdx.x) wait_for_previous_kernel();      // the scores are filled with -inf
-      if (r < nrows) {
+      finish_head(it.heads - 1, ss);
+      head_it += (uint32_t)it.heads;
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_at(l_acc_empty + 8 * buf);       // projections and logits of the item have been read
+      if (item == cluster_id) wait_for_previous_kernel();         // the scores are filled with -inf
+      if (part == 0 && r < it.nrows && ok) {
         if (nonfinite) atomicOr(prm.status, kStatusNonFinite);
-        else atomic_max_float(prm.s_query + row0 + r, best);
+        else atomic_max_float(prm.s_query + it.row0 + r, best);
       }
     }
   }
 
   tc_fence_before();
   __syncthreads();
-  if (warp == 5) tmem_dealloc(tmem_base, kTmemCols);
+  cluster_sync_all();                      // nothing of the peer may still point at this CTA
+  if (warp == 9) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols)
+                 : "memory");
+  }
   if (threadIdx.x == 0 && *abort_flag) atomicOr(prm.status, kStatusTimeout);
 }
 
