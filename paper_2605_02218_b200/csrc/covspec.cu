@@ -21,7 +21,6 @@
 #include "identity_tc.cuh"
 #include "relevance_tc.cuh"
 #include "relevance_vis.cuh"
-#include "relevance_pair.cuh"
 #include "subspace_tc.cuh"
 #include "subspace_fused.cuh"
 #include "score_kernels.cuh"
@@ -67,7 +66,6 @@ struct Plan {
   int tiles[T_COUNT] = {0};
   int t_max = 0, p_max = 0, m_max = 0, win_max = 0, nbot_max = 0;
   int n_tiles = 0;                            // 128-token tiles over all requests
-  int n_pairs = 0;                            // pairs of neighbouring tiles of one request
   int n_gram_tiles = 0, n_ptiles = 0;         // lower-triangle Gram items / row tiles of the subspace blocks (stage 2)
   int tile_rows = 128;                        // rows of a subspace-block tile: 64 when that still gives every tile a CTA
   int tile_ctas = 0, servers = 0;             // CTAs of the subspace kernel that carry tiles / that only factor
@@ -220,7 +218,7 @@ int get_plan(covspec_ctx* ctx, const covspec_problem* p, cudaStream_t stream) {
   pl.keep_offsets.assign(B + 1, 0);
   pl.tile_list.clear();
   pl.presel_offsets.assign(B + 1, 0);
-  pl.n_stage2 = 0; pl.t_max = 0; pl.p_max = 0; pl.m_max = 0; pl.n_tiles = 0; pl.n_pairs = 0;
+  pl.n_stage2 = 0; pl.t_max = 0; pl.p_max = 0; pl.m_max = 0; pl.n_tiles = 0;
   pl.n_gram_tiles = 0; pl.n_ptiles = 0;
   pl.win_max = 0; pl.nbot_max = 0;
   long long g_off = 0, c_off = 0;
@@ -239,8 +237,6 @@ int get_plan(covspec_ctx* ctx, const covspec_problem* p, cudaStream_t stream) {
     for (int i = 0; i < r.n; i += tc::kTileM)
       pl.tile_list.push_back(make_int4(r.vis_off + i, std::min(tc::kTileM, r.n - i), r.txt_off, r.t));
     pl.n_tiles += (r.n + tc::kTileM - 1) / tc::kTileM;
-    r.pair_off = pl.n_pairs;
-    pl.n_pairs += ((r.n + tc::kTileM - 1) / tc::kTileM + 1) / 2;
     r.gram_tile_off = pl.n_gram_tiles;
     r.g_off = g_off;
     r.c_off = c_off;
@@ -616,52 +612,6 @@ int launch_identity_tc(const void* X, const void* Q, long long rows_x, long long
   return COVSPEC_OK;
 }
 
-// Eq. 10 on the tensor cores, two-SM form (relevance_pair.cuh): query embedding (MODE 1), -inf fill,
-// fused projection + cosine max over pairs of token tiles.
-int relevance_pair(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cudaStream_t s) {
-  const covspec_config& cfg = ctx->cfg;
-  const Plan& pl = ctx->plan;
-  int P = ctx->P, d = cfg.d;
-  const void *X = p->X, *Q = p->Q, *Wk = p->Wk, *Wq = p->Wq;
-  if (ctx->split_tc) { X = ctx->X3; Q = ctx->Q3; Wk = ctx->Wk3; Wq = ctx->Wq3; d = ctx->d3; }
-  __nv_bfloat16* qn = reinterpret_cast<__nv_bfloat16*>(ctx->Qn);
-  CUtensorMap map_x, map_wk, map_q, map_wq, map_qn, map_qnl;
-  long long lo_off = (long long)cfg.max_total_txt * P;   // lo parts follow the hi parts
-  int st;
-  if ((st = make_map_bf16(&map_x, X, pl.total_vis, d, tc::kTileM))) return st;
-  if ((st = make_map_bf16(&map_wk, Wk, P, d, tc::kTileN / 2))) return st;
-  if ((st = make_map_bf16(&map_q, Q, pl.total_txt, d, tc::kTileM))) return st;
-  if ((st = make_map_bf16(&map_wq, Wq, P, d, tc::kTileN / 2))) return st;
-  if ((st = make_map_bf16(&map_qn, qn, pl.total_txt, P, tc::kTT / 2))) return st;
-  if ((st = make_map_bf16(&map_qnl, qn + lo_off, pl.total_txt, P, tc::kTT / 2))) return st;
-  int n_hp = (cfg.n_heads + 1) / 2;
-  tc2::PairParams prm{};
-  prm.plan = ctx->d_plan; prm.batch = p->batch;
-  prm.n_groups = n_hp; prm.hp_per_group = 1;
-  prm.n_heads = cfg.n_heads; prm.k_chunks = (d + tc::kBK - 1) / tc::kBK; prm.P = P;
-  prm.status = ctx->status;
-  const int max_clusters = ctx->num_sms / 2;
-  // query side
-  prof_mark(ctx, ST_QEMBED, 0, s);
-  prm.rows_total = pl.total_txt;
-  prm.n_items = (int)((pl.total_txt + 2 * tc::kTileM - 1) / (2 * tc::kTileM)) * prm.n_groups;
-  prm.qn_out = qn; prm.qn_lo_off = lo_off; prm.s_query = nullptr;
-  prm.fill = s_query; prm.fill_n = pl.total_vis;          // -inf for the visual-side launch below
-  int grid = 2 * std::min(prm.n_items, max_clusters);
-  tc2::relevance_pair_kernel<1><<<grid, tc2::kPairThreads, tc2::kSmemBytes2, s>>>(map_q, map_wq, map_qn, map_qnl, prm);
-  LAUNCH_CHECK(ctx);
-  prof_mark(ctx, ST_QEMBED, 1, s);
-  // visual side
-  prof_mark(ctx, ST_RELEVANCE, 0, s);
-  prm.n_items = pl.n_pairs * prm.n_groups;
-  prm.qn_out = nullptr; prm.s_query = s_query; prm.fill = nullptr;
-  grid = 2 * std::min(prm.n_items, max_clusters);
-  tc2::relevance_pair_kernel<0><<<grid, tc2::kPairThreads, tc2::kSmemBytes2, s>>>(map_x, map_wk, map_qn, map_qnl, prm);
-  LAUNCH_CHECK(ctx);
-  prof_mark(ctx, ST_RELEVANCE, 1, s);
-  return COVSPEC_OK;
-}
-
 // Eq. 10 on the tensor cores: query embedding (MODE 1), -inf fill, fused projection + cosine max.
 int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cudaStream_t s) {
   const covspec_config& cfg = ctx->cfg;
@@ -688,7 +638,7 @@ int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cud
   if ((st = make_map_bf16(&map_wq, Wq, P, d, group_heads * tc::kHeadDim))) return st;
   if ((st = make_map_bf16(&map_qn, qn, pl.total_txt, P, query_rows))) return st;
   if ((st = make_map_bf16(&map_qnl, qn + lo_off, pl.total_txt, P, query_rows))) return st;
-  tc::Params prm{};
+  tc::QueryParams prm{};
   prm.n_heads = cfg.n_heads; prm.k_chunks = (d + tc::kBK - 1) / tc::kBK; prm.P = P;
   prm.status = ctx->status;
   // query side
@@ -742,14 +692,13 @@ int launch_activity(covspec_ctx* ctx, const covspec_problem* p, float* s_act, bo
   LayerPtrs lp{};
   for (int l = 0; l <= cfg.act_layers; ++l) lp.h[l] = p->Hs[l];
   if (background) {
-    // beside the two-SM relevance kernel only one block per SM fits (shared-memory reserve)
-    int per_sm = cfg.relevance_path == 2 ? 1 : cfg.activity_overlap;
+    int per_sm = cfg.activity_overlap;
     // One block per SM reads about 1.8 TB/s beside the relevance kernel; where that would end after the
     // kernel (about 1.1 PFLOP/s) a second one is added (batch of 16 x 576 tokens, d = 2048: 115 -> 71 us).
     // Where it ends before, a second block only slows the kernel down (video: 3570 -> 3940 us a call).
     const double stream_s = (double)(cfg.act_layers + 1) * rowsX * cfg.d * ctx->esize / 1.8e12;
     const double kernel_s = 2.0 * rowsX * (ctx->split_tc ? ctx->d3 : cfg.d) * ctx->P / 1.1e15;
-    if (per_sm == 1 && cfg.relevance_path != 2 && stream_s > kernel_s) per_sm = 2;
+    if (per_sm == 1 && stream_s > kernel_s) per_sm = 2;
     unsigned grid = (unsigned)std::min<long long>((rowsX + 15) / 16, (long long)ctx->num_sms * per_sm);
     if (cfg.act_layers <= 4)
       activity_stream_kernel<T, 4><<<grid, 512, 0, s>>>(lp, cfg.act_layers, rowsX, cfg.d, s_act);
@@ -817,7 +766,7 @@ int score_impl(covspec_ctx* ctx, const covspec_problem* p, float* s_query, float
       split3_kernel<<<grid, 256, 0, s>>>(jobs, ctx->d_plan, B, cfg.d, ctx->dp);
       LAUNCH_CHECK(ctx);
     }
-    int st = cfg.relevance_path == 2 ? relevance_pair(ctx, p, s_query, s) : relevance_tc(ctx, p, s_query, s);
+    int st = relevance_tc(ctx, p, s_query, s);
     if (st) return st;
   } else if (identity_tc) {
     prof_mark(ctx, ST_RELEVANCE, 0, s);
@@ -1203,10 +1152,6 @@ int covspec_prune_init(const covspec_config* cfg, covspec_ctx** out) {
                              tc::kVisSmem) == cudaSuccess &&
         cudaFuncSetAttribute(tc::query_embed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              tc::kQuerySmem) == cudaSuccess &&
-        cudaFuncSetAttribute(tc2::relevance_pair_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             tc2::kSmemBytes2) == cudaSuccess &&
-        cudaFuncSetAttribute(tc2::relevance_pair_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             tc2::kSmemBytes2) == cudaSuccess &&
         cudaFuncSetAttribute(sub::gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              sub::kGramSmem) == cudaSuccess &&
         cudaFuncSetAttribute(sub::subspace_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,

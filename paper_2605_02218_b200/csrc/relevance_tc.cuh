@@ -2,10 +2,13 @@
 // the query side: Qp = Q * Wq^T, normalised per head and written as bf16 hi + lo for the visual side
 // (relevance_vis.cuh).
 //
-// Work item of the query side: one 128-row tile of all query elements, one pair of heads.  Warp roles
+// Work item of the query side: one 128-row tile of all query elements, one or two heads.  Warp roles
 // (192 threads): warps 0-3 epilogue (one TMEM lane = one query element each), warp 4 TMA producer, warp 5 MMA
 // issuer and TMEM owner; two accumulators, so that the epilogue of an item runs beside the next one's main
 // loop.  Two 96 KB stages of two chunks instead of four of one were slower (15.0 -> 17.6 us at d = 2048).
+// With few items up to four CTAs of a cluster take a part of an item's inner dimension each and push their sums to the
+// first one: an item alone takes as long as its chain of chunks (512 cycles each, the time shared memory takes to write and read
+// one; one float32 request, 48 chunks: 17.2 -> 11.6 us).
 // Every mbarrier wait is bounded; on expiry the CTA raises a status bit, leaves its loops, frees TMEM and exits.
 #pragma once
 #include "tc_common.cuh"
@@ -18,7 +21,6 @@ constexpr int kTileM = 128;            // tokens per tile (UMMA M)
 constexpr int kTileN = 256;            // projected features per pass: one pair of heads (UMMA N)
 constexpr int kHeadDim = 128;
 constexpr int kBK = 64;                // bf16 elements per k-chunk = one 128-byte swizzle row
-constexpr int kTT = 64;                // query elements per logits tile (UMMA N of the 2nd product)
 constexpr int kHalf = 64;              // features of a restaged half head (one 128-byte swizzle row)
 constexpr int kBytesA = kTileM * kBK * 2;          // 16 KB
 constexpr int kBytesB = kTileN * kBK * 2;          // 32 KB
@@ -36,30 +38,27 @@ constexpr int kQuerySplitMax = 4;
 constexpr int kQueryPartBytes = kTileM * 32 * 4;
 static_assert((kQuerySplitMax - 1) * (kHeadDim / 32) * kQueryPartBytes <= kQueryStages * kBytesStage, "partial sums in the ring");
 
-struct Params {
-  const ReqPlan* plan;
-  int batch;
-  int n_items;          // (tile, pair of heads) pairs
-  int n_groups;         // pairs of heads (query side: groups of group_heads)
-  int group_heads;      // query side: heads per item, 2 or 1
-  int split;            // query side: CTAs (one cluster) that share an item's inner dimension; more than 1: one item of
-                        // one head per cluster
+struct QueryParams {
+  int n_items;          // (128-row tile, group of heads) pairs
+  int n_groups;         // groups of heads
+  int group_heads;      // heads per item, 2 or 1
+  int split;            // CTAs (one cluster) that share an item's inner dimension; more than 1: one item of one head per
+                        // cluster
   int n_heads;
   int k_chunks;         // ceil(d / 64)
   int P;                // n_heads * 128
-  long long rows_total; // query side: number of query rows
-  float* s_query;       // visual side, out (pre-filled with -inf)
-  __nv_bfloat16* qn_out;// query side, out: hi [rows_total, P] followed by lo at qn_out + qn_lo_off
+  long long rows_total; // query rows
+  __nv_bfloat16* qn_out;// out: hi [rows_total, P] followed by lo at qn_out + qn_lo_off
   long long qn_lo_off;
-  float* fill;          // query side: score array to fill with -inf for the visual side's launch that follows
-  long long fill_n;     //             (nullptr: nothing to fill)
+  float* fill;          // score array to fill with -inf for the visual side's launch that follows
+  long long fill_n;     // (nullptr: nothing to fill)
   int* status;
 };
 
 __global__ void __launch_bounds__(192, 1)
 query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
                    const __grid_constant__ CUtensorMap map_b,   // Wq: [P, d]
-                   const Params prm) {
+                   const QueryParams prm) {
   extern __shared__ __align__(1024) uint8_t rel_smem_raw[];
   uint8_t* smem = rel_smem_raw;
   if (smem_u32(smem) & 1023u) {          // the swizzled tiles need a 1024-byte aligned base

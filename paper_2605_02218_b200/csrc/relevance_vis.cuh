@@ -81,6 +81,12 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
       : "memory");
 }
 
+// Largest of three, NaN if one of them is.
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
 // One poll that never suspends the thread (try_wait may, while the current chunk's products are still to be issued).
 __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
@@ -327,11 +333,13 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
                    l_logit_empty = map_to_cta(logit_empty, 0);       // [2] each: 8 bytes apart
     uint32_t n = 0, head_it = 0, lt = 0;
     bool ok = aligned;                                     // a thread that gave up stays for the barriers
+    Item next = decode(cluster_id);
     for (int item = cluster_id; item < prm.n_items; item += n_clusters, ++n) {
-      const Item it = decode(item);
+      const Item it = next;
+      next = decode(min(item + n_clusters, prm.n_items - 1));       // its loads are back by the time it is needed
       const uint32_t buf = n & 1u;
       const int ntt = it.tiles0 + it.tiles1;
-      float best = -INFINITY, top = -INFINITY, ss = 0.f;    // top: largest product of the head so far
+      float best = -INFINITY, top = -INFINITY, ss = 0.f;    // top: largest product of the head so far (NaN if one is)
       bool nonfinite = false;
       ok = ok && mbar_wait(&acc_full[buf], (n >> 1) & 1u, abort_flag);
       tc_fence_after();
@@ -344,17 +352,25 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
         const int T = seg ? it.T1 : it.T0;
         if (seg == it.mine) {
           const uint32_t cols = t_lane + buf * kTileN + h * kHeadDim;
-          const int c_end = (part + 1) * (width >> 1);
+          const int c0 = part * (width >> 1), c_end = c0 + (width >> 1);
 #pragma unroll 1
-          for (int c = part * (width >> 1); c < c_end; c += 16) {
-            float v[16];
-            tmem_ld16(cols + c, v);
+          for (int c = c0; c < c_end; c += 32) {
+            float v[32];
+            if (c_end - c >= 32) {
+              tmem_ld32(cols + c, v);
+            } else {
+              float u[16];
+              tmem_ld16(cols + c, u);
 #pragma unroll
-            for (int e = 0; e < 16; ++e)
-              if (j0 + c + e < T) {
-                nonfinite |= v[e] != v[e];
-                top = fmaxf(top, v[e]);
-              }
+              for (int e = 0; e < 32; ++e) v[e] = e < 16 ? u[e] : -INFINITY;
+            }
+            if (j0 + c + 32 > T) {
+#pragma unroll
+              for (int e = 0; e < 32; ++e)
+                if (j0 + c + e >= T) v[e] = -INFINITY;
+            }
+#pragma unroll
+            for (int e = 0; e < 32; e += 2) top = max3_nan(top, v[e], v[e + 1]);
           }
         }
         tc_fence_before();
@@ -367,11 +383,11 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
       auto finish_head = [&](int h, float ss_h) {
         read_logits(h, ntt - 1);
         float* x = exchange + ((head_it + (uint32_t)h) & 1u) * 256 + r;
-        if (part == 1) { x[0] = ss_h; x[128] = nonfinite ? __int_as_float(0x7fc00000) : top; }
+        if (part == 1) { x[0] = ss_h; x[128] = top; }
         named_barrier(1, kVisEpiWarps * 32);
         if (part == 0) {
           const float s = ss_h + x[0], o = x[128];
-          nonfinite |= o != o || !(s <= 3.402823466e38f);
+          nonfinite |= o != o || top != top || !(s <= 3.402823466e38f);
           float inv = 0.f;
           if (s > 1.17549435e-38f) { inv = rsqrtf(s); inv = inv * (1.5f - 0.5f * s * inv * inv); }
           best = fmaxf(best, fmaxf(top, o) * inv);
