@@ -127,8 +127,25 @@ def load_library():
     lib.covspec_profile_stage_count.argtypes = []
     lib.covspec_profile_stage_name.argtypes = [C.c_int]
     lib.covspec_profile_stage_name.restype = C.c_char_p
+    _bind_native(lib)
     _lib = lib
     return lib
+
+
+_native = None
+
+
+def _bind_native(lib):
+    """Loads _binding.so, the native part of this binding, and gives it the library's functions."""
+    global _native
+    try:
+        from . import _binding
+    except ImportError as e:
+        raise RuntimeError("the native part of the binding is missing: build it with "
+                           "`python -m paper_2605_02218_b200.build`") from e
+    _binding.bind(*(C.cast(f, C.c_void_p).value for f in
+                    (lib.covspec_correct, lib.covspec_branch_candidates_host, lib.covspec_query_score_static)))
+    _native = _binding
 
 
 def default_config(**overrides) -> Config:
@@ -400,15 +417,14 @@ def query_score_static(X: torch.Tensor, Q: torch.Tensor, vis_offsets, txt_offset
     allocate device memory (a serving loop with a fully committed memory pool, a process whose
     allocator belongs to another framework).  The library call itself allocates nothing; pass
     `out` (float32, one element per visual token) to keep this wrapper allocation-free as well."""
-    lib = load_library()
+    if _native is None:
+        load_library()
     assert X.is_cuda and Q.is_cuda and X.is_contiguous() and Q.is_contiguous() and X.dtype == Q.dtype
-    vis, vis_p = _i32(vis_offsets)
-    txt, txt_p = _i32(txt_offsets)
+    vis = np.ascontiguousarray(vis_offsets, dtype=np.int32)
+    txt = np.ascontiguousarray(txt_offsets, dtype=np.int32)
     if out is None:
         out = torch.empty(int(vis[-1]), dtype=torch.float32, device=X.device)
-    dtype = COVSPEC_BF16 if X.dtype == torch.bfloat16 else COVSPEC_F32
-    st = lib.covspec_query_score_static(dtype, X.shape[1], len(vis) - 1, _ptr(X), vis_p, _ptr(Q),
-                                        txt_p, _ptr(out), _stream())
+    st = _native.static_score(X, Q, vis, txt, out)
     if st:
         raise CovspecError(st, "covspec_query_score_static")
     return out
@@ -422,26 +438,18 @@ def correct(z_draft: torch.Tensor, z_target: torch.Tensor, uniforms: torch.Tenso
     """covspec_correct: gating (Eq. 16-17), acceptance probability (Eq. 5) and the residual
     correction draw (Eq. 6) for every row of two logit matrices [rows, ld] (ld >= vocab).
     Returns (margin, gate, accept, resid_mass, token) device tensors."""
-    lib = _lib or load_library()
-    assert z_draft.is_cuda and z_draft.is_contiguous() and z_target.is_contiguous()
-    assert z_draft.shape == z_target.shape and z_draft.dtype == z_target.dtype
-    rows, ld = z_draft.shape
-    dev = z_draft.device
-    # five allocations (7.3 us; two that are cut into rows take 8.9) and plain integers for the addresses: on a drafted
-    # block of a few positions the call takes longer here than on the device
-    margin = torch.empty(rows, dtype=torch.float32, device=dev)
-    gate = torch.empty(rows, dtype=torch.int32, device=dev)
-    accept = torch.empty(rows, dtype=torch.float32, device=dev)
-    mass = torch.empty(rows, dtype=torch.float32, device=dev)
-    token = torch.empty(rows, dtype=torch.int32, device=dev)
-    st = lib.covspec_correct(_LOGIT_DTYPES[z_draft.dtype], rows, ld if vocab is None else vocab, ld, z_draft.data_ptr(),
-                             z_target.data_ptr(), None if drafted is None else drafted.data_ptr(),
-                             None if uniforms is None else uniforms.data_ptr(), gamma,
-                             margin.data_ptr(), gate.data_ptr(), accept.data_ptr(), mass.data_ptr(), token.data_ptr(),
-                             _raw_stream())
-    if st:
-        raise CovspecError(st, "covspec_correct")
-    return margin, gate, accept, mass, token
+    if _native is None:
+        load_library()
+    # native: on a drafted block of a few positions the call would take longer in Python than on the device
+    got = _native.correct(z_draft, z_target, uniforms, gamma, drafted, vocab)
+    if type(got) is tuple:
+        return got
+    if got is None:                      # not what the call takes: say why
+        assert z_draft.is_cuda and z_draft.is_contiguous() and z_target.is_contiguous()
+        assert z_draft.shape == z_target.shape and z_draft.dtype == z_target.dtype
+        rows, ld = z_draft.shape
+        raise TypeError(f"covspec_correct: {_LOGIT_DTYPES[z_draft.dtype]} logits with arguments that are no tensors")
+    raise CovspecError(got, "covspec_correct")
 
 
 def fanout(f0: int, rho: float, j: int) -> int:
@@ -458,6 +466,11 @@ def branch_candidates(z_draft: torch.Tensor, fanouts, drafted: Optional[torch.Te
     excluded.  `fanouts`: one int per row.  Returns (cand int32 device tensor, offsets numpy)."""
     lib = _lib or load_library()
     rows, ld = z_draft.shape
+    off = np.empty(rows + 1, dtype=np.int32)
+    got = _native.candidates(z_draft, fanouts, off, drafted, vocab)
+    if isinstance(got, torch.Tensor):
+        return got, off
+    # fan-outs that are no list of ints, and the fan-outs and row lengths that the host-offset form does not take (-3)
     vocab = ld if vocab is None else vocab
     f = np.asarray(fanouts, dtype=np.int64)
     assert len(f) == rows
@@ -468,7 +481,7 @@ def branch_candidates(z_draft: torch.Tensor, fanouts, drafted: Optional[torch.Te
     dtype, z, out = _LOGIT_DTYPES[z_draft.dtype], z_draft.data_ptr(), cand.data_ptr()
     y, stream = None if drafted is None else drafted.data_ptr(), _raw_stream()
     st = lib.covspec_branch_candidates_host(dtype, rows, vocab, ld, z, y, off.ctypes.data, most, out, stream)
-    if st == -3:                         # a fan-out or a row length that the host-offset form does not take
+    if st == -3:
         d_off = torch.from_numpy(off).to(z_draft.device)
         st = lib.covspec_branch_candidates(dtype, rows, vocab, ld, z, y, d_off.data_ptr(), most, out, stream)
     if st:

@@ -1,10 +1,12 @@
 """Builds libcovspec.so in-tree with nvcc for sm_100a (no torch extension machinery: the library
-is a plain C ABI loaded through ctypes)."""
+is a plain C ABI loaded through ctypes), and _binding.so, the native part of the Python binding, with g++ against
+torch's headers."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -12,6 +14,8 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcovspec.so")
 LIB_DEBUG = os.path.join(HERE, "libcovspec_debug.so")     # the same sources with -DCOVSPEC_DEBUG_BOUNDS
 SOURCES = ["covspec.cu"]
+BINDING = os.path.join(HERE, "_binding.so")
+BINDING_SOURCE = os.path.join(CSRC, "binding.cpp")
 
 
 def _newest(paths):
@@ -21,7 +25,7 @@ def _newest(paths):
 def needs_build(lib: str = LIB) -> bool:
     if not os.path.exists(lib):
         return True
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + \
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != os.path.basename(BINDING_SOURCE)] + \
            [os.path.join(ROOT, "include", "covspec.h")]
     return _newest(deps) > os.path.getmtime(lib)
 
@@ -29,6 +33,8 @@ def needs_build(lib: str = LIB) -> bool:
 def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False) -> str:
     """Builds the library if a source is newer than it.  debug_bounds=True builds the checked variant
     (libcovspec_debug.so): index-driven accesses test their index and report COVSPEC_ERR_BOUNDS."""
+    if not debug_bounds:
+        build_binding(force)
     LIB = LIB_DEBUG if debug_bounds else globals()["LIB"]
     if not force and not needs_build(LIB):
         return LIB
@@ -49,6 +55,26 @@ def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False
     if verbose:
         sys.stderr.write(res.stderr)
     return LIB
+
+
+def build_binding(force: bool = False) -> str:
+    if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING_SOURCE) <= os.path.getmtime(BINDING):
+        return BINDING
+    import torch
+    base = os.path.dirname(torch.__file__)
+    libs = os.path.join(base, "lib")
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-shared", "-fPIC", "-std=c++17",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", os.path.join(base, "include"), "-I", os.path.join(base, "include", "torch", "csrc", "api", "include"),
+           "-I", sysconfig.get_paths()["include"], "-I", os.path.join(cuda, "include"),
+           "-o", BINDING, BINDING_SOURCE, "-L", libs, "-lc10", "-lc10_cuda", "-ltorch", "-ltorch_cpu", "-ltorch_python",
+           "-Wl,-rpath," + libs]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+        raise RuntimeError("g++ failed building " + os.path.basename(BINDING))
+    return BINDING
 
 
 if __name__ == "__main__":
