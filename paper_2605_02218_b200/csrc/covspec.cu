@@ -682,6 +682,16 @@ int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cud
 }
 
 // ---- Eq. 10-12 -------------------------------------------------------------------------------
+// Estimates for the choice between the forms of Eq. 11: the snapshot stack by one background block per SM (1.8 TB/s) and the
+// relevance kernel (1.1 PFLOP/s).
+struct ActivityTimes { double stream_s, kernel_s; };
+ActivityTimes activity_times(const covspec_ctx* ctx) {
+  const covspec_config& cfg = ctx->cfg;
+  const double rows = (double)ctx->plan.total_vis;
+  return ActivityTimes{(cfg.act_layers + 1) * rows * cfg.d * ctx->esize / 1.8e12,
+                       2.0 * rows * (ctx->split_tc ? ctx->d3 : cfg.d) * ctx->P / 1.1e15};
+}
+
 // Eq. 11 on `s`: the full-rate kernel, or (background = true) the small persistent grid that runs
 // beside the relevance kernel.
 template <typename T>
@@ -694,11 +704,11 @@ int launch_activity(covspec_ctx* ctx, const covspec_problem* p, float* s_act, bo
   if (background) {
     int per_sm = cfg.activity_overlap;
     // One block per SM reads about 1.8 TB/s beside the relevance kernel; where that would end after the
-    // kernel (about 1.1 PFLOP/s) a second one is added (batch of 16 x 576 tokens, d = 2048: 115 -> 71 us).
+    // kernel a second one is added (batch of 16 x 576 tokens, d = 2048: 115 -> 71 us).
     // Where it ends before, a second block only slows the kernel down (video: 3570 -> 3940 us a call).
-    const double stream_s = (double)(cfg.act_layers + 1) * rowsX * cfg.d * ctx->esize / 1.8e12;
-    const double kernel_s = 2.0 * rowsX * (ctx->split_tc ? ctx->d3 : cfg.d) * ctx->P / 1.1e15;
-    if (per_sm == 1 && stream_s > kernel_s) per_sm = 2;
+    const ActivityTimes t = activity_times(ctx);
+    if (per_sm == 1 && t.stream_s > t.kernel_s) per_sm = 2;
+    if (cfg.act_layers > 8) per_sm = 1;                  // 40 registers a thread: two blocks would keep the kernel's CTA out
     unsigned grid = (unsigned)std::min<long long>((rowsX + 15) / 16, (long long)ctx->num_sms * per_sm);
     if (cfg.act_layers <= 4)
       activity_stream_kernel<T, 4><<<grid, 512, 0, s>>>(lp, cfg.act_layers, rowsX, cfg.d, s_act);

@@ -134,12 +134,14 @@ __device__ __forceinline__ void load8_stream(const __nv_bfloat16* p, float (&v)[
 // Eq. 11 as a background stream: the same arithmetic as activity_kernel, but a small persistent
 // grid (one or two blocks per SM, rows handed out round-robin) whose loads bypass L1 and are marked
 // evict-first in L2.  Few blocks matter: every resident block reserves 1 KB of the SM's shared
-// memory, and the relevance kernel's CTA fits beside at most two of them.  The fused call runs it beside the tensor-core relevance kernel, which leaves
+// memory, and the relevance kernel's CTA fits beside at most two of them, of 32 registers a thread (two blocks of 40 registers,
+// as six layers took with two iterations in flight, keep that CTA out until the stream has ended: 12 requests of 2987-5975
+// tokens, d = 3936, 1244 us a call with a smaller CTA, 1510 with this one).  The fused call runs it beside the tensor-core relevance kernel, which leaves
 // HBM almost idle and most issue slots free: at a fraction of the HBM rate the whole snapshot stack
 // is read before the relevance kernel ends, without evicting the operand tiles that kernel re-reads
 // from L2.
 template <typename T, int MAXL>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(512, MAXL <= 8 ? 4 : 3)
 activity_stream_kernel(LayerPtrs hs, int n_layers /* = act_layers */, long long rows, int d,
                        float* __restrict__ s_act) {
   const int lane = threadIdx.x & 31;
@@ -149,7 +151,7 @@ activity_stream_kernel(LayerPtrs hs, int n_layers /* = act_layers */, long long 
 #pragma unroll
     for (int l = 0; l < MAXL; ++l) acc[l] = 0.f;
     size_t base = (size_t)row * d;
-#pragma unroll 2
+#pragma unroll (MAXL <= 4 ? 2 : 1)
     for (int k = lane * 8; k < d; k += 256) {
       float prev[8], cur[8];
       load8_stream(reinterpret_cast<const T*>(hs.h[0]) + base + k, prev);
