@@ -749,6 +749,12 @@ int score_impl(covspec_ctx* ctx, const covspec_problem* p, float* s_query, float
   // context's side stream (fork here, join before the scores are fused).
   // The identity kernel reads X once and is done early: the full-rate activity kernel fills the SMs it leaves.
   bool overlap = (use_tc || identity_tc) && cfg.act_layers > 0 && cfg.activity_overlap > 0;
+  // Two background blocks per SM read 3.6 TB/s, the kernel that has the GPU to itself 6.3: a long stream beside a short
+  // relevance kernel (few heads) is faster after it.  In units of stream_s the first takes 0.5 and the second 0.29.
+  if (use_tc && cfg.activity_overlap == 1) {
+    const ActivityTimes t = activity_times(ctx);
+    if (t.stream_s > 150e-6 && t.kernel_s < 0.2 * t.stream_s) overlap = false;
+  }
   auto fork_activity = [&]() -> int {
     CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
     prof_mark(ctx, ST_ACTIVITY, 0, ctx->side);
