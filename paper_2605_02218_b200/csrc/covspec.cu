@@ -604,8 +604,8 @@ int launch_identity_tc(const void* X, const void* Q, long long rows_x, long long
   if ((st = make_map_bf16(&map_x, X, rows_x, d, prm.tile_rows))) return st;
   if ((st = make_map_bf16(&map_q, Q, rows_q, d, prm.n_cols))) return st;
   const int smem = prm.stages * prm.stage_bytes + slack + ident::kTailBytes + 1024;
-  ident::identity_tc_kernel<<<blocks, ident::kIdThreads, smem, s>>>(map_x, map_q, reqs, prm);
-  CUDA_TRY(cudaGetLastError());
+  CUDA_TRY(launch_clusters(1, status == nullptr, ident::identity_tc_kernel, dim3((unsigned)blocks), ident::kIdThreads, (size_t)smem, s,
+                           map_x, map_q, reqs, prm));
   CUDA_TRY(launch_dependent(ident::identity_exact_kernel, dim3((unsigned)((rows + 7) / 8)), 256, 0, s,
                             static_cast<const __nv_bfloat16*>(X), static_cast<const __nv_bfloat16*>(Q), inv_q, reqs, prm, d,
                             (int)first, (int)rows));

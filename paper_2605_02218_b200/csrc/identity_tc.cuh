@@ -196,6 +196,10 @@ identity_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // Without an activity stream beside it (no status word) the second kernel may come up already; its blocks would
+  // take that stream's places otherwise.  Not before this CTA has its TMEM: the next call's first kernel allocates too.
+  if (prm.status == nullptr) launch_dependents_now();
+  wait_for_previous_kernel();
 
   // tile_rows = 64: two blocks share a 128-token tile (the MMA still computes 128 rows: the upper 64 read whatever
   // follows in the ring and go nowhere)
@@ -383,6 +387,7 @@ identity_exact_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* 
                       int first, int rows) {
   const int row = first + (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
   wait_for_previous_kernel();
+  launch_dependents_now();
   if (row >= first + rows) return;
   const uint32_t code = __float_as_uint(prm.s_query[row]);
   if ((code & kCode) != kCode) return;                   // not finite
