@@ -124,8 +124,8 @@ __device__ __forceinline__ bool jacobi_sweeps(float* C, int ldc, int w, float s1
 // shuffle joins the sums and no barrier separates the rounds.  The search ends as soon as np - 1
 // consecutive rounds (every pair once) have passed without a rotation, wherever in a sweep that
 // happens.  A round is a chain of shared load, eight-term sums, shuffle, threshold and, where a pair
-// rotates, root, quotient, reciprocal root and store: w = 32 took 640 cycles a round on two warps with a
-// barrier per round.
+// rotates, two reciprocal roots and store: w = 32 took 640 cycles a round on two warps with a
+// barrier per round, 485 with root, quotient and reciprocal root, 445 now (packed sums as well: 505, their chain is the longer).
 __host__ __device__ __forceinline__ int ritz_row(int row) {      // place of a row inside its column
   return (row & 1) * 16 + (row & 2) * 4 + (row >> 2);
 }
@@ -171,26 +171,27 @@ __device__ __noinline__ bool jacobi_warp32(int c_off, int w, float s1, int max_s
     const float thr2 = fmaxf(1e-12f * al * be, abs2 * fminf(al, be));
     const bool rotate = active && g2 > thr2 && g2 > 1e-37f;
     if (__any_sync(0xffffffffu, rotate)) {
-      // tan of the rotation angle: t = sign(d g) 2|g| / (|d| + sqrt(d^2 + 4 g^2)), d = |b|^2 - |a|^2
-      // (hardware root, quotient and reciprocal root, a few units in the last place each: the
-      // rotation is orthogonal to float32 accuracy for whatever t comes out)
-      float d = be - al, r, t, c;
-      asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d * d + 4.f * g2));
-      asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(t) : "f"(2.f * ga), "f"(fabsf(d) + r));
-      if (d < 0.f) t = -t;
-      asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(c) : "f"(t * t + 1.f));
-      const float sn = t * c;
+      // with d = |b|^2 - |a|^2 and theta the smaller of the two angles that make the columns orthogonal:
+      // cos 2 theta = |d| / sqrt(d^2 + 4 g^2), sin 2 theta = sign(d) 2 g / sqrt(d^2 + 4 g^2), then the half-angle formulas
+      // (hardware reciprocal roots, a few units in the last place each: the rotation is orthogonal to float32
+      // accuracy up to those, and the columns' lengths are taken again when the vectors are written)
+      const float d = be - al;
+      float ih, ic;
+      asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(ih) : "f"(fmaf(d, d, 4.f * g2)));
+      const float c2 = ih > 0.f ? fmaf(0.5f * fabsf(d), ih, 0.5f) : 1.f;      // 0: the root is beyond the float32 range
+      asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(ic) : "f"(c2));
+      const float c = c2 * ic, sn = (d < 0.f ? -ga : ga) * ih * ic;
       if (rotate) {
+        const f32x2 cc = pack2(c, c), ss = pack2(sn, sn), ns = pack2(-sn, -sn);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          float ya[4], yb[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            ya[e] = c * xa[4 * q + e] - sn * xb[4 * q + e];
-            yb[e] = sn * xa[4 * q + e] + c * xb[4 * q + e];
-          }
-          ca[q] = make_float4(ya[0], ya[1], ya[2], ya[3]);
-          cb[q] = make_float4(yb[0], yb[1], yb[2], yb[3]);
+          float2 a01, a23, b01, b23;
+          const f32x2 x0 = pack2(xa[4 * q], xa[4 * q + 1]), x1 = pack2(xa[4 * q + 2], xa[4 * q + 3]);
+          const f32x2 y0 = pack2(xb[4 * q], xb[4 * q + 1]), y1 = pack2(xb[4 * q + 2], xb[4 * q + 3]);
+          a01 = unpack2(fma2(ns, y0, mul2(cc, x0))); a23 = unpack2(fma2(ns, y1, mul2(cc, x1)));
+          b01 = unpack2(fma2(cc, y0, mul2(ss, x0))); b23 = unpack2(fma2(cc, y1, mul2(ss, x1)));
+          ca[q] = make_float4(a01.x, a01.y, a23.x, a23.y);
+          cb[q] = make_float4(b01.x, b01.y, b23.x, b23.y);
         }
       }
       __syncwarp();

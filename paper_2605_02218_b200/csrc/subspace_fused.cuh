@@ -628,7 +628,9 @@ __device__ __noinline__ void team_ritz(const double* pbase, int nt, int p, int w
   }
   epi_sync();
   const float s1 = sqrtf(*s_scale);
-  if (conv_tol > 0.f && p < m) {
+  // `first` .. : the threads that look at the estimate
+  auto settled = [&](int first, int count) {
+    if (!(conv_tol > 0.f) || p >= m) return;
     // Has the iteration settled?  The basis vectors converge to eigenvectors in order, so
     // theta_k ~ sqrt(B'_kk) estimates the k-th eigenvalue of G and theta_min the first one left
     // out of the basis.  After q multiplications a kept direction k still carries about
@@ -640,14 +642,14 @@ __device__ __noinline__ void team_ritz(const double* pbase, int nt, int p, int w
     for (int i = lane; i < p; i += 32) tmin = fminf(tmin, dg[i]);
     tmin = warp_min(tmin);
     float worst = 0.f;
-    for (int i = et; i < r; i += kEpiThreads) {
+    for (int i = et - first; i < r; i += count) {
       float th = dg[i];
       if (th - tmin > 1e-3f * s1 && th > 0.f)
         worst = fmaxf(worst, 2.f * (th / s1) * __powf(tmin / th, (float)steps));
     }
     worst = warp_max(worst);
     if (lane == 0 && worst > conv_tol) atomicOr(status, kStatusNoConverge);
-  }
+  };
   const int nact = small ? 32 : min(kEpiThreads, ((((w + 1) >> 1) * 4) + 31) & ~31);
   if (et == 0) *s_flag = 0;
   epi_sync();
@@ -658,6 +660,9 @@ __device__ __noinline__ void team_ritz(const double* pbase, int nt, int p, int w
     else if (w <= 96) converged = jacobi_sweeps<24>(C, ldc, w, s1, max_sweeps, nact, s_flag);
     else converged = jacobi_sweeps<(kPMax + 3) / 4>(C, ldc, w, s1, max_sweeps, nact, s_flag);
     if (!converged && et == 0) atomicOr(status, kStatusNoConverge);
+    if (!small) settled(0, nact);
+  } else if (small) {
+    settled(32, kEpiThreads - 32);               // beside the rotations, which are one warp's
   }
   named_barrier(3, kEpiThreads);
   for (int k = warp; k < w; k += 8) {
