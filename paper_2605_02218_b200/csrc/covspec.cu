@@ -634,7 +634,8 @@ int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cud
   const int vis_heads = cfg.n_heads == 1 || n_pairs * cfg.n_heads <= n_clusters ? 1 : 2;
   const int query_rows = std::min(tc::kLogitN, (pl.t_max + 31) / 32 * 32) / 2;      // per CTA of a pair
   if ((st = make_map_bf16(&map_wk, Wk, P, d, vis_heads * tc::kHeadDim / 2))) return st;
-  if ((st = make_map_bf16(&map_q, Q, pl.total_txt, d, tc::kTileM))) return st;
+  const int tile_rows = (int)std::min<long long>(tc::kTileM, round_up(pl.total_txt, 8));
+  if ((st = make_map_bf16(&map_q, Q, pl.total_txt, d, tile_rows))) return st;
   if ((st = make_map_bf16(&map_wq, Wq, P, d, group_heads * tc::kHeadDim))) return st;
   if ((st = make_map_bf16(&map_qn, qn, pl.total_txt, P, query_rows))) return st;
   if ((st = make_map_bf16(&map_qnl, qn + lo_off, pl.total_txt, P, query_rows))) return st;
@@ -649,16 +650,10 @@ int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cud
   prm.n_items = q_tiles * prm.n_groups;
   prm.qn_out = qn; prm.qn_lo_off = lo_off;
   prm.fill = s_query; prm.fill_n = pl.total_vis;          // -inf for the visual-side launch below
-  // few items share their inner dimension among the CTAs of a cluster, as long as that leaves half the SMs
-  prm.split = 1;
-  if (group_heads == 1)
-    for (int sp = tc::kQuerySplitMax; sp > 1 && prm.split == 1; sp /= 2)
-      if (prm.n_items * sp <= ctx->num_sms / 2 && prm.k_chunks >= 4 * sp) prm.split = sp;
-  // In clusters of two where nothing is shared: they take both SMs of a pair, so that the other pairs are free for the visual
-  // side's clusters.
-  const int q_cluster = prm.split > 1 ? prm.split : 2;
-  int grid = prm.split > 1 ? prm.n_items * prm.split : 2 * std::min((prm.n_items + 1) / 2, n_clusters);
-  CUDA_TRY(launch_clusters(q_cluster, false, tc::query_embed_kernel, dim3(grid), 192, tc::kQuerySmem, s, map_q, map_wq, prm));
+  prm.tile_rows = tile_rows;
+  // in clusters of two: the CTAs take both SMs of a pair, so that the other pairs are free for the visual side's clusters
+  int grid = 2 * std::min((prm.n_items + 1) / 2, n_clusters);
+  CUDA_TRY(launch_clusters(2, false, tc::query_embed_kernel, dim3(grid), 192, tc::kQuerySmem, s, map_q, map_wq, prm));
   LAUNCH_CHECK(ctx);
   prof_mark(ctx, ST_QEMBED, 1, s);
   // visual side

@@ -6,9 +6,9 @@
 // (192 threads): warps 0-3 epilogue (one TMEM lane = one query element each), warp 4 TMA producer, warp 5 MMA
 // issuer and TMEM owner; two accumulators, so that the epilogue of an item runs beside the next one's main
 // loop.  Two 96 KB stages of two chunks instead of four of one were slower (15.0 -> 17.6 us at d = 2048).
-// With few items up to four CTAs of a cluster take a part of an item's inner dimension each and push their sums to the
-// first one: an item alone takes as long as its chain of chunks (512 cycles each, the time shared memory takes to write and read
-// one; one float32 request, 48 chunks: 17.2 -> 11.6 us).
+// An item takes as long as its chain of chunks, each the time shared memory takes to write and read it (512 cycles with one
+// head and 128 rows): where all query elements fit one tile, only their rows are loaded.  Sharing the inner dimension among
+// four CTAs gained about 1 us of a call with one request and moved scores by 1e-6, enough to exchange near-tied tokens.
 // Every mbarrier wait is bounded; on expiry the CTA raises a status bit, leaves its loops, frees TMEM and exits.
 #pragma once
 #include "tc_common.cuh"
@@ -33,17 +33,12 @@ constexpr int kQueryMaxStages = kQueryStages * kBytesStage / (kBytesA + kHeadDim
 // activity stream gather on few SMs, and the visual side's CTAs do not fit there until the stream has ended.
 constexpr int kQuerySmem = 225 * 1024;
 static_assert(kQueryStages * kBytesStage + 1024 <= kQuerySmem, "ring and barriers");
-// An item's first CTA receives the other CTAs' sums in its ring: [CTA - 1][group of 32 features][8 vectors of 4][128 rows].
-constexpr int kQuerySplitMax = 4;
-constexpr int kQueryPartBytes = kTileM * 32 * 4;
-static_assert((kQuerySplitMax - 1) * (kHeadDim / 32) * kQueryPartBytes <= kQueryStages * kBytesStage, "partial sums in the ring");
 
 struct QueryParams {
   int n_items;          // (128-row tile, group of heads) pairs
   int n_groups;         // groups of heads
   int group_heads;      // heads per item, 2 or 1
-  int split;            // CTAs (one cluster) that share an item's inner dimension; more than 1: one item of one head per
-                        // cluster
+  int tile_rows;        // rows that are loaded of a tile: 128, or fewer where one tile holds all query elements
   int n_heads;
   int k_chunks;         // ceil(d / 64)
   int P;                // n_heads * 128
@@ -134,22 +129,19 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
     }
   };
 
-  const int first_item = blockIdx.x / prm.split, stride = gridDim.x / prm.split, part = blockIdx.x % prm.split;
   const int stage_bytes = kBytesA + prm.group_heads * kHeadDim * kBK * 2, stages = kQueryStages * kBytesStage / stage_bytes;
-  const int per = (prm.k_chunks + prm.split - 1) / prm.split;
-  const int kc0 = part * per, kc1 = min(prm.k_chunks, kc0 + per);
 
   if (warp == 4) {
     // ---------------------------------------------------------------- TMA producer
     if (lane == 0) {
       uint32_t it = 0;
       bool ok = true;
-      for (int item = first_item; item < prm.n_items && ok; item += stride) {
+      for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x) {
         const int row0 = item / prm.n_groups * kTileM, head0 = item % prm.n_groups * prm.group_heads;
-        for (int kc = kc0; kc < kc1; ++kc, ++it) {
+        for (int kc = 0; kc < prm.k_chunks; ++kc, ++it) {
           const int s = it % stages;
           if (!(ok = mbar_wait(&empty[s], ((it / stages) & 1u) ^ 1u, abort_flag))) break;
-          mbar_expect_tx(&full[s], stage_bytes);
+          mbar_expect_tx(&full[s], stage_bytes - (kTileM - prm.tile_rows) * kBK * 2);
           const uint32_t dst = smem_u32(smem + s * stage_bytes);
           tma_load_2d(dst, &map_a, kc * kBK, row0, &full[s]);
           tma_load_2d(dst + kBytesA, &map_b, kc * kBK, head0 * kHeadDim, &full[s]);
@@ -162,14 +154,14 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
     if (lane == 0) {
       uint32_t it = 0, n = 0;
       bool ok = true;
-      for (int item = first_item; item < prm.n_items && ok; item += stride, ++n) {
+      for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x, ++n) {
         const uint32_t buf = n & 1u;
         if (!(ok = mbar_wait(&acc_empty[buf], ((n >> 1) & 1u) ^ 1u, abort_flag))) break;
         tc_fence_after();
         // a lone last head takes half the columns (see relevance_vis_kernel)
         const int head0 = item % prm.n_groups * prm.group_heads;
         const uint32_t idesc = umma_idesc(kTileM, min(prm.group_heads, prm.n_heads - head0) * kHeadDim);
-        for (int kc = kc0; kc < kc1; ++kc, ++it) {
+        for (int kc = 0; kc < prm.k_chunks; ++kc, ++it) {
           const int s = it % stages;
           if (!(ok = mbar_wait(&full[s], (it / stages) & 1u, abort_flag))) break;
           tc_fence_after();
@@ -177,18 +169,18 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
           const uint64_t adesc = umma_desc(addr), bdesc = umma_desc(addr + kBytesA);
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k)
-            umma_bf16(tmem_base + buf * kTileN, adesc + 2 * k, bdesc + 2 * k, idesc, (kc - kc0) | k);
+            umma_bf16(tmem_base + buf * kTileN, adesc + 2 * k, bdesc + 2 * k, idesc, (kc | k) != 0);
           umma_commit(&empty[s]);
         }
         if (ok) umma_commit(&acc_full[buf]);
       }
     }
     __syncwarp();
-  } else if (prm.split == 1) {
+  } else {
     // ---------------------------------------------------------------- epilogue (warps 0-3)
     uint32_t n = 0;
     bool ok = true;
-    for (int item = first_item; item < prm.n_items && ok; item += stride, ++n) {
+    for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x, ++n) {
       const int row0 = item / prm.n_groups * kTileM, head0 = item % prm.n_groups * prm.group_heads;
       const long long rem = prm.rows_total - row0;
       const uint32_t buf = n & 1u;
@@ -201,43 +193,6 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
       tc_fence_before();
       mbar_arrive(&acc_empty[buf]);
     }
-  } else {
-    if (!mbar_wait(&acc_full[0], 0, abort_flag)) atomicOr(prm.status, kStatusTimeout);
-    tc_fence_after();
-  }
-  if (prm.split > 1) {
-    // every CTA's products are complete and its ring is idle: the other CTAs push their sums to the first one, which adds
-    // them up in the order of the inner dimension
-    const int row0 = first_item / prm.n_groups * kTileM, head = first_item % prm.n_groups;
-    const long long rem = prm.rows_total - row0;
-    const int nrows = rem < kTileM ? (int)rem : kTileM;
-    const bool work = warp < 4 && warp * 32 < nrows;         // whole warps
-    __syncwarp();
-    cluster_sync_all();
-    if (work && part != 0) {
-#pragma unroll 1
-      for (int c4 = 0; c4 < kHeadDim / 32; ++c4) {
-        float v[32];
-        tmem_ld32(t_lane + c4 * 32, v);
-        const uint32_t dst = map_to_cta(smem + ((part - 1) * (kHeadDim / 32) + c4) * kQueryPartBytes + r * 16, 0);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) store_at(dst + q * kTileM * 16, v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-      }
-    }
-    __syncwarp();
-    cluster_sync_all();
-    if (work && part == 0 && *abort_flag == 0)
-      store_head(row0, nrows, head, [&](int c4, float (&v)[32]) {
-        tmem_ld32(t_lane + c4 * 32, v);
-        for (int c = 1; c < prm.split; ++c) {
-          const float4* src = reinterpret_cast<const float4*>(smem + ((c - 1) * (kHeadDim / 32) + c4) * kQueryPartBytes) + r;
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const float4 w = src[q * kTileM];
-            v[4 * q] += w.x; v[4 * q + 1] += w.y; v[4 * q + 2] += w.z; v[4 * q + 3] += w.w;
-          }
-        }
-      });
   }
 
   tc_fence_before();

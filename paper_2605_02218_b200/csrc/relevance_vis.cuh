@@ -48,7 +48,7 @@ constexpr int kVisHeadBytes = kHeadDim / 2 * kBK * 2;      // 8 KB: this CTA's h
 constexpr int kLogitN = 128;                              // query elements per logits tile (UMMA N of the 2nd product)
 constexpr int kQueryRing = 28 * 1024;
 constexpr int kMaxQuerySlots = 8;
-constexpr int kVisSmem = kVisRing + 4 * kBytesKp + kQueryRing + 1024 /*barriers*/ + 2048 /*exchange*/;
+constexpr int kVisSmem = kVisRing + 4 * kBytesKp + kQueryRing + 1024 /*barriers*/ + 1024 /*exchange*/;
 static_assert(kVisSmem <= kQuerySmem, "see kQuerySmem");
 
 // ---- two-CTA forms of the building blocks of tc_common.cuh ----
@@ -107,7 +107,7 @@ struct VisParams {
   int n_tiles;
   int n_items;          // (pair of tiles, group of heads) pairs
   int n_groups;         // groups of heads
-  int group_heads;      // heads per group, 2 or 1 (1: the weight map's boxes are 64 rows high instead of 128)
+  int group_heads;      // heads per group, 2 or 1 (the weight map's boxes are 64 rows high per head)
   int stages;           // of the main ring, kBytesA + group_heads * kVisHeadBytes each
   int n_heads;
   int k_chunks;         // ceil(d / 64)
@@ -140,7 +140,7 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
   uint64_t* kp_free = kp_ready + 1;                      // both
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(kp_free + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  float* exchange = reinterpret_cast<float*>(q_smem + kQueryRing + 1024);      // [2][norm, largest logit][128]
+  float* exchange = reinterpret_cast<float*>(q_smem + kQueryRing + 1024);      // [2][128] largest logit of the second thread
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
@@ -382,14 +382,14 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
       // largest product over the length (rounding keeps the order, so scaling after the maximum changes nothing)
       auto finish_head = [&](int h, float ss_h) {
         read_logits(h, ntt - 1);
-        float* x = exchange + ((head_it + (uint32_t)h) & 1u) * 256 + r;
-        if (part == 1) { x[0] = ss_h; x[128] = top; }
+        float* x = exchange + ((head_it + (uint32_t)h) & 1u) * 128 + r;
+        if (part == 1) *x = top;
         named_barrier(1, kVisEpiWarps * 32);
         if (part == 0) {
-          const float s = ss_h + x[0], o = x[128];
-          nonfinite |= o != o || top != top || !(s <= 3.402823466e38f);
+          const float o = *x;
+          nonfinite |= o != o || top != top || !(ss_h <= 3.402823466e38f);
           float inv = 0.f;
-          if (s > 1.17549435e-38f) { inv = rsqrtf(s); inv = inv * (1.5f - 0.5f * s * inv * inv); }
+          if (ss_h > 1.17549435e-38f) { inv = rsqrtf(ss_h); inv = inv * (1.5f - 0.5f * ss_h * inv * inv); }
           best = fmaxf(best, fmaxf(top, o) * inv);
         }
         top = -INFINITY;
@@ -421,6 +421,19 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
                 make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
             *reinterpret_cast<uint4*>(rowp + 2 * kBytesKp + chunk * 16) =
                 make_uint4(pl[4 * q], pl[4 * q + 1], pl[4 * q + 2], pl[4 * q + 3]);
+          }
+        }
+        if (part == 0) {
+          // the other half of the squared length: one thread adds up all features in their order
+#pragma unroll 1
+          for (int c2 = 0; c2 < 2; ++c2) {
+            float v[32];
+            tmem_ld32(cols + kHalf + c2 * 32, v);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+              float a = v[2 * e], b = v[2 * e + 1];
+              ss += a * a + b * b;
+            }
           }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
