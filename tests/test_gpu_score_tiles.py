@@ -1,6 +1,5 @@
 """Relevance kernel and Gram kernel at the edges of their work split: pairs of token tiles (odd numbers of tiles, pairs
-that belong to two requests), logits tiles of up to 128 query elements, items of one and two heads, the shared inner dimension
-of the query side, the shared columns of the Gram items, CTAs with many row tiles."""
+that belong to two requests), logits tiles of up to 128 query elements, items of one and two heads, the shared columns of the Gram items, CTAs with many row tiles."""
 import numpy as np
 import pytest
 import torch
@@ -30,7 +29,7 @@ def _query_scores(wl, path):
     ([128, 1, 300], [32, 33, 65], 3, 72),                           # pairs of two requests, a lone last head, a partial chunk
     ([130, 257, 64, 500, 127], [1, 128, 129, 300, 64], 2, 200),     # logits tiles of every width, up to three of them
     ([128 * 151 + 5], [40], 1, 64),                                 # more single-head items than clusters
-    ([576], [31], 16, 2048),                                        # one item per cluster; four CTAs share a query item
+    ([576], [31], 16, 2048),                                        # one item per cluster; a query tile of 31 rows
     ([700] * 9, [96, 97, 2, 64, 31, 160, 7, 128, 255], 7, 328),     # several items per cluster
 ])
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
@@ -74,3 +73,19 @@ def test_more_row_tiles_per_cta_than_are_looked_up_in_advance():
     wl = workloads.make_workload("many-tiles-per-cta", seed=33, dtype=torch.bfloat16, batch=2500, n_vis=(40, 90), n_txt=1, d=64,
                                  n_heads=1, rank=4, keep_ratio=0.2, act_layers=1)
     parity.run_gpu(wl, requests=[0, 1, 777, 1480, 2110, 2400, 2499])
+
+
+@pytest.mark.parametrize("layers,n,d", [(4, 16384, 2048),      # long enough for the stream to follow the relevance kernel
+                                        (10, 700, 256), (6, 3000, 1024), (4, 300, 264)])
+def test_activity_is_the_same_wherever_it_runs(layers, n, d):
+    wl = _workload("activity", [n], [9], d=d, n_heads=1, act_layers=layers)
+    got = []
+    for overlap in (0, 1, 2):
+        pr = api.Pruner.for_workload(wl, activity_overlap=overlap)
+        got.append([t.clone() for t in pr.score(pr.marshal(wl))])
+        assert pr.device_status() == 0
+        pr.close()
+    for other in got[1:]:
+        for a, b in zip(got[0], other):
+            assert torch.equal(a, b)
+
