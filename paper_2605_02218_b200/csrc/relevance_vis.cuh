@@ -12,13 +12,17 @@
 // so the projected embeddings never leave the SM.
 //
 // Why two SMs: a CTA fetches its own tokens and only its half of the weights, 32 KB per 64 features and 512 tensor
-// cycles.  One SM alone needs 48 KB for its 128 x 256 products, 96 bytes a cycle, and an SM gets about 64 from L2:
-// its main loop ran at two thirds of the tensor rate.  The query elements are shared the same way.
+// cycles.  The time of a chunk follows what shared memory writes and reads for it (128 bytes a cycle), whatever the depth
+// of the ring: 96 KB for the 128 x 256 products of one SM, 786 cycles measured, about 80 KB here, 725-750 (the tensor pipe is
+// busy 76 % of the time; 16,384 tokens, d = 3584, 28 heads: 308 us).  Under the power limit of long runs the kernel went
+// from 1.35 to 1.42 PFLOP/s.  The query elements are shared the same way.
 //
 // The second product and the epilogue of one item run beside the main loop of the next: TMEM holds two
 // accumulators of 256 columns, and the logits of a head take the place of that head's own columns, which have
 // been read by then.  The main loop, the logits and their operands have issuing threads of their own, so
 // nothing interleaves them but the tensor pipe; a head is restaged while the logits of the one before are read.
+// Below d = 2048 that chain is the longer one (per head 1.3 k cycles of restaging, 24 products of about 128 cycles each
+// whatever their width up to 128, the reading): 148 tiles, 16 heads, d = 256, 256 query elements 170 -> 104 us.
 // The tiles of a pair may belong to two requests (tiles are paired across the whole batch): such a pair goes
 // through the query elements of both, and each CTA looks at its own request's logits.
 //
