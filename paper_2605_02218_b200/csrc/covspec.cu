@@ -629,13 +629,13 @@ int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cud
   long long lo_off = (long long)cfg.max_total_txt * P;   // lo parts follow the hi parts
   int st;
   if ((st = make_map_bf16(&map_x, X, pl.total_vis, d, tc::kTileM))) return st;
-  // Visual side: one head per item while the items with one head leave no cluster more than one.
+  // Visual side: one head per item while the items with one head leave no cluster more than one (its main loop is the
+  // shorter then: 4 x 64 instead of 4 x 128 cycles of products per chunk).
   const int n_pairs = (pl.n_tiles + 1) / 2, n_clusters = ctx->num_sms / 2;
   const int vis_heads = cfg.n_heads == 1 || n_pairs * cfg.n_heads <= n_clusters ? 1 : 2;
   const int query_rows = std::min(tc::kLogitN, (pl.t_max + 31) / 32 * 32) / 2;      // per CTA of a pair
   if ((st = make_map_bf16(&map_wk, Wk, P, d, vis_heads * tc::kHeadDim / 2))) return st;
-  const int tile_rows = (int)std::min<long long>(tc::kTileM, round_up(pl.total_txt, 8));
-  if ((st = make_map_bf16(&map_q, Q, pl.total_txt, d, tile_rows))) return st;
+  if ((st = make_map_bf16(&map_q, Q, pl.total_txt, d, tc::kTileM))) return st;
   if ((st = make_map_bf16(&map_wq, Wq, P, d, group_heads * tc::kHeadDim))) return st;
   if ((st = make_map_bf16(&map_qn, qn, pl.total_txt, P, query_rows))) return st;
   if ((st = make_map_bf16(&map_qnl, qn + lo_off, pl.total_txt, P, query_rows))) return st;
@@ -650,7 +650,6 @@ int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cud
   prm.n_items = q_tiles * prm.n_groups;
   prm.qn_out = qn; prm.qn_lo_off = lo_off;
   prm.fill = s_query; prm.fill_n = pl.total_vis;          // -inf for the visual-side launch below
-  prm.tile_rows = tile_rows;
   // in clusters of two: the CTAs take both SMs of a pair, so that the other pairs are free for the visual side's clusters
   int grid = 2 * std::min((prm.n_items + 1) / 2, n_clusters);
   CUDA_TRY(launch_clusters(2, false, tc::query_embed_kernel, dim3(grid), 192, tc::kQuerySmem, s, map_q, map_wq, prm));

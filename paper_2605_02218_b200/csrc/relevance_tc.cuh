@@ -6,9 +6,9 @@
 // (192 threads): warps 0-3 epilogue (one TMEM lane = one query element each), warp 4 TMA producer, warp 5 MMA
 // issuer and TMEM owner; two accumulators, so that the epilogue of an item runs beside the next one's main
 // loop.  Two 96 KB stages of two chunks instead of four of one were slower (15.0 -> 17.6 us at d = 2048).
-// An item takes as long as its chain of chunks, each the time shared memory takes to write and read it (512 cycles with one
-// head and 128 rows): where all query elements fit one tile, only their rows are loaded.  Sharing the inner dimension among
-// four CTAs gained about 1 us of a call with one request and moved scores by 1e-6, enough to exchange near-tied tokens.
+// An item takes as long as its chain of chunks (about 500 cycles each with one head).  Sharing the inner dimension among
+// four CTAs gained about 1 us of a call with one request and moved scores by 1e-6, enough to exchange near-tied tokens;
+// loading only the rows that a lone tile has gained nothing.
 // Every mbarrier wait is bounded; on expiry the CTA raises a status bit, leaves its loops, frees TMEM and exits.
 #pragma once
 #include "tc_common.cuh"
@@ -38,7 +38,6 @@ struct QueryParams {
   int n_items;          // (128-row tile, group of heads) pairs
   int n_groups;         // groups of heads
   int group_heads;      // heads per item, 2 or 1
-  int tile_rows;        // rows that are loaded of a tile: 128, or fewer where one tile holds all query elements
   int n_heads;
   int k_chunks;         // ceil(d / 64)
   int P;                // n_heads * 128
@@ -134,17 +133,18 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
   if (warp == 4) {
     // ---------------------------------------------------------------- TMA producer
     if (lane == 0) {
-      uint32_t it = 0;
+      int s = 0;
+      uint32_t ph = 1;
       bool ok = true;
       for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x) {
         const int row0 = item / prm.n_groups * kTileM, head0 = item % prm.n_groups * prm.group_heads;
-        for (int kc = 0; kc < prm.k_chunks; ++kc, ++it) {
-          const int s = it % stages;
-          if (!(ok = mbar_wait(&empty[s], ((it / stages) & 1u) ^ 1u, abort_flag))) break;
-          mbar_expect_tx(&full[s], stage_bytes - (kTileM - prm.tile_rows) * kBK * 2);
+        for (int kc = 0; kc < prm.k_chunks; ++kc) {
+          if (!(ok = mbar_wait(&empty[s], ph, abort_flag))) break;
+          mbar_expect_tx(&full[s], stage_bytes);
           const uint32_t dst = smem_u32(smem + s * stage_bytes);
           tma_load_2d(dst, &map_a, kc * kBK, row0, &full[s]);
           tma_load_2d(dst + kBytesA, &map_b, kc * kBK, head0 * kHeadDim, &full[s]);
+          if (++s == stages) { s = 0; ph ^= 1u; }
         }
       }
     }
@@ -152,7 +152,8 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
   } else if (warp == 5) {
     // ---------------------------------------------------------------- MMA issuer
     if (lane == 0) {
-      uint32_t it = 0, n = 0;
+      int s = 0;
+      uint32_t ph = 0, n = 0;
       bool ok = true;
       for (int item = blockIdx.x; item < prm.n_items && ok; item += gridDim.x, ++n) {
         const uint32_t buf = n & 1u;
@@ -161,9 +162,8 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
         // a lone last head takes half the columns (see relevance_vis_kernel)
         const int head0 = item % prm.n_groups * prm.group_heads;
         const uint32_t idesc = umma_idesc(kTileM, min(prm.group_heads, prm.n_heads - head0) * kHeadDim);
-        for (int kc = 0; kc < prm.k_chunks; ++kc, ++it) {
-          const int s = it % stages;
-          if (!(ok = mbar_wait(&full[s], (it / stages) & 1u, abort_flag))) break;
+        for (int kc = 0; kc < prm.k_chunks; ++kc) {
+          if (!(ok = mbar_wait(&full[s], ph, abort_flag))) break;
           tc_fence_after();
           const uint32_t addr = smem_u32(smem + s * stage_bytes);
           const uint64_t adesc = umma_desc(addr), bdesc = umma_desc(addr + kBytesA);
@@ -171,6 +171,7 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
           for (int k = 0; k < kBK / 16; ++k)
             umma_bf16(tmem_base + buf * kTileN, adesc + 2 * k, bdesc + 2 * k, idesc, (kc | k) != 0);
           umma_commit(&empty[s]);
+          if (++s == stages) { s = 0; ph ^= 1u; }
         }
         if (ok) umma_commit(&acc_full[buf]);
       }
