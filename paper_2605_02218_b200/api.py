@@ -411,6 +411,31 @@ class Pruner:
             raise CovspecError(st, "device status")
 
 
+def _addr(t, name: str, dtype: torch.dtype, device: torch.device, least: int):
+    """The address of a tensor that kernels on `device` read or write `least` elements of `dtype` from: the
+    library takes addresses only, so what does not fit is refused here.  Pinned host memory is within a kernel's
+    reach too.  None stays None."""
+    if t is None:
+        return None
+    if not isinstance(t, torch.Tensor):
+        raise TypeError(f"{name}: a tensor is required, not {type(t).__name__}")
+    if t.dtype != dtype:
+        raise TypeError(f"{name}: {dtype} is required, not {t.dtype}")
+    if t.device != device and not (t.device.type == "cpu" and t.is_pinned()):
+        raise ValueError(f"{name}: on {t.device}, the call is on {device}")
+    if not t.is_contiguous():
+        raise ValueError(f"{name}: a contiguous tensor is required")
+    if t.numel() < least:
+        raise ValueError(f"{name}: {t.numel()} elements, {least} are used")
+    return t.data_ptr()
+
+
+def _c_int(v, name: str) -> int:
+    if not -2 ** 31 <= v < 2 ** 31:
+        raise ValueError(f"{name}: {v} is no 32-bit integer")
+    return v
+
+
 def query_score_static(X: torch.Tensor, Q: torch.Tensor, vis_offsets, txt_offsets,
                        out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """covspec_query_score_static: Eq. 10 with the identity embedding for callers that must not
@@ -425,9 +450,30 @@ def query_score_static(X: torch.Tensor, Q: torch.Tensor, vis_offsets, txt_offset
     if out is None:
         out = torch.empty(int(vis[-1]), dtype=torch.float32, device=X.device)
     st = _native.static_score(X, Q, vis, txt, out)
+    if st is None:
+        st = _static_score(X, Q, vis, txt, out)
     if st:
         raise CovspecError(st, "covspec_query_score_static")
     return out
+
+
+def _static_score(X, Q, vis, txt, out) -> int:
+    """The call for arguments of every kind that the library can take; says what is wrong with others."""
+    if X.dtype not in (torch.bfloat16, torch.float32):
+        raise TypeError(f"X: bfloat16 or float32 is required, not {X.dtype}")
+    d = _c_int(X.shape[1], "d")
+    if Q.shape[1] != d:
+        raise ValueError(f"Q: {Q.shape[1]} features, X has {d}")
+    if vis.size < 2 or vis.size != txt.size:
+        raise ValueError(f"{vis.size} and {txt.size} offsets: one more than requests is required of both")
+    rows_x, rows_q = int(vis[-1]), int(txt[-1])      # the library refuses offsets that do not ascend from 0
+    ip = C.POINTER(C.c_int)
+    with torch.cuda.device(X.device):
+        return load_library().covspec_query_score_static(
+            COVSPEC_BF16 if X.dtype == torch.bfloat16 else COVSPEC_F32, d, vis.size - 1,
+            _addr(X, "X", X.dtype, X.device, rows_x * d), vis.ctypes.data_as(ip),
+            _addr(Q, "Q", X.dtype, X.device, rows_q * d), txt.ctypes.data_as(ip),
+            _addr(out, "out", torch.float32, X.device, rows_x), _stream())
 
 
 _LOGIT_DTYPES = {torch.float32: COVSPEC_F32, torch.bfloat16: COVSPEC_BF16, torch.float16: COVSPEC_F16}
@@ -444,12 +490,29 @@ def correct(z_draft: torch.Tensor, z_target: torch.Tensor, uniforms: torch.Tenso
     got = _native.correct(z_draft, z_target, uniforms, gamma, drafted, vocab)
     if type(got) is tuple:
         return got
-    if got is None:                      # not what the call takes: say why
-        assert z_draft.is_cuda and z_draft.is_contiguous() and z_target.is_contiguous()
-        assert z_draft.shape == z_target.shape and z_draft.dtype == z_target.dtype
-        rows, ld = z_draft.shape
-        raise TypeError(f"covspec_correct: {_LOGIT_DTYPES[z_draft.dtype]} logits with arguments that are no tensors")
-    raise CovspecError(got, "covspec_correct")
+    if got is not None:
+        raise CovspecError(got, "covspec_correct")
+    return _correct(z_draft, z_target, uniforms, gamma, drafted, vocab)
+
+
+def _correct(z_draft, z_target, uniforms, gamma, drafted, vocab):
+    """The call for arguments of every kind that the library can take; says what is wrong with others."""
+    assert z_draft.is_cuda and z_draft.is_contiguous() and z_target.is_contiguous()
+    assert z_draft.shape == z_target.shape and z_draft.dtype == z_target.dtype
+    rows, ld = z_draft.shape
+    dtype, dev = _LOGIT_DTYPES[z_draft.dtype], z_draft.device
+    vocab = ld if vocab is None else _c_int(vocab, "vocab")
+    zt = _addr(z_target, "z_target", z_draft.dtype, dev, z_draft.numel())
+    y, u = _addr(drafted, "drafted", torch.int32, dev, rows), _addr(uniforms, "uniforms", torch.float32, dev, rows)
+    margin, accept, mass = (torch.empty(rows, dtype=torch.float32, device=dev) for _ in range(3))
+    gate, token = (torch.empty(rows, dtype=torch.int32, device=dev) for _ in range(2))
+    with torch.cuda.device(dev):
+        st = load_library().covspec_correct(dtype, _c_int(rows, "rows"), vocab, ld, z_draft.data_ptr(), zt, y, u, gamma,
+                                            margin.data_ptr(), gate.data_ptr(), accept.data_ptr(), mass.data_ptr(),
+                                            token.data_ptr(), _stream())
+    if st:
+        raise CovspecError(st, "covspec_correct")
+    return margin, gate, accept, mass, token
 
 
 def fanout(f0: int, rho: float, j: int) -> int:
@@ -471,19 +534,24 @@ def branch_candidates(z_draft: torch.Tensor, fanouts, drafted: Optional[torch.Te
     if isinstance(got, torch.Tensor):
         return got, off
     # fan-outs that are no list of ints, and the fan-outs and row lengths that the host-offset form does not take (-3)
-    vocab = ld if vocab is None else vocab
+    if not z_draft.is_cuda:
+        raise ValueError(f"z_draft: on {z_draft.device}, a CUDA device is required")
+    dtype, dev = _LOGIT_DTYPES[z_draft.dtype], z_draft.device
+    z = _addr(z_draft, "z_draft", z_draft.dtype, dev, 0)
+    y = _addr(drafted, "drafted", torch.int32, dev, rows)
+    vocab = ld if vocab is None else _c_int(vocab, "vocab")
     f = np.asarray(fanouts, dtype=np.int64)
     assert len(f) == rows
     off = np.zeros(rows + 1, dtype=np.int32)
     np.cumsum(f, out=off[1:])
     total, most = int(off[-1]), int(f.max()) if rows else 0
-    cand = torch.empty(max(total, 1), dtype=torch.int32, device=z_draft.device)
-    dtype, z, out = _LOGIT_DTYPES[z_draft.dtype], z_draft.data_ptr(), cand.data_ptr()
-    y, stream = None if drafted is None else drafted.data_ptr(), _raw_stream()
-    st = lib.covspec_branch_candidates_host(dtype, rows, vocab, ld, z, y, off.ctypes.data, most, out, stream)
-    if st == -3:
-        d_off = torch.from_numpy(off).to(z_draft.device)
-        st = lib.covspec_branch_candidates(dtype, rows, vocab, ld, z, y, d_off.data_ptr(), most, out, stream)
+    cand = torch.empty(max(total, 1), dtype=torch.int32, device=dev)
+    with torch.cuda.device(dev):
+        args = (dtype, _c_int(rows, "rows"), vocab, ld, z, y)
+        st = lib.covspec_branch_candidates_host(*args, off.ctypes.data, most, cand.data_ptr(), _stream())
+        if st == -3:
+            d_off = torch.from_numpy(off).to(dev)
+            st = lib.covspec_branch_candidates(*args, d_off.data_ptr(), most, cand.data_ptr(), _stream())
     if st:
         raise CovspecError(st, "covspec_branch_candidates")
     return (cand if total else cand[:0]), off

@@ -1,7 +1,9 @@
 // Native part of the Python binding (api.py) for the calls that are shorter on the device than their submission from Python:
-// the result tensors, the addresses and the call into the library in one step.  Everything that is not the usual case
-// (other argument types, errors) goes back to Python.  The library's functions are handed over as addresses by api.py, so
-// that they come from the library it has loaded (bind).
+// the checks, the result tensors, the addresses and the call into the library in one step.  The library sees addresses only,
+// so every tensor is held against what the kernels will read or write of it.  Everything that is not the usual case (other
+// argument types, tensors that do not fit, another device than the current one) goes back to Python, which says what is wrong
+// or makes the call itself.  The library's functions are handed over as addresses by api.py, so that they come from the
+// library it has loaded (bind).
 #include <Python.h>
 
 #include <ATen/ops/empty.h>
@@ -10,7 +12,7 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
-#include <vector>
+#include <climits>
 
 namespace {
 
@@ -40,6 +42,13 @@ int dtype_code(const at::Tensor& t) {
     default: return -1;
   }
 }
+// Dense memory of at least `least` elements of this type on the call's device.
+bool fits(const at::Tensor& t, at::ScalarType type, const at::Device& dev, long long least) {
+  return t.device() == dev && t.scalar_type() == type && t.is_contiguous() && t.numel() >= least;
+}
+// The call's tensors lie on the current device, whose stream takes the launch.
+bool on_current_device(const at::Tensor& t) { return t.is_cuda() && t.device().index() == c10::cuda::current_device(); }
+bool is_int(long long v) { return v >= INT_MIN && v <= INT_MAX; }
 bool int_arg(PyObject* o, long long& v) {
   v = PyLong_AsLongLong(o);
   return !(v == -1 && PyErr_Occurred());
@@ -69,22 +78,26 @@ int call(F f, A... args) {
 }
 void* current_stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
-// correct(z_draft, z_target, uniforms or None, gamma, drafted or None, vocab) -> (status, margin, gate, accept, mass, token);
-// None where an argument is not what the Python function's checks let through.
+// correct(z_draft, z_target, uniforms or None, gamma, drafted or None, vocab) -> (margin, gate, accept, mass, token), or the
+// library's status; None where an argument is not of the usual kind.
 PyObject* correct(PyObject*, PyObject* const* a, Py_ssize_t n) {
   HANDLE_TH_ERRORS
   if (n != 6 || !THPVariable_Check(a[0]) || !THPVariable_Check(a[1]) || !(a[2] == Py_None || THPVariable_Check(a[2])) ||
       !(a[4] == Py_None || THPVariable_Check(a[4])))
     Py_RETURN_NONE;
   const at::Tensor &zd = THPVariable_Unpack(a[0]), &zt = THPVariable_Unpack(a[1]);
-  if (!zd.is_cuda() || zd.dim() != 2 || !zd.is_contiguous() || !zt.is_contiguous() || !zd.sizes().equals(zt.sizes()) ||
-      zd.scalar_type() != zt.scalar_type() || dtype_code(zd) < 0)
+  if (!on_current_device(zd) || zd.dim() != 2 || !zd.is_contiguous() || dtype_code(zd) < 0 || !zd.sizes().equals(zt.sizes()) ||
+      !fits(zt, zd.scalar_type(), zd.device(), zd.numel()))
+    Py_RETURN_NONE;
+  const long long rows = zd.size(0), ld = zd.size(1);
+  if ((a[2] != Py_None && !fits(THPVariable_Unpack(a[2]), at::kFloat, zd.device(), rows)) ||
+      (a[4] != Py_None && !fits(THPVariable_Unpack(a[4]), at::kInt, zd.device(), rows)))
     Py_RETURN_NONE;
   const double gamma = PyFloat_AsDouble(a[3]);
   if (gamma == -1.0 && PyErr_Occurred()) return nullptr;
-  const long long rows = zd.size(0), ld = zd.size(1);
   long long vocab = ld;
   if (a[5] != Py_None && !int_arg(a[5], vocab)) return nullptr;
+  if (!is_int(vocab) || !is_int(rows)) Py_RETURN_NONE;
   const auto f32 = zd.options().dtype(at::kFloat), i32 = zd.options().dtype(at::kInt);
   at::Tensor margin = at::empty({rows}, f32), gate = at::empty({rows}, i32), accept = at::empty({rows}, f32),
              mass = at::empty({rows}, f32), token = at::empty({rows}, i32);
@@ -112,13 +125,15 @@ PyObject* candidates(PyObject*, PyObject* const* a, Py_ssize_t n) {
   HANDLE_TH_ERRORS
   if (n != 5 || !THPVariable_Check(a[0]) || !PyList_CheckExact(a[1]) || !(a[3] == Py_None || THPVariable_Check(a[3]))) Py_RETURN_NONE;
   const at::Tensor& z = THPVariable_Unpack(a[0]);
-  if (z.dim() != 2 || dtype_code(z) < 0) Py_RETURN_NONE;
+  if (!on_current_device(z) || z.dim() != 2 || !z.is_contiguous() || dtype_code(z) < 0) Py_RETURN_NONE;
   const long long rows = z.size(0), ld = z.size(1);
+  if (a[3] != Py_None && !fits(THPVariable_Unpack(a[3]), at::kInt, z.device(), rows)) Py_RETURN_NONE;
   IntArray off;
   if (!off.get(a[2], true)) return nullptr;
   if (PyList_GET_SIZE(a[1]) != rows || off.size() != rows + 1 || rows < 1) Py_RETURN_NONE;
   long long vocab = ld, total = 0, most = 0;
   if (a[4] != Py_None && !int_arg(a[4], vocab)) return nullptr;
+  if (!is_int(vocab) || !is_int(rows)) Py_RETURN_NONE;
   off.data()[0] = 0;
   for (long long r = 0; r < rows; ++r) {
     PyObject* item = PyList_GET_ITEM(a[1], r);
@@ -140,18 +155,23 @@ PyObject* candidates(PyObject*, PyObject* const* a, Py_ssize_t n) {
   END_HANDLE_TH_ERRORS
 }
 
-// static_score(X, Q, vis, txt: int32 arrays, out) -> the library's status
+// static_score(X, Q, vis, txt: int32 arrays, out) -> the library's status; None where an argument is not of the usual kind.
 PyObject* static_score(PyObject*, PyObject* const* a, Py_ssize_t n) {
   HANDLE_TH_ERRORS
-  if (n != 5 || !THPVariable_Check(a[0]) || !THPVariable_Check(a[1]) || !THPVariable_Check(a[4])) {
-    PyErr_SetString(PyExc_TypeError, "tensors required");
-    return nullptr;
-  }
+  if (n != 5 || !THPVariable_Check(a[0]) || !THPVariable_Check(a[1]) || !THPVariable_Check(a[4])) Py_RETURN_NONE;
   IntArray vis, txt;
   if (!vis.get(a[2], false) || !txt.get(a[3], false)) return nullptr;
   const at::Tensor &x = THPVariable_Unpack(a[0]), &q = THPVariable_Unpack(a[1]), &out = THPVariable_Unpack(a[4]);
-  const int st = call(g_static, x.scalar_type() == at::kBFloat16 ? 1 : 0, (int)x.size(1), (int)vis.size() - 1, x.data_ptr(), vis.data(),
-                          q.data_ptr(), txt.data(), static_cast<float*>(out.data_ptr()), current_stream());
+  const at::ScalarType type = x.scalar_type();
+  if (!on_current_device(x) || (type != at::kBFloat16 && type != at::kFloat) || x.dim() != 2 || q.dim() != 2 || x.size(1) != q.size(1) ||
+      !is_int(x.size(1)) || vis.size() < 2 || vis.size() != txt.size() || !is_int(vis.size()))
+    Py_RETURN_NONE;
+  // the library refuses offsets that do not ascend from 0, so the last ones say what is read
+  const long long d = x.size(1), rows_x = vis.data()[vis.size() - 1], rows_q = txt.data()[txt.size() - 1];
+  if (!fits(x, type, x.device(), rows_x * d) || !fits(q, type, x.device(), rows_q * d) || !fits(out, at::kFloat, x.device(), rows_x))
+    Py_RETURN_NONE;
+  const int st = call(g_static, type == at::kBFloat16 ? 1 : 0, (int)d, (int)vis.size() - 1, x.data_ptr(), vis.data(), q.data_ptr(),
+                      txt.data(), static_cast<float*>(out.data_ptr()), current_stream());
   return PyLong_FromLong(st);
   END_HANDLE_TH_ERRORS
 }

@@ -55,3 +55,79 @@ def test_fanouts_of_every_form_give_the_same_candidates(vocab, fan):
     with pytest.raises(api.CovspecError) as e:
         api.branch_candidates(d["z_draft"], [-1, 2, 2], d["drafted"], vocab=d["vocab"])
     assert e.value.status == -2
+
+
+def _z(rows=4, ld=64, dtype=torch.float16):
+    return torch.zeros(rows, ld, dtype=dtype, device="cuda:0")
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("error,kw", [
+    (TypeError, dict(uniforms=lambda: torch.zeros(4, dtype=torch.float64, device="cuda:0"))),
+    (TypeError, dict(uniforms=lambda: [0.0] * 4)),
+    (ValueError, dict(uniforms=lambda: torch.zeros(4))),                              # not on the device
+    (ValueError, dict(uniforms=lambda: torch.zeros(3, device="cuda:0"))),             # too short
+    (ValueError, dict(uniforms=lambda: torch.zeros(1, device="cuda:0").expand(4))),   # no dense memory
+    (TypeError, dict(drafted=lambda: torch.zeros(4, dtype=torch.int64, device="cuda:0"))),
+    (ValueError, dict(drafted=lambda: torch.zeros(4, dtype=torch.int32))),
+    (ValueError, dict(drafted=lambda: torch.zeros(3, dtype=torch.int32, device="cuda:0"))),
+    (ValueError, dict(drafted=lambda: torch.zeros(8, dtype=torch.int32, device="cuda:0")[::2])),
+    (ValueError, dict(z_target=lambda: _z().cpu())),
+    (ValueError, dict(vocab=lambda: 2 ** 32 + 32)),
+])
+def test_correct_refuses_memory_that_the_kernel_must_not_read(error, kw):
+    # all of these return before anything is launched
+    args = dict(z_draft=_z(), z_target=_z(), uniforms=torch.zeros(4, device="cuda:0"), gamma=0.02,
+                drafted=torch.zeros(4, dtype=torch.int32, device="cuda:0"))
+    with pytest.raises(error):
+        api.correct(**{**args, **{k: make() for k, make in kw.items()}})
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("fans", [[2] * 4, (2,) * 4])                   # the native call and the general one
+@pytest.mark.parametrize("error,kw", [
+    (ValueError, dict(z_draft=lambda: _z().cpu())),
+    (ValueError, dict(z_draft=lambda: _z(4, 128)[:, :64])),              # rows are not back to back
+    (KeyError, dict(z_draft=lambda: _z(dtype=torch.float64))),
+    (TypeError, dict(drafted=lambda: torch.zeros(4, dtype=torch.int64, device="cuda:0"))),
+    (ValueError, dict(drafted=lambda: torch.zeros(3, dtype=torch.int32, device="cuda:0"))),
+    (ValueError, dict(drafted=lambda: torch.zeros(4, dtype=torch.int32))),
+    (ValueError, dict(vocab=lambda: 2 ** 32 + 32)),
+])
+def test_candidates_refuse_memory_that_the_kernel_must_not_read(error, kw, fans):
+    args = dict(z_draft=_z(), fanouts=fans, drafted=torch.zeros(4, dtype=torch.int32, device="cuda:0"))
+    with pytest.raises(error):
+        api.branch_candidates(**{**args, **{k: make() for k, make in kw.items()}})
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("error,kw", [
+    (TypeError, dict(X=lambda: _z(), Q=lambda: _z())),                   # float16
+    (ValueError, dict(Q=lambda: torch.zeros(4, 32, device="cuda:0"))),   # another width
+    (ValueError, dict(vis_offsets=lambda: [0, 5])),                      # past the end of X
+    (ValueError, dict(txt_offsets=lambda: [0, 5])),
+    (ValueError, dict(vis_offsets=lambda: [0, 2, 4])),                   # more requests than in the other list
+    (ValueError, dict(vis_offsets=lambda: [4], txt_offsets=lambda: [4])),
+    (TypeError, dict(out=lambda: torch.zeros(4, dtype=torch.bfloat16, device="cuda:0"))),
+    (ValueError, dict(out=lambda: torch.zeros(3, device="cuda:0"))),
+    (ValueError, dict(out=lambda: torch.zeros(4))),
+    (ValueError, dict(out=lambda: torch.zeros(8, device="cuda:0")[::2])),
+])
+def test_static_score_refuses_memory_that_the_kernel_must_not_touch(error, kw):
+    args = dict(X=_z(dtype=torch.float32), Q=_z(dtype=torch.float32), vis_offsets=[0, 4], txt_offsets=[0, 4])
+    with pytest.raises(error):
+        api.query_score_static(**{**args, **{k: make() for k, make in kw.items()}})
+
+
+@pytest.mark.gpu
+def test_pinned_host_memory_is_taken_and_gives_the_same():
+    d = workloads.make_logits(seed=3, rows=4, vocab=1000, dtype=torch.float16, device="cuda:0")
+    z, y = d["z_draft"], d["drafted"]
+    want = api.correct(z, d["z_target"], d["uniforms"], 0.02, y, vocab=1000)
+    got = api.correct(z, d["z_target"], d["uniforms"].cpu().pin_memory(), 0.02, y.cpu().pin_memory(), vocab=1000)
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(want, got))
+    want, off = api.branch_candidates(z, [3, 2, 1, 0], y, vocab=1000)
+    got, off2 = api.branch_candidates(z, [3, 2, 1, 0], y.cpu().pin_memory(), vocab=1000)
+    torch.cuda.synchronize()
+    assert torch.equal(want, got) and np.array_equal(off, off2)
