@@ -266,7 +266,7 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
         const Item it = decode(item);
         const int ntt = it.tiles0 + it.tiles1;
         for (int h = 0; h < it.heads && ok; ++h, ++head_it) {
-          if (!(ok = mbar_wait(kp_ready, head_it & 1u, abort_flag))) break;      // both CTAs have restaged this head
+          if (!(ok = mbar_wait_cluster(kp_ready, head_it & 1u, abort_flag))) break;      // both CTAs have restaged this head
           const uint32_t kp_addr = smem_u32(kp_smem);
           const uint32_t d_col = tmem_base + (n & 1u) * kTileN + h * kHeadDim;
           for (int i = 0; i < ntt && ok; ++i, ++lt) {
@@ -443,7 +443,7 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_at(l_kp_ready);
+        if (lane == 0) mbar_arrive_release_at(l_kp_ready);
         if (h > 0) finish_head(h - 1, ss_before);
         for (int i = 0; i + 1 < ntt; ++i) read_logits(h, i);
       }

@@ -41,18 +41,39 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// The same for arrivals with release semantics at cluster scope (mbar_arrive_release_at).
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 // Bounded wait.  Returns false when `limit` polls expired or another role already gave up.
-__device__ __forceinline__ bool mbar_wait_limited(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                                  uint32_t limit) {
+template <typename Poll>
+__device__ __forceinline__ bool wait_limited(Poll poll, volatile int* abort_flag, uint32_t limit) {
   for (uint32_t i = 0; i < limit; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (poll()) return true;
     if ((i & 255u) == 255u && *abort_flag) return false;
   }
   *abort_flag = 1;
   return false;
 }
+__device__ __forceinline__ bool mbar_wait_limited(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                                  uint32_t limit) {
+  return wait_limited([&] { return mbar_try_wait(bar, parity); }, abort_flag, limit);
+}
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
   return mbar_wait_limited(bar, parity, abort_flag, kSpinLimit);
+}
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  return wait_limited([&] { return mbar_try_wait_cluster(bar, parity); }, abort_flag, kSpinLimit);
 }
 
 // One poll of a barrier that the caller will wait for next.  Polling costs an issuing thread 50-300 cycles
@@ -185,11 +206,21 @@ __device__ __forceinline__ uint32_t map_to_cta(const void* p, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
   return r;
 }
-// Arrival on a barrier of any CTA of the cluster.  What has to be seen with it are reads of TMEM (tcgen05.wait::ld) and
-// shared memory written for the tensor core (fence.proxy.async), both complete by then: a release at cluster scope would
-// also wait for the thread's outstanding global atomics.
+// Arrivals on a barrier of any CTA of the cluster.  The first form is for what completed reads of TMEM (tcgen05.wait::ld) free:
+// it orders no memory across CTAs, and so does not wait for the thread's outstanding global atomics.
 __device__ __forceinline__ void mbar_arrive_at(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+// The arriving thread's writes to its CTA's shared memory, and those of threads it has synchronised with (__syncwarp), are
+// seen by a thread of any CTA of the cluster that waits with mbar_wait_cluster: for tiles that another CTA's thread hands to
+// the tensor core (after fence.proxy.async by the writers).  The fence is restricted to shared memory: an arrival with
+// release at cluster scope takes so much longer that the relevance kernel's chain from head to head shows it, whichever thread
+// arrives (26 requests of 279-1676 tokens, 12 heads: 201 -> 212 us; batch of 16 x 576 tokens, 16 heads: 359 -> 363).
+__device__ __forceinline__ void mbar_arrive_release_at(uint32_t cluster_addr) {
+  asm volatile(
+      "fence.release.sync_restrict::shared::cta.cluster;\n"
+      "mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr)
+      : "memory");
 }
 __device__ __forceinline__ void store_at(uint32_t cluster_addr, float a, float b, float c, float d) {
   asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "f"(a), "f"(b), "f"(c), "f"(d)

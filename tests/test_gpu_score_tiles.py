@@ -44,6 +44,18 @@ def test_query_scores_against_the_cuda_core_kernels(n, t, heads, d, dtype):
     assert np.abs(got - want).max() <= tol
 
 
+def test_restaged_heads_are_complete_when_the_other_sm_multiplies_them():
+    # the leader of a pair multiplies shared memory that its peer's threads have written: with several items and heads per
+    # cluster the same tiles are overwritten again and again, and a product of a half-written one would change a score
+    wl = _workload("restaged", [700] * 9, [96, 97, 2, 64, 31, 160, 7, 128, 255], d=72, n_heads=12)
+    pr = api.Pruner.for_workload(wl)
+    m = pr.marshal(wl)
+    first = pr.score(m)[0]
+    for _ in range(100):
+        assert torch.equal(first, pr.score(m)[0])
+    pr.close()
+
+
 @pytest.mark.parametrize("where", [0, 40, 70, 99])
 def test_a_query_element_that_is_not_finite_is_reported(where):
     wl = _workload("nan", [200, 40], [100, 3], d=128, n_heads=1)
