@@ -88,11 +88,13 @@ typedef struct {
                              M <= 16384 and B_vis <= 8192 per request                              */
   int ritz_window;     /* basis vectors above the cut at r that take part in the final Rayleigh-Ritz
                           step together with the eig_oversample ones below it (default 16; >= p: all) */
-  int activity_overlap; /* > 0: while Eq. 10 runs on the tensor cores (which leaves HBM idle), Eq. 11
-                          streams the snapshot stack on a second stream of the context with at least this
-                          many 512-thread blocks per SM (1 or 2; default 1: two where one would take longer
-                          than Eq. 10), joined before Eq. 12; 0: the two
-                          scores are computed one after the other on the caller's stream           */
+  int activity_overlap; /* where Eq. 11 runs while Eq. 10 is on the tensor cores with heads, whose kernel leaves HBM
+                          idle.  1 (default): on a second stream of the context beside Eq. 10, joined before Eq. 12,
+                          with as many warps per SM as let it end before Eq. 10 does, or, where that is estimated to
+                          be faster (a long stack and few heads), after Eq. 10 on the caller's stream; 2: always
+                          beside, with 32 warps per SM; 0: always after.  With the identity embedding on the
+                          tensor cores any value > 0 runs it on the second stream after the first kernel.  The
+                          scores are the same bits in all forms                                        */
   float conv_tol;      /* the subspace iteration behind Eq. 14 runs a fixed number of steps; after the
                           last one the library estimates, from the Ritz values, how far the energies
                           can still be from those of the exact truncated SVD (relative to the largest

@@ -676,14 +676,28 @@ int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cud
 }
 
 // ---- Eq. 10-12 -------------------------------------------------------------------------------
-// Estimates for the choice between the forms of Eq. 11: the snapshot stack by one background block per SM (1.8 TB/s) and the
-// relevance kernel (1.1 PFLOP/s).
-struct ActivityTimes { double stream_s, kernel_s; };
-ActivityTimes activity_times(const covspec_ctx* ctx) {
+// Where Eq. 11 runs with activity_overlap = 1: after the relevance kernel at the full rate of activity_kernel, or beside it
+// with `warps` warps per SM (activity_stream_kernel).
+//
+// After: 6.3 TB/s (5.0 with more than four layers, no better than beside with more than eight), and the relevance
+// kernels alone before it, which take about what reading X takes, 12 us and half of their products' time.  Beside: 4.25 (4.0) TB/s
+// and nothing else, as long as the products take less.  So a long stack beside few heads goes after (8 requests of 4000 tokens,
+// d = 3584, 1 head: 4 layers 265 us after, 287 beside; 8 layers 490 and 524), with 3 heads beside (312 and 287).  float32 inputs
+// are split beside the stream and gain nothing after (671 and 673).
+//
+// Warps: enough to end at 70 % of the relevance kernel's time (1.1 PFLOP/s).  More of them only take its bandwidth and power
+// early; at 125 % the stream ends last (video 3480 -> 4020 us a call, 24 requests of 61,505 tokens in all 1073 -> 1225).
+struct ActivityPlan { bool beside; int warps; };
+ActivityPlan plan_activity(const covspec_ctx* ctx) {
   const covspec_config& cfg = ctx->cfg;
-  const double rows = (double)ctx->plan.total_vis;
-  return ActivityTimes{(cfg.act_layers + 1) * rows * cfg.d * ctx->esize / 1.8e12,
-                       2.0 * rows * (ctx->split_tc ? ctx->d3 : cfg.d) * ctx->P / 1.1e15};
+  const double rows = (double)ctx->plan.total_vis, x_bytes = rows * cfg.d * ctx->esize, bytes = (cfg.act_layers + 1) * x_bytes;
+  const int width = (cfg.n_heads + 1) / 2 * 2 * ctx->hd;                  // an odd head takes the time of two
+  const double kernel_s = 2.0 * rows * (ctx->split_tc ? ctx->d3 : cfg.d) * width / 1.1e15;
+  const bool few = cfg.act_layers <= 4;
+  const double beside_s = bytes / (few ? 4.25e12 : 4.0e12), after_s = bytes / (few ? 6.3e12 : 5.0e12);
+  const bool after = !ctx->split_tc && cfg.act_layers <= 8 && beside_s > after_s + x_bytes / 5.9e12 + 12e-6 + 0.5 * kernel_s;
+  const double warps = ceil(kStreamWarps * beside_s / (0.7 * kernel_s));
+  return ActivityPlan{!after, (int)std::min((double)kStreamWarps, std::max(8.0, warps))};
 }
 
 // Eq. 11 on `s`: the full-rate kernel, or (background = true) the small persistent grid that runs
@@ -696,20 +710,16 @@ int launch_activity(covspec_ctx* ctx, const covspec_problem* p, float* s_act, bo
   LayerPtrs lp{};
   for (int l = 0; l <= cfg.act_layers; ++l) lp.h[l] = p->Hs[l];
   if (background) {
-    int per_sm = cfg.activity_overlap;
-    // One block per SM reads about 1.8 TB/s beside the relevance kernel; where that would end after the
-    // kernel a second one is added (batch of 16 x 576 tokens, d = 2048: 115 -> 71 us).
-    // Where it ends before, a second block only slows the kernel down (video: 3570 -> 3940 us a call).
-    const ActivityTimes t = activity_times(ctx);
-    if (per_sm == 1 && t.stream_s > t.kernel_s) per_sm = 2;
-    if (cfg.act_layers > 8) per_sm = 1;                  // 40 registers a thread: two blocks would keep the kernel's CTA out
-    unsigned grid = (unsigned)std::min<long long>((rowsX + 15) / 16, (long long)ctx->num_sms * per_sm);
-    if (cfg.act_layers <= 4)
-      activity_stream_kernel<T, 4><<<grid, 512, 0, s>>>(lp, cfg.act_layers, rowsX, cfg.d, s_act);
-    else if (cfg.act_layers <= 8)
-      activity_stream_kernel<T, 8><<<grid, 512, 0, s>>>(lp, cfg.act_layers, rowsX, cfg.d, s_act);
-    else
-      activity_stream_kernel<T, 16><<<grid, 512, 0, s>>>(lp, cfg.act_layers, rowsX, cfg.d, s_act);
+    const int warps = cfg.activity_overlap == 2 ? kStreamWarps : plan_activity(ctx).warps;
+    // two iterations in flight where every lane has the same number of them (else the lanes part ways in the last pair)
+    auto launch = [&](void (*kernel)(LayerPtrs, int, long long, int, float*, int)) {
+      const unsigned grid = (unsigned)std::min<long long>((rowsX + warps - 1) / warps, ctx->num_sms);
+      kernel<<<grid, 32 * kStreamWarps, 0, s>>>(lp, cfg.act_layers, rowsX, cfg.d, s_act, warps);
+    };
+    const bool even = cfg.d % 256 == 0;
+    if (cfg.act_layers > 8) launch(activity_stream_kernel<T, 16, 2>);
+    else if (cfg.act_layers > 4) launch(even ? activity_stream_kernel<T, 8, 2> : activity_stream_kernel<T, 8, 1>);
+    else launch(even ? activity_stream_kernel<T, 4, 2> : activity_stream_kernel<T, 4, 1>);
   } else {
     unsigned grid = (unsigned)((rowsX + 7) / 8);
     if (cfg.act_layers <= 4)
@@ -743,12 +753,7 @@ int score_impl(covspec_ctx* ctx, const covspec_problem* p, float* s_query, float
   // context's side stream (fork here, join before the scores are fused).
   // The identity kernel reads X once and is done early: the full-rate activity kernel fills the SMs it leaves.
   bool overlap = (use_tc || identity_tc) && cfg.act_layers > 0 && cfg.activity_overlap > 0;
-  // Two background blocks per SM read 3.6 TB/s, the kernel that has the GPU to itself 6.3: a long stream beside a short
-  // relevance kernel (few heads) is faster after it.  In units of stream_s the first takes 0.5 and the second 0.29.
-  if (use_tc && cfg.activity_overlap == 1) {
-    const ActivityTimes t = activity_times(ctx);
-    if (t.stream_s > 150e-6 && t.kernel_s < 0.2 * t.stream_s) overlap = false;
-  }
+  if (use_tc && cfg.activity_overlap == 1 && !plan_activity(ctx).beside) overlap = false;
   auto fork_activity = [&]() -> int {
     CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
     prof_mark(ctx, ST_ACTIVITY, 0, ctx->side);
@@ -1176,11 +1181,16 @@ int covspec_prune_init(const covspec_config* cfg, covspec_ctx** out) {
       return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                   cudaSharedmemCarveoutMaxShared) == cudaSuccess;
     };
-    ok = max_shared(activity_stream_kernel<__nv_bfloat16, 4>) && max_shared(activity_stream_kernel<__nv_bfloat16, 8>) &&
-         max_shared(activity_stream_kernel<__nv_bfloat16, 16>) && max_shared(activity_stream_kernel<float, 4>) &&
-         max_shared(activity_stream_kernel<float, 8>) && max_shared(activity_stream_kernel<float, 16>) &&
+    auto streams = [&](auto* tag) {
+      using T = std::remove_pointer_t<decltype(tag)>;
+      return max_shared(activity_stream_kernel<T, 4, 1>) && max_shared(activity_stream_kernel<T, 4, 2>) &&
+             max_shared(activity_stream_kernel<T, 8, 1>) && max_shared(activity_stream_kernel<T, 8, 2>) &&
+             max_shared(activity_stream_kernel<T, 16, 2>);
+    };
+    ok = streams((__nv_bfloat16*)nullptr) && streams((float*)nullptr) &&
          max_shared(activity_kernel<__nv_bfloat16, 4>) && max_shared(activity_kernel<__nv_bfloat16, 8>) &&
-         max_shared(activity_kernel<__nv_bfloat16, 16>);      // beside the identity kernel
+         max_shared(activity_kernel<__nv_bfloat16, 16>) &&    // beside the identity kernel
+         max_shared(split3_kernel);                           // before the stream on the same SMs, which then keeps its split
   }
   if (ok) {
     // tensor maps over the workspace arrays of the subspace iteration (fixed for the context)

@@ -47,6 +47,9 @@ namespace tc {
 constexpr int kVisRing = 128 * 1024;
 constexpr int kVisMaxStages = 8;
 constexpr int kVisThreads = 384;
+// Bounds for 64 registers a thread: 24,576 of the SM's 65,536, which is what a block of the activity stream leaves (score_kernels.cuh).
+// The kernel takes 62 without spills; with 80 it is 0 to 3 % faster by itself, and no stream block of enough warps fits beside it.
+constexpr int kVisMaxThreads = 512;
 constexpr int kVisEpiWarps = 8;
 constexpr int kVisHeadBytes = kHeadDim / 2 * kBK * 2;      // 8 KB: this CTA's half of a head's weight chunk
 constexpr int kLogitN = 128;                              // query elements per logits tile (UMMA N of the 2nd product)
@@ -121,7 +124,7 @@ struct VisParams {
   int* status;
 };
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kVisThreads, 2)   // (80 registers: see kVisThreads)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kVisMaxThreads, 2)
 relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d]
                      const __grid_constant__ CUtensorMap map_w,   // Wk: [P, d]
                      const __grid_constant__ CUtensorMap map_q,   // Qn hi: [sum T, P]

@@ -131,27 +131,31 @@ __device__ __forceinline__ void load8_stream(const __nv_bfloat16* p, float (&v)[
   v[6] = __uint_as_float(t.w << 16); v[7] = __uint_as_float(t.w & 0xffff0000u);
 }
 
-// Eq. 11 as a background stream: the same arithmetic as activity_kernel, but a small persistent
-// grid (one or two blocks per SM, rows handed out round-robin) whose loads bypass L1 and are marked
-// evict-first in L2.  Few blocks matter: every resident block reserves 1 KB of the SM's shared
-// memory, and the relevance kernel's CTA fits beside at most two of them, of 32 registers a thread (two blocks of 40 registers,
-// as six layers took with two iterations in flight, keep that CTA out until the stream has ended: 12 requests of 2987-5975
-// tokens, d = 3936, 1244 us a call with a smaller CTA, 1510 with this one).  The fused call runs it beside the tensor-core relevance kernel, which leaves
-// HBM almost idle and most issue slots free: at a fraction of the HBM rate the whole snapshot stack
-// is read before the relevance kernel ends, without evicting the operand tiles that kernel re-reads
-// from L2.
-template <typename T, int MAXL>
-__global__ void __launch_bounds__(512, MAXL <= 8 ? 4 : 3)
+// Eq. 11 as a background stream: the same arithmetic as activity_kernel, but a persistent grid of one block per SM whose
+// first `block_warps` warps work (rows handed out round-robin), with loads that bypass L1 and are marked evict-first in L2.
+// The score runs it beside the tensor-core relevance kernel, which leaves HBM almost idle and most issue slots free: at a
+// fraction of the HBM rate the whole snapshot stack is read before the relevance kernel ends, without evicting
+// the operand tiles that kernel re-reads from L2.
+//
+// One block of 1024 threads and 40 registers a thread: it fits beside a CTA of the relevance kernel (24,576 registers, see
+// there) and never beside another one of its own.  Smaller blocks gather where the query embedding leaves SMs free, three or
+// four on one, and the relevance kernel's CTAs cannot start there before the stream has ended: with two blocks of 512
+// threads, calls back to back, 12 heads, d = 2048: 16 x 576 tokens and six layers 124 us a call, 96 now; 10 x 1640
+// tokens and ten layers 359 and 230; 8 x 4000 tokens, d = 3584, four layers 517 and 390.
+constexpr int kStreamWarps = 32;
+template <typename T, int MAXL, int UNROLL>
+__global__ void __maxnreg__(40)
 activity_stream_kernel(LayerPtrs hs, int n_layers /* = act_layers */, long long rows, int d,
-                       float* __restrict__ s_act) {
-  const int lane = threadIdx.x & 31;
-  const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
-  for (long long row = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); row < rows; row += warps) {
+                       float* __restrict__ s_act, int block_warps) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp >= block_warps) return;
+  const long long warps = (long long)gridDim.x * block_warps;
+  for (long long row = (long long)blockIdx.x * block_warps + warp; row < rows; row += warps) {
     float acc[MAXL];
 #pragma unroll
     for (int l = 0; l < MAXL; ++l) acc[l] = 0.f;
     size_t base = (size_t)row * d;
-#pragma unroll (MAXL <= 4 ? 2 : 1)
+#pragma unroll UNROLL
     for (int k = lane * 8; k < d; k += 256) {
       float prev[8], cur[8];
       load8_stream(reinterpret_cast<const T*>(hs.h[0]) + base + k, prev);

@@ -88,7 +88,8 @@ def test_more_row_tiles_per_cta_than_are_looked_up_in_advance():
 
 
 @pytest.mark.parametrize("layers,n,d", [(4, 16384, 2048),      # long enough for the stream to follow the relevance kernel
-                                        (10, 700, 256), (6, 3000, 1024), (4, 300, 264)])
+                                        (10, 700, 256), (6, 3000, 1024), (4, 300, 264), (1, 5, 64), (8, 4800, 1336),
+                                        (16, 129, 520)])
 def test_activity_is_the_same_wherever_it_runs(layers, n, d):
     wl = _workload("activity", [n], [9], d=d, n_heads=1, act_layers=layers)
     got = []
