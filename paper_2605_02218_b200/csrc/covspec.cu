@@ -71,6 +71,7 @@ struct Plan {
   int tile_ctas = 0, servers = 0;             // CTAs of the subspace kernel that carry tiles / that only factor
   int pow_grid = 0;                           // CTAs of the power step
   std::vector<int4> tile_list;                // 128-token tiles: first row of X, rows, first query row, query elements
+  int pair_queries = 0;                       // most query elements of a pair of neighbouring tiles (of one request or two)
   std::vector<int> sched;                     // [pow_grid + 1] offsets + item lists (longest first) + places (see FusedParams)
   bool one_request_ctas = false;              // no CTA of the subspace kernel carries tiles of two requests
   long long total_vis = 0, total_txt = 0, total_keep = 0, total_presel = 0;
@@ -263,6 +264,11 @@ int get_plan(covspec_ctx* ctx, const covspec_problem* p, cudaStream_t stream) {
     if (r.p > pl.p_max) pl.p_max = r.p;
     if (r.m > pl.m_max) pl.m_max = r.m;
     if (r.n > n_max) n_max = r.n;
+  }
+  pl.pair_queries = 0;
+  for (int i = 0; i < pl.n_tiles; i += 2) {
+    const int4 a = pl.tile_list[i], c = pl.tile_list[std::min(i + 1, pl.n_tiles - 1)];
+    pl.pair_queries = std::max(pl.pair_queries, a.w + (a.z != c.z ? c.w : 0));
   }
   pl.total_vis = p->vis_offsets[B]; pl.total_txt = p->txt_offsets[B];
   pl.total_keep = pl.keep_offsets[B]; pl.total_presel = pl.presel_offsets[B];
@@ -633,7 +639,7 @@ int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cud
   // shorter then: 4 x 64 instead of 4 x 128 cycles of products per chunk).
   const int n_pairs = (pl.n_tiles + 1) / 2, n_clusters = ctx->num_sms / 2;
   const int vis_heads = cfg.n_heads == 1 || n_pairs * cfg.n_heads <= n_clusters ? 1 : 2;
-  const int query_rows = std::min(tc::kLogitN, (pl.t_max + 31) / 32 * 32) / 2;      // per CTA of a pair
+  const int query_rows = std::min(tc::kLogitN, (pl.pair_queries + 31) / 32 * 32) / 2;      // per CTA of a pair
   if ((st = make_map_bf16(&map_wk, Wk, P, d, vis_heads * tc::kHeadDim / 2))) return st;
   if ((st = make_map_bf16(&map_q, Q, pl.total_txt, d, tc::kTileM))) return st;
   if ((st = make_map_bf16(&map_wq, Wq, P, d, group_heads * tc::kHeadDim))) return st;

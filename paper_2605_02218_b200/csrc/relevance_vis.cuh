@@ -23,8 +23,11 @@
 // nothing interleaves them but the tensor pipe; a head is restaged while the logits of the one before are read.
 // Below d = 2048 that chain is the longer one (per head 1.3 k cycles of restaging, 24 products of about 128 cycles each
 // whatever their width up to 128, the reading): 148 tiles, 16 heads, d = 256, 256 query elements 170 -> 104 us.
-// The tiles of a pair may belong to two requests (tiles are paired across the whole batch): such a pair goes
-// through the query elements of both, and each CTA looks at its own request's logits.
+// The tiles of a pair may belong to two requests (tiles are paired across the whole batch).  Their query elements are
+// neighbouring rows, so such a pair goes through them as through one request's, and each CTA looks at its own columns (512
+// requests of 100 tokens, d = 512, 8 heads, 32 and 64 query elements each: 221 and 246 us with logits tiles of one
+// request each, 164 and 191 now).  Both requests' products are computed for all 256 rows, which shows where nearly all pairs are
+// such ones and the logits are most of the work: with 256 query elements each 615 us, 602 on one SM per tile.
 //
 // Warp roles per CTA (384 threads): 0-7 epilogue (a TMEM lane = a token; warps w and w + 4 share 32 tokens, each
 // taking half of the columns), 8 TMA producer of the main ring, 9 TMEM owner and, in the leader CTA, MMA issuer of
@@ -178,12 +181,12 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
   const uint32_t tmem_base = *tmem_slot;
   const int n_clusters = gridDim.x >> 1, cluster_id = blockIdx.x >> 1;
 
-  // Item -> this CTA's tile rows, first head and heads of the group, and the query rows of the pair's requests (one
-  // segment, or two where the tiles belong to different requests); every role walks the same list.
+  // Item -> this CTA's tile rows, first head and heads of the group, the query rows of the pair (of one request, or of two
+  // neighbouring ones) and this CTA's own among them; every role walks the same list.
   struct Item {
     int row0, nrows, head0, heads;
-    int txt0, T0, tiles0, txt1, T1, tiles1;    // per segment: first query row, query elements, logits tiles (0: no segment)
-    int mine;                              // this CTA's segment
+    int txt0, T, tiles;                    // first query row, query elements, logits tiles of the pair
+    int own0, own1;                        // this CTA's query elements
   };
   auto decode = [&](int item) {
     Item it;
@@ -192,20 +195,18 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
     it.heads = min(prm.group_heads, prm.n_heads - it.head0);
     const int4 a = prm.tiles[2 * pair], b = prm.tiles[min(2 * pair + 1, prm.n_tiles - 1)];
     const bool two = a.z != b.z;           // requests (each has query rows of its own)
-    it.txt0 = a.z; it.T0 = a.w; it.tiles0 = (a.w + kLogitN - 1) / kLogitN;
-    it.txt1 = b.z; it.T1 = b.w; it.tiles1 = two ? (b.w + kLogitN - 1) / kLogitN : 0;
-    it.mine = rank != 0 && two ? 1 : 0;
+    it.txt0 = a.z;
+    it.T = a.w + (two ? b.w : 0);
+    it.tiles = (it.T + kLogitN - 1) / kLogitN;
+    it.own0 = two && rank != 0 ? a.w : 0;
+    it.own1 = two && rank == 0 ? a.w : it.T;
     const bool exists = 2 * pair + (int)rank < prm.n_tiles;      // no tile: all rows read as zeros
     it.row0 = exists ? (rank != 0 ? b.x : a.x) : prm.rows_total;
     it.nrows = exists ? (rank != 0 ? b.y : a.y) : 0;
     return it;
   };
-  // Logits tile i of an item: its segment, first query element in it and width (a multiple of 32)
-  auto logits_tile = [&](const Item& it, int i, int& seg, int& j0, int& width) {
-    seg = i >= it.tiles0 ? 1 : 0;
-    j0 = (seg ? i - it.tiles0 : i) * kLogitN;
-    width = min(kLogitN, ((seg ? it.T1 : it.T0) - j0 + 31) & ~31);
-  };
+  // Width of logits tile i of an item (a multiple of 32)
+  auto logits_width = [&](const Item& it, int i) { return min(kLogitN, (it.T - i * kLogitN + 31) & ~31); };
   const int stage_bytes = kBytesA + prm.group_heads * kVisHeadBytes;
   const int q_bytes = prm.query_rows * kHalf * 2, q_slots = min(kMaxQuerySlots, kQueryRing / q_bytes);
 
@@ -215,7 +216,7 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
       int s = 0;
       uint32_t ph = 1;
       bool ok = true;
-            for (int item = cluster_id; item < prm.n_items && ok; item += n_clusters) {
+      for (int item = cluster_id; item < prm.n_items && ok; item += n_clusters) {
         const Item it = decode(item);
         // the CTA's half of the group's features (a lone last head: 64 of the 128 rows are used)
         const int wrow = it.head0 * kHeadDim + (int)rank * it.heads * (kHeadDim / 2);
@@ -267,19 +268,17 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
       bool ok = true;
       for (int item = cluster_id; item < prm.n_items && ok; item += n_clusters, ++n) {
         const Item it = decode(item);
-        const int ntt = it.tiles0 + it.tiles1;
+        const int ntt = it.tiles;
         for (int h = 0; h < it.heads && ok; ++h, ++head_it) {
           if (!(ok = mbar_wait_cluster(kp_ready, head_it & 1u, abort_flag))) break;      // both CTAs have restaged this head
           const uint32_t kp_addr = smem_u32(kp_smem);
           const uint32_t d_col = tmem_base + (n & 1u) * kTileN + h * kHeadDim;
           for (int i = 0; i < ntt && ok; ++i, ++lt) {
-            int seg, j0, width;
-            logits_tile(it, i, seg, j0, width);
             // the tile before the last has been read (its barrier is used again), and within a head the last one
             // too: it lies in the same columns
             if (lt >= 2 && !(ok = mbar_wait(&logit_empty[lt & 1u], ((lt - 2) >> 1) & 1u, abort_flag))) break;
             if (i > 0 && !(ok = mbar_wait(&logit_empty[(lt - 1) & 1u], ((lt - 1) >> 1) & 1u, abort_flag))) break;
-            const uint32_t idesc = umma_idesc(2 * kTileM, width);
+            const uint32_t idesc = umma_idesc(2 * kTileM, logits_width(it, i));
             // logits = sum over the two halves of Kp_hi Qn_hi^T + Kp_lo Qn_hi^T + Kp_hi Qn_lo^T
             for (int half = 0; half < 2 && ok; ++half) {
               const uint64_t hi = umma_desc(kp_addr + half * kBytesKp), lo = umma_desc(kp_addr + (2 + half) * kBytesKp);
@@ -314,12 +313,10 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
       wait_for_previous_kernel();              // the unit query elements are complete
       for (int item = cluster_id; item < prm.n_items && ok; item += n_clusters) {
         const Item it = decode(item);
-        const int ntt = it.tiles0 + it.tiles1;
+        const int ntt = it.tiles;
         for (int h = 0; h < it.heads && ok; ++h)
           for (int i = 0; i < ntt && ok; ++i) {
-            int seg, j0, width;
-            logits_tile(it, i, seg, j0, width);
-            const int y = (seg ? it.txt1 : it.txt0) + j0 + (int)rank * (width >> 1);
+            const int y = it.txt0 + i * kLogitN + (int)rank * (logits_width(it, i) >> 1);
             for (int p = 0; p < 4; ++p) {      // half, hi / lo: the order in which the logits issuer uses them
               if (!(ok = mbar_wait(&q_empty[qs], ph, abort_flag))) break;
               if (leader) mbar_expect_tx(&q_full[qs], 2 * q_bytes);
@@ -345,25 +342,25 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
       const Item it = next;
       next = decode(min(item + n_clusters, prm.n_items - 1));       // its loads are back by the time it is needed
       const uint32_t buf = n & 1u;
-      const int ntt = it.tiles0 + it.tiles1;
+      const int ntt = it.tiles;
       float best = -INFINITY, top = -INFINITY, ss = 0.f;    // top: largest product of the head so far (NaN if one is)
       bool nonfinite = false;
       ok = ok && mbar_wait(&acc_full[buf], (n >> 1) & 1u, abort_flag);
       tc_fence_after();
-      // logits tile i of head h: this thread's half of the columns
+      // logits tile i of head h: this thread's half of the CTA's own columns
       auto read_logits = [&](int h, int i) {
-        int seg, j0, width;
-        logits_tile(it, i, seg, j0, width);
         ok = ok && mbar_wait(&logit_full[lt & 1u], (lt >> 1) & 1u, abort_flag);
         tc_fence_after();
-        const int T = seg ? it.T1 : it.T0;
-        if (seg == it.mine) {
+        const int lo = max(it.own0 - i * kLogitN, 0), hi = min(it.own1 - i * kLogitN, kLogitN);
+        if (lo < hi) {
           const uint32_t cols = t_lane + buf * kTileN + h * kHeadDim;
-          const int c0 = part * (width >> 1), c_end = c0 + (width >> 1);
+          // from the 16 columns that lo lies in; the tile's width is a multiple of 32, so what is read has been written
+          const int first = lo & ~15, half = ((hi - first + 1) / 2 + 15) & ~15;
+          const int c0 = first + part * half, c_end = part ? hi : min(hi, first + half);
 #pragma unroll 1
           for (int c = c0; c < c_end; c += 32) {
             float v[32];
-            if (c_end - c >= 32) {
+            if (c_end - c > 16) {
               tmem_ld32(cols + c, v);
             } else {
               float u[16];
@@ -371,10 +368,10 @@ relevance_vis_kernel(const __grid_constant__ CUtensorMap map_x,   // X: [rows, d
 #pragma unroll
               for (int e = 0; e < 32; ++e) v[e] = e < 16 ? u[e] : -INFINITY;
             }
-            if (j0 + c + 32 > T) {
+            if (c < lo || c + 32 > hi) {
 #pragma unroll
               for (int e = 0; e < 32; ++e)
-                if (j0 + c + e >= T) v[e] = -INFINITY;
+                if (c + e < lo || c + e >= hi) v[e] = -INFINITY;
             }
 #pragma unroll
             for (int e = 0; e < 32; e += 2) top = max3_nan(top, v[e], v[e + 1]);

@@ -31,6 +31,9 @@ def _query_scores(wl, path):
     ([128 * 151 + 5], [40], 1, 64),                                 # more single-head items than clusters
     ([576], [31], 16, 2048),                                        # one item per cluster; a query tile of 31 rows
     ([700] * 9, [96, 97, 2, 64, 31, 160, 7, 128, 255], 7, 328),     # several items per cluster
+    ([100, 90, 128, 77, 5, 60], [16, 16, 1, 15, 17, 31], 2, 128),   # pairs of two requests: columns from 16, 1 and 17 on
+    ([100, 90, 128, 77, 5, 60, 9], [100, 100, 127, 2, 128, 129, 64], 3, 72),   # a request's columns in two logits tiles
+    ([60] * 160, [33] * 160, 1, 64),                                # every pair of two requests, several items per cluster
 ])
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 def test_query_scores_against_the_cuda_core_kernels(n, t, heads, d, dtype):
