@@ -7,11 +7,16 @@ when the compiled library is missing, and every call raises on a non-zero status
 from __future__ import annotations
 
 import ctypes as C
+import importlib.machinery
+import importlib.util
 import os
+import warnings
 from typing import Optional
 
 import numpy as np
 import torch
+
+from . import build as _build
 
 # COVSPEC_LIBRARY selects another build of the same library (the checked one, libcovspec_debug.so)
 _LIB_PATH = os.environ.get("COVSPEC_LIBRARY") or \
@@ -75,7 +80,7 @@ _lib = None
 
 def load_library():
     """Loads libcovspec.so (built by paper_2605_02218_b200.build).  Raises if it is missing."""
-    global _lib
+    global _lib, _native
     if _lib is not None:
         return _lib
     if not os.path.exists(_LIB_PATH):
@@ -127,7 +132,7 @@ def load_library():
     lib.covspec_profile_stage_count.argtypes = []
     lib.covspec_profile_stage_name.argtypes = [C.c_int]
     lib.covspec_profile_stage_name.restype = C.c_char_p
-    _bind_native(lib)
+    _native = _load_native(lib, _build.binding_path())
     _lib = lib
     return lib
 
@@ -135,17 +140,22 @@ def load_library():
 _native = None
 
 
-def _bind_native(lib):
-    """Loads _binding.so, the native part of this binding, and gives it the library's functions."""
-    global _native
+def _load_native(lib, path: str):
+    """The native part of the binding with the library's functions given to it, or None: the three calls that it makes
+    shorter then go through ctypes."""
+    if not os.path.exists(path):
+        return None
     try:
-        from . import _binding
+        loader = importlib.machinery.ExtensionFileLoader(__package__ + "._binding", path)
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader(loader.name, loader))
+        loader.exec_module(module)
     except ImportError as e:
-        raise RuntimeError("the native part of the binding is missing: build it with "
-                           "`python -m paper_2605_02218_b200.build`") from e
-    _binding.bind(*(C.cast(f, C.c_void_p).value for f in
-                    (lib.covspec_correct, lib.covspec_branch_candidates_host, lib.covspec_query_score_static)))
-    _native = _binding
+        warnings.warn(f"{path} does not load, calls go through ctypes (build it again with "
+                      f"`python -m paper_2605_02218_b200.build`): {e}", RuntimeWarning)
+        return None
+    module.bind(*(C.cast(f, C.c_void_p).value for f in
+                  (lib.covspec_correct, lib.covspec_branch_candidates_host, lib.covspec_query_score_static)))
+    return module
 
 
 def default_config(**overrides) -> Config:
@@ -442,14 +452,14 @@ def query_score_static(X: torch.Tensor, Q: torch.Tensor, vis_offsets, txt_offset
     allocate device memory (a serving loop with a fully committed memory pool, a process whose
     allocator belongs to another framework).  The library call itself allocates nothing; pass
     `out` (float32, one element per visual token) to keep this wrapper allocation-free as well."""
-    if _native is None:
+    if _lib is None:
         load_library()
     assert X.is_cuda and Q.is_cuda and X.is_contiguous() and Q.is_contiguous() and X.dtype == Q.dtype
     vis = np.ascontiguousarray(vis_offsets, dtype=np.int32)
     txt = np.ascontiguousarray(txt_offsets, dtype=np.int32)
     if out is None:
         out = torch.empty(int(vis[-1]), dtype=torch.float32, device=X.device)
-    st = _native.static_score(X, Q, vis, txt, out)
+    st = None if _native is None else _native.static_score(X, Q, vis, txt, out)
     if st is None:
         st = _static_score(X, Q, vis, txt, out)
     if st:
@@ -484,10 +494,10 @@ def correct(z_draft: torch.Tensor, z_target: torch.Tensor, uniforms: torch.Tenso
     """covspec_correct: gating (Eq. 16-17), acceptance probability (Eq. 5) and the residual
     correction draw (Eq. 6) for every row of two logit matrices [rows, ld] (ld >= vocab).
     Returns (margin, gate, accept, resid_mass, token) device tensors."""
-    if _native is None:
+    if _lib is None:
         load_library()
     # native: on a drafted block of a few positions the call would take longer in Python than on the device
-    got = _native.correct(z_draft, z_target, uniforms, gamma, drafted, vocab)
+    got = None if _native is None else _native.correct(z_draft, z_target, uniforms, gamma, drafted, vocab)
     if type(got) is tuple:
         return got
     if got is not None:
@@ -530,7 +540,7 @@ def branch_candidates(z_draft: torch.Tensor, fanouts, drafted: Optional[torch.Te
     lib = _lib or load_library()
     rows, ld = z_draft.shape
     off = np.empty(rows + 1, dtype=np.int32)
-    got = _native.candidates(z_draft, fanouts, off, drafted, vocab)
+    got = None if _native is None else _native.candidates(z_draft, fanouts, off, drafted, vocab)
     if isinstance(got, torch.Tensor):
         return got, off
     # fan-outs that are no list of ints, and the fan-outs and row lengths that the host-offset form does not take (-3)

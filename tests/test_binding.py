@@ -1,9 +1,49 @@
 """The native part of the Python binding: what the calls refuse, and that every form of fan-outs gives the same answer."""
+import sys
+
 import numpy as np
 import pytest
 import torch
 
-from paper_2605_02218_b200 import api, workloads
+from paper_2605_02218_b200 import api, build, workloads
+
+
+def test_the_native_part_holds_to_one_python_and_one_torch():
+    lib = api.load_library()
+    assert api._native is not None
+    path = build.binding_path()
+    assert torch.__version__ in path and sys.implementation.cache_tag in path
+    assert api._load_native(lib, path.replace("torch-", "torch-0")) is None       # another version's: not there
+
+
+def test_a_native_part_that_does_not_load_is_named_and_done_without(tmp_path):
+    broken = tmp_path / "_binding.so"
+    broken.write_bytes(b"no library")
+    with pytest.warns(RuntimeWarning, match="_binding.so"):
+        assert api._load_native(api.load_library(), str(broken)) is None
+
+
+def test_a_failed_build_of_the_native_part_leaves_the_library(monkeypatch, capsys):
+    monkeypatch.setattr(build, "build_binding", lambda force=False: (_ for _ in ()).throw(RuntimeError("no Python.h")))
+    assert build.build() == build.LIB and "no Python.h" in capsys.readouterr().err
+
+
+@pytest.mark.gpu
+def test_without_the_native_part_the_calls_give_the_same(monkeypatch):
+    d = workloads.make_logits(seed=4, rows=8, vocab=40000, dtype=torch.float16, device="cuda:0")
+    wl = workloads.make_workload("static", seed=5, dtype=torch.bfloat16, batch=3, n_vis=(90, 300), n_txt=(1, 20), d=264, n_heads=0,
+                                 rank=8, keep_ratio=0.2, act_layers=0, device="cuda:0")
+
+    def calls():
+        cand, off = api.branch_candidates(d["z_draft"], [8, 5, 3, 2, 1, 0, 1, 2], d["drafted"], vocab=40000)
+        return [*api.correct(d["z_draft"], d["z_target"], d["uniforms"], 0.02, d["drafted"], vocab=40000), cand,
+                torch.from_numpy(off), api.query_score_static(wl.X, wl.Q, wl.vis_offsets, wl.txt_offsets)]
+    want = calls()
+    monkeypatch.setattr(api, "_native", None)
+    for a, b in zip(want, calls()):
+        assert torch.equal(a, b)
+    with pytest.raises(TypeError):
+        api.correct(d["z_draft"], d["z_target"], d["uniforms"].double(), 0.02)
 
 
 def test_correct_refuses_what_it_does_not_take():
