@@ -38,11 +38,11 @@ import torch
 from paper_2605_02218_b200 import workloads
 
 # dram__bytes_read.sum + dram__bytes_write.sum of the visual-side relevance kernel from one ncu
-# capture on c5 cut to one request (16384 tokens: 148.6 MB, of which the 25.7 MB of projection
+# capture on c5 cut to one request (16384 tokens: 148.7 MB, of which the 25.7 MB of projection
 # weights are read once per launch and the rest grows with the tokens), scaled to the tokens one
 # launch of the full workload processes; see the summary named here.
-NCU_RELEVANCE_TRAFFIC = {"bytes_per_token": (148.589e6 - 25.69e6) / 16384, "fixed_bytes": 25.69e6, "config": "c5",
-                         "source": "profiles/relevance_tc_kernel_c5_one_request.md"}
+NCU_RELEVANCE_TRAFFIC = {"bytes_per_token": (148.652e6 - 25.69e6) / 16384, "fixed_bytes": 25.69e6, "config": "c5",
+                         "source": "profiles/relevance_vis_kernel_one_request.md"}
 NCU_CORRECT_BYTES_PER_ROW = 366.5e6 / 512          # profiles/correct_kernel_vocab152k.md
 
 METRIC = "visual_tokens_pruned_per_s"

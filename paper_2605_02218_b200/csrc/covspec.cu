@@ -618,7 +618,7 @@ int launch_identity_tc(const void* X, const void* Q, long long rows_x, long long
   return COVSPEC_OK;
 }
 
-// Eq. 10 on the tensor cores: query embedding (MODE 1), -inf fill, fused projection + cosine max.
+// Eq. 10 on the tensor cores: query embedding, which also fills the scores with -inf, then the fused projection + cosine max.
 int relevance_tc(covspec_ctx* ctx, const covspec_problem* p, float* s_query, cudaStream_t s) {
   const covspec_config& cfg = ctx->cfg;
   const Plan& pl = ctx->plan;

@@ -29,8 +29,8 @@ constexpr int kBytesKp = kTileM * kHalf * 2;       // 16 KB: [128 x 64] of one h
 constexpr int kTmemCols = 512;
 constexpr int kQueryStages = 4;        // of two heads (48 KB); six of one
 constexpr int kQueryMaxStages = kQueryStages * kBytesStage / (kBytesA + kHeadDim * kBK * 2);
-// As much shared memory as the visual side takes, although 193 KB would do: with more room the blocks of the
-// activity stream gather on few SMs, and the visual side's CTAs do not fit there until the stream has ended.
+// 193 KB would do.  A little more than the visual side's 222 KB, so that what finds room beside one finds room beside the other:
+// with smaller blocks of the activity stream than today's one per SM, more room made those gather on few SMs.
 constexpr int kQuerySmem = 225 * 1024;
 static_assert(kQueryStages * kBytesStage + 1024 <= kQuerySmem, "ring and barriers");
 
@@ -89,16 +89,16 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
       prm.fill[i] = -INFINITY;
   }
 
-  // Epilogue of one head: unit-length bf16 slices (hi and lo) of the tile's projected query elements; load gives 32
-  // features of the thread's row.
+  // Epilogue of one head: unit-length bf16 slices (hi and lo) of the tile's projected query elements, which lie from
+  // column `cols` of TMEM on.
   const int r = (warp & 3) * 32 + lane;                    // row inside the tile = TMEM lane
   const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-  auto store_head = [&](int row0, int nrows, int head, auto&& load) {
+  auto store_head = [&](int row0, int nrows, int head, uint32_t cols) {
     float ss = 0.f;
 #pragma unroll 1
     for (int c4 = 0; c4 < 4; ++c4) {
       float v[32];
-      load(c4, v);
+      tmem_ld32(cols + c4 * 32, v);
 #pragma unroll
       for (int e = 0; e < 32; ++e) ss += v[e] * v[e];
     }
@@ -108,7 +108,7 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
 #pragma unroll 1
     for (int c4 = 0; c4 < 4; ++c4) {
       float v[32];
-      load(c4, v);
+      tmem_ld32(cols + c4 * 32, v);
       if (r < nrows) {
         __nv_bfloat16* dst = prm.qn_out + (size_t)(row0 + r) * prm.P + (size_t)head * kHeadDim + c4 * 32;
 #pragma unroll
@@ -189,8 +189,7 @@ query_embed_kernel(const __grid_constant__ CUtensorMap map_a,   // Q: [rows, d]
       tc_fence_after();
       const int heads = min(prm.group_heads, prm.n_heads - head0);
       for (int h = 0; h < heads; ++h)
-        store_head(row0, rem < kTileM ? (int)rem : kTileM, head0 + h,
-                   [&](int c4, float (&v)[32]) { tmem_ld32(t_lane + buf * kTileN + h * kHeadDim + c4 * 32, v); });
+        store_head(row0, rem < kTileM ? (int)rem : kTileM, head0 + h, t_lane + buf * kTileN + h * kHeadDim);
       tc_fence_before();
       mbar_arrive(&acc_empty[buf]);
     }

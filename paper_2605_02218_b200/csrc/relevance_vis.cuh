@@ -12,10 +12,11 @@
 // so the projected embeddings never leave the SM.
 //
 // Why two SMs: a CTA fetches its own tokens and only its half of the weights, 32 KB per 64 features and 512 tensor
-// cycles.  The time of a chunk follows what shared memory writes and reads for it (128 bytes a cycle), whatever the depth
-// of the ring: 96 KB for the 128 x 256 products of one SM, 786 cycles measured, about 80 KB here, 725-750 (the tensor pipe is
-// busy 76 % of the time; 16,384 tokens, d = 3584, 28 heads: 308 us).  Under the power limit of long runs the kernel went
-// from 1.35 to 1.42 PFLOP/s.  The query elements are shared the same way.
+// cycles.  Measured per chunk, whatever the depth of the ring: 786 cycles for the 128 x 256 products of one SM, which write and
+// read 96 KB of shared memory (768 cycles at 128 bytes a cycle); 725-750 here with about 80 KB (640), of which some
+// 100 are not explained (the tensor pipe is busy 76 % of the time; 16,384 tokens, d = 3584, 28 heads: 308 us).  Under the power
+// limit of long runs the kernel went from 1.35 to 1.42 PFLOP/s, the three hi and lo products of the logits counted.  The
+// query elements are shared the same way.
 //
 // The second product and the epilogue of one item run beside the main loop of the next: TMEM holds two
 // accumulators of 256 columns, and the logits of a head take the place of that head's own columns, which have

@@ -266,13 +266,14 @@ __device__ __forceinline__ void factor_diag_thread(double* D, const double* d0, 
 constexpr int kEpiThreads = 256;         // warps 0-7
 
 // What the kernel needs to know of a tile.  Every role looks its tiles up once per step; the search through the requests is a
-// chain of loads that the acquiring loads of the counters send to L2 each time (64 requests: 5 k cycles a tile and step
+// chain of loads that the acquiring loads of the counters send to L2 each time (64 requests: 3.3 k cycles a tile and step
 // in the epilogue alone), so a CTA's first kCachedTiles tiles are looked up once per launch.
 struct TileItem {
   int b, tile;              // request, tile of the request
   int m, p, r, win, presel_off, ptile_off;
 };
 constexpr int kCachedTiles = 16;
+static_assert(8 * 8 + 8 * 4 + sizeof(TileItem) * kCachedTiles <= 1024, "barriers, single words and tiles lie in the last KB of the tail");
 
 // The part behind the ring: the triangular factor, its reciprocal diagonal (a scratch array of p floats
 // while a factor is being made), barriers, then single words.

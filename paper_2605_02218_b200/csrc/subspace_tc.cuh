@@ -104,8 +104,8 @@ struct GramParams {
   int split;            // CTAs that share an item's columns (1, 2 or 4; more than 1: one item per CTA)
   int* status;
 };
-// The time of a chunk follows the traffic of shared memory, 128 bytes a cycle: it is written once and its operands are read
-// once per product (one 128 x 128 item: 64 KB, 508 cycles, with two ring stages or six).  Where a call has few items, 2 or 4
+// A chunk is written to shared memory once and its operands are read once per product, 64 KB for one 128 x 128 item, 512
+// cycles at 128 bytes a cycle: 508 measured (within the error of the clock), with two ring stages or six.  Where a call has few items, 2 or 4
 // CTAs take the columns of one between them, each with the whole row tile: 64 and 48 KB per chunk instead of 96 for a
 // 128 x 256 block (one float32 request 20.4 -> 16.0 us, one bf16 request 16.1 -> 11.7, 16 requests of 288 rows
 // 24.2 -> 20.2).  Every element is still summed by one accumulator in the order of the inner dimension.

@@ -222,10 +222,6 @@ __device__ __forceinline__ void mbar_arrive_release_at(uint32_t cluster_addr) {
       "mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr)
       : "memory");
 }
-__device__ __forceinline__ void store_at(uint32_t cluster_addr, float a, float b, float c, float d) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "f"(a), "f"(b), "f"(c), "f"(d)
-               : "memory");
-}
 
 // Self-test of the bounded wait: one thread waits on a barrier that nothing signals; the wait gives
 // up after `limit` polls and the time-out is recorded in the status word, exactly as the kernels do.

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2605_02218_b200 import workloads
+from paper_2605_02218_b200 import api, workloads
 from tests import parity
 
 pytestmark = pytest.mark.gpu
@@ -79,10 +79,16 @@ def test_zero_token_on_the_tensor_core_path():
 
 @pytest.mark.parametrize("kw", [SMALL[2], SMALL[7]], ids=lambda kw: f"seed{kw['seed']}")
 def test_two_sm_relevance_kernel(kw):
-    # relevance_path = 2: the cta_group::2 form of the relevance kernel (pairs of token tiles on pairs
-    # of SMs) gives the same scores; ragged sizes, an odd number of tiles, more than 256 query elements
+    # the relevance kernel (pairs of token tiles on pairs of SMs) at ragged sizes, an odd number of tiles, more than
+    # 256 query elements; relevance_path = 2, which once chose it, is still taken and gives the same bits as 0
     wl = workloads.make_workload(f"pair{kw['seed']}", **kw)
     _report(wl.name, parity.run_gpu(wl, pruner_kw=dict(relevance_path=2)))
+    got = []
+    for path in (0, 2):
+        pr = api.Pruner.for_workload(wl.to("cuda:0"), relevance_path=path)
+        got.append(pr.score(pr.marshal(wl.to("cuda:0")))[0].clone())
+        pr.close()
+    assert torch.equal(*got)
 
 
 @pytest.mark.parametrize("d", [136, 1104])

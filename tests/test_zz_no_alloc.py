@@ -64,6 +64,57 @@ def test_static_query_score_matches_context_entry_point_twice_in_a_row():
 
 
 @pytest.mark.gpu
+def test_static_calls_back_to_back_and_in_a_graph():
+    """A call's first kernel comes up while the call before it still runs, over one scratch array: calls on different inputs with
+    nothing between them give what each gives alone, and so do calls in a captured graph, behind another kernel, a copy and
+    a fork of streams, which a launch of that kind cannot overlap."""
+    from paper_2605_02218_b200 import api, build
+    build.build()
+    wls = [workloads.make_workload("static", n_heads=0, rank=8, keep_ratio=0.2, act_layers=0, dtype=torch.bfloat16, seed=50 + i, **kw)
+           .to("cuda:0") for i, kw in enumerate([dict(batch=5, n_vis=(90, 700), n_txt=(1, 50), d=264),
+                                                 dict(batch=70, n_vis=(20, 150), n_txt=(1, 9), d=512),      # several launches
+                                                 dict(batch=1, n_vis=(576, 576), n_txt=(32, 32), d=1024)])]
+    run = lambda wl, out: api.query_score_static(wl.X, wl.Q, wl.vis_offsets, wl.txt_offsets, out=out)
+    want = []
+    for wl in wls:
+        want.append(run(wl, torch.full((wl.total_vis,), float("nan"), device="cuda:0")).clone())
+        torch.cuda.synchronize()
+    order = [0, 1, 2, 2, 0, 1, 0, 2, 1, 1] * 5
+    outs = [torch.full((wls[i].total_vis,), float("nan"), device="cuda:0") for i in order]
+    torch.cuda.synchronize()
+    for i, out in zip(order, outs):
+        run(wls[i], out)
+    torch.cuda.synchronize()
+    assert all(torch.equal(want[i], out) for i, out in zip(order, outs))
+
+    got = [torch.empty_like(w) for w in want] * 2
+    got = [t.clone() for t in got]
+    stage = torch.empty_like(wls[1].X)
+    side = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        run(wls[0], got[0])                                   # first node
+        run(wls[2], got[2])                                   # behind a call
+        stage.copy_(wls[1].X)
+        run(wls[1], got[1])                                   # behind a copy
+        got[3].zero_()
+        run(wls[0], got[3])                                   # behind a fill
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            got[5].zero_()
+        got[4].zero_()
+        torch.cuda.current_stream().wait_stream(side)
+        run(wls[2], got[5])                                   # behind a join
+        run(wls[1], got[4])
+    for _ in range(3):
+        for t in got:
+            t.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(want[i % 3], t) for i, t in enumerate(got))
+
+
+@pytest.mark.gpu
 def test_static_entry_point_rejects_what_does_not_fit():
     from paper_2605_02218_b200 import api, build
     build.build()
