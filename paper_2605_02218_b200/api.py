@@ -16,8 +16,6 @@ from typing import Optional
 import numpy as np
 import torch
 
-from . import build as _build
-
 # COVSPEC_LIBRARY selects another build of the same library (the checked one, libcovspec_debug.so)
 _LIB_PATH = os.environ.get("COVSPEC_LIBRARY") or \
     os.path.join(os.path.dirname(os.path.abspath(__file__)), "libcovspec.so")
@@ -132,7 +130,8 @@ def load_library():
     lib.covspec_profile_stage_count.argtypes = []
     lib.covspec_profile_stage_name.argtypes = [C.c_int]
     lib.covspec_profile_stage_name.restype = C.c_char_p
-    _native = _load_native(lib, _build.binding_path())
+    from .build import binding_path
+    _native = _load_native(lib, binding_path())
     _lib = lib
     return lib
 
